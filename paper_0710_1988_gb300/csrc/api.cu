@@ -133,6 +133,7 @@ extern "C" int wd_create(const int lat[4], const void *links, double kappa, doub
   h->prof.d_sites = nullptr;
   h->links32 = nullptr;
   h->links16 = nullptr;
+  h->links_fx = nullptr;
   h->mixed_bits = 32;
   h->mixed_delta = 0.0;
   h->mixed_inner_max = 300;
@@ -162,6 +163,7 @@ extern "C" int wd_create(const int lat[4], const void *links, double kappa, doub
   if (e == cudaSuccess) e = cudaMemset(h->prof.d_sites, 0, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess)
     e = cudaMemcpy(h->links, links, sizeof(double2) * 36 * V, cudaMemcpyDefault);
+  if (e == cudaSuccess) e = fx_links_create(h);
   if (e == cudaSuccess) {
     cudaMemPoolProps props;
     std::memset(&props, 0, sizeof(props));
@@ -173,10 +175,20 @@ extern "C" int wd_create(const int lat[4], const void *links, double kappa, doub
       uint64_t thr = UINT64_MAX;
       e = cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
+    // the scratch of one operator product, mapped here and not in the first call
+    void *p = nullptr;
+    if (e == cudaSuccess && h->links_fx != nullptr) {
+      if (cudaMallocFromPoolAsync(&p, 200 * (size_t)V, h->pool, 0) == cudaSuccess) {
+        cudaFreeAsync(p, 0);
+        cudaStreamSynchronize(0);
+      }
+      cudaGetLastError();
+    }
   }
   if (e != cudaSuccess) {
     int rc = cuda_fail(e, "wd_create");
     if (h->links) cudaFree(h->links);
+    if (h->links_fx) cudaFree(h->links_fx);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     h->prof.destroy();
     delete h;
@@ -253,6 +265,7 @@ extern "C" void wd_destroy(wd_handle h) {
   if (h->ev_in) cudaEventDestroy(h->ev_in);
   if (h->ev_out) cudaEventDestroy(h->ev_out);
   if (h->links) cudaFree(h->links);
+  if (h->links_fx) cudaFree(h->links_fx);
   if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
 }

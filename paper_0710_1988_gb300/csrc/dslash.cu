@@ -17,6 +17,7 @@
 #include "cplx.cuh"
 #include "wd_internal.h"
 #include "kernels.cuh"
+#include "fx.cuh"
 #include "spin.cuh"
 
 namespace wd {
@@ -199,6 +200,254 @@ wilson_f64_kernel(const double2 *__restrict__ links, const double2 *__restrict__
   }
 }
 
+// ----------------------------------------------------------------- fixed-point form
+
+// Links -> fixed-point slices [tile][mu][entry][32], sites parity by parity
+// when all extents are even (g.split), and a check that every link may be used
+// so: entries within 1 in modulus (to rounding) and every row and column
+// summing to between 0.5 and 2.5 in |re| + |im| (a 3x3 unitary matrix:
+// between 1 and sqrt(6)), which bounds the sums of fx.cuh and keeps the
+// links' own rounding below FP64's.  *bad counts links that fail.
+__global__ void __launch_bounds__(128)
+fx_links_kernel(const double2 *__restrict__ U, int4 *__restrict__ L, LatticeGeom g,
+                int *__restrict__ bad) {
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  const Nbrs32 nb = neighbours32((unsigned)s, g);
+  int4 *l = L + fx_at(g.split ? nb.par * (unsigned)(g.V / 2) + ((unsigned)s >> 1) : (unsigned)s, 36);
+  bool ok = true;
+  for (int mu = 0; mu < 4; ++mu) {
+    double row[3] = {0.0, 0.0, 0.0}, col[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double2 u = U[(s * 4 + mu) * 9 + i];
+      const double a = fabs(u.x), b = fabs(u.y);
+      ok = ok && a <= 1.0 + 0x1p-20 && b <= 1.0 + 0x1p-20 && a + b <= 1.5;   // false for NaN
+      row[i / 3] += a + b;
+      col[i % 3] += a + b;
+      const double hr = ok ? rint(u.x * 0x1p30) : 0.0, hi = ok ? rint(u.y * 0x1p30) : 0.0;
+      const double lr = ok ? rint(fma(u.x, 0x1p30, -hr) * 0x1p29) : 0.0;
+      const double li = ok ? rint(fma(u.y, 0x1p30, -hi) * 0x1p29) : 0.0;
+      l[(mu * 9 + i) * FX_TILE] = make_int4((int)hr, (int)lr, (int)hi, (int)li);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      ok = ok && row[i] >= 0.5 && row[i] <= 2.5 && col[i] >= 0.5 && col[i] <= 2.5;
+  }
+  if (!ok) atomicAdd(bad, 1);
+}
+
+// Spinors -> fixed point (fx.cuh), one thread per site and system.
+__global__ void __launch_bounds__(128)
+fx_encode_kernel(const double2 *__restrict__ in, FxVec out, long long sites, size_t tiled,
+                 const int *__restrict__ status, unsigned mask) {
+  const int r = blockIdx.y;
+  if (status != nullptr && !((mask >> status[r]) & 1u)) return;
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= sites) return;
+  double2 p[12];
+  load_spinor(in + ((long long)r * sites + s) * 12, p);
+  int e = 0;
+  unsigned long long any = 0;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    e = max(e, max(exp_bits(p[c].x), exp_bits(p[c].y)));
+    any |= (unsigned long long)(__double_as_longlong(p[c].x) | __double_as_longlong(p[c].y)) << 1;
+  }
+  const int E = fx_site_exponent(e, any == 0);
+  out.e[(long long)r * sites + s] = E;
+  int4 *o = out.v + (size_t)r * 12 * tiled + fx_at((unsigned)s, 12);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) o[c * FX_TILE] = fx_slices(p[c], max(e, 1));
+}
+
+// sum over the eight hops of one site in FP64: the sites next to a value that
+// fixed point does not hold
+template <bool DAG>
+__device__ __noinline__ void hops_f64(const double2 *__restrict__ psi,
+                                      const double2 *__restrict__ links, const Nbrs32 &nb,
+                                      long long s, double2 *acc) {
+  constexpr int F = DAG ? +1 : -1;
+  double2 t[12];
+  hop_pair<0, F, true>(psi, links, nb.up[0], s, nb.dn[0], t);
+  hop_pair<1, F, false>(psi, links, nb.up[1], s, nb.dn[1], t);
+  hop_pair<2, F, false>(psi, links, nb.up[2], s, nb.dn[2], t);
+  hop_pair<3, F, false>(psi, links, nb.up[3], s, nb.dn[3], t);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[c] = t[c];
+}
+
+// wilson_f64_kernel's result with the hops in fixed point; `in` is the
+// encoded form of in64.  A block covers 128 sites, two lanes (l, l + 16) a
+// site.  Blocks are numbered system fastest: the nrhs blocks of one range of
+// sites share its links through L2.
+constexpr int FX_SITES = 128;
+
+constexpr size_t FX_SMEM = 2 * FX_SITES / 32 * 2 * sizeof(FxStage);   // two stages a warp
+
+template <bool DAG, int EPI>
+__global__ void __launch_bounds__(2 * FX_SITES, 2)
+wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec in,
+                 const double2 *__restrict__ in64, double2 *__restrict__ out, LatticeGeom g,
+                 size_t tiled, double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
+                 double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
+                 unsigned long long *__restrict__ sites) {
+  const int r = (int)(blockIdx.x % (unsigned)nrhs);
+  const long long sb = blockIdx.x / (unsigned)nrhs;
+  if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
+  if (sites != nullptr && sb == 0 && threadIdx.x == 0)
+    atomicAdd(sites, (unsigned long long)g.V);  // work accounting for the profiler
+  const int sp = (threadIdx.x >> 4) & 1;
+  const long long at = sb * FX_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+  const bool valid = at < g.V;
+  const unsigned s = valid ? (unsigned)at : (unsigned)g.V - 1;   // idle lanes repeat the last site
+  const size_t V = (size_t)g.V;
+  const Nbrs32 nb = neighbours32(s, g);
+  const int *ev = in.e + (size_t)r * V;
+  int eu[4], ed[4], E = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    eu[m] = __ldg(ev + nb.up[m]);
+    ed[m] = __ldg(ev + nb.dn[m]);
+    E = max(E, max(eu[m], ed[m]));
+  }
+  extern __shared__ __align__(128) unsigned char fx_smem[];
+  FxStage *stage = reinterpret_cast<FxStage *>(fx_smem) + 2 * (threadIdx.x >> 5);
+  longlong2 up[3], low[3];
+  {
+    const int4 *psi = in.v + (size_t)r * 12 * tiled;
+    const unsigned half = g.split, odd = (unsigned)(g.V / 2);
+    const unsigned here = g.split ? (nb.par ? odd : 0u) + (s >> 1) : s;
+    const unsigned other = g.split && !nb.par ? odd : 0u;
+    fx_hops<(DAG ? +1 : -1)>(
+        stage, [&](int m, bool fwd) {
+          return L + fx_at(fwd ? here : other + (nb.dn[m] >> half), 36) + m * 9 * FX_TILE;
+        },
+        [&](int m, bool fwd) { return psi + fx_at(fwd ? nb.up[m] : nb.dn[m], 12); }, sp, E, eu, ed,
+        up, low);
+  }
+  // the warp's 16 sites of hop sums through shared memory, so that its reads
+  // and writes of the FP64 vectors are contiguous
+  double2 *hop = reinterpret_cast<double2 *>(stage);   // 13 a site: no bank conflicts
+  double2 *mine = hop + (threadIdx.x & 15) * 13;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    mine[3 * sp + a] = make_double2(fx_to_double(up[a].x, E), fx_to_double(up[a].y, E));
+    mine[6 + 3 * sp + a] = make_double2(fx_to_double(low[a].x, E), fx_to_double(low[a].y, E));
+  }
+  __syncwarp();
+  if (E == FX_SPECIAL && sp == 0 && valid) {
+    hops_f64<DAG>(in64 + (size_t)r * 12 * V, links, nb, s, mine);
+  }
+  __syncwarp();
+  double red[3] = {0.0, 0.0, 0.0};
+  const long long first = sb * FX_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
+  const size_t base = ((size_t)r * V + first) * 12;
+  const int count = 12 * (int)max(0LL, min(16LL, g.V - first));
+  const double tmu = DAG ? -mu : mu;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int c = q * 32 + (threadIdx.x & 31);
+    if (c < count) {
+      const double2 p = __ldg(in64 + base + c), d = hop[c + c / 12];
+      double2 v;
+      v.x = fma(-kappa, d.x, p.x);
+      v.y = fma(-kappa, d.y, p.y);
+      if (tmu != 0.0) {  // + i mu gamma5 psi, gamma5 = diag(1, 1, -1, -1)
+        const double m = c % 12 < 6 ? tmu : -tmu;
+        v.x = fma(-m, p.y, v.x);
+        v.y = fma(m, p.x, v.y);
+      }
+      out[base + c] = v;
+      if (EPI != EPI_NONE) {  // <aux, out> or <out, in>, and <out, out>
+        const double2 a = EPI == EPI_DOT ? __ldg(aux + base + c) : v;
+        const double2 b = EPI == EPI_DOT ? v : p;
+        red[0] = fma(a.x, b.x, red[0]);
+        red[0] = fma(a.y, b.y, red[0]);
+        red[1] = fma(a.x, b.y, red[1]);
+        red[1] = fma(-a.y, b.x, red[1]);
+        red[2] = fma(v.x, v.x, red[2]);
+        red[2] = fma(v.y, v.y, red[2]);
+      }
+    }
+  }
+  if (EPI != EPI_NONE) {
+    block_sum<3>(red);
+    if (threadIdx.x == 0) {
+      const long long nsb = gridDim.x / (unsigned)nrhs;
+      double *dst = partial + ((long long)r * nsb + sb) * 3;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) dst[q] = red[q];
+    }
+  }
+}
+
+// The handle's fixed-point links, or none where they do not fit fx.cuh's
+// bounds or the memory: the FP64 kernel then serves.
+cudaError_t fx_links_create(wd_context *h) {
+  h->links_fx = nullptr;
+  if (h->V >= (1LL << 31)) return cudaSuccess;
+  int *bad = nullptr, hbad = 1;
+  if (cudaMalloc(&h->links_fx, sizeof(int4) * 36 * fx_sites(h->V)) != cudaSuccess) {
+    cudaGetLastError();
+    h->links_fx = nullptr;
+    return cudaSuccess;
+  }
+  cudaError_t e = cudaMalloc(&bad, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(bad, 0, sizeof(int));
+  if (e == cudaSuccess) {
+    fx_links_kernel<<<(unsigned)((h->V + 127) / 128), 128>>>(h->links, h->links_fx, geom_of(h), bad);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
+  if (bad) cudaFree(bad);
+  if (hbad != 0) {
+    cudaFree(h->links_fx);
+    h->links_fx = nullptr;
+  }
+  return e;
+}
+
+static cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,
+                                    const int *status, unsigned mask, cudaStream_t s) {
+  fx_encode_kernel<<<dim3((unsigned)((sites + 127) / 128), nrhs), 128, 0, s>>>(in, f, sites, fx_sites(sites), status, mask);
+  return cudaGetLastError();
+}
+
+static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 *in, double2 *out,
+                                    int nrhs, int dagger, int epi, const double2 *aux,
+                                    double *partial, const int *status, cudaStream_t s,
+                                    unsigned mask, unsigned long long *cnt) {
+  const unsigned grid = (unsigned)((h->V + FX_SITES - 1) / FX_SITES) * (unsigned)nrhs;
+  const LatticeGeom g = geom_of(h);
+#define WFX(D, E)                                                                                \
+  wilson_fx_kernel<D, E><<<grid, 2 * FX_SITES, FX_SMEM, s>>>(h->links_fx, h->links, f, in, out, g,              \
+                                              fx_sites(h->V), h->kappa,                       \
+                                              h->mu, nrhs, aux, partial, status, mask, cnt)
+  static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
+  if (attr_device != h->device) {
+    const void *k[6] = {(const void *)wilson_fx_kernel<false, EPI_NONE>, (const void *)wilson_fx_kernel<false, EPI_DOT>,
+                        (const void *)wilson_fx_kernel<false, EPI_TSTT>, (const void *)wilson_fx_kernel<true, EPI_NONE>,
+                        (const void *)wilson_fx_kernel<true, EPI_DOT>, (const void *)wilson_fx_kernel<true, EPI_TSTT>};
+    for (const void *f : k) {
+      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
+      if (e != cudaSuccess) return e;
+    }
+    attr_device = h->device;
+  }
+  if (dagger) {
+    if (epi == EPI_DOT) WFX(true, EPI_DOT);
+    else if (epi == EPI_TSTT) WFX(true, EPI_TSTT);
+    else WFX(true, EPI_NONE);
+  } else {
+    if (epi == EPI_DOT) WFX(false, EPI_DOT);
+    else if (epi == EPI_TSTT) WFX(false, EPI_TSTT);
+    else WFX(false, EPI_NONE);
+  }
+#undef WFX
+  return cudaGetLastError();
+}
+
 LatticeGeom geom_of(const wd_context *h) {
   LatticeGeom g;
   for (int i = 0; i < 4; ++i) g.L[i] = h->dims[i];
@@ -210,6 +459,8 @@ LatticeGeom geom_of(const wd_context *h) {
     g.dsh[i] = 31 + l;
     g.dm[i] = (1ULL << g.dsh[i]) / d + 1;
   }
+  g.split = 1;
+  for (int i = 0; i < 4; ++i) g.split &= h->dims[i] % 2 == 0;
   return g;
 }
 
@@ -228,10 +479,24 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
                                   unsigned mask) {
   if (h->eo)  // even-odd Schur operator on even half vectors
     return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask);
-  dim3 grid(wilson_blocks(h), nrhs);
-  LatticeGeom g = geom_of(h);
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
+  if (h->links_fx != nullptr && (long long)wilson_blocks(h) * nrhs <= 0x7fffffffLL) {
+    // scratch for the encoded input, stream-ordered; without it the FP64 kernel
+    const size_t nv = (size_t)nrhs * fx_sites(h->V);
+    int4 *buf = nullptr;
+    if (cudaMallocFromPoolAsync((void **)&buf, nv * (12 * sizeof(int4) + sizeof(int)), h->pool, s) == cudaSuccess) {
+      const FxVec f{buf, reinterpret_cast<int *>(buf + 12 * nv)};
+      cudaError_t e = launch_fx_encode(in, f, h->V, nrhs, status, mask, s);
+      if (e == cudaSuccess)
+        e = launch_wilson_fx(h, f, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
+      cudaError_t e2 = cudaFreeAsync(buf, s);
+      return e != cudaSuccess ? e : e2;
+    }
+    cudaGetLastError();
+  }
+  dim3 grid(wilson_blocks(h), nrhs);
+  LatticeGeom g = geom_of(h);
   if (dagger) {
     if (epi == EPI_DOT)
       wilson_f64_kernel<true, EPI_DOT><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);

@@ -1,0 +1,261 @@
+// Block fixed point for the FP64 Wilson operator.
+//
+// This GPU issues 1.7 FP64 FMAs per clock and SM (DFMA probe), so a site
+// update's ~930 FP64 instructions take 550 clocks of its SM; integer
+// multiply-adds of 32 x 32 + 64 bits go at about 30, 32-bit integer adds at
+// 120.  The hops' products are therefore formed in integers.  A spinor site
+// (24 reals) shares the largest exponent field E of its entries and holds
+// each as X = round(x 2^(1078 - E)), |X| <= 2^56: entries down to 2^-3 of the
+// site's largest are held exactly, smaller ones to 2^-57 of it.  X is stored
+// as two signed slices, X = hi 2^29 + lo with |lo| <= 2^28, |hi| <= 2^27, so
+// that a spin projection and the sums and differences of a complex product
+// add slices without carries (|hi| <= 2^29, |lo| <= 2^30).  A link entry is
+// u = uh 2^-30 + ul 2^-59, |ul| <= 2^28.
+//
+//   u x = [uh hi + (uh lo + ul hi) 2^-29] 2^(E - 1079)  (+ ul lo 2^-58, left
+//         out: below half a unit of X)
+//
+// takes three multiply-adds per real product, exact in 64-bit sums: with
+// every row and column of a link summing to at most 2.5 in |re| + |im| (3x3
+// unitary: sqrt(6)), one hop's component is below 2.5 * 2^58 units, the sum
+// over the eight hops below 2^62.4 and the middle sums below 2^63.  A sum
+// over hops is aligned to the largest E of the neighbours and rounded once
+// to FP64 at the end.  Its error is a few units of 2^-57 of the largest
+// neighbour entry; the eight hops' FP64 roundings leave more (2-norm against
+// 64-bit torch arithmetic, whose own rounding is in both: 1.0e-16 against
+// 1.1e-16).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "spin.cuh"
+
+namespace wd {
+
+// Layout: tiles of 32 sites, [tile][component][32] (12 components of a
+// spinor, 4 x 9 entries of a site's links), so that a warp's loads of one
+// component are contiguous and the components lie at fixed offsets.
+constexpr int FX_TILE = 32;
+__device__ __forceinline__ size_t fx_at(unsigned s, unsigned comps) {
+  return (size_t)(s >> 5) * (FX_TILE * comps) + (s & 31);
+}
+inline size_t fx_sites(long long sites) { return (size_t)((sites + FX_TILE - 1) / FX_TILE * FX_TILE); }
+
+constexpr int FX_SPECIAL = 0x7fffffff;   // a site whose FP64 values must be used
+constexpr int FX_EMIN = 200, FX_EMAX = 1900;
+
+__device__ __forceinline__ int exp_bits(double x) {
+  return (__double2hiint(x) >> 20) & 0x7ff;
+}
+
+// shared exponent of a site from the largest exponent field of its entries:
+// E for values in range, 0 for a site of zeros, FX_SPECIAL for infinities,
+// NaN and magnitudes near the ends of FP64's range.  allzero: every entry is 0.
+__device__ __forceinline__ int fx_site_exponent(int emax, bool allzero) {
+  if (emax >= FX_EMIN && emax <= FX_EMAX) return emax;
+  return allzero ? 0 : FX_SPECIAL;
+}
+
+// (hi, lo) slices of x against the site exponent E >= x's own exponent field
+__device__ __forceinline__ int2 fx_slices(double x, int E) {
+  const long long b = __double_as_longlong(x);
+  const int be = (int)((unsigned long long)b >> 52) & 0x7ff;
+  const long long M = (b & 0xFFFFFFFFFFFFFLL) | (be ? 1LL << 52 : 0LL);
+  const int r = min(E - be, 62);
+  long long X = ((M << 3) + (long long)((1ULL << r) >> 1)) >> r;
+  X = b < 0 ? -X : X;
+  const int lo = ((int)(unsigned)X << 3) >> 3;       // low 29 bits, signed
+  return make_int2((int)((X - lo) >> 29), lo);
+}
+
+__device__ __forceinline__ int4 fx_slices(double2 x, int E) {
+  const int2 a = fx_slices(x.x, E), b = fx_slices(x.y, E);
+  return make_int4(a.x, a.y, b.x, b.y);
+}
+
+// T 2^(E - 1079) rounded to FP64, FX_EMIN <= E <= FX_EMAX
+__device__ __forceinline__ double fx_to_double(long long T, int E) {
+  const unsigned long long a = T < 0 ? 0ULL - (unsigned long long)T : (unsigned long long)T;
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << (lz & 63);
+  unsigned long long bits = (m >> 11) + ((m >> 10) & 1ULL) +
+                            ((unsigned long long)((unsigned)E + 6u - (unsigned)lz) << 52);
+  bits |= (unsigned long long)T & 0x8000000000000000ULL;
+  return a == 0 ? 0.0 : __longlong_as_double((long long)bits);
+}
+
+// Sums of one complex product chain U h in three real products each (Gauss):
+// with U = a + i b, h = c + i d,
+//   k1 = (a + b) c, k2 = a (d - c), k3 = b (c + d): U h = (k1 - k3) + i (k1 + k2),
+// and with a - b in k1, conj(U) h = (k1 + k3) + i (k1 + k2).  Each real product
+// adds its high part and its two middle parts.
+struct FxAcc {
+  long long h1, m1, h2, m2, h3, m3;
+};
+
+// h as (c, d - c, c + d), each (hi, lo)
+struct FxArg {
+  int2 c, m, p;
+  __device__ __forceinline__ FxArg() {}
+  __device__ __forceinline__ explicit FxArg(int4 v)
+      : c(make_int2(v.x, v.y)), m(make_int2(v.z - v.x, v.w - v.y)), p(make_int2(v.x + v.z, v.y + v.w)) {}
+};
+
+__device__ __forceinline__ void fx_mac(long long &h, long long &m, int uh, int ul, int2 x) {
+  h += (long long)uh * x.x;
+  m += (long long)uh * x.y;
+  m += (long long)ul * x.x;
+}
+
+template <bool CONJ>
+__device__ __forceinline__ void fx_cmac(FxAcc &s, int4 u, const FxArg &x) {
+  fx_mac(s.h1, s.m1, CONJ ? u.x - u.z : u.x + u.z, CONJ ? u.y - u.w : u.y + u.w, x.c);
+  fx_mac(s.h2, s.m2, u.x, u.y, x.m);
+  fx_mac(s.h3, s.m3, u.z, u.w, x.p);
+}
+
+template <bool CONJ>
+__device__ __forceinline__ longlong2 fx_value(const FxAcc &s) {   // m1 starts at 2^28: rounded
+  const long long rm = CONJ ? s.m1 + s.m3 : s.m1 - s.m3, im = s.m1 + s.m2;
+  return make_longlong2((CONJ ? s.h1 + s.h3 : s.h1 - s.h3) + (rm >> 29), s.h1 + s.h2 + (im >> 29));
+}
+
+// round((x) 2^-d) for 0 <= d <= 63, |x| < 2^62
+__device__ __forceinline__ long long fx_align(long long x, int d) {
+  return (x + (long long)((1ULL << d) >> 1)) >> d;
+}
+
+// a + f b for a factor f = 1, i, -1, -i (F = 0, 1, 2, 3), slice by slice
+template <int F>
+__device__ __forceinline__ int4 fx_add(int4 a, int4 b) {
+  if (F == 0) return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+  if (F == 1) return make_int4(a.x - b.z, a.y - b.w, a.z + b.x, a.w + b.y);
+  if (F == 2) return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+  return make_int4(a.x + b.z, a.y + b.w, a.z - b.x, a.w - b.y);
+}
+
+template <int F>
+__device__ __forceinline__ longlong2 fx_add(longlong2 a, longlong2 b) {
+  if (F == 0) return make_longlong2(a.x + b.x, a.y + b.y);
+  if (F == 1) return make_longlong2(a.x - b.y, a.y + b.x);
+  if (F == 2) return make_longlong2(a.x - b.x, a.y - b.y);
+  return make_longlong2(a.x + b.y, a.y - b.x);
+}
+
+// One hop is shared by two lanes of a warp, one per upper spin sp: with h_sp =
+// psi_sp + S (B psi)_sp the lane forms chi_sp = U h_sp and adds it to the
+// output's spin sp and, times S B^dagger, to one lower spin (spin.cuh): LOW =
+// 3 - sp for mu = x, y and 2 + sp for mu = z, t, the one its h_sp came from.
+// The factors of sp = 0 and 1 are equal (x, t) or opposite (y, z):
+//   projection, S = -1:      x: i   y: sgn   z: i sgn   t: -1    sgn = 1 - 2 sp
+//   reconstruction, S = +1:  x: i   y: -sgn  z: i sgn   t:  1
+// Splitting a site over two lanes halves its registers (128 at four warps per
+// scheduler; one lane a site spills) and its chain, and both read one link.
+template <int MU, int S>
+struct FxSpin {
+  static constexpr bool SGN = MU == 1 || MU == 2;
+  static constexpr int P0 = MU == 0 || MU == 2 ? 1 : MU == 1 ? 0 : 2;   // without sgn
+  static constexpr int R0 = MU == 0 || MU == 2 ? 1 : MU == 1 ? 2 : 0;
+  static constexpr int P = S < 0 ? P0 : (P0 + 2) & 3;
+  static constexpr int R = S > 0 ? R0 : (R0 + 2) & 3;
+};
+
+// A hop's operands staged in shared memory for the 16 sites of a warp.
+struct FxStage {
+  int4 u[9][16];      // the link's entries
+  int4 psi[12][16];   // the neighbour's components
+};
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;"
+               ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// Both lanes of a site copy its operands: l, q: the link's and the
+// neighbour's first component.
+__device__ __forceinline__ void fx_fetch(FxStage &st, const int4 *l, const int4 *q) {
+  const int site = threadIdx.x & 15, half = (threadIdx.x >> 4) & 1;
+#pragma unroll
+  for (int c = 0; c < 12; c += 2) cp_async16(&st.psi[c + half][site], q + (c + half) * FX_TILE);
+#pragma unroll
+  for (int c = 0; c < 8; c += 2) cp_async16(&st.u[c + half][site], l + (c + half) * FX_TILE);
+  if (half == 0) cp_async16(&st.u[8][site], l + 8 * FX_TILE);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The lane's part of one hop, in units 2^(Eq + d - 1079): up += chi, low +=
+// (factor without sgn) chi, low lying in the neighbour's spin cl.
+template <int MU, int S, bool ADJ>
+__device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
+                                       longlong2 (&up)[3], longlong2 (&low)[3]) {
+  using W = FxSpin<MU, S>;
+  const int site = threadIdx.x & 15, sgn = 1 - 2 * sp;
+  FxArg h[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    int4 q = st.psi[3 * cl + b][site];
+    if (W::SGN) q = make_int4(sgn * q.x, sgn * q.y, sgn * q.z, sgn * q.w);
+    h[b] = FxArg(fx_add<W::P>(st.psi[3 * sp + b][site], q));
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    FxAcc s = {0, 1LL << 28, 0, 0, 0, 0};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) fx_cmac<ADJ>(s, st.u[ADJ ? 3 * b + a : 3 * a + b][site], h[b]);
+    longlong2 chi = fx_value<ADJ>(s);
+    if (d != 0) chi = make_longlong2(fx_align(chi.x, d), fx_align(chi.y, d));
+    up[a] = fx_add<0>(up[a], chi);
+    low[a] = fx_add<W::R>(low[a], chi);
+  }
+}
+
+// The eight hops of a site for one lane: up is the sum's spin sp, low its
+// spin 2 + sp, in units 2^(E - 1079).  The next hop's operands are copied to
+// shared memory (st: two stages of this warp) while one hop is computed: the
+// copies wait for L2 and hold no registers (through L1, which serves a third
+// of them: a 10-system apply at 16^4 0.288 ms with the staging, 0.301 with
+// plain loads, 0.332 with copies past L1; the arithmetic alone 0.237).  The y and z hops come first in
+// their lower sums, whose factor sgn is then applied once; between them the
+// lanes exchange the x and y hops' lower sums, which belong to the other.
+template <int F, class LinkAt, class SiteAt>
+__device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, int sp, int E,
+                                        const int (&eu)[4], const int (&ed)[4],
+                                        longlong2 (&up)[3], longlong2 (&low)[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) up[a] = low[a] = make_longlong2(0, 0);
+#define FX_FETCH(B, M, FWD) fx_fetch(st[B], link(M, FWD), site(M, FWD));
+#define FX_READY(N)                                            \
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); \
+  __syncwarp();
+#define FX_SIGN                                                                                    \
+  if (sp) {                                                                                        \
+    _Pragma("unroll") for (int a = 0; a < 3; ++a) low[a] = make_longlong2(-low[a].x, -low[a].y);   \
+  }
+#define FX_PAIR(M, CL, NEXT, WAIT)                                      \
+  FX_FETCH(1, M, false)                                                 \
+  FX_READY(1)                                                           \
+  fx_hop<M, F, false>(st[0], sp, CL, min(E - eu[M], 63), up, low);      \
+  __syncwarp();                                                         \
+  NEXT                                                                  \
+  FX_READY(WAIT)                                                        \
+  fx_hop<M, -F, true>(st[1], sp, CL, min(E - ed[M], 63), up, low);      \
+  __syncwarp();
+  FX_FETCH(0, 1, true)
+  FX_PAIR(1, 3 - sp, FX_FETCH(0, 0, true), 1)
+  FX_SIGN
+  FX_PAIR(0, 3 - sp, FX_FETCH(0, 2, true), 1)
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    low[a] = make_longlong2(__shfl_xor_sync(0xffffffffu, low[a].x, 16),
+                            __shfl_xor_sync(0xffffffffu, low[a].y, 16));
+  FX_SIGN
+  FX_PAIR(2, 2 + sp, FX_FETCH(0, 3, true), 1)
+  FX_SIGN
+  FX_PAIR(3, 2 + sp, , 0)
+#undef FX_PAIR
+#undef FX_SIGN
+#undef FX_READY
+#undef FX_FETCH
+}
+
+}  // namespace wd

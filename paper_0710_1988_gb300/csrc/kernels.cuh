@@ -16,6 +16,7 @@ struct LatticeGeom {
   // l = ceil(log2 d), dm = floor(2^dsh / d) + 1, exact for n < 2^31.
   unsigned long long dm[3];
   int dsh[3];
+  int split;   // all extents even: the fixed-point links are stored parity by parity
 };
 
 enum { EPI_NONE = 0, EPI_DOT = 1, EPI_TSTT = 2 };
@@ -50,7 +51,14 @@ struct BicgScalars {
 };
 
 LatticeGeom geom_of(const wd_context *h);
+
+// Fixed-point spinors (fx.cuh): v [rhs][tile][12][32], e [rhs][sites].
+struct FxVec {
+  int4 *v;
+  int *e;
+};
 int wilson_blocks(const wd_context *h);
+cudaError_t fx_links_create(wd_context *h);
 
 // Wilson apply with an optional fused reduction epilogue; blocks of systems
 // whose status is not in `mask` do nothing (status == nullptr: all act).

@@ -96,6 +96,7 @@ __device__ __forceinline__ Nbrs neighbours(long long s, const int (&L)[4]) {
 // 32-bit arithmetic and the geometry's multiply-shift divisions.
 struct Nbrs32 {
   unsigned up[4], dn[4];
+  unsigned par;   // (x + y + z + t) & 1
 };
 
 __device__ __forceinline__ unsigned fast_div(unsigned n, unsigned long long m, int sh) {
@@ -111,6 +112,7 @@ __device__ __forceinline__ Nbrs32 neighbours32(unsigned s, const LatticeGeom &g)
   const unsigned y = q0 - q1 * L1;
   const unsigned t = fast_div(q1, g.dm[2], g.dsh[2]);
   const unsigned z = q1 - t * L2;
+  nb.par = (x + y + z + t) & 1u;
   const unsigned sy = L0, sz = sy * L1, st = sz * L2;
   nb.up[0] = x + 1 == L0 ? s - (L0 - 1) : s + 1;
   nb.dn[0] = x == 0 ? s + (L0 - 1) : s - 1;

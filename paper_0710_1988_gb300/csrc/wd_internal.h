@@ -76,6 +76,7 @@ struct wd_context {
   double mu;
   int device;
   double2 *links;   // device, [V][4][3][3] complex128
+  int4 *links_fx;   // fixed-point links [tile][4][9][32] (fx.cuh), nullptr: not usable
   cudaMemPool_t pool;  // this handle's scratch pool
   wd::Profiler prof;   // optional kernel timing
   float4 *links32;     // FP32 rows 0, 1 of every link (mixed precision), lazily built
