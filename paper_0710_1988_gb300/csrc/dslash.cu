@@ -408,7 +408,7 @@ cudaError_t fx_links_create(wd_context *h) {
   return e;
 }
 
-static cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,
+cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,
                                     const int *status, unsigned mask, cudaStream_t s) {
   fx_encode_kernel<<<dim3((unsigned)((sites + 127) / 128), nrhs), 128, 0, s>>>(in, f, sites, fx_sites(sites), status, mask);
   return cudaGetLastError();

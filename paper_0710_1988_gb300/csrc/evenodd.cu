@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "cplx.cuh"
+#include "fx.cuh"
 #include "kernels.cuh"
 #include "spin.cuh"
 #include "wd_internal.h"
@@ -141,6 +142,244 @@ wilson_eo_kernel(const double2 *__restrict__ links, const double2 *__restrict__ 
   }
 }
 
+// ----------------------------------------------------------------- fixed-point form
+
+// D_{pout, 1-pout} src at site s in FP64, from the FP64 values of the sites
+// that fixed point does not hold and the fixed-point ones of the others: the
+// sites next to such a value.
+template <int MU, int S, bool ADJ>
+__device__ __forceinline__ void hop_mixed(const double2 *__restrict__ src, const int4 *__restrict__ psi,
+                                          const int *__restrict__ e, const double2 *__restrict__ links,
+                                          unsigned q, long long ql, double2 (&acc)[12]) {
+  double2 p[12], h[6], c[6];
+  const int E = e[q >> 1];
+  const int4 *x = psi + fx_at(q >> 1, 12);
+#pragma unroll
+  for (int i = 0; i < 12; ++i)
+    p[i] = E == FX_SPECIAL ? src[(size_t)(q >> 1) * 12 + i] : fx_decode(x[i * FX_TILE], E);
+  project<MU, S>(p, h);
+  su3_mul_eo<ADJ>(links + (ql * 4 + MU) * 9, h, c);
+  reconstruct<MU, S>(acc, c);
+}
+
+template <bool DAG>
+__device__ __noinline__ void hops_mixed(const double2 *__restrict__ src, const int4 *__restrict__ psi,
+                                        const int *__restrict__ e, const double2 *__restrict__ links,
+                                        const Nbrs32 nb, unsigned s, double2 *out) {
+  constexpr int F = DAG ? +1 : -1;
+  constexpr int B = -F;
+  double2 acc[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
+  hop_mixed<0, F, false>(src, psi, e, links, nb.up[0], s, acc);
+  hop_mixed<0, B, true>(src, psi, e, links, nb.dn[0], nb.dn[0], acc);
+  hop_mixed<1, F, false>(src, psi, e, links, nb.up[1], s, acc);
+  hop_mixed<1, B, true>(src, psi, e, links, nb.dn[1], nb.dn[1], acc);
+  hop_mixed<2, F, false>(src, psi, e, links, nb.up[2], s, acc);
+  hop_mixed<2, B, true>(src, psi, e, links, nb.dn[2], nb.dn[2], acc);
+  hop_mixed<3, F, false>(src, psi, e, links, nb.up[3], s, acc);
+  hop_mixed<3, B, true>(src, psi, e, links, nb.dn[3], nb.dn[3], acc);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) out[c] = acc[c];
+}
+
+constexpr int EO_SITES = 128;                                          // per block, two lanes each
+constexpr size_t EO_SMEM = 2 * EO_SITES / 32 * 2 * sizeof(FxStage);    // two stages a warp
+
+// wilson_eo_kernel's modes with the hops in fixed point (fx.cuh): src is the
+// encoded operand, src64 its FP64 values at least where it has FX_SPECIAL.
+// EO_SCHUR1 writes the odd vector in fixed point (outfx) for the second half
+// hop, and in FP64 (out) only the sites that need it.
+template <bool DAG, int MODE, int EPI>
+__global__ void __launch_bounds__(2 * EO_SITES, 2)
+wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec src,
+                    const double2 *__restrict__ src64, const double2 *__restrict__ same,
+                    double2 *__restrict__ out, FxVec outfx, LatticeGeom g, size_t tiled, int pout,
+                    double kappa, double mu, double inv_1mu2, int nrhs,
+                    const double2 *__restrict__ aux, double *__restrict__ partial,
+                    const int *__restrict__ status, unsigned mask,
+                    unsigned long long *__restrict__ sites) {
+  const int r = (int)(blockIdx.x % (unsigned)nrhs);
+  const long long sb = blockIdx.x / (unsigned)nrhs;
+  if (status != nullptr && !((mask >> status[r]) & 1u)) return;
+  if (sites != nullptr && sb == 0 && threadIdx.x == 0)
+    atomicAdd(sites, (unsigned long long)g.V);  // two half hops = one full MVP of work
+  const unsigned Vh = (unsigned)(g.V / 2);
+  const int sp = (threadIdx.x >> 4) & 1;
+  const long long at = sb * EO_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+  const bool valid = at < Vh;
+  const unsigned i = valid ? (unsigned)at : Vh - 1;   // idle lanes repeat the last site
+  // the site of parity pout in the x-pair (2i, 2i + 1)
+  const unsigned q0 = fast_div(2 * i, g.dm[0], g.dsh[0]);
+  const unsigned q1 = fast_div(q0, g.dm[1], g.dsh[1]);
+  const unsigned q2 = fast_div(q1, g.dm[2], g.dsh[2]);
+  const unsigned yzt = (q0 - q1 * (unsigned)g.L[1]) + (q1 - q2 * (unsigned)g.L[2]) + q2;
+  const unsigned s = 2 * i + ((int)(yzt & 1u) != pout ? 1u : 0u);
+  const Nbrs32 nb = neighbours32(s, g);
+  const int *ev = src.e + (size_t)r * Vh;
+  const int4 *psi = src.v + (size_t)r * 12 * tiled;
+  int eu[4], ed[4], E = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    eu[m] = __ldg(ev + (nb.up[m] >> 1));
+    ed[m] = __ldg(ev + (nb.dn[m] >> 1));
+    E = max(E, max(eu[m], ed[m]));
+  }
+  extern __shared__ __align__(128) unsigned char eo_smem[];
+  FxStage *stage = reinterpret_cast<FxStage *>(eo_smem) + 2 * (threadIdx.x >> 5);
+  longlong2 up[3], low[3];
+  const unsigned here = (pout ? Vh : 0u) + i, other = pout ? 0u : Vh;
+  fx_hops<(DAG ? +1 : -1)>(
+      stage, [&](int m, bool fwd) {
+        return L + fx_at(fwd ? here : other + (nb.dn[m] >> 1), 36) + m * 9 * FX_TILE;
+      },
+      [&](int m, bool fwd) { return psi + fx_at((fwd ? nb.up[m] : nb.dn[m]) >> 1, 12); }, sp, E,
+      eu, ed, up, low);
+  const size_t off = (size_t)r * 12 * Vh;
+  const double tmu = DAG ? -mu : mu;
+  if (MODE == EO_SCHUR1 && tmu == 0.0 && __all_sync(0xffffffffu, E != FX_SPECIAL)) {
+    // h itself: the sums' slices, without a way through FP64
+    int bits = fx_sum_bits(up, low);
+    bits = max(bits, __shfl_xor_sync(0xffffffffu, bits, 16));
+    if (valid) {
+      int4 *o = outfx.v + (size_t)r * 12 * tiled + fx_at(i, 12);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int2 ux = fx_reslice(up[a].x, bits), uy = fx_reslice(up[a].y, bits);
+        const int2 lx = fx_reslice(low[a].x, bits), ly = fx_reslice(low[a].y, bits);
+        o[(3 * sp + a) * FX_TILE] = make_int4(ux.x, ux.y, uy.x, uy.y);
+        o[(6 + 3 * sp + a) * FX_TILE] = make_int4(lx.x, lx.y, ly.x, ly.y);
+      }
+      if (sp == 0) outfx.e[(size_t)r * Vh + i] = bits ? E + bits - 57 : 0;
+    }
+    return;
+  }
+  // the warp's 16 sites of hop sums through shared memory
+  double2 *hop = reinterpret_cast<double2 *>(stage);   // 13 a site: no bank conflicts
+  double2 *mine = hop + (threadIdx.x & 15) * 13;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    mine[3 * sp + a] = make_double2(fx_to_double(up[a].x, E), fx_to_double(up[a].y, E));
+    mine[6 + 3 * sp + a] = make_double2(fx_to_double(low[a].x, E), fx_to_double(low[a].y, E));
+  }
+  __syncwarp();
+  if (E == FX_SPECIAL && sp == 0 && valid) hops_mixed<DAG>(src64 + off, psi, ev, links, nb, s, mine);
+  __syncwarp();
+  if (MODE == EO_SCHUR1) {   // (1 - i mu g5) h / (1 + mu^2)
+    double2 v[6];
+    int e = 0;
+    unsigned long long any = 0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const double2 h = mine[(c < 3 ? 0 : 3) + 3 * sp + c];
+      const double gm = c < 3 ? tmu : -tmu;
+      v[c].x = (h.x + gm * h.y) * inv_1mu2;
+      v[c].y = (h.y - gm * h.x) * inv_1mu2;
+      e = max(e, max(exp_bits(v[c].x), exp_bits(v[c].y)));
+      any |= (unsigned long long)(__double_as_longlong(v[c].x) | __double_as_longlong(v[c].y)) << 1;
+    }
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+    any |= __shfl_xor_sync(0xffffffffu, any, 16);
+    const int Eo = fx_site_exponent(e, any == 0);
+    if (valid) {
+      int4 *o = outfx.v + (size_t)r * 12 * tiled + fx_at(i, 12);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const int comp = (c < 3 ? 0 : 3) + 3 * sp + c;
+        o[comp * FX_TILE] = fx_slices(v[c], max(e, 1));
+        if (Eo == FX_SPECIAL) out[off + (size_t)i * 12 + comp] = v[c];
+      }
+      if (sp == 0) outfx.e[(size_t)r * Vh + i] = Eo;
+    }
+    return;
+  }
+  double red[3] = {0.0, 0.0, 0.0};
+  const long long first = sb * EO_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
+  const size_t base = off + (size_t)first * 12;
+  const int count = 12 * (int)max(0LL, min(16LL, (long long)Vh - first));
+  const double k2 = kappa * kappa;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int c = q * 32 + (threadIdx.x & 31);
+    if (c < count) {
+      const double2 sm = __ldg(same + base + c), h = hop[c + c / 12];
+      double2 v;
+      if (MODE == EO_SCHUR2) {    // (1 + i mu g5) same - kappa^2 h
+        double2 d = sm;
+        if (tmu != 0.0 || exp_bits(sm.x) == 0x7ff || exp_bits(sm.y) == 0x7ff) {
+          const double gm = c % 12 < 6 ? tmu : -tmu;
+          d.x = sm.x - gm * sm.y;
+          d.y = sm.y + gm * sm.x;
+        }
+        v.x = fma(-k2, h.x, d.x);
+        v.y = fma(-k2, h.y, d.y);
+      } else {                    // same + kappa h
+        v.x = fma(kappa, h.x, sm.x);
+        v.y = fma(kappa, h.y, sm.y);
+      }
+      out[base + c] = v;
+      if (EPI != EPI_NONE) {  // <aux, out> or <out, same>, and <out, out>
+        const double2 a = EPI == EPI_DOT ? __ldg(aux + base + c) : v;
+        const double2 b = EPI == EPI_DOT ? v : sm;
+        red[0] = fma(a.x, b.x, fma(a.y, b.y, red[0]));
+        red[1] = fma(a.x, b.y, fma(-a.y, b.x, red[1]));
+        red[2] = fma(v.x, v.x, fma(v.y, v.y, red[2]));
+      }
+    }
+  }
+  if (EPI != EPI_NONE) {
+    block_sum<3>(red);
+    if (threadIdx.x == 0) {
+      const long long nsb = gridDim.x / (unsigned)nrhs;
+      double *d = partial + ((long long)r * nsb + sb) * 3;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) d[q] = red[q];
+    }
+  }
+}
+
+template <bool DAG, int MODE, int EPI>
+static cudaError_t launch_eo_fx1(const wd_context *h, FxVec src, const double2 *src64,
+                                 const double2 *same, double2 *out, FxVec outfx, int pout, int nrhs,
+                                 const double2 *aux, double *partial, const int *status,
+                                 unsigned mask, unsigned long long *cnt, cudaStream_t s) {
+  static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
+  if (attr_device != h->device) {
+    const cudaError_t e = cudaFuncSetAttribute(wilson_eo_fx_kernel<DAG, MODE, EPI>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EO_SMEM);
+    if (e != cudaSuccess) return e;
+    attr_device = h->device;
+  }
+  const unsigned grid = (unsigned)((h->V / 2 + EO_SITES - 1) / EO_SITES) * (unsigned)nrhs;
+  const double inv = 1.0 / std::fma(h->mu, h->mu, 1.0);
+  wilson_eo_fx_kernel<DAG, MODE, EPI><<<grid, 2 * EO_SITES, EO_SMEM, s>>>(
+      h->links_fx, h->links, src, src64, same, out, outfx, geom_of(h), fx_sites(h->V / 2), pout,
+      h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt);
+  return cudaGetLastError();
+}
+
+// Stream-ordered scratch for `count` encoded batches of half vectors; v is
+// nullptr when the memory is not there.
+struct FxScratch {
+  FxVec f[2];
+  int4 *buf = nullptr;
+  cudaStream_t s;
+  FxScratch(const wd_context *h, int nrhs, int count, cudaStream_t stream) : s(stream) {
+    if (h->links_fx == nullptr || (h->V / 2 + EO_SITES - 1) / EO_SITES * nrhs > 0x7fffffffLL) return;
+    const size_t nv = (size_t)nrhs * fx_sites(h->V / 2), one = nv * 12 * sizeof(int4) + nv * sizeof(int);
+    if (cudaMallocFromPoolAsync((void **)&buf, count * one, h->pool, s) != cudaSuccess) {
+      cudaGetLastError();
+      buf = nullptr;
+      return;
+    }
+    for (int i = 0; i < count; ++i)
+      f[i] = FxVec{buf + i * 12 * nv, reinterpret_cast<int *>(buf + count * 12 * nv) + i * nv};
+  }
+  ~FxScratch() {
+    if (buf) cudaFreeAsync(buf, s);
+  }
+};
+
 int eo_blocks(const wd_context *h) { return (int)((h->V / 2 + 127) / 128); }
 
 template <bool DAG>
@@ -181,6 +420,27 @@ cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double
   if (ensure_eo_tmp(h, nrhs)) return cudaErrorMemoryAllocation;
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
+  FxScratch fx(h, nrhs, 2, s);
+  if (fx.buf) {
+    cudaError_t e = launch_fx_encode(in, fx.f[0], h->V / 2, nrhs, status, mask, s);
+    if (e != cudaSuccess) return e;
+#define EO_FX(D, M, E, SRC, SRC64, SAME, OUT, OUTFX, POUT, CNT)                                     \
+  launch_eo_fx1<D, M, E>(h, SRC, SRC64, SAME, OUT, OUTFX, POUT, nrhs, aux, partial, status, mask, CNT, s)
+#define EO_FX_PAIR(D, E)                                                                            \
+  {                                                                                                 \
+    e = EO_FX(D, EO_SCHUR1, EPI_NONE, fx.f[0], in, nullptr, h->eo_tmp, fx.f[1], 1, nullptr);        \
+    return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, fx.f[1], h->eo_tmp, in, out, fx.f[0], 0, cnt); \
+  }
+    if (dagger) {
+      if (epi == EPI_DOT) EO_FX_PAIR(true, EPI_DOT)
+      if (epi == EPI_TSTT) EO_FX_PAIR(true, EPI_TSTT)
+      EO_FX_PAIR(true, EPI_NONE)
+    }
+    if (epi == EPI_DOT) EO_FX_PAIR(false, EPI_DOT)
+    if (epi == EPI_TSTT) EO_FX_PAIR(false, EPI_TSTT)
+    EO_FX_PAIR(false, EPI_NONE)
+#undef EO_FX_PAIR
+  }
   dim3 grid(eo_blocks(h), nrhs);
   if (dagger) {
     launch_eo<true>(EO_SCHUR1, EPI_NONE, grid, s, h, in, nullptr, h->eo_tmp, 1, nullptr, nullptr, status, mask, nullptr);
@@ -238,6 +498,21 @@ static unsigned grid_for(long long n) {
   return (unsigned)(b > 1216 ? 1216 : (b < 1 ? 1 : b));
 }
 
+// out (parity pout) = same + kappa D src
+static cudaError_t launch_eo_axpy(const wd_context *h, const double2 *src, const double2 *same,
+                                  double2 *out, int pout, int nrhs, cudaStream_t s) {
+  FxScratch fx(h, nrhs, 1, s);
+  if (fx.buf) {
+    const cudaError_t e = launch_fx_encode(src, fx.f[0], h->V / 2, nrhs, nullptr, M_ALL, s);
+    return e != cudaSuccess ? e
+                            : launch_eo_fx1<false, EO_AXPY, EPI_NONE>(h, fx.f[0], src, same, out, FxVec{nullptr, nullptr}, pout, nrhs,
+                                                                      nullptr, nullptr, nullptr, M_ALL, nullptr, s);
+  }
+  launch_eo<false>(EO_AXPY, EPI_NONE, dim3(eo_blocks(h), nrhs), s, h, src, same, out, pout, nullptr,
+                   nullptr, nullptr, M_ALL, nullptr);
+  return cudaGetLastError();
+}
+
 // b_hat = b_e + kappa D_eo A_oo^{-1} b_o  for nrhs full vectors B
 cudaError_t launch_eo_prepare(wd_context *h, const double2 *B, double2 *Bhat, double2 *be,
                               double2 *bo, int nrhs, cudaStream_t s) {
@@ -246,9 +521,7 @@ cudaError_t launch_eo_prepare(wd_context *h, const double2 *B, double2 *Bhat, do
   const long long nh = (long long)nrhs * 12 * (h->V / 2);
   eo_split_kernel<<<dim3(grid_for(h->V), nrhs), 256, 0, s>>>(B, be, bo, g, 0);
   aoo_inv_kernel<<<grid_for(nh), 256, 0, s>>>(bo, bo, h->mu, nh);
-  launch_eo<false>(EO_AXPY, EPI_NONE, dim3(eo_blocks(h), nrhs), s, h, bo, be, Bhat, 0, nullptr,
-                   nullptr, nullptr, M_ALL, nullptr);
-  return cudaGetLastError();
+  return launch_eo_axpy(h, bo, be, Bhat, 0, nrhs, s);
 }
 
 // X (full) from x_e: x_o = A_oo^{-1} (b_o + kappa D_oe x_e)
@@ -258,8 +531,8 @@ cudaError_t launch_eo_reconstruct(wd_context *h, const double2 *B, const double2
   const LatticeGeom g = geom_of(h);
   const long long nh = (long long)nrhs * 12 * (h->V / 2);
   eo_split_kernel<<<dim3(grid_for(h->V), nrhs), 256, 0, s>>>(B, be, bo, g, 0);
-  launch_eo<false>(EO_AXPY, EPI_NONE, dim3(eo_blocks(h), nrhs), s, h, Xe, bo, be, 1, nullptr,
-                   nullptr, nullptr, M_ALL, nullptr);  // be <- b_o + kappa D_oe x_e (odd)
+  const cudaError_t e = launch_eo_axpy(h, Xe, bo, be, 1, nrhs, s);  // be <- b_o + kappa D_oe x_e (odd)
+  if (e != cudaSuccess) return e;
   aoo_inv_kernel<<<grid_for(nh), 256, 0, s>>>(be, bo, h->mu, nh);
   eo_split_kernel<<<dim3(grid_for(h->V), nrhs), 256, 0, s>>>(X, const_cast<double2 *>(Xe), bo, g, 1);
   return cudaGetLastError();

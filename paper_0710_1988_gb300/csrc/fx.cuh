@@ -84,6 +84,31 @@ __device__ __forceinline__ double fx_to_double(long long T, int E) {
   return a == 0 ? 0.0 : __longlong_as_double((long long)bits);
 }
 
+// X 2^(E - 1078) of a stored site's component
+__device__ __forceinline__ double2 fx_decode(int4 v, int E) {
+  const long long re = ((long long)v.x << 29) + v.y, im = ((long long)v.z << 29) + v.w;
+  return make_double2(fx_to_double(re, E + 1), fx_to_double(im, E + 1));
+}
+
+// Sums T 2^(E - 1079) of a site, shared by the lanes l and l + 16 (six complex
+// components each), as slices of X 2^(E' - 1078): returns E'.  bits: the
+// bit length of the largest |T| of the site.
+__device__ __forceinline__ int fx_sum_bits(const longlong2 (&a)[3], const longlong2 (&b)[3]) {
+  unsigned long long m = 0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    m |= (unsigned long long)(a[i].x ^ (a[i].x >> 63)) | (unsigned long long)(a[i].y ^ (a[i].y >> 63)) |
+         (unsigned long long)(b[i].x ^ (b[i].x >> 63)) | (unsigned long long)(b[i].y ^ (b[i].y >> 63));
+  return 64 - __clzll((long long)m);
+}
+
+__device__ __forceinline__ int2 fx_reslice(long long T, int bits) {
+  const int k = bits - 56;
+  const long long X = k > 0 ? (T + (1LL << (k - 1))) >> k : T << -k;
+  const int lo = ((int)(unsigned)X << 3) >> 3;
+  return make_int2((int)((X - lo) >> 29), lo);
+}
+
 // Sums of one complex product chain U h in three real products each (Gauss):
 // with U = a + i b, h = c + i d,
 //   k1 = (a + b) c, k2 = a (d - c), k3 = b (c + d): U h = (k1 - k3) + i (k1 + k2),

@@ -59,6 +59,9 @@ struct FxVec {
 };
 int wilson_blocks(const wd_context *h);
 cudaError_t fx_links_create(wd_context *h);
+// Encode nrhs vectors of `sites` sites (systems in mask).
+cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,
+                             const int *status, unsigned mask, cudaStream_t s);
 
 // Wilson apply with an optional fused reduction epilogue; blocks of systems
 // whose status is not in `mask` do nothing (status == nullptr: all act).

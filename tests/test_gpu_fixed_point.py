@@ -121,3 +121,90 @@ def test_unit_links_are_exact(wdl):
     psi = (rng.integers(-64, 65, size=(L.volume(dims), 4, 3))
            + 1j * rng.integers(-64, 65, size=(L.volume(dims), 4, 3))) / 8.0
     assert np.array_equal(_apply(wdl, dims, U, psi, 0.125), dirac.apply_A(U, psi, dims, 0.125))
+
+
+def _schur(wdl, dims, U, half, kappa, mu=0.0, dagger=False):
+    import torch
+    op = wdl.WilsonOperator(dims, cuda(U), kappa, mu)
+    op.set_operator(True)
+    out = torch.empty(half.size, dtype=torch.complex128, device="cuda:0")
+    op.apply(cuda(half), out, dagger=dagger)
+    got = host(out).reshape(half.shape)
+    op.close()
+    return got
+
+
+def _two_hop_max(half, dims):
+    """Largest |re| or |im| of the even sites within two hops, at the even sites."""
+    v = L.volume(dims)
+    full = np.zeros((v, 4, 3), dtype=np.complex128)
+    even = _even_sites(dims)
+    full[even] = half
+    m = _local_max(full, dims)
+    return _local_max(np.broadcast_to(m[:, None, None] + 0j, (v, 1, 1)), dims)[even]
+
+
+def _even_sites(dims):
+    s = np.arange(L.volume(dims))
+    x, s = s % dims[0], s // dims[0]
+    y, s = s % dims[1], s // dims[1]
+    z, t = s % dims[2], s // dims[2]
+    return (x + y + z + t) % 2 == 0
+
+
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((4, 2, 2, 2), 3), ((2, 2, 2, 10), 2),
+                                       ((6, 4, 2, 6), 2), ((34, 2, 4, 2), 1), ((8, 8, 2, 4), 3)])
+@pytest.mark.parametrize("mu", [0.0, 0.07])
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("spread", [0.0, 20.0])
+def test_schur_edges_and_magnitudes(wdl, dims, nrhs, mu, dagger, spread):
+    """Each half hop leaves 64 units of 2^-53 of its largest entry and grows
+    entries by at most 2^5: 2^12 units of kappa^2 M over two hops, 64 of M."""
+    from oracle import evenodd
+    rng = np.random.Generator(np.random.PCG64(18))
+    U = L.gauge_field(dims, 0.9, 43)
+    half = L.gaussian_spinor(dims, 44, nrhs=nrhs)[:, : L.volume(dims) // 2]
+    half = half * 10.0 ** rng.uniform(-spread, spread, size=half.shape[:2])[:, :, None, None]
+    half[:, 0] = 0.0
+    got = _schur(wdl, dims, U, half, 0.14, mu, dagger)
+    g5 = lambda z: dirac.gamma5(z.reshape(-1, 4, 3))
+    for r in range(nrhs):
+        if dagger:
+            ref = g5(evenodd.schur_apply(U, dims, 0.14, -mu, g5(half[r]).ravel()))
+        else:
+            ref = evenodd.schur_apply(U, dims, 0.14, mu, half[r].ravel())
+        ref = ref.reshape(half[r].shape)
+        bound = (4096 * 0.14 ** 2 + 64) * 2.0 ** -53 * _two_hop_max(half[r], dims)
+        assert np.all(np.abs(got[r] - ref).max(axis=(-1, -2)) <= bound)
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.07])
+def test_schur_values_outside_fixed_point_match_the_fp64_kernel(wdl, mu):
+    """As for the full operator; the scaled link reaches two hops."""
+    dims = (8, 4, 4, 8)
+    v = L.volume(dims)
+    U = L.gauge_field(dims, 0.5, 53)
+    U2 = U.copy()
+    far = v - 1
+    U2[far, 0] *= 4.0
+    half = L.gaussian_spinor(dims, 54)[: v // 2]
+    half[7, 0, 1] = np.inf
+    half[100, 2, 0] = complex(0.0, np.nan)
+    half[150] *= 1e-310
+    half[160] *= 1e300
+    half[170] = 0.0
+    half[171] = 5e-324
+    a, b = _schur(wdl, dims, U, half, 0.14, mu), _schur(wdl, dims, U2, half, 0.14, mu)
+    hit = np.zeros((v, 1, 1), dtype=np.complex128)
+    hit[[far, far - 7]] = 1.0             # the ends of the scaled x link
+    even = _even_sites(dims)
+    keep = _local_max(hit, dims)[even] == 0.0
+    for x, y in ((a.real[keep], b.real[keep]), (a.imag[keep], b.imag[keep])):
+        assert np.array_equal(np.isnan(x), np.isnan(y))
+        inf = np.isinf(y)
+        assert np.array_equal(inf, np.isinf(x)) and np.array_equal(x[inf], y[inf])
+    clean = half.copy()
+    clean[~np.isfinite(clean)] = 0.0
+    bound = ((4096 * 0.14 ** 2 + 64) * 2.0 ** -53 * _two_hop_max(clean, dims))[keep][:, None, None]
+    fin = np.isfinite(b[keep])
+    assert np.all(np.abs(a[keep] - b[keep])[fin] <= np.broadcast_to(bound, a[keep].shape)[fin])
