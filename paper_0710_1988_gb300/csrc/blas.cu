@@ -369,7 +369,6 @@ int ts_dot_blocks(long long n, int k, int nrhs) {
 // lane keeps half of its values, sends the other half to its partner and
 // adds what it receives, so lane i ends with the warp sum of value i after
 // 16 + 8 + 4 + 2 + 1 additions (a shuffle tree per value would take 160).
-template <int Q = 16>   // complex sums of the tile written (the first Q of the 16)
 __device__ __forceinline__ void ts_tile_reduce(double (&vals)[32], double2 *__restrict__ partial) {
   __shared__ double red[32][TS_THREADS / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -387,13 +386,13 @@ __device__ __forceinline__ void ts_tile_reduce(double (&vals)[32], double2 *__re
   red[lane][wid] = vals[0];
   __syncthreads();
   const long long tile = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  for (int q = threadIdx.x; q < Q; q += blockDim.x) {
+  for (int q = threadIdx.x; q < 16; q += blockDim.x) {
     double a = 0.0, b = 0.0;
     for (int w2 = 0; w2 < TS_THREADS / 32; ++w2) {
       a += red[q * 2][w2];
       b += red[q * 2 + 1][w2];
     }
-    partial[tile * Q + q] = make_double2(a, b);
+    partial[tile * 16 + q] = make_double2(a, b);
   }
 }
 
@@ -486,164 +485,12 @@ cudaError_t launch_ts_dot(const double2 *V, int k, const double2 *W, int nrhs, i
   return cudaGetLastError();
 }
 
-// ----------------------------------------------------------------- first Gram-Schmidt pass, double-float
-
-// h = V^dagger w for one vector w with every product and sum carried as a
-// pair of FP32 numbers (about 48 significant bits), on this GPU's FP32 pipe
-// instead of its much slower FP64 one.  It serves the first pass of
-// classical Gram-Schmidt applied twice: the second pass, in FP64, measures
-// and removes whatever this one left (its coefficients h2 = V^dagger(w - V h)
-// are then of the order of 2^-48 ||w|| instead of 2^-53), and the Hessenberg
-// column h + h2 is exact to FP64 rounding.  An operand outside FP32's range
-// contributes nothing here and is removed by the FP64 pass.
-//  * split: x = hi + lo with hi the top 24 significant bits of x (bit
-//    operations, no FP64 instruction) and lo the next 24 (x - hi rounded).
-//  * product: Dekker's exact product by FMA, p + e = ah bh, plus the cross
-//    terms ah bl + al bh (al bl is below 2^-48 of the product).
-//  * sum: Knuth's TwoSum of the running high part and p; the rounding error
-//    and the low parts accumulate in the low word.
-__device__ __forceinline__ void split_df(double x, float &hi, float &lo) {
-  const long long b = __double_as_longlong(x);
-  const unsigned sign = (unsigned)((unsigned long long)b >> 32) & 0x80000000u;
-  const int e = (int)((b >> 52) & 0x7FF);
-  const int fe = e - 1023 + 127;
-  if (fe <= 0 || fe >= 255) {   // zero, or outside FP32's normal range
-    hi = 0.f;
-    lo = 0.f;
-    return;
-  }
-  hi = __uint_as_float(sign | ((unsigned)fe << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu));
-  const unsigned rem = (unsigned)b & 0x1FFFFFFFu;       // the 29 fraction bits below hi
-  if (rem == 0u || e < 949) {                            // nothing left, or 2^(e-1075) underflows
-    lo = 0.f;
-    return;
-  }
-  const float scale = __uint_as_float((unsigned)(e - 948) << 23);   // 2^(e - 1075)
-  lo = __uint_as_float(__float_as_uint(__uint2float_rn(rem) * scale) | sign);
-}
-
-__device__ __forceinline__ void df_mac(float ah, float al, float bh, float bl, float &sh,
-                                       float &sl) {
-  const float p = ah * bh;
-  float e = fmaf(ah, bh, -p);
-  e = fmaf(ah, bl, fmaf(al, bh, e));
-  const float sum = sh + p;
-  const float t = sum - sh;
-  const float err = (sh - (sum - t)) + (p - t);
-  sl += err + e;
-  sh = sum;
-}
-
-// Tiles of DF_JT basis vectors: a tile's loads are issued together before
-// its arithmetic (the FP32 arithmetic is too quick to hide the loads the way
-// the FP64 pipe does in ts_dot_kernel), and the small tile leaves registers
-// for four blocks per SM (63 registers, no spills): the kernel is bound by
-// instruction issue and latency, so occupancy pays (16^4 tall-skinny time per
-// step: 8-vector tiles at three blocks 477 ms, 4 at five 464, 4 at four 450).
-constexpr int DF_JT = 4;
-
-static void ts_dot_df_grid(long long n, int k, dim3 *grid) {
-  const int gy = (k + DF_JT - 1) / DF_JT;
-  long long gx = TS_MAX_BLOCKS / gy;
-  const long long need = (n + TS_THREADS - 1) / TS_THREADS;
-  if (gx > need) gx = need;
-  if (gx < 8) gx = need < 8 ? need : 8;
-  if (gx < 1) gx = 1;
-  *grid = dim3((unsigned)gx, gy, 1);
-}
-
-__global__ void __launch_bounds__(TS_THREADS, 4)
-ts_dot_df_kernel(const float2 *__restrict__ Vh, const float2 *__restrict__ Vl, int k,
-                 const double2 *__restrict__ W, long long n, double2 *__restrict__ partial,
-                 const int *__restrict__ status) {
-  if (status != nullptr && *status != 0) return;
-  const int j0 = blockIdx.y * DF_JT;
-  const int nj = min(DF_JT, k - j0);
-  float arh[DF_JT], arl[DF_JT], aih[DF_JT], ail[DF_JT];
-#pragma unroll
-  for (int j = 0; j < DF_JT; ++j) arh[j] = arl[j] = aih[j] = ail[j] = 0.f;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    float2 vh[DF_JT], vl[DF_JT];
-#pragma unroll
-    for (int j = 0; j < DF_JT; ++j) {   // rows past the last vector reread it and add nothing
-      const long long o = (long long)(j0 + (j < nj ? j : nj - 1)) * n + i;
-      vh[j] = __ldg(Vh + o);
-      vl[j] = __ldg(Vl + o);
-    }
-    const double2 w = __ldg(W + i);
-    float wrh, wrl, wih, wil;
-    split_df(w.x, wrh, wrl);
-    split_df(w.y, wih, wil);
-#pragma unroll
-    for (int j = 0; j < DF_JT; ++j) {
-      float vrh = vh[j].x, vrl = vl[j].x, vih = vh[j].y, vil = vl[j].y;
-      if (j >= nj) vrh = vrl = vih = vil = 0.f;
-      // conj(v) w = (vr wr + vi wi) + i (vr wi - vi wr)
-      df_mac(vrh, vrl, wrh, wrl, arh[j], arl[j]);
-      df_mac(vih, vil, wih, wil, arh[j], arl[j]);
-      df_mac(vrh, vrl, wih, wil, aih[j], ail[j]);
-      df_mac(-vih, -vil, wrh, wrl, aih[j], ail[j]);
-    }
-  }
-  // the tile's DF_JT complex sums in the first 2 DF_JT of the 32 reduced values
-  double vals[32];
-#pragma unroll
-  for (int j = 0; j < DF_JT; ++j) {
-    vals[2 * j] = (double)arh[j] + (double)arl[j];
-    vals[2 * j + 1] = (double)aih[j] + (double)ail[j];
-  }
-#pragma unroll
-  for (int q = 2 * DF_JT; q < 32; ++q) vals[q] = 0.0;
-  ts_tile_reduce<DF_JT>(vals, partial);
-}
-
-// Each complex128 entry of v as FP32 pairs in two planes: vh[i] = (Re hi,
-// Im hi), vl[i] = (Re lo, Im lo).  The basis in the form the double-float
-// dot reads (both planes) and the FP32 Gram-Schmidt correction reads (the
-// high plane: half the bytes of v), written once per basis vector.
-__global__ void __launch_bounds__(256)
-split_df_kernel(const double2 *__restrict__ v, float2 *__restrict__ vh, float2 *__restrict__ vl,
-                long long count, const int *__restrict__ status) {
-  if (status != nullptr && *status != 0) return;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double2 a = v[i];
-    float rh, rl, ih, il;
-    split_df(a.x, rh, rl);
-    split_df(a.y, ih, il);
-    vh[i] = make_float2(rh, ih);
-    vl[i] = make_float2(rl, il);
-  }
-}
-
-cudaError_t launch_split_df(const double2 *v, float2 *vh, float2 *vl, long long count,
-                            const int *status, cudaStream_t s) {
-  ProfLaunch prof_(PC_TS, s);
-  long long blocks = (count + 255) / 256;
-  if (blocks > 4 * 1216) blocks = 4 * 1216;
-  if (blocks < 1) blocks = 1;
-  split_df_kernel<<<(unsigned)blocks, 256, 0, s>>>(v, vh, vl, count, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ts_dot_df(const float2 *Vh, const float2 *Vl, int k, const double2 *w,
-                             long long n, double2 *partial, const int *status, cudaStream_t s) {
-  ProfLaunch prof_(PC_TS, s);
-  if (k < 1 || k > 4096) return cudaErrorInvalidValue;
-  dim3 grid;
-  ts_dot_df_grid(n, k, &grid);
-  ts_dot_df_kernel<<<grid, TS_THREADS, 0, s>>>(Vh, Vl, k, w, n, partial, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ts_dot_df_finalize(const double2 *partial, long long n, int k, double2 *C,
-                                      int ldc, const int *status, cudaStream_t s) {
-  ProfLaunch prof_(PC_TS, s);
-  dim3 grid;
-  ts_dot_df_grid(n, k, &grid);
-  ts_dot_finalize_kernel<<<(k + 3) / 4, 128, 0, s>>>(partial, grid.x, grid.y, DF_JT, 1, k, 1, C,
-                                                     ldc, nullptr, 0, status);
+cudaError_t launch_ts_dot_finalize_grid(const double2 *partial, int gx, int gy, int JT, int RT, int k,
+                                        int nrhs, double2 *C, int ldc, double2 *C2, int ldc2,
+                                        const int *status, cudaStream_t s) {
+  const int P = k * nrhs;  // one warp per pair, four warps per block
+  ts_dot_finalize_kernel<<<(P + 3) / 4, 128, 0, s>>>(partial, gx, gy, JT, RT, k, nrhs, C, ldc, C2,
+                                                     ldc2, status);
   return cudaGetLastError();
 }
 
@@ -655,10 +502,8 @@ cudaError_t launch_ts_dot_finalize(const double2 *partial, long long n, int k, i
   ts_dot_grid(n, k, nrhs, &grid);
   int JT, RT;
   ts_dot_tile(nrhs, &JT, &RT);
-  const int P = k * nrhs;  // one warp per pair, four warps per block
-  ts_dot_finalize_kernel<<<(P + 3) / 4, 128, 0, s>>>(partial, grid.x, grid.y, JT, RT, k, nrhs,
-                                                     C, ldc, C2, ldc2, status);
-  return cudaGetLastError();
+  return launch_ts_dot_finalize_grid(partial, (int)grid.x, (int)grid.y, JT, RT, k, nrhs, C, ldc, C2, ldc2,
+                                     status, s);
 }
 
 constexpr int TU_THREADS = 256;
@@ -719,111 +564,6 @@ cudaError_t launch_ts_update(const double2 *V, int kv, const double2 *Y, int ldy
   return cudaSuccess;
 }
 
-// ----------------------------------------------------------------- CGS correction
-
-// w -= V h for the second pass of classical Gram-Schmidt, whose coefficients
-// h are of the order of the first pass's rounding (|h| ~ eps ||w||): the
-// correction V h then needs only FP32 accuracy relative to itself, which is
-// far below FP64 rounding of w, while its products would cost FP64 FMAs.
-// FP32 path, taken when ||h||^2 <= 1e-20 (||w0||^2 - ||hsum||^2) (the
-// correction below 1e-10 of the vector it corrects; ||w0||^2 from the Wilson
-// kernel's partials, hsum the coefficients of both passes): V and h are
-// truncated to FP32 by bit operations (no FP64 instruction), the products
-// accumulate in FP32, and w is updated in FP64.  Otherwise the FP64 form of
-// ts_update.  Every block forms the decision from the same device data in
-// the same order, so all take the same path.
-__device__ __forceinline__ float f32_trunc(double x) {
-  const long long b = __double_as_longlong(x);
-  const unsigned sign = (unsigned)((unsigned long long)b >> 32) & 0x80000000u;
-  const int fe = (int)((b >> 52) & 0x7FF) - 1023 + 127;
-  if (fe <= 0) return __uint_as_float(sign);                 // below FP32's normal range
-  if (fe >= 255) return __uint_as_float(sign | 0x7F7FFFFFu);  // clamp (not met here)
-  return __uint_as_float(sign | ((unsigned)fe << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu));
-}
-
-__device__ __forceinline__ double f64_widen(float x) {
-  const unsigned u = __float_as_uint(x);
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  const unsigned e = (u >> 23) & 0xFF;
-  if (e == 0) return __longlong_as_double((long long)sign);  // zero (subnormals flushed)
-  return __longlong_as_double((long long)(sign | ((unsigned long long)(e - 127 + 1023) << 52) |
-                                          ((unsigned long long)(u & 0x7FFFFFu) << 29)));
-}
-
-__global__ void __launch_bounds__(TU_THREADS)
-ts_update_correction_kernel(const double2 *__restrict__ V, const float2 *__restrict__ Vh, int kv,
-                            const double2 *__restrict__ h, const double2 *__restrict__ hsum,
-                            int ldh, const double *__restrict__ part_w, int nbw, double2 *w,
-                            long long n, const int *__restrict__ status) {
-  if (status != nullptr && *status != 0) return;
-  __shared__ float2 hf[TU_MAXK];
-  __shared__ double2 hd[TU_MAXK];
-  __shared__ int use32;
-  if (threadIdx.x < 32) {
-    double w2 = 0.0, s2 = 0.0, c2 = 0.0;
-    for (int b = threadIdx.x; b < nbw; b += 32) w2 += part_w[(long long)b * 3 + 2];
-    for (int r = threadIdx.x; r < kv; r += 32) {
-      c2 += cnorm2(h[r]);
-      s2 += cnorm2(hsum[(long long)r * ldh]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      w2 += __shfl_xor_sync(0xffffffffu, w2, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      c2 += __shfl_xor_sync(0xffffffffu, c2, o);
-    }
-    if (threadIdx.x == 0) use32 = c2 <= 1e-20 * (w2 - s2) ? 1 : 0;
-  }
-  for (int r = threadIdx.x; r < kv; r += blockDim.x) {
-    hd[r] = h[r];
-    hf[r] = make_float2(f32_trunc(h[r].x), f32_trunc(h[r].y));
-  }
-  __syncthreads();
-  const bool fp32 = use32 != 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    double2 o = w[i];
-    if (fp32) {
-      float ax = 0.f, ay = 0.f;
-      for (int r = 0; r < kv; ++r) {
-        float vx, vy;
-        if (Vh != nullptr) {   // the same truncation, stored: half the bytes of V
-          const float2 v = __ldg(Vh + (long long)r * n + i);
-          vx = v.x;
-          vy = v.y;
-        } else {
-          const double2 v = __ldg(V + (long long)r * n + i);
-          vx = f32_trunc(v.x);
-          vy = f32_trunc(v.y);
-        }
-        const float2 c = hf[r];
-        ax = fmaf(vx, c.x, fmaf(-vy, c.y, ax));
-        ay = fmaf(vx, c.y, fmaf(vy, c.x, ay));
-      }
-      o.x -= f64_widen(ax);
-      o.y -= f64_widen(ay);
-    } else {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int r = 0; r < kv; ++r) acc = cfma(__ldg(V + (long long)r * n + i), hd[r], acc);
-      o = csub(o, acc);
-    }
-    w[i] = o;
-  }
-}
-
-cudaError_t launch_ts_update_correction(const double2 *V, const float2 *Vh, int kv,
-                                        const double2 *h, const double2 *hsum, int ldh,
-                                        const double *part_w, int nbw, double2 *w, long long n,
-                                        const int *status, cudaStream_t s) {
-  ProfLaunch prof_(PC_TS, s);
-  if (kv > TU_MAXK || kv < 1) return cudaErrorInvalidValue;
-  long long blocks = (n + TU_THREADS - 1) / TU_THREADS;
-  if (blocks > 1216) blocks = 1216;
-  ts_update_correction_kernel<<<(unsigned)blocks, TU_THREADS, 0, s>>>(V, Vh, kv, h, hsum, ldh,
-                                                                     part_w, nbw, w, n, status);
-  return cudaGetLastError();
-}
-
 // ----------------------------------------------------------------- Arnoldi helpers
 
 __global__ void arnoldi_normalize_finalize_kernel(const double *__restrict__ pw, int nb,
@@ -844,20 +584,6 @@ __global__ void arnoldi_normalize_finalize_kernel(const double *__restrict__ pw,
       *m_eff = j + 1;
     }
   }
-}
-
-__global__ void scale_by_inverse_entry_kernel(double2 *__restrict__ v,
-                                              const double2 *__restrict__ w,
-                                              const double2 *__restrict__ H, int idx,
-                                              long long n, const int *__restrict__ status) {
-  if (status != nullptr && *status != 0) return;  // uniform over the grid
-  __shared__ double s_inv;  // one division per block, not per thread
-  if (threadIdx.x == 0) s_inv = 1.0 / H[idx].x;
-  __syncthreads();
-  const double inv = s_inv;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    v[i] = cscale(inv, w[i]);
 }
 
 cudaError_t launch_arnoldi_normalize_finalize(const double *partial_w, int nb,
@@ -882,14 +608,6 @@ cudaError_t launch_norm_finalize(const double *partial, int nb, int stride, doub
                                  cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
   norm_finalize_kernel<<<1, 256, 0, s>>>(partial, nb, stride, dst);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scale_by_inverse_entry(double2 *v, const double2 *w, const double2 *H,
-                                          int idx, long long n, const int *status,
-                                          cudaStream_t s) {
-  ProfLaunch prof_(PC_STREAM, s);
-  scale_by_inverse_entry_kernel<<<stream_blocks(n), SB_THREADS, 0, s>>>(v, w, H, idx, n, status);
   return cudaGetLastError();
 }
 

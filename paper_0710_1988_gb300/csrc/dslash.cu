@@ -467,7 +467,8 @@ LatticeGeom geom_of(const wd_context *h) {
 int eo_blocks(const wd_context *h);
 cudaError_t launch_schur_f64_epi(const wd_context *h, const double2 *in, double2 *out, int nrhs,
                                  int dagger, int epi, const double2 *aux, double *partial,
-                                 const int *status, cudaStream_t s, unsigned mask);
+                                 const int *status, cudaStream_t s, unsigned mask,
+                                 const FxVec *pre);
 
 int wilson_blocks(const wd_context *h) {
   return h->eo ? eo_blocks(h) : (int)((h->V + 127) / 128);
@@ -476,12 +477,14 @@ int wilson_blocks(const wd_context *h) {
 cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double2 *out,
                                   int nrhs, int dagger, int epi, const double2 *aux,
                                   double *partial, const int *status, cudaStream_t s,
-                                  unsigned mask) {
+                                  unsigned mask, const FxVec *pre) {
   if (h->eo)  // even-odd Schur operator on even half vectors
-    return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask);
+    return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, pre);
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
   if (h->links_fx != nullptr && (long long)wilson_blocks(h) * nrhs <= 0x7fffffffLL) {
+    if (pre != nullptr)
+      return launch_wilson_fx(h, *pre, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
     // scratch for the encoded input, stream-ordered; without it the FP64 kernel
     const size_t nv = (size_t)nrhs * fx_sites(h->V);
     int4 *buf = nullptr;

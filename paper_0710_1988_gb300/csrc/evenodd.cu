@@ -415,21 +415,24 @@ static int ensure_eo_tmp(wd_context *h, int nrhs) {
 // reduction epilogues of the full operator on the second half hop.
 cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double2 *out, int nrhs,
                                  int dagger, int epi, const double2 *aux, double *partial,
-                                 const int *status, cudaStream_t s, unsigned mask) {
+                                 const int *status, cudaStream_t s, unsigned mask,
+                                 const FxVec *pre) {
   wd_context *h = const_cast<wd_context *>(hc);
   if (ensure_eo_tmp(h, nrhs)) return cudaErrorMemoryAllocation;
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
-  FxScratch fx(h, nrhs, 2, s);
+  FxScratch fx(h, nrhs, pre ? 1 : 2, s);
   if (fx.buf) {
-    cudaError_t e = launch_fx_encode(in, fx.f[0], h->V / 2, nrhs, status, mask, s);
+    const FxVec tmp = fx.f[0], src = pre ? *pre : fx.f[1];
+    cudaError_t e = cudaSuccess;
+    if (!pre) e = launch_fx_encode(in, src, h->V / 2, nrhs, status, mask, s);
     if (e != cudaSuccess) return e;
 #define EO_FX(D, M, E, SRC, SRC64, SAME, OUT, OUTFX, POUT, CNT)                                     \
   launch_eo_fx1<D, M, E>(h, SRC, SRC64, SAME, OUT, OUTFX, POUT, nrhs, aux, partial, status, mask, CNT, s)
 #define EO_FX_PAIR(D, E)                                                                            \
   {                                                                                                 \
-    e = EO_FX(D, EO_SCHUR1, EPI_NONE, fx.f[0], in, nullptr, h->eo_tmp, fx.f[1], 1, nullptr);        \
-    return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, fx.f[1], h->eo_tmp, in, out, fx.f[0], 0, cnt); \
+    e = EO_FX(D, EO_SCHUR1, EPI_NONE, src, in, nullptr, h->eo_tmp, tmp, 1, nullptr);                \
+    return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, tmp, h->eo_tmp, in, out, tmp, 0, cnt);       \
   }
     if (dagger) {
       if (epi == EPI_DOT) EO_FX_PAIR(true, EPI_DOT)

@@ -65,10 +65,11 @@ cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nr
 
 // Wilson apply with an optional fused reduction epilogue; blocks of systems
 // whose status is not in `mask` do nothing (status == nullptr: all act).
+// pre: `in` already in fixed point (used when the handle has such links).
 cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double2 *out,
                                   int nrhs, int dagger, int epi, const double2 *aux,
                                   double *partial, const int *status, cudaStream_t s,
-                                  unsigned mask = M_ACTIVE);
+                                  unsigned mask = M_ACTIVE, const FxVec *pre = nullptr);
 
 // ----------------------------------------------------------------- BLAS1
 // Number of blocks (per system) every streaming kernel uses; fixed so that
@@ -122,37 +123,16 @@ cudaError_t launch_ts_dot(const double2 *V, int k, const double2 *W, int nrhs, i
 cudaError_t launch_ts_dot_finalize(const double2 *partial, long long n, int k, int nrhs,
                                    double2 *C, int ldc, double2 *C2, int ldc2,
                                    const int *status, cudaStream_t s);
-// launch_ts_dot for one vector (nrhs = 1, no gamma5) in double-float
-// arithmetic (about 48 bits, on the FP32 pipe): the first pass of CGS2, whose
-// error the FP64 second pass removes.  V in the split form of
-// launch_split_df (k vectors of n entries in each plane).  Its partials (at
-// most ts_dot_partial_count(n, k, 1)) are summed by launch_ts_dot_df_finalize
-// into C[j * ldc], j < k.
-cudaError_t launch_ts_dot_df(const float2 *Vh, const float2 *Vl, int k, const double2 *w,
-                             long long n, double2 *partial, const int *status, cudaStream_t s);
-// vh[i] = (Re hi, Im hi), vl[i] = (Re lo, Im lo) of v[i] (hi: the top 24
-// significant bits, lo: the next 24; an entry outside FP32's normal range
-// gives zeros), i < count.
-cudaError_t launch_split_df(const double2 *v, float2 *vh, float2 *vl, long long count,
-                            const int *status, cudaStream_t s);
-cudaError_t launch_ts_dot_df_finalize(const double2 *partial, long long n, int k, double2 *C,
-                                      int ldc, const int *status, cudaStream_t s);
+// the same sum of partials laid out [(gy rows, gx blocks)][JT x RT]
+cudaError_t launch_ts_dot_finalize_grid(const double2 *partial, int gx, int gy, int JT, int RT, int k,
+                                        int nrhs, double2 *C, int ldc, double2 *C2, int ldc2,
+                                        const int *status, cudaStream_t s);
 // OUT[c][i] = (beta_one ? IN[c][i] : 0) + sign * sum_j V[j][i] Y[j*ldy + c],
 // c < ncol, kv <= 128.  OUT may alias IN (in-place update) but not V.
 cudaError_t launch_ts_update(const double2 *V, int kv, const double2 *Y, int ldy, int ncol,
                              const double2 *IN, double2 *OUT, int beta_one, double sign,
                              long long n, const int *status, cudaStream_t s);
 
-// w -= V h for the second classical Gram-Schmidt pass: FP32 products when
-// ||h||^2 <= 1e-20 (||w0||^2 - ||hsum||^2) (part_w: Wilson-kernel partials,
-// [3 b + 2] = block b's share of ||w0||^2; hsum: column of both passes'
-// coefficients, stride ldh), else FP64 (blas.cu).
-// Vh: nullptr, or V's high FP32 parts in the layout of launch_split_df (read
-// instead of V on the FP32 path).
-cudaError_t launch_ts_update_correction(const double2 *V, const float2 *Vh, int kv,
-                                        const double2 *h, const double2 *hsum, int ldh,
-                                        const double *part_w, int nbw, double2 *w, long long n,
-                                        const int *status, cudaStream_t s);
 // The same product on the tensor cores (exact-split BF16 emulation to FP64
 // accuracy, tc_gemm.cu): kv <= 88, any ncol; OUT may alias IN but not V.
 // scratch: ts_update_tc_scratch_bytes(kv, ncol, n) device bytes; *err (device)
@@ -173,10 +153,38 @@ cudaError_t launch_arnoldi_normalize_finalize(const double *partial_w, int nb,
 // *dst = sqrt(sum_i partial[i*stride]) for i < nb (deterministic order)
 cudaError_t launch_norm_finalize(const double *partial, int nb, int stride, double2 *dst,
                                  cudaStream_t s);
-// v = w / Re(H[idx]) unless *status != 0
-cudaError_t launch_scale_by_inverse_entry(double2 *v, const double2 *w, const double2 *H,
-                                          int idx, long long n, const int *status,
-                                          cudaStream_t s);
+// ----------------------------------------------------------------- Gram-Schmidt in fixed point (fx_basis.cu)
+// Basis vectors of n entries (n even) in fixed point: planes hi, lo [vector][n]
+// and exponents ex [vector][fxb_chunks(n)].
+struct FxBasis {
+  int2 *hi, *lo;
+  int *ex;
+};
+long long fxb_chunks(long long n);
+// `count` vectors from w, the first into slot j of b: v = w / Re(H[idx]) (H nullptr: v = w);
+// v (may be w, or nullptr) gets the FP64 values, fx (one vector; fx.v may be
+// nullptr) the site-wise form of the operator.  Nothing when *status != 0.
+cudaError_t launch_fxb_encode(const double2 *w, const double2 *H, int idx, double2 *v, FxBasis b,
+                              long long j, int count, FxVec fx, long long n, const int *status,
+                              cudaStream_t s);
+// C[j ldc] = <V_j, w> (g5: <V_j, gamma5 w>), j < k, and C2[j ldc2] += it when C2 != nullptr.
+// partial: fxb_dot_partials(n, k) complex numbers.  V: the FP64 vectors.
+size_t fxb_dot_partials(long long n, int k);
+cudaError_t launch_fxb_dot(FxBasis b, const double2 *V, int k, const double2 *w, int g5, long long n,
+                           double2 *partial, double2 *C, int ldc, double2 *C2, int ldc2,
+                           const int *status, cudaStream_t s);
+// w -= sum_j V_j h[j ldh] (add: w +=), k <= 128
+cudaError_t launch_fxb_update(FxBasis b, const double2 *V, int k, const double2 *h, int ldh, int add,
+                              double2 *w, long long n, const int *status, cudaStream_t s);
+// w -= V h for the second classical Gram-Schmidt pass: FP32 products when
+// ||h||^2 <= 1e-20 (||w0||^2 - ||hsum||^2) (part_w: Wilson-kernel partials,
+// [3 b + 2] = block b's share of ||w0||^2; hsum: column of both passes'
+// coefficients, stride ldh), else FP64.  part_n[2 c] = chunk c's share of
+// ||w||^2 afterwards.
+cudaError_t launch_fxb_correction(FxBasis b, const double2 *V, int k, const double2 *h,
+                                  const double2 *hsum, int ldh, const double *part_w, int nbw,
+                                  double2 *w, long long n, double *part_n, const int *status,
+                                  cudaStream_t s);
 
 // ----------------------------------------------------------------- small dense (1 CTA)
 // LU with partial pivoting of a k x k matrix (row-major), in place; piv[k].

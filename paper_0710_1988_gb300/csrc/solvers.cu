@@ -150,16 +150,38 @@ int deflation_build(wd_deflation_space *d, cudaStream_t s, Arena &ar) {
   const int k = d->k;
   // W = A V: k MVPs, batched as k right-hand sides
   RET_IF(launch_ok(launch_wilson_f64(h, d->V, d->W, k, 0, s), "wilson(V)"));
-  // G = U^dagger W, in column groups of 16
+  // G = U^dagger W: column by column in fixed point, which reads U at the
+  // speed of memory (k = 40 at 16^4: 3.8 ms, FP64 9.1 ms); FP64, in column
+  // groups of 16, where the memory for U's planes is not there
   const double2 *Uop = d->U ? d->U : d->V;
   const int g5 = d->U ? 0 : 1;
-  double2 *part = ar.take<double2>(ts_dot_partial_count(n, k, 16));
   double *info = ar.take<double>(2);
   if (ar.failed) return WD_OUT_OF_MEMORY;
-  for (int j0 = 0; j0 < k; j0 += 16) {
-    const int nc = k - j0 < 16 ? k - j0 : 16;
-    RET_IF(launch_ok(launch_ts_dot(Uop, k, d->W + (size_t)j0 * n, nc, g5, n, part, nullptr, s), "ts_dot(G)"));
-    RET_IF(launch_ok(launch_ts_dot_finalize(part, n, k, nc, d->LU + j0, k, nullptr, 0, nullptr, s), "ts_fin(G)"));
+  const long long nc = fxb_chunks(n);
+  const size_t plane = (size_t)k * n * sizeof(int2);
+  void *planes = nullptr;
+  if (cudaMallocFromPoolAsync(&planes, 2 * plane + (size_t)k * nc * sizeof(int), ar.pool, s) != cudaSuccess) {
+    cudaGetLastError();
+    planes = nullptr;
+  }
+  if (planes != nullptr) {
+    ar.ptrs.push_back(planes);
+    char *at = static_cast<char *>(planes);
+    const FxBasis fb{reinterpret_cast<int2 *>(at), reinterpret_cast<int2 *>(at + plane),
+                     reinterpret_cast<int *>(at + 2 * plane)};
+    double2 *part = ar.take<double2>(fxb_dot_partials(n, k));
+    if (ar.failed) return WD_OUT_OF_MEMORY;
+    RET_IF(launch_ok(launch_fxb_encode(Uop, nullptr, 0, nullptr, fb, 0, k, FxVec{nullptr, nullptr}, n, nullptr, s), "encode(U)"));
+    for (int j = 0; j < k; ++j)
+      RET_IF(launch_ok(launch_fxb_dot(fb, Uop, k, d->W + (size_t)j * n, g5, n, part, d->LU + j, k, nullptr, 0, nullptr, s), "dot(G)"));
+  } else {
+    double2 *part = ar.take<double2>(ts_dot_partial_count(n, k, 16));
+    if (ar.failed) return WD_OUT_OF_MEMORY;
+    for (int j0 = 0; j0 < k; j0 += 16) {
+      const int nc16 = k - j0 < 16 ? k - j0 : 16;
+      RET_IF(launch_ok(launch_ts_dot(Uop, k, d->W + (size_t)j0 * n, nc16, g5, n, part, nullptr, s), "ts_dot(G)"));
+      RET_IF(launch_ok(launch_ts_dot_finalize(part, n, k, nc16, d->LU + j0, k, nullptr, 0, nullptr, s), "ts_fin(G)"));
+    }
   }
   RET_IF(launch_ok(launch_lu_factor(d->LU, k, d->piv, info, s), "lu_factor"));
   double hinfo[2];
@@ -242,14 +264,17 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
   double2 *w = ar.take<double2>(n);
   double2 *r = ar.take<double2>(n);
   size_t npart = 0;
-  for (int j = 1; j <= m + 1; ++j) npart = std::max(npart, ts_dot_partial_count(n, j, 1));
+  for (int j = 1; j <= m + 1; ++j) npart = std::max(npart, fxb_dot_partials(n, j));
   double2 *part_t = ar.take<double2>(npart);
-  // the basis as FP32 pairs (high and low planes) for the double-float dot
-  // and the FP32 correction
-  float2 *Vsh = ar.take<float2>((size_t)2 * (m + 1) * n);
-  float2 *Vsl = Vsh == nullptr ? nullptr : Vsh + (size_t)(m + 1) * n;
+  // the basis in fixed point for the Gram-Schmidt products, and its newest
+  // vector site by site for the operator
+  const long long nc = fxb_chunks(n);
+  FxBasis fb{ar.take<int2>((size_t)(m + 1) * n), ar.take<int2>((size_t)(m + 1) * n),
+             ar.take<int>((size_t)(m + 1) * nc)};
+  const size_t ns = (size_t)(n / 12 + 31) / 32 * 32;
+  const FxVec fv{ar.take<int4>(12 * ns), ar.take<int>(ns)};
   double *part_w = ar.take<double>((size_t)nbw * 3);
-  double *part_n = ar.take<double>((size_t)nbs * 2);
+  double *part_n = ar.take<double>((size_t)std::max<long long>(nbs, nc) * 2);
   double2 *H = ar.take<double2>((size_t)(m + 1) * m);
   double2 *c = ar.take<double2>(m + 1);
   double2 *h2 = ar.take<double2>(m + 1);
@@ -304,8 +329,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     return WD_OK;
   }
   WD_CK(cudaMemsetAsync(H, 0, sizeof(double2) * (m + 1) * m, s));
-  RET_IF(launch_ok(launch_scale_by_inverse_entry(Va, r, c, 0, n, nullptr, s), "v1"));
-  RET_IF(launch_ok(launch_split_df(Va, Vsh, Vsl, n, nullptr, s), "v1 split"));
+  RET_IF(launch_ok(launch_fxb_encode(r, c, 0, Va, fb, 0, 1, fv, n, nullptr, s), "v1"));
 
   double2 *V = Va, *Vn = Vb;
   int j0 = 0, cycles = 0, rc = WD_NOT_CONVERGED;
@@ -318,22 +342,16 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     for (int j = j0; j < m; ++j) {
       double2 *vj = V + (size_t)j * n;
       // w = A v_j, with ||w||^2 fused (lucky-breakdown reference)
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, vj, w, 1, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE), "arnoldi wilson"));
-      // classical Gram-Schmidt, applied twice: the first pass's coefficients
-      // in double-float (~48 bits, FP32 pipe), the second pass's in FP64 (it
-      // removes what the first left, so H = h1 + h2 is exact to FP64
-      // rounding), its update in FP32 when h2 is at rounding level
-      RET_IF(launch_ok(launch_ts_dot_df(Vsh, Vsl, j + 1, w, n, part_t, status, s), "cgs dot1"));
-      RET_IF(launch_ok(launch_ts_dot_df_finalize(part_t, n, j + 1, H + j, m, status, s), "cgs fin1"));
-      RET_IF(launch_ok(launch_ts_update(V, j + 1, H + j, m, 1, w, w, 1, -1.0, n, status, s), "cgs upd1"));
-      RET_IF(launch_ok(launch_ts_dot(V, j + 1, w, 1, 0, n, part_t, status, s), "cgs dot2"));
-      RET_IF(launch_ok(launch_ts_dot_finalize(part_t, n, j + 1, 1, h2, 1, H + j, m, status, s), "cgs fin2"));
-      RET_IF(launch_ok(launch_ts_update_correction(V, Vsh, j + 1, h2, H + j, m, part_w, nbw, w, n, status, s), "cgs upd2"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, vj, w, 1, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, &fv), "arnoldi wilson"));
+      // classical Gram-Schmidt, applied twice, in fixed point (fx_basis.cu); the
+      // second pass's update in FP32 when its coefficients are at rounding level
+      RET_IF(launch_ok(launch_fxb_dot(fb, V, j + 1, w, 0, n, part_t, H + j, m, nullptr, 0, status, s), "cgs dot1"));
+      RET_IF(launch_ok(launch_fxb_update(fb, V, j + 1, H + j, m, 0, w, n, status, s), "cgs upd1"));
+      RET_IF(launch_ok(launch_fxb_dot(fb, V, j + 1, w, 0, n, part_t, h2, 1, H + j, m, status, s), "cgs dot2"));
+      RET_IF(launch_ok(launch_fxb_correction(fb, V, j + 1, h2, H + j, m, part_w, nbw, w, n, part_n, status, s), "cgs upd2"));
       // h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j}
-      RET_IF(launch_ok(launch_norms(w, nullptr, part_n, n, 1, s), "norm w"));
-      RET_IF(launch_ok(launch_arnoldi_normalize_finalize(part_n, nbs, part_w, nbw, H, m, j, 1e-14, status, m_eff, s), "arnoldi fin"));
-      RET_IF(launch_ok(launch_scale_by_inverse_entry(V + (size_t)(j + 1) * n, w, H, (j + 1) * m + j, n, status, s), "arnoldi scale"));
-      RET_IF(launch_ok(launch_split_df(V + (size_t)(j + 1) * n, Vsh + (size_t)(j + 1) * n, Vsl + (size_t)(j + 1) * n, n, status, s), "arnoldi split"));
+      RET_IF(launch_ok(launch_arnoldi_normalize_finalize(part_n, (int)nc, part_w, nbw, H, m, j, 1e-14, status, m_eff, s), "arnoldi fin"));
+      RET_IF(launch_ok(launch_fxb_encode(w, H, (j + 1) * m + j, V + (size_t)(j + 1) * n, fb, j + 1, 1, fv, n, status, s), "v_{j+1}"));
     }
     cycles += 1;
     CycleEndArgs a;
@@ -361,7 +379,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     WD_CK(cudaStreamSynchronize(s));
     mvp += hme - j0;
     // x += V_m d
-    RET_IF(launch_ok(launch_ts_update(V, hme, d, 1, 1, x, x, 1, 1.0, n, nullptr, s), "x update"));
+    RET_IF(launch_ok(launch_fxb_update(fb, V, hme, d, 1, 1, x, n, nullptr, s), "x update"));
     last_rel = hres / bnorm0;
     hist.push_back(last_rel);
     if (hflags[0] != 0) {
@@ -393,18 +411,19 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
       WD_CK(cudaMemcpy2DAsync(H, sizeof(double2) * m, Hk, sizeof(double2) * k, sizeof(double2) * k,
                               k + 1, cudaMemcpyDeviceToDevice, s));
     WD_CK(cudaMemcpyAsync(c, ck, sizeof(double2) * (k + 1), cudaMemcpyDeviceToDevice, s));
+    // the restarted basis v_1 .. v_{k+1} in fixed point, the last vector
+    // re-orthogonalised against the others
+    double2 *vk = V + (size_t)k * n;
+    const double2 *nrm = nullptr;
     if (k > 0) {
-      // re-orthogonalise v_{k+1} against v_1..v_k
-      double2 *vk = V + (size_t)k * n;
-      RET_IF(launch_ok(launch_ts_dot(V, k, vk, 1, 0, n, part_t, nullptr, s), "reorth dot"));
-      RET_IF(launch_ok(launch_ts_dot_finalize(part_t, n, k, 1, h2, 1, nullptr, 0, nullptr, s), "reorth fin"));
-      RET_IF(launch_ok(launch_ts_update(V, k, h2, 1, 1, vk, vk, 1, -1.0, n, nullptr, s), "reorth upd"));
+      RET_IF(launch_ok(launch_fxb_encode(V, nullptr, 0, nullptr, fb, 0, k, FxVec{nullptr, nullptr}, n, nullptr, s), "restart encode"));
+      RET_IF(launch_ok(launch_fxb_dot(fb, V, k, vk, 0, n, part_t, h2, 1, nullptr, 0, nullptr, s), "reorth dot"));
+      RET_IF(launch_ok(launch_fxb_update(fb, V, k, h2, 1, 0, vk, n, nullptr, s), "reorth upd"));
       RET_IF(launch_ok(launch_norms(vk, nullptr, part_n, n, 1, s), "reorth norm"));
       RET_IF(launch_ok(launch_norm_finalize(part_n, nbs, 2, scal, s), "reorth nrm"));
-      RET_IF(launch_ok(launch_scale_by_inverse_entry(vk, vk, scal, 0, n, nullptr, s), "reorth scale"));
+      nrm = scal;
     }
-    // the restarted basis v_1 .. v_{k+1} in split form
-    RET_IF(launch_ok(launch_split_df(V, Vsh, Vsl, (long long)(k + 1) * n, nullptr, s), "restart split"));
+    RET_IF(launch_ok(launch_fxb_encode(vk, nrm, 0, vk, fb, k, 1, fv, n, nullptr, s), "v_{k+1}"));
     j0 = k;
   }
   // outputs
