@@ -27,86 +27,7 @@ __device__ __forceinline__ bool sys_on(const int *status, unsigned mask, int r) 
   return status == nullptr || ((mask >> status[r]) & 1u);
 }
 
-// ----------------------------------------------------------------- BiCGStab updates
-
-__global__ void __launch_bounds__(SB_THREADS)
-bicg_update_p_kernel(double2 *__restrict__ p, const double2 *__restrict__ rv,
-                     const double2 *__restrict__ vv, const BicgScalars *__restrict__ sc,
-                     const int *__restrict__ status, long long n) {
-  const int r = blockIdx.y;
-  if (!sys_on(status, M_ACTIVE, r)) return;  // uniform per block
-  // beta = (rho / rho_old) (alpha / omega), once per block: two complex
-  // divisions in every thread cost more FP64 issue than the few elements
-  // each thread updates
-  __shared__ double2 s_bm[2];
-  if (threadIdx.x == 0) {
-    const BicgScalars S = sc[r];
-    const double2 beta = cmul(cdiv(S.rho, S.rho_old), cdiv(S.alpha, S.omega));
-    s_bm[0] = beta;
-    s_bm[1] = cneg(cmul(beta, S.omega));
-  }
-  __syncthreads();
-  const double2 beta = s_bm[0], mbo = s_bm[1];
-  const long long off = (long long)r * n;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double2 pi = p[off + i], vi = vv[off + i], ri = rv[off + i];
-    // p = r + beta (p - omega v) = r + beta p - (beta omega) v: 8 FMA
-    p[off + i] = cfma(mbo, vi, cfma(beta, pi, ri));
-  }
-}
-
-__global__ void __launch_bounds__(SB_THREADS)
-bicg_update_s_kernel(double2 *__restrict__ s, const double2 *__restrict__ rv,
-                     const double2 *__restrict__ vv, const BicgScalars *__restrict__ sc,
-                     const int *__restrict__ status, long long n) {
-  const int r = blockIdx.y;
-  if (!sys_on(status, M_ACTIVE, r)) return;
-  const double2 al = sc[r].alpha;
-  const double2 mal = make_double2(-al.x, -al.y);
-  const long long off = (long long)r * n;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    s[off + i] = cfma(mal, vv[off + i], rv[off + i]);  // s = r - alpha v
-}
-
-__global__ void __launch_bounds__(SB_THREADS)
-bicg_update_xr_kernel(double2 *__restrict__ x, double2 *__restrict__ rv,
-                      const double2 *__restrict__ p, const double2 *__restrict__ sv,
-                      const double2 *__restrict__ t, const double2 *__restrict__ rhat,
-                      const BicgScalars *__restrict__ sc, const int *__restrict__ status,
-                      double *__restrict__ partial, long long n) {
-  const int r = blockIdx.y;
-  if (!sys_on(status, M_ACTIVE, r)) return;
-  const double2 al = sc[r].alpha, om = sc[r].omega;
-  const double2 mom = make_double2(-om.x, -om.y);
-  const long long off = (long long)r * n;
-  double red[3] = {0.0, 0.0, 0.0};
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double2 si = sv[off + i];
-    double2 xi = x[off + i];
-    xi = cfma(al, p[off + i], xi);      // x += alpha p + omega s
-    xi = cfma(om, si, xi);
-    x[off + i] = xi;
-    const double2 ri = cfma(mom, t[off + i], si);  // r = s - omega t
-    rv[off + i] = ri;
-    const double2 h = rhat[off + i];
-    red[0] = fma(h.x, ri.x, red[0]);
-    red[0] = fma(h.y, ri.y, red[0]);
-    red[1] = fma(h.x, ri.y, red[1]);
-    red[1] = fma(-h.y, ri.x, red[1]);
-    red[2] = fma(ri.x, ri.x, red[2]);
-    red[2] = fma(ri.y, ri.y, red[2]);
-  }
-  block_sum<3>(red);
-  if (threadIdx.x == 0) {
-    double *d = partial + ((long long)r * gridDim.x + blockIdx.x) * 3;
-    d[0] = red[0];
-    d[1] = red[1];
-    d[2] = red[2];
-  }
-}
+// ----------------------------------------------------------------- vectors and norms
 
 __global__ void __launch_bounds__(SB_THREADS)
 sub_norm_kernel(double2 *__restrict__ out, const double2 *__restrict__ a,
@@ -168,29 +89,6 @@ restart_vectors_kernel(double2 *__restrict__ rhat, const double2 *__restrict__ r
   }
 }
 
-cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v,
-                                 const BicgScalars *sc, const int *status, long long n,
-                                 int nrhs, cudaStream_t s) {
-  ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_p_kernel<<<dim3(stream_blocks(n), nrhs), SB_THREADS, 0, s>>>(p, r, v, sc, status, n);
-  return cudaGetLastError();
-}
-cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v,
-                                 const BicgScalars *sc, const int *status, long long n,
-                                 int nrhs, cudaStream_t s) {
-  ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_s_kernel<<<dim3(stream_blocks(n), nrhs), SB_THREADS, 0, s>>>(sv, r, v, sc, status, n);
-  return cudaGetLastError();
-}
-cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, const double2 *sv,
-                                  const double2 *t, const double2 *rhat, const BicgScalars *sc,
-                                  const int *status, double *partial, long long n, int nrhs,
-                                  cudaStream_t s) {
-  ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_xr_kernel<<<dim3(stream_blocks(n), nrhs), SB_THREADS, 0, s>>>(
-      x, r, p, sv, t, rhat, sc, status, partial, n);
-  return cudaGetLastError();
-}
 cudaError_t launch_sub_norm(double2 *out, const double2 *a, const double2 *b, const int *status,
                             unsigned mask, double *partial, long long n, int nrhs,
                             cudaStream_t s) {
@@ -233,10 +131,16 @@ __device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
   S.rho_old = make_double2(1.0, 0.0);
   S.alpha = make_double2(1.0, 0.0);
   S.omega = make_double2(1.0, 0.0);
+  S.beta = S.rho;
+  S.mbo = cneg(S.rho);
   S.rhat_norm = sqrt(rr);
   S.rnorm = sqrt(rr);
 }
 
+// One block per system.  An FP64 division, square root or hypot is a chain of
+// some ten FP64 instructions of 64 clocks each, so the independent ones of a
+// kind go to different warps (the solver waits for this kernel three times an
+// iteration).
 __global__ void __launch_bounds__(256)
 bicg_finalize_kernel(int kind, const double *__restrict__ partial, int nb, BicgScalars *sc,
                      int *status, double *hist, int hist_len) {
@@ -263,37 +167,60 @@ bicg_finalize_kernel(int kind, const double *__restrict__ partial, int nb, BicgS
   }
   if (kind == FIN_ALPHA || kind == FIN_OMEGA || kind == FIN_RHO) {
     if (st != ST_ACTIVE) return;
+    __shared__ double sum[3];
+    __shared__ double2 quot[2];
+    __shared__ double root[2];
+    BicgScalars &S = sc[r];
     double v[3];
     reduce_partials<3>(partial, nb, r, v);
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) sum[q] = v[q];
+    }
+    __syncthreads();
+    const double2 d = make_double2(sum[0], sum[1]);
+    const double n2 = sum[2];
+    if (threadIdx.x == 0) {
+      if (kind == FIN_ALPHA) quot[0] = cdiv(S.rho, d);
+      else if (kind == FIN_OMEGA) quot[0].x = n2 == 0.0 ? 0.0 : d.x / n2;
+      else quot[0] = cdiv(d, S.rho);   // rho / rho_old
+    } else if (threadIdx.x == 32) {
+      if (kind == FIN_OMEGA) quot[0].y = n2 == 0.0 ? 0.0 : d.y / n2;
+      else root[0] = sqrt(n2);
+    } else if (threadIdx.x == 64 && kind != FIN_OMEGA) {
+      root[1] = hypot(d.x, d.y);
+    } else if (threadIdx.x == 96 && kind == FIN_RHO) {
+      quot[1] = cdiv(S.alpha, S.omega);
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
-    BicgScalars &S = sc[r];
     if (kind == FIN_ALPHA) {  // <r_hat, v>, ||v||^2
-      const double2 rv = make_double2(v[0], v[1]);
       S.mvp += 1;
-      if (hypot(rv.x, rv.y) <= 1e-30 * S.rhat_norm * sqrt(v[2])) {
+      if (root[1] <= 1e-30 * S.rhat_norm * root[0]) {
         status[r] = ST_BREAKDOWN;
         return;
       }
-      S.alpha = cdiv(S.rho, rv);
+      S.alpha = quot[0];
     } else if (kind == FIN_OMEGA) {  // <t, s>, ||t||^2
-      if (v[2] == 0.0) {  // t = A s = 0 means s = 0: x += alpha p finishes
-        S.omega = make_double2(0.0, 0.0);
-      } else {
-        S.mvp += 1;
-        S.omega = cdiv(make_double2(v[0], v[1]), make_double2(v[2], 0.0));
-      }
+      // t = A s = 0 means s = 0: omega = 0, x += alpha p finishes
+      if (n2 != 0.0) S.mvp += 1;
+      S.omega = quot[0];
     } else {  // FIN_RHO: <r_hat, r>, ||r||^2
+      const double rnorm = root[0], rel = rnorm / S.bnorm;
+      const double2 beta = cmul(quot[0], quot[1]);
+      S.beta = beta;
+      S.mbo = cneg(cmul(beta, S.omega));
       S.rho_old = S.rho;
-      S.rho = make_double2(v[0], v[1]);
-      S.rnorm = sqrt(v[2]);
+      S.rho = d;
+      S.rnorm = rnorm;
       S.iters += 1;
       if (hist != nullptr && S.iters <= hist_len)
-        hist[(long long)r * hist_len + S.iters - 1] = S.rnorm / S.bnorm;
-      if (S.rnorm / S.bnorm <= S.tol)
+        hist[(long long)r * hist_len + S.iters - 1] = rel;
+      if (rel <= S.tol)
         status[r] = ST_RECURSIVE;
       else if (S.iters >= S.max_iter)
         status[r] = ST_MAXITER;
-      else if (hypot(S.rho.x, S.rho.y) <= 1e-30 * S.rhat_norm * S.rnorm)
+      else if (root[1] <= 1e-30 * S.rhat_norm * rnorm)
         status[r] = ST_BREAKDOWN;
     }
     return;

@@ -258,7 +258,7 @@ fx_encode_kernel(const double2 *__restrict__ in, FxVec out, long long sites, siz
   out.e[(long long)r * sites + s] = E;
   int4 *o = out.v + (size_t)r * 12 * tiled + fx_at((unsigned)s, 12);
 #pragma unroll
-  for (int c = 0; c < 12; ++c) o[c * FX_TILE] = fx_slices(p[c], max(e, 1));
+  for (int c = 0; c < 12; ++c) o[c * FX_TILE] = fx_slices(p[c], max(e, FX_EMIN));
 }
 
 // sum over the eight hops of one site in FP64: the sites next to a value that
@@ -340,7 +340,7 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
     hops_f64<DAG>(in64 + (size_t)r * 12 * V, links, nb, s, mine);
   }
   __syncwarp();
-  double red[3] = {0.0, 0.0, 0.0};
+  double2 dv[6], da[6];   // the epilogue's operands
   const long long first = sb * FX_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
   const size_t base = ((size_t)r * V + first) * 12;
   const int count = 12 * (int)max(0LL, min(16LL, g.V - first));
@@ -359,26 +359,20 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
         v.y = fma(m, p.x, v.y);
       }
       out[base + c] = v;
-      if (EPI != EPI_NONE) {  // <aux, out> or <out, in>, and <out, out>
-        const double2 a = EPI == EPI_DOT ? __ldg(aux + base + c) : v;
-        const double2 b = EPI == EPI_DOT ? v : p;
-        red[0] = fma(a.x, b.x, red[0]);
-        red[0] = fma(a.y, b.y, red[0]);
-        red[1] = fma(a.x, b.y, red[1]);
-        red[1] = fma(-a.y, b.x, red[1]);
-        red[2] = fma(v.x, v.x, red[2]);
-        red[2] = fma(v.y, v.y, red[2]);
+      if (EPI != EPI_NONE) {
+        dv[q] = v;
+        da[q] = EPI == EPI_DOT ? __ldg(aux + base + c) : p;
       }
+    } else if (EPI != EPI_NONE) {
+      dv[q] = da[q] = make_double2(0.0, 0.0);
     }
   }
-  if (EPI != EPI_NONE) {
-    block_sum<3>(red);
-    if (threadIdx.x == 0) {
-      const long long nsb = gridDim.x / (unsigned)nrhs;
-      double *dst = partial + ((long long)r * nsb + sb) * 3;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) dst[q] = red[q];
-    }
+  if (EPI != EPI_NONE) {  // <aux, out> or <out, in>, and <out, out>
+    __shared__ double sums[2 * FX_SITES / 32][3];
+    double2 d = fx_warp_dots<6>(da, dv);
+    if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, in>: the conjugate
+    const long long nsb = gridDim.x / (unsigned)nrhs;
+    fx_block_dots<2 * FX_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
   }
 }
 

@@ -286,14 +286,14 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         const int comp = (c < 3 ? 0 : 3) + 3 * sp + c;
-        o[comp * FX_TILE] = fx_slices(v[c], max(e, 1));
+        o[comp * FX_TILE] = fx_slices(v[c], max(e, FX_EMIN));
         if (Eo == FX_SPECIAL) out[off + (size_t)i * 12 + comp] = v[c];
       }
       if (sp == 0) outfx.e[(size_t)r * Vh + i] = Eo;
     }
     return;
   }
-  double red[3] = {0.0, 0.0, 0.0};
+  double2 dv[6], da[6];   // the epilogue's operands
   const long long first = sb * EO_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
   const size_t base = off + (size_t)first * 12;
   const int count = 12 * (int)max(0LL, min(16LL, (long long)Vh - first));
@@ -318,23 +318,20 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
         v.y = fma(kappa, h.y, sm.y);
       }
       out[base + c] = v;
-      if (EPI != EPI_NONE) {  // <aux, out> or <out, same>, and <out, out>
-        const double2 a = EPI == EPI_DOT ? __ldg(aux + base + c) : v;
-        const double2 b = EPI == EPI_DOT ? v : sm;
-        red[0] = fma(a.x, b.x, fma(a.y, b.y, red[0]));
-        red[1] = fma(a.x, b.y, fma(-a.y, b.x, red[1]));
-        red[2] = fma(v.x, v.x, fma(v.y, v.y, red[2]));
+      if (EPI != EPI_NONE) {
+        dv[q] = v;
+        da[q] = EPI == EPI_DOT ? __ldg(aux + base + c) : sm;
       }
+    } else if (EPI != EPI_NONE) {
+      dv[q] = da[q] = make_double2(0.0, 0.0);
     }
   }
-  if (EPI != EPI_NONE) {
-    block_sum<3>(red);
-    if (threadIdx.x == 0) {
-      const long long nsb = gridDim.x / (unsigned)nrhs;
-      double *d = partial + ((long long)r * nsb + sb) * 3;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) d[q] = red[q];
-    }
+  if (EPI != EPI_NONE) {  // <aux, out> or <out, same>, and <out, out>
+    __shared__ double sums[2 * EO_SITES / 32][3];
+    double2 d = fx_warp_dots<6>(da, dv);
+    if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, same>: the conjugate
+    const long long nsb = gridDim.x / (unsigned)nrhs;
+    fx_block_dots<2 * EO_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
   }
 }
 

@@ -56,32 +56,59 @@ __device__ __forceinline__ int fx_site_exponent(int emax, bool allzero) {
   return allzero ? 0 : FX_SPECIAL;
 }
 
-// (hi, lo) slices of x against the site exponent E >= x's own exponent field
-__device__ __forceinline__ int2 fx_slices(double x, int E) {
-  const long long b = __double_as_longlong(x);
-  const int be = (int)((unsigned long long)b >> 52) & 0x7ff;
-  const long long M = (b & 0xFFFFFFFFFFFFFLL) | (be ? 1LL << 52 : 0LL);
-  const int r = min(E - be, 62);
-  long long X = ((M << 3) + (long long)((1ULL << r) >> 1)) >> r;
-  X = b < 0 ? -X : X;
-  const int lo = ((int)(unsigned)X << 3) >> 3;       // low 29 bits, signed
-  return make_int2((int)((X - lo) >> 29), lo);
+// Slices of x against a shared exponent E >= FX_EMIN, x's own exponent field
+// at most E (zeros and subnormals give 0): hi 2^LO + lo = |x| 2^(1049 + LO - E)
+// with the sign on both, |lo| <= 2^(LO - 1).  LO = 29: rounded, the form above;
+// LO = 30: cut off at its last bit (2^-57 of the largest), without spin
+// projections and complex sums the middle products then still fit.  About 17
+// instructions; the shift saturates (PTX), so E needs no clamp.
+template <int LO>
+__device__ __forceinline__ int2 fx_cut(double x, int E) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const unsigned be = (h >> 20) & 0x7ffu;
+  const unsigned long long t = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | l) << 11;
+  unsigned long long Y;
+  asm("shr.u64 %0, %1, %2;" : "=l"(Y) : "l"(t), "r"((unsigned)E - be + 7u));
+  if (LO == 29) Y = (Y + 1) >> 1;
+  const int lo = (int)((unsigned)Y << (32 - LO)) >> (32 - LO);
+  const int hi = (int)((Y + (1ULL << (LO - 1))) >> LO);
+  const int s = (int)h >> 31;
+  return make_int2((hi ^ s) - s, (lo ^ s) - s);
 }
+
+__device__ __forceinline__ int2 fx_slices(double x, int E) { return fx_cut<29>(x, E); }
 
 __device__ __forceinline__ int4 fx_slices(double2 x, int E) {
   const int2 a = fx_slices(x.x, E), b = fx_slices(x.y, E);
   return make_int4(a.x, a.y, b.x, b.y);
 }
 
-// T 2^(E - 1079) rounded to FP64, FX_EMIN <= E <= FX_EMAX
+__device__ __forceinline__ int4 fx_cut30(double2 x, int E) {
+  const int2 a = fx_cut<30>(x.x, E), b = fx_cut<30>(x.y, E);
+  return make_int4(a.x, a.y, b.x, b.y);
+}
+
+// T 2^(E - 1079) rounded to FP64 (halves away from zero), |T| < 2^63,
+// 70 <= E <= 1970
 __device__ __forceinline__ double fx_to_double(long long T, int E) {
-  const unsigned long long a = T < 0 ? 0ULL - (unsigned long long)T : (unsigned long long)T;
-  const int lz = __clzll((long long)a);
-  const unsigned long long m = a << (lz & 63);
-  unsigned long long bits = (m >> 11) + ((m >> 10) & 1ULL) +
-                            ((unsigned long long)((unsigned)E + 6u - (unsigned)lz) << 52);
-  bits |= (unsigned long long)T & 0x8000000000000000ULL;
-  return a == 0 ? 0.0 : __longlong_as_double((long long)bits);
+  const long long s = T >> 63;
+  const unsigned long long a = (unsigned long long)((T ^ s) - s);
+  const int lz = __clzll((long long)a);                       // 1 .. 64
+  const unsigned long long m = ((a << (lz - 1)) + 0x200) >> 10;   // top bit at 52, or 53 after a carry
+  const unsigned hi = (unsigned)(m >> 32) + (((unsigned)E + 6u - (unsigned)lz) << 20);
+  return __hiloint2double((int)(a == 0 ? 0u : hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)m);
+}
+
+// acc += a b: one 32 x 32 + 64-bit multiply-add.  (Sums of products written in
+// C are taken apart into more instructions; only fx_mac below is the faster
+// for it.)
+__device__ __forceinline__ void fx_wide(long long &acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+
+// T 2^(E - 1079) for any E
+__device__ __forceinline__ double fx_scaled(long long T, int E) {
+  return E >= 70 && E <= 1970 ? fx_to_double(T, E) : ldexp((double)T, E - 1079);
 }
 
 // X 2^(E - 1078) of a stored site's component
@@ -281,6 +308,102 @@ __device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, i
 #undef FX_SIGN
 #undef FX_READY
 #undef FX_FETCH
+}
+
+// ----------------------------------------------------------------- a warp's entries
+
+// Shared exponent of N entries a lane over the warp: the largest exponent
+// field (at least FX_EMIN) and, in ok, whether fixed point holds every value.
+template <int N>
+__device__ __forceinline__ int fx_warp_exponent(const double2 (&x)[N], bool &ok) {
+  int e = 0;
+  unsigned long long any = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    e = max(e, max(exp_bits(x[i].x), exp_bits(x[i].y)));
+    any |= (unsigned long long)(__double_as_longlong(x[i].x) | __double_as_longlong(x[i].y)) << 1;
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  ok = e <= FX_EMAX && (e >= FX_EMIN || !__any_sync(0xffffffffu, any != 0));
+  return max(e, FX_EMIN);
+}
+
+// <a, v> and ||v||^2 over N <= 8 entries a lane of a warp, in fixed point
+// against the warp's exponents: lane 0 returns (re, ||v||^2), lane 16 (im, ).
+// A lane's sums are below 2^58 (middle 2^60), the warp's below 2^63; a product
+// leaves out 2^-56 of the maxima's, a lane's sum is rounded at 2^-54.  In FP64 this is
+// six FMAs an entry, 76 clocks of a subpartition each for a warp, and as many
+// for every addition of the warp's reduction.
+template <int N>
+__device__ __forceinline__ double2 fx_warp_dots(const double2 (&a)[N], const double2 (&v)[N]) {
+  bool oka, okv;
+  const int ea = fx_warp_exponent(a, oka), ev = fx_warp_exponent(v, okv);
+  const bool upper = threadIdx.x & 16;
+  if (oka && okv) {
+    long long rh = 0, rm = 1LL << 29, ih = 0, im = 1LL << 29, nh = 0, nm = 1LL << 28;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int4 x = fx_cut30(a[i], ea), y = fx_cut30(v[i], ev);
+      fx_wide(rh, x.x, y.x);
+      fx_wide(rm, x.x, y.y);
+      fx_wide(rm, x.y, y.x);
+      fx_wide(rh, x.z, y.z);
+      fx_wide(rm, x.z, y.w);
+      fx_wide(rm, x.w, y.z);
+      fx_wide(ih, x.x, y.z);
+      fx_wide(im, x.x, y.w);
+      fx_wide(im, x.y, y.z);
+      fx_wide(ih, -x.z, y.x);
+      fx_wide(im, -x.z, y.y);
+      fx_wide(im, -x.w, y.x);
+      fx_wide(nh, y.x, y.x);
+      fx_wide(nm, y.x, y.y);
+      fx_wide(nh, y.z, y.z);
+      fx_wide(nm, y.z, y.w);
+    }
+    const long long tr = rh + (rm >> 30), ti = ih + (im >> 30);
+    long long t = (upper ? ti : tr) + __shfl_xor_sync(0xffffffffu, upper ? tr : ti, 16);
+    long long u = nh + (nm >> 29);
+    u += __shfl_xor_sync(0xffffffffu, u, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      t += __shfl_xor_sync(0xffffffffu, t, o);
+      u += __shfl_xor_sync(0xffffffffu, u, o);
+    }
+    return make_double2(fx_scaled(t, ea + ev - 1019), fx_scaled(u, ev + ev - 1019));
+  }
+  double s[3] = {0.0, 0.0, 0.0};   // values that fixed point does not hold
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    s[0] = fma(a[i].x, v[i].x, fma(a[i].y, v[i].y, s[0]));
+    s[1] = fma(a[i].x, v[i].y, fma(-a[i].y, v[i].x, s[1]));
+    s[2] = fma(v[i].x, v[i].x, fma(v[i].y, v[i].y, s[2]));
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+  return make_double2(upper ? s[1] : s[0], s[2]);
+}
+
+// Sum of the warps' fx_warp_dots over the block, written as its three
+// partials <a, v> re, im and ||v||^2.  sh: WARPS entries.
+template <int WARPS>
+__device__ __forceinline__ void fx_block_dots(double2 d, double (*sh)[3], double *dst) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) {
+    sh[w][0] = d.x;
+    sh[w][2] = d.y;
+  } else if (lane == 16) {
+    sh[w][1] = d.x;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < WARPS; ++i) s += sh[i][threadIdx.x];
+    dst[threadIdx.x] = s;
+  }
 }
 
 }  // namespace wd

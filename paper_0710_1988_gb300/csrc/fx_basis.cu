@@ -63,7 +63,7 @@ __device__ __forceinline__ int fxb_exponent(const double2 (&x)[4], int *raw, int
     m = max(m, red[2 * i]);
     z |= red[2 * i + 1];
   }
-  *raw = max(m, 1);
+  *raw = max(m, FX_EMIN);
   return fx_site_exponent(m, z == 0);
 }
 
@@ -116,7 +116,7 @@ fxb_encode_kernel(const double2 *w, const double2 *__restrict__ H, int idx, doub
       if (base + c >= n) continue;
       const unsigned site = (unsigned)((base + c) / 12);
       const int e = site_e[s];
-      fx.v[fx_at(site, 12) + (c - 12 * s) * FX_TILE] = fx_slices(x[q], max(e, 1));
+      fx.v[fx_at(site, 12) + (c - 12 * s) * FX_TILE] = fx_slices(x[q], max(e, FX_EMIN));
       if (c == 12 * s) fx.e[site] = fx_site_exponent(e, site_nz[s] == 0);
     }
   }
@@ -162,17 +162,11 @@ __device__ __forceinline__ void fxb_commit() { asm volatile("cp.async.commit_gro
 template <int N>
 __device__ __forceinline__ void fxb_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// acc += a b: one 32 x 32 + 64-bit multiply-add (the compiler would otherwise
-// take the sums of products apart into twice the instructions)
-__device__ __forceinline__ void fxb_wide(long long &acc, int a, int b) {
-  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
-}
-
 // one real product: (ah, al) (bh, bl) into the high and middle sums
 __device__ __forceinline__ void fxb_mac(long long &h, long long &m, int ah, int al, int bh, int bl) {
-  fxb_wide(h, ah, bh);
-  fxb_wide(m, ah, bl);
-  fxb_wide(m, al, bh);
+  fx_wide(h, ah, bh);
+  fx_wide(m, ah, bl);
+  fx_wide(m, al, bh);
 }
 
 // ----------------------------------------------------------------- dot
@@ -264,7 +258,7 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
     const int jl = lane >> 1;   // this lane's vector
     if (jl < nj) {
       const int Ev = b.ex[(long long)(j0 + jl) * nc + c];
-      if (Ew != FX_SPECIAL && Ev != FX_SPECIAL) sum += ldexp((double)tsum[warp][lane], Ev + Ew - 2098);
+      if (Ew != FX_SPECIAL && Ev != FX_SPECIAL) sum += fx_scaled(tsum[warp][lane], Ev + Ew - 1019);
     }
     __syncwarp();
     // chunks that fixed point does not hold, in FP64
@@ -445,15 +439,7 @@ fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (!(q < 2 ? in0 : in1)) continue;
-    double re, im2;
-    const int E = G - 1019;   // T 2^(E - 1079)
-    if (E >= 70 && E <= 1970) {
-      re = fx_to_double(rh[q], E);
-      im2 = fx_to_double(ih[q], E);
-    } else {
-      re = ldexp((double)rh[q], G - 2098);
-      im2 = ldexp((double)ih[q], G - 2098);
-    }
+    double re = fx_scaled(rh[q], G - 1019), im2 = fx_scaled(ih[q], G - 1019);
     if (add) {
       re = -re;
       im2 = -im2;

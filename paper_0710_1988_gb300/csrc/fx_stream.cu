@@ -1,0 +1,260 @@
+// BiCGStab's vector updates in FP64 storage with fixed-point arithmetic.
+//
+// p = r + beta p - beta omega v, s = r - alpha v, and x += alpha p + omega s,
+// r = s - omega t with <rhat, r> and ||r||^2 take 8, 4 and 18 FP64 FMAs an
+// entry, 4.8, 2.4 and 11 clocks of an SM, where memory delivers their 64, 48 and
+// 112 bytes in 3, 2.2 and 5.3.  So p, x and the dots are formed in integers
+// (fx.cuh: shared exponent, two slices, three multiply-adds a real product, one
+// FP64 addition a real), and s and r, four FMAs an entry each, stay on the FP64
+// pipe beside them.  A warp works on 16 sites (192 entries, six a lane) that
+// share one exponent per operand; a scalar has its own.  Products are kept at
+// 2^-58 of (scalar x largest entry) and leave out 2^-56 of it at most, 2^-58 in
+// the mean: below the two roundings of the FP64 form.  Tiles with infinities,
+// NaN or magnitudes near the ends of FP64's range take FP64.  p and s also leave
+// in the operator's form, site by site, through shared memory so that the
+// writes are contiguous.
+//
+// 16^4, 10 systems, us a launch (FP64 with its separate encoding -> here):
+// p 173 -> 124 (all FP64 but one term: 148), s 97 -> 84 (in integers 111),
+// x and r 285 -> 189 (r in integers too: 219; its memory takes 130).
+#include "cplx.cuh"
+#include "fx.cuh"
+#include "kernels.cuh"
+#include "wd_internal.h"
+
+namespace wd {
+
+namespace {
+
+constexpr int FXS_WARPS = 8, FXS_THREADS = 32 * FXS_WARPS;
+constexpr int FXS_TILE = 192;   // entries of a warp's tile
+
+// a scalar in slices against its own exponent field e (0: not held)
+struct FxScalar {
+  int4 s;
+  int e;
+};
+
+__device__ __forceinline__ FxScalar fxs_scalar(double2 c, bool &ok) {
+  FxScalar r;
+  r.e = max(exp_bits(c.x), exp_bits(c.y));
+  const bool zero = ((__double_as_longlong(c.x) | __double_as_longlong(c.y)) << 1) == 0;
+  ok = ok && (zero || (r.e >= FX_EMIN && r.e <= FX_EMAX));
+  r.e = max(r.e, FX_EMIN);
+  r.s = fx_cut30(c, r.e);
+  return r;
+}
+
+// c z in units 2^(Ec + Ez - 1023 - 1079): |value| < 2^60
+__device__ __forceinline__ longlong2 fxs_mul(const FxScalar &c, int4 z) {
+  long long rh = 0, rm = 1LL << 25, ih = 0, im = 1LL << 25;
+  fx_wide(rh, c.s.x, z.x);
+  fx_wide(rm, c.s.x, z.y);
+  fx_wide(rm, c.s.y, z.x);
+  fx_wide(rh, -c.s.z, z.z);
+  fx_wide(rm, -c.s.z, z.w);
+  fx_wide(rm, -c.s.w, z.z);
+  fx_wide(ih, c.s.x, z.z);
+  fx_wide(im, c.s.x, z.w);
+  fx_wide(im, c.s.y, z.z);
+  fx_wide(ih, c.s.z, z.x);
+  fx_wide(im, c.s.z, z.y);
+  fx_wide(im, c.s.w, z.x);
+  return make_longlong2((rh << 4) + (rm >> 26), (ih << 4) + (im >> 26));
+}
+
+// whether the units of c z can be applied by fx_to_double
+__device__ __forceinline__ bool fxs_in_range(const FxScalar &c, int E) {
+  const int u = c.e + E - 1023;
+  return u >= 70 && u <= 1970;
+}
+
+// a + c1 z1 + c2 z2: E1, E2 the shared exponents of z1, z2
+__device__ __forceinline__ double2 fxs_axpy2(double2 a, const FxScalar &c1, double2 z1, int E1,
+                                             const FxScalar &c2, double2 z2, int E2) {
+  const longlong2 t = fxs_mul(c1, fx_cut30(z1, E1)), u = fxs_mul(c2, fx_cut30(z2, E2));
+  const int E = c1.e + E1 - 1023, F = c2.e + E2 - 1023;
+  const int dt = min(max(F - E, 0), 63), du = min(max(E - F, 0), 63);
+  const long long re = fx_align(t.x, dt) + fx_align(u.x, du), im = fx_align(t.y, dt) + fx_align(u.y, du);
+  const int G = max(E, F);
+  return make_double2(a.x + fx_to_double(re, G), a.y + fx_to_double(im, G));
+}
+
+struct FxsTile {
+  int4 v[16 * 13];   // 13 a site: no bank conflicts
+  int e[16];
+  int nz[16];
+};
+
+// The warp's 16 sites of x (entry q 32 + lane) into the operator's form;
+// first: its first site, count: its entries.
+__device__ __forceinline__ void fxs_emit(FxsTile &t, const double2 (&x)[6], FxVec fx, int r,
+                                         long long sites, size_t tiled, long long first, int count) {
+  const int lane = threadIdx.x & 31;
+  if (lane < 16) t.e[lane] = t.nz[lane] = 0;
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int s = (q * 32 + lane) / 12;
+    atomicMax(&t.e[s], max(exp_bits(x[q].x), exp_bits(x[q].y)));
+    if ((__double_as_longlong(x[q].x) | __double_as_longlong(x[q].y)) << 1) t.nz[s] = 1;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int c = q * 32 + lane, s = c / 12;
+    t.v[c + s] = fx_slices(x[q], max(t.e[s], FX_EMIN));
+  }
+  __syncwarp();
+  const int site = lane & 15;
+  if (12 * site < count) {
+    int4 *o = fx.v + (size_t)r * 12 * tiled + fx_at((unsigned)(first + site), 12);
+#pragma unroll
+    for (int c = 0; c < 12; c += 2) o[(c + (lane >> 4)) * FX_TILE] = t.v[site * 13 + c + (lane >> 4)];
+    if (lane < 16) fx.e[(size_t)r * sites + first + site] = fx_site_exponent(t.e[site], t.nz[site] == 0);
+  }
+  __syncwarp();
+}
+
+}  // namespace
+
+// TWO: out = a + beta out + mbo z (the p update); else out = a - alpha z (s)
+template <bool TWO>
+__global__ void __launch_bounds__(FXS_THREADS, 2)
+bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, const double2 *__restrict__ z,
+                      FxVec fx, size_t tiled, const BicgScalars *__restrict__ sc,
+                      const int *__restrict__ status, long long n) {
+  const int r = blockIdx.y;
+  if (!((M_ACTIVE >> status[r]) & 1u)) return;   // uniform per block
+  extern __shared__ __align__(16) unsigned char fxs_smem[];
+  FxsTile &tile = reinterpret_cast<FxsTile *>(fxs_smem)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const double2 c1 = TWO ? sc[r].beta : cneg(sc[r].alpha), c2 = TWO ? sc[r].mbo : c1;
+  bool held = true;
+  const FxScalar s1 = fxs_scalar(c1, held), s2 = fxs_scalar(c2, held);
+  const size_t off = (size_t)r * n;
+  const long long tiles = (n + FXS_TILE - 1) / FXS_TILE;
+  for (long long t = (long long)blockIdx.x * FXS_WARPS + (threadIdx.x >> 5); t < tiles;
+       t += (long long)gridDim.x * FXS_WARPS) {
+    const long long base = t * FXS_TILE;
+    const int count = (int)min((long long)FXS_TILE, n - base);
+    double2 y[6], w[6], x[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int c = q * 32 + lane;
+      const size_t i = off + base + c;
+      const bool in = c < count;
+      x[q] = in ? a[i] : make_double2(0.0, 0.0);
+      w[q] = in ? z[i] : make_double2(0.0, 0.0);
+      if (TWO) y[q] = in ? out[i] : make_double2(0.0, 0.0);
+    }
+    bool ok = false;
+    int Ey = FX_EMIN, Ez = FX_EMIN;
+    if (TWO) {
+      bool o1;
+      Ez = fx_warp_exponent(w, ok);
+      Ey = fx_warp_exponent(y, o1);
+      ok = ok && o1 && held && fxs_in_range(s1, Ey) && fxs_in_range(s2, Ez);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      if (TWO)
+        x[q] = ok ? fxs_axpy2(x[q], s1, y[q], Ey, s2, w[q], Ez) : cfma(c2, w[q], cfma(c1, y[q], x[q]));
+      else
+        x[q] = cfma(c1, w[q], x[q]);
+      const int c = q * 32 + lane;
+      if (c < count) out[off + base + c] = x[q];
+    }
+    if (fx.v != nullptr) fxs_emit(tile, x, fx, r, n / 12, tiled, base / 12, count);
+  }
+}
+
+__global__ void __launch_bounds__(FXS_THREADS, 2)
+bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, const double2 *__restrict__ p,
+                         const double2 *__restrict__ sv, const double2 *__restrict__ t,
+                         const double2 *__restrict__ rhat, const BicgScalars *__restrict__ sc,
+                         const int *__restrict__ status, double *__restrict__ partial, long long n) {
+  const int r = blockIdx.y;
+  if (!((M_ACTIVE >> status[r]) & 1u)) return;
+  __shared__ double sums[FXS_WARPS][3];
+  const int lane = threadIdx.x & 31;
+  const double2 al = sc[r].alpha, om = sc[r].omega;
+  bool held = true;
+  const FxScalar sa = fxs_scalar(al, held), so = fxs_scalar(om, held);
+  const size_t off = (size_t)r * n;
+  const long long tiles = (n + FXS_TILE - 1) / FXS_TILE;
+  const double2 zero = make_double2(0.0, 0.0);
+  double2 dots = zero;
+  for (long long w = (long long)blockIdx.x * FXS_WARPS + (threadIdx.x >> 5); w < tiles;
+       w += (long long)gridDim.x * FXS_WARPS) {
+    const long long base = w * FXS_TILE;
+    const int count = (int)min((long long)FXS_TILE, n - base);
+    double2 s[6], u[6], h[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const size_t i = off + base + q * 32 + lane;
+      const bool in = q * 32 + lane < count;
+      s[q] = in ? sv[i] : zero;
+      u[q] = in ? p[i] : zero;
+      h[q] = in ? x[i] : zero;
+    }
+    bool os, ok;
+    const int Es = fx_warp_exponent(s, os), Ep = fx_warp_exponent(u, ok);
+    ok = ok && os && held && fxs_in_range(sa, Ep) && fxs_in_range(so, Es);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {   // x += alpha p + omega s
+      const double2 xi = ok ? fxs_axpy2(h[q], sa, u[q], Ep, so, s[q], Es)
+                            : cfma(om, s[q], cfma(al, u[q], h[q]));
+      if (q * 32 + lane < count) x[off + base + q * 32 + lane] = xi;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const size_t i = off + base + q * 32 + lane;
+      const bool in = q * 32 + lane < count;
+      u[q] = in ? t[i] : zero;
+      h[q] = in ? rhat[i] : zero;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {   // r = s - omega t
+      s[q] = cfma(cneg(om), u[q], s[q]);
+      if (q * 32 + lane < count) rv[off + base + q * 32 + lane] = s[q];
+    }
+    const double2 d = fx_warp_dots<6>(h, s);
+    dots = cadd(dots, d);
+  }
+  fx_block_dots<FXS_WARPS>(dots, sums, partial + ((long long)r * gridDim.x + blockIdx.x) * 3);
+}
+
+// blocks (per system) of the update kernels: a tile a warp up to four blocks per SM
+int fxs_blocks(long long n) {
+  const long long b = ((n + FXS_TILE - 1) / FXS_TILE + FXS_WARPS - 1) / FXS_WARPS;
+  return (int)(b > 608 ? 608 : b < 1 ? 1 : b);
+}
+
+cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v, FxVec fx,
+                                 const BicgScalars *sc, const int *status, long long n,
+                                 int nrhs, cudaStream_t s) {
+  ProfLaunch prof_(PC_STREAM, s);
+  bicg_update_fx_kernel<true><<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, FXS_WARPS * sizeof(FxsTile), s>>>(
+      p, r, v, fx, fx_sites(n / 12), sc, status, n);
+  return cudaGetLastError();
+}
+cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v, FxVec fx,
+                                 const BicgScalars *sc, const int *status, long long n,
+                                 int nrhs, cudaStream_t s) {
+  ProfLaunch prof_(PC_STREAM, s);
+  bicg_update_fx_kernel<false><<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, FXS_WARPS * sizeof(FxsTile), s>>>(
+      sv, r, v, fx, fx_sites(n / 12), sc, status, n);
+  return cudaGetLastError();
+}
+cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, const double2 *sv,
+                                  const double2 *t, const double2 *rhat, const BicgScalars *sc,
+                                  const int *status, double *partial, long long n, int nrhs,
+                                  cudaStream_t s) {
+  ProfLaunch prof_(PC_STREAM, s);
+  bicg_update_xr_fx_kernel<<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc,
+                                                                             status, partial, n);
+  return cudaGetLastError();
+}
+
+}  // namespace wd

@@ -41,6 +41,7 @@ constexpr unsigned M_ALL = 0xffffffffu;
 // BiCGStab scalars of one system, device resident.
 struct BicgScalars {
   double2 rho, rho_old, alpha, omega;
+  double2 beta, mbo;   // of the next p = r + beta p + mbo v: (rho / rho_old)(alpha / omega), -beta omega
   double bnorm, rhat_norm, rnorm, true_rel, tol;
   int iters, max_iter, restarts, max_restarts;
   long long mvp, mvp_extra;
@@ -76,10 +77,14 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
 // the reduction order, and hence every result, is reproducible.
 int stream_blocks(long long n);
 
-cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v,
+// BiCGStab updates of the active systems in fixed point (fx_stream.cu); n a
+// multiple of 12.  fx (v may be nullptr): the result site by site for the
+// operator.  update_xr writes fxs_blocks(n) partials (<rhat, r>, ||r||^2) a system.
+int fxs_blocks(long long n);
+cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v, FxVec fx,
                                  const BicgScalars *sc, const int *status, long long n,
                                  int nrhs, cudaStream_t s);
-cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v,
+cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v, FxVec fx,
                                  const BicgScalars *sc, const int *status, long long n,
                                  int nrhs, cudaStream_t s);
 cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, const double2 *sv,

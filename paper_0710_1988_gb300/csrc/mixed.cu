@@ -520,15 +520,7 @@ bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *__restrict__ r,
                        const int *__restrict__ status, long long n4) {
   const int q = blockIdx.y;
   if (!on32(status, M_ACTIVE, q)) return;  // uniform per block
-  // beta in FP64 once per block (as in bicg_update_p_kernel)
-  __shared__ float2 s_bm[2];
-  if (threadIdx.x == 0) {
-    const BicgScalars S = sc[q];
-    s_bm[0] = f2(cmul(cdiv(S.rho, S.rho_old), cdiv(S.alpha, S.omega)));
-    s_bm[1] = make_float2(-(float)S.omega.x, -(float)S.omega.y);
-  }
-  __syncthreads();
-  const float2 beta = s_bm[0], mom = s_bm[1];
+  const float2 beta = f2(sc[q].beta), mom = make_float2(-(float)sc[q].omega.x, -(float)sc[q].omega.y);
   const long long off = (long long)q * n4;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x) {
@@ -657,6 +649,7 @@ __global__ void reliable_finalize_kernel(const double *__restrict__ partial, int
   S.rnorm = sqrt(v[2]);
   S.true_rel = S.rnorm / S.bnorm;
   S.rho = make_double2(v[0], v[1]);  // <rhat, r> with the replaced residual
+  S.beta = cmul(cdiv(S.rho, S.rho_old), cdiv(S.alpha, S.omega));
   if (st == ST_BREAKDOWN || st == ST_MAXITER) return;  // final: record only
   if (S.true_rel <= S.tol_outer) {
     status[r] = ST_DONE;
@@ -666,6 +659,7 @@ __global__ void reliable_finalize_kernel(const double *__restrict__ partial, int
     S.rho_old = make_double2(1.0, 0.0);
     S.alpha = make_double2(1.0, 0.0);
     S.omega = make_double2(1.0, 0.0);
+    S.beta = S.rho;
     S.rhat_norm = S.rnorm;
     S.restarts += 1;
     status[r] = ST_RESTART;

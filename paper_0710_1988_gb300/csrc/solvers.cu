@@ -49,12 +49,25 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   double2 *r = ar.take<double2>(vec), *rhat = ar.take<double2>(vec);
   double2 *p = ar.take<double2>(vec), *v = ar.take<double2>(vec);
   double2 *sv = ar.take<double2>(vec), *t = ar.take<double2>(vec);
-  double *part_s = ar.take<double>((size_t)nrhs * nbs * 3);
+  const size_t ns = (size_t)(n / 12 + 31) / 32 * 32 * nrhs;
+  const int nbx = fxs_blocks(n);
+  double *part_s = ar.take<double>((size_t)nrhs * std::max(nbs, nbx) * 3);
   double *part_w = ar.take<double>((size_t)nrhs * nbw * 3);
   BicgScalars *sc = ar.take<BicgScalars>(nrhs);
   int *status = ar.take<int>(nrhs);
   double *hist = hist_len > 0 ? ar.take<double>((size_t)nrhs * hist_len) : nullptr;
   if (ar.failed) return WD_OUT_OF_MEMORY;
+  // p or s in the operator's fixed-point form, written by their updates
+  FxVec fv{nullptr, nullptr};   // without the memory the operator encodes for itself, or runs in FP64
+  if (h->links_fx != nullptr) {
+    fv = FxVec{ar.take<int4>(12 * ns), ar.take<int>(ns)};
+    if (ar.failed) {
+      cudaGetLastError();
+      ar.failed = false;
+      fv = FxVec{nullptr, nullptr};
+    }
+  }
+  const FxVec *pre = fv.v != nullptr ? &fv : nullptr;
 
   std::vector<BicgScalars> hsc(nrhs);
   for (auto &q : hsc) {
@@ -85,14 +98,14 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   for (;;) {
     if (++guard > (long long)max_iter + 64) break;  // every pass does >= 1 iteration
     for (int it = 0; it < CHUNK; ++it) {
-      RET_IF(launch_ok(launch_bicg_update_p(p, r, v, sc, status, n, nrhs, s), "update_p"));
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, p, v, nrhs, 0, EPI_DOT, rhat, part_w, status, s, M_ACTIVE), "wilson_dot"));
+      RET_IF(launch_ok(launch_bicg_update_p(p, r, v, fv, sc, status, n, nrhs, s), "update_p"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, p, v, nrhs, 0, EPI_DOT, rhat, part_w, status, s, M_ACTIVE, pre), "wilson_dot"));
       RET_IF(launch_ok(launch_bicg_finalize(FIN_ALPHA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_alpha"));
-      RET_IF(launch_ok(launch_bicg_update_s(sv, r, v, sc, status, n, nrhs, s), "update_s"));
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, sv, t, nrhs, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE), "wilson_tstt"));
+      RET_IF(launch_ok(launch_bicg_update_s(sv, r, v, fv, sc, status, n, nrhs, s), "update_s"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, sv, t, nrhs, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, pre), "wilson_tstt"));
       RET_IF(launch_ok(launch_bicg_finalize(FIN_OMEGA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_omega"));
       RET_IF(launch_ok(launch_bicg_update_xr(X, r, p, sv, t, rhat, sc, status, part_s, n, nrhs, s), "update_xr"));
-      RET_IF(launch_ok(launch_bicg_finalize(FIN_RHO, part_s, nbs, sc, status, hist, hist_len, nrhs, s), "fin_rho"));
+      RET_IF(launch_ok(launch_bicg_finalize(FIN_RHO, part_s, nbx, sc, status, hist, hist_len, nrhs, s), "fin_rho"));
     }
     WD_CK(cudaMemcpyAsync(hst.data(), status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
     WD_CK(cudaStreamSynchronize(s));

@@ -87,3 +87,32 @@ def test_cycles_match_oracle(wdl, dims, m, k, kind):
         assert np.linalg.norm(host(X) - ref) <= 1e-9 * np.linalg.norm(ref)
         defl.close()
     op.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1, 1), (17, 1, 1, 1), (3, 3, 7, 1), (4, 4, 4, 1), (5, 13, 1, 1),
+                                  (11, 7, 5, 3)])
+@pytest.mark.parametrize("kind", ["plain", "spread", "point", "tiny_chunk"])
+@pytest.mark.parametrize("iters", [1, 3])
+def test_bicgstab_steps_match_oracle(wdl, dims, kind, iters):
+    """Whole BiCGStab iterations (fx_stream.cu: updates and dots on tiles of 16
+    sites) from the same start.  Three steps at kappa = 0.1, where A is within
+    0.8 of the unit matrix, amplify rounding by less than 1e3: 1e-12.  A system
+    whose rho vanishes to rounding (a point source far from its own images:
+    the oracle breaks down at its second step) has no such bar and is left out."""
+    U = L.gauge_field(dims, 0.5, 95)
+    A, _ = oracle_ops(U, dims, 0.1)
+    b = _source(dims, kind)
+    if kind == "tiny_chunk":
+        b = L.gaussian_spinor(dims, 92).reshape(-1, 12)
+        b[16:48] *= 1e-260               # two tiles that fixed point does not hold
+        b = b.ravel()
+    batch = np.stack([b, L.gaussian_spinor(dims, 96).ravel()])
+    op = wdl.WilsonOperator(dims, cuda(U), 0.1)
+    X = cuda(np.zeros_like(batch))
+    op.dbicgstab(cuda(batch), X, None, tol=1e-15, max_iter=iters)
+    for got, rhs in zip(host(X), batch):
+        ref, so = krylov.bicgstab(A, rhs, tol=1e-15, max_iter=iters)
+        if so.breakdown:
+            continue
+        assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+    op.close()
