@@ -376,6 +376,176 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   }
 }
 
+// ----------------------------------------------------------------- few sites
+
+// b times 1, i, -1, -i (f = 0 .. 3) added to a, slice by slice
+__device__ __forceinline__ int4 fx_add_turned(int4 a, int4 b, int f) {
+  const int m1 = f == 1 || f == 2 ? -1 : 0, m2 = f >= 2 ? -1 : 0;   // signs of the real and the imaginary part
+  const int rh = f & 1 ? b.z : b.x, rl = f & 1 ? b.w : b.y, ih = f & 1 ? b.x : b.z, il = f & 1 ? b.y : b.w;
+  return make_int4(a.x + ((rh ^ m1) - m1), a.y + ((rl ^ m1) - m1), a.z + ((ih ^ m2) - m2),
+                   a.w + ((il ^ m2) - m2));
+}
+
+__device__ __forceinline__ longlong2 shfl_xor(longlong2 v, int lane) {
+  return make_longlong2(__shfl_xor_sync(0xffffffffu, v.x, lane), __shfl_xor_sync(0xffffffffu, v.y, lane));
+}
+
+// The same product for few sites, where the time is one warp's chain: lane =
+// (site of 2) 16 + (upper spin) 8 + (hop of 8), so a lane encodes one
+// neighbour's half of the spins, forms one hop's chi and the eight hops of a
+// site are summed over lanes; no encoded copy, one launch.  It issues about
+// twice the instructions a site of wilson_fx_kernel.
+constexpr int FX_FEW_SITES = 8;   // sites a block, two a warp
+
+template <bool DAG, int EPI>
+__global__ void __launch_bounds__(16 * FX_FEW_SITES)
+wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links,
+                     const double2 *__restrict__ in, double2 *__restrict__ out, LatticeGeom g,
+                     double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
+                     double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
+                     unsigned long long *__restrict__ sites) {
+  const int r = (int)(blockIdx.x % (unsigned)nrhs);
+  const long long sb = blockIdx.x / (unsigned)nrhs;
+  if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
+  if (sites != nullptr && sb == 0 && threadIdx.x == 0)
+    atomicAdd(sites, (unsigned long long)g.V);  // work accounting for the profiler
+  const int lane = threadIdx.x & 31, sp = (lane >> 3) & 1, m = (lane >> 1) & 3;
+  const bool fwd = !(lane & 1);
+  const int local = threadIdx.x >> 4;   // site of the block
+  const long long at = sb * FX_FEW_SITES + local;
+  const bool valid = at < g.V;
+  const unsigned s = valid ? (unsigned)at : (unsigned)g.V - 1;   // idle lanes repeat the last site
+  const size_t V = (size_t)g.V;
+  // this lane's neighbour
+  const unsigned q0 = fast_div(s, g.dm[0], g.dsh[0]), q1 = fast_div(q0, g.dm[1], g.dsh[1]);
+  const unsigned t = fast_div(q1, g.dm[2], g.dsh[2]);
+  const unsigned x = s - q0 * g.L[0], y = q0 - q1 * g.L[1], z = q1 - t * g.L[2];
+  const unsigned pos = m == 0 ? x : m == 1 ? y : m == 2 ? z : t;
+  const unsigned ext = m == 0 ? g.L[0] : m == 1 ? g.L[1] : m == 2 ? g.L[2] : g.L[3];
+  const unsigned step = (m > 0 ? g.L[0] : 1u) * (m > 1 ? g.L[1] : 1u) * (m > 2 ? g.L[2] : 1u);
+  const unsigned q = fwd ? (pos + 1 == ext ? s - pos * step : s + step)
+                         : (pos == 0 ? s + (ext - 1) * step : s - step);
+  const unsigned ls = fwd ? s : q;                            // the link's site
+  const unsigned odd = (x + y + z + t + (fwd ? 0 : 1)) & 1u;  // its parity on even extents
+  const int4 *l = L + fx_at(g.split ? odd * (unsigned)(V / 2) + (ls >> 1) : ls, 36) + m * 9 * FX_TILE;
+  int4 u[9];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      int4 e = __ldg(l + (fwd ? 3 * a + b : 3 * b + a) * FX_TILE);
+      if (!fwd) e = make_int4(e.x, e.y, -e.z, -e.w);   // backward: the adjoint
+      u[3 * a + b] = e;
+    }
+  const double2 *psi = in + ((size_t)r * V + q) * 12;
+  const int low_spin = m < 2 ? 3 - sp : 2 + sp;   // fx.cuh
+  double2 pu[3], pl[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    pu[b] = __ldg(psi + 3 * sp + b);
+    pl[b] = __ldg(psi + 3 * low_spin + b);
+  }
+  int e = 0;
+  unsigned long long any = 0;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    e = max(max(e, max(exp_bits(pu[b].x), exp_bits(pu[b].y))), max(exp_bits(pl[b].x), exp_bits(pl[b].y)));
+    any |= (unsigned long long)(__double_as_longlong(pu[b].x) | __double_as_longlong(pu[b].y) |
+                                __double_as_longlong(pl[b].x) | __double_as_longlong(pl[b].y)) << 1;
+  }
+  // the two lanes of a hop hold the neighbour's four spins between them
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
+  any |= __shfl_xor_sync(0xffffffffu, any, 8);
+  const int Eq = fx_site_exponent(e, any == 0);
+  int E = Eq;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+  constexpr int F = DAG ? +1 : -1;
+  const bool plus = fwd == (F > 0);   // the hop's projector is 1 + gamma_mu
+  const int P0 = m == 0 ? 1 : m == 1 ? 2 * sp : m == 2 ? 1 + 2 * sp : 2;     // projection of 1 - gamma_mu
+  const int R0 = m == 0 ? 1 : m == 1 ? 2 - 2 * sp : m == 2 ? 1 + 2 * sp : 0;  // reconstruction of 1 + gamma_mu
+  const int P = plus ? (P0 + 2) & 3 : P0, R = plus ? R0 : (R0 + 2) & 3;
+  const int raw = max(e, FX_EMIN);
+  FxArg h[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) h[b] = FxArg(fx_add_turned(fx_slices(pu[b], raw), fx_slices(pl[b], raw), P));
+  longlong2 up[3], low[3];
+  const int d = min(E - Eq, 63);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    FxAcc acc = {0, 1LL << 28, 0, 0, 0, 0};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) fx_cmac<false>(acc, u[3 * a + b], h[b]);
+    const longlong2 chi = fx_value<false>(acc);
+    up[a] = make_longlong2(fx_align(chi.x, d), fx_align(chi.y, d));
+    const long long re = R & 1 ? up[a].y : up[a].x, im = R & 1 ? up[a].x : up[a].y;
+    low[a] = make_longlong2(R == 1 || R == 2 ? -re : re, R >= 2 ? -im : im);
+    // x and y hops: the lower spin 3 - sp is the other lane's 2 + sp
+    const longlong2 other = shfl_xor(low[a], 8);
+    if (m < 2) low[a] = other;
+  }
+  // sum over the hops: z, t lanes keep the lower spin, x, y lanes the upper
+  const bool lower = lane & 4;
+  longlong2 sum[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const longlong2 got = shfl_xor(lower ? up[a] : low[a], 4), keep = lower ? low[a] : up[a];
+    sum[a] = make_longlong2(keep.x + got.x, keep.y + got.y);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+      const longlong2 v = shfl_xor(sum[a], o);
+      sum[a] = make_longlong2(sum[a].x + v.x, sum[a].y + v.y);
+    }
+  }
+  const int j = lane & 3;   // colour of this lane's entry (3: none)
+  const longlong2 T = j == 0 ? sum[0] : j == 1 ? sum[1] : sum[2];
+  double2 hop = make_double2(fx_to_double(T.x, E), fx_to_double(T.y, E));
+  const int c = 3 * ((lower ? 2 : 0) + sp) + j;
+  // values that fixed point does not hold
+  __shared__ double2 exact[FX_FEW_SITES][12];
+  if (__any_sync(0xffffffffu, E == FX_SPECIAL)) {
+    if (E == FX_SPECIAL && (lane & 15) == 0)
+      hops_f64<DAG>(in + (size_t)r * 12 * V, links, neighbours32(s, g), s, exact[local]);
+    __syncwarp();
+    if (E == FX_SPECIAL && j < 3) hop = exact[local][c];
+  }
+  double2 dv[1] = {make_double2(0.0, 0.0)}, da[1] = {make_double2(0.0, 0.0)};
+  if (valid && j < 3) {
+    const size_t i = ((size_t)r * V + s) * 12 + c;
+    const double2 p = __ldg(in + i);
+    const double tmu = DAG ? -mu : mu;
+    double2 v;
+    v.x = fma(-kappa, hop.x, p.x);
+    v.y = fma(-kappa, hop.y, p.y);
+    if (tmu != 0.0) {  // + i mu gamma5 psi, gamma5 = diag(1, 1, -1, -1)
+      const double mm = lower ? -tmu : tmu;
+      v.x = fma(-mm, p.y, v.x);
+      v.y = fma(mm, p.x, v.y);
+    }
+    out[i] = v;
+    if (EPI != EPI_NONE) {
+      dv[0] = v;
+      da[0] = EPI == EPI_DOT ? __ldg(aux + i) : p;
+    }
+  }
+  if (EPI != EPI_NONE) {  // <aux, out> or <out, in>, and <out, out>
+    __shared__ double sums[FX_FEW_SITES / 2][3];
+    double2 dd = fx_warp_dots<1>(da, dv);
+    if (EPI == EPI_TSTT && lane == 16) dd.x = -dd.x;   // <out, in>: the conjugate
+    const long long nsb = gridDim.x / (unsigned)nrhs;
+    fx_block_dots<FX_FEW_SITES / 2>(dd, sums, partial + ((long long)r * nsb + sb) * 3);
+  }
+}
+
+// Whether the few-site kernel serves nrhs systems of the full operator: up to
+// where the two forms take the same time, sites x systems (us an apply, this
+// kernel against encoding + wilson_fx_kernel): 256: 7.6 / 18.3, 4096: 10.3 /
+// 18.5, 8192: 14.4 / 18.5, 10395: 16.5 / 26.3, 16384: 24.6 / 18.5.  The solvers'
+// products (epi) come with their input encoded, 4.8 us less.
+static bool fx_few(const wd_context *h, int nrhs, int epi) {
+  return !h->eo && h->links_fx != nullptr && h->V * nrhs <= (epi == EPI_NONE ? 12288 : 6144);
+}
+
 // The handle's fixed-point links, or none where they do not fit fx.cuh's
 // bounds or the memory: the FP64 kernel then serves.
 cudaError_t fx_links_create(wd_context *h) {
@@ -442,6 +612,29 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
   return cudaGetLastError();
 }
 
+static cudaError_t launch_wilson_fx_few(const wd_context *h, const double2 *in, double2 *out, int nrhs,
+                                        int dagger, int epi, const double2 *aux, double *partial,
+                                        const int *status, cudaStream_t s, unsigned mask,
+                                        unsigned long long *cnt) {
+  const unsigned grid = (unsigned)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES) * (unsigned)nrhs;
+  const LatticeGeom g = geom_of(h);
+#define WFEW(D, E)                                                                              \
+  wilson_fx_few_kernel<D, E><<<grid, 16 * FX_FEW_SITES, 0, s>>>(h->links_fx, h->links, in, out, g, \
+                                                                h->kappa, h->mu, nrhs, aux,       \
+                                                                partial, status, mask, cnt)
+  if (dagger) {
+    if (epi == EPI_DOT) WFEW(true, EPI_DOT);
+    else if (epi == EPI_TSTT) WFEW(true, EPI_TSTT);
+    else WFEW(true, EPI_NONE);
+  } else {
+    if (epi == EPI_DOT) WFEW(false, EPI_DOT);
+    else if (epi == EPI_TSTT) WFEW(false, EPI_TSTT);
+    else WFEW(false, EPI_NONE);
+  }
+#undef WFEW
+  return cudaGetLastError();
+}
+
 LatticeGeom geom_of(const wd_context *h) {
   LatticeGeom g;
   for (int i = 0; i < 4; ++i) g.L[i] = h->dims[i];
@@ -464,8 +657,13 @@ cudaError_t launch_schur_f64_epi(const wd_context *h, const double2 *in, double2
                                  const int *status, cudaStream_t s, unsigned mask,
                                  const FxVec *pre);
 
-int wilson_blocks(const wd_context *h) {
+int wilson_blocks(const wd_context *h, int nrhs) {
+  if (fx_few(h, nrhs, EPI_DOT)) return (int)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES);
   return h->eo ? eo_blocks(h) : (int)((h->V + 127) / 128);
+}
+
+bool wilson_takes_encoded(const wd_context *h, int nrhs) {
+  return h->links_fx != nullptr && !fx_few(h, nrhs, EPI_DOT);
 }
 
 cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double2 *out,
@@ -476,7 +674,9 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
     return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, pre);
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
-  if (h->links_fx != nullptr && (long long)wilson_blocks(h) * nrhs <= 0x7fffffffLL) {
+  if (fx_few(h, nrhs, epi))
+    return launch_wilson_fx_few(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
+  if (h->links_fx != nullptr && (long long)wilson_blocks(h, nrhs) * nrhs <= 0x7fffffffLL) {
     if (pre != nullptr)
       return launch_wilson_fx(h, *pre, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
     // scratch for the encoded input, stream-ordered; without it the FP64 kernel
@@ -492,7 +692,7 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
     }
     cudaGetLastError();
   }
-  dim3 grid(wilson_blocks(h), nrhs);
+  dim3 grid(wilson_blocks(h, nrhs), nrhs);
   LatticeGeom g = geom_of(h);
   if (dagger) {
     if (epi == EPI_DOT)

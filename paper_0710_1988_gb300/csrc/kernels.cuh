@@ -58,7 +58,9 @@ struct FxVec {
   int4 *v;
   int *e;
 };
-int wilson_blocks(const wd_context *h);
+// blocks (partials a system) of a product of nrhs systems, and whether it reads `pre`
+int wilson_blocks(const wd_context *h, int nrhs);
+bool wilson_takes_encoded(const wd_context *h, int nrhs);
 cudaError_t fx_links_create(wd_context *h);
 // Encode nrhs vectors of `sites` sites (systems in mask).
 cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,

@@ -44,7 +44,7 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
                      int nrhs, double tol, int max_iter, wd_stats *stats, cudaStream_t s,
                      double *hist_host, int hist_len, Arena &ar) {
   const long long n = op_n(h);
-  const int nbs = stream_blocks(n), nbw = wilson_blocks(h);
+  const int nbs = stream_blocks(n), nbw = wilson_blocks(h, nrhs);
   const size_t vec = (size_t)nrhs * n;
   double2 *r = ar.take<double2>(vec), *rhat = ar.take<double2>(vec);
   double2 *p = ar.take<double2>(vec), *v = ar.take<double2>(vec);
@@ -59,7 +59,7 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   if (ar.failed) return WD_OUT_OF_MEMORY;
   // p or s in the operator's fixed-point form, written by their updates
   FxVec fv{nullptr, nullptr};   // without the memory the operator encodes for itself, or runs in FP64
-  if (h->links_fx != nullptr) {
+  if (wilson_takes_encoded(h, nrhs)) {
     fv = FxVec{ar.take<int4>(12 * ns), ar.take<int>(ns)};
     if (ar.failed) {
       cudaGetLastError();
@@ -271,7 +271,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
                 wd_stats *stats, cudaStream_t s, double *hist_host, int hist_len, Arena &ar) {
   h->gmresdr_hist.clear();
   const long long n = op_n(h);
-  const int nbs = stream_blocks(n), nbw = wilson_blocks(h);
+  const int nbs = stream_blocks(n), nbw = wilson_blocks(h, 1);
   double2 *Va = ar.take<double2>((size_t)(m + 1) * n);
   double2 *Vb = ar.take<double2>((size_t)(m + 1) * n);
   double2 *w = ar.take<double2>(n);
@@ -285,7 +285,8 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
   FxBasis fb{ar.take<int2>((size_t)(m + 1) * n), ar.take<int2>((size_t)(m + 1) * n),
              ar.take<int>((size_t)(m + 1) * nc)};
   const size_t ns = (size_t)(n / 12 + 31) / 32 * 32;
-  const FxVec fv{ar.take<int4>(12 * ns), ar.take<int>(ns)};
+  FxVec fv{nullptr, nullptr};
+  if (wilson_takes_encoded(h, 1)) fv = FxVec{ar.take<int4>(12 * ns), ar.take<int>(ns)};
   double *part_w = ar.take<double>((size_t)nbw * 3);
   double *part_n = ar.take<double>((size_t)std::max<long long>(nbs, nc) * 2);
   double2 *H = ar.take<double2>((size_t)(m + 1) * m);
@@ -355,7 +356,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     for (int j = j0; j < m; ++j) {
       double2 *vj = V + (size_t)j * n;
       // w = A v_j, with ||w||^2 fused (lucky-breakdown reference)
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, vj, w, 1, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, &fv), "arnoldi wilson"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, vj, w, 1, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, fv.v ? &fv : nullptr), "arnoldi wilson"));
       // classical Gram-Schmidt, applied twice, in fixed point (fx_basis.cu); the
       // second pass's update in FP32 when its coefficients are at rounding level
       RET_IF(launch_ok(launch_fxb_dot(fb, V, j + 1, w, 0, n, part_t, H + j, m, nullptr, 0, status, s), "cgs dot1"));

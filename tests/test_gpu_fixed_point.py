@@ -49,7 +49,11 @@ def _apply(wdl, dims, U, psi, kappa, mu=0.0, dagger=False):
     return got
 
 
-@pytest.mark.parametrize("dims,nrhs", [((1, 1, 1, 1), 1), ((3, 5, 1, 1), 2), ((4, 4, 1, 1), 1),
+@pytest.mark.parametrize("dims,nrhs", [((13, 9, 7, 15), 1), ((16, 16, 6, 8), 1), ((11, 9, 7, 2), 9),
+                                       # the same edges in the form for more than 12288 sites x systems
+                                       ((17, 1, 1, 1), 742), ((31, 1, 1, 1), 400), ((43, 3, 1, 1), 98),
+                                       ((8, 4, 4, 1), 97), ((2, 2, 2, 4), 400), ((1, 1, 1, 1), 12300),
+                                       ((1, 1, 1, 1), 1), ((3, 5, 1, 1), 2), ((4, 4, 1, 1), 1),
                                        ((17, 1, 1, 1), 1), ((31, 1, 1, 1), 1), ((2, 2, 2, 4), 3),
                                        ((11, 3, 1, 1), 1), ((127, 1, 1, 1), 2), ((8, 4, 4, 1), 1),
                                        ((43, 3, 1, 1), 3), ((6, 2, 4, 8), 2), ((9, 7, 5, 3), 4)])
@@ -63,13 +67,14 @@ def test_edges_and_magnitudes(wdl, dims, nrhs, dagger, spread):
     psi[:, 0] = 0.0
     got = _apply(wdl, dims, U, psi, 0.14, 0.07, dagger)
     f = dirac.apply_A_dagger if dagger else dirac.apply_A
-    for r in range(nrhs):
+    for r in sorted({0, 1 % nrhs, 2 % nrhs, nrhs // 2, nrhs - 1}):
         ref = f(U, psi[r], dims, 0.14, 0.07)
         bound = 64 * 2.0 ** -53 * _local_max(psi[r], dims)
         assert np.all(np.abs(got[r] - ref).max(axis=(-1, -2)) <= bound)
 
 
-def test_values_outside_fixed_point_match_the_fp64_kernel(wdl):
+@pytest.mark.parametrize("nrhs", [1, 40])     # few sites in all, and many
+def test_values_outside_fixed_point_match_the_fp64_kernel(wdl, nrhs):
     """Infinities, NaN, subnormal and very large entries beside ordinary ones:
     the same finite values, and the same infinities and NaN, as the FP64
     kernel gives (an operator whose only difference is one scaled link, which
@@ -86,8 +91,8 @@ def test_values_outside_fixed_point_match_the_fp64_kernel(wdl):
     psi[160] *= 1e300
     psi[170] = 0.0
     psi[171] = 5e-324
-    a = _apply(wdl, dims, U, psi, 0.14)
-    b = _apply(wdl, dims, U2, psi, 0.14)
+    a = _apply(wdl, dims, U, np.stack([psi] * nrhs), 0.14)[-1]
+    b = _apply(wdl, dims, U2, np.stack([psi] * nrhs), 0.14)[-1]
     keep = np.ones(L.volume(dims), dtype=bool)
     keep[[far, far - 5]] = False          # the two ends of the scaled x link
     a, b = a[keep], b[keep]
