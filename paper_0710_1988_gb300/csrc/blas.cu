@@ -8,6 +8,7 @@
 // finalizer sums the partials in block order.
 #include <cstdio>
 
+#include "bicg_fin.cuh"
 #include "cplx.cuh"
 #include "kernels.cuh"
 #include "wd_internal.h"
@@ -137,10 +138,7 @@ __device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
   S.rnorm = sqrt(rr);
 }
 
-// One block per system.  An FP64 division, square root or hypot is a chain of
-// some ten FP64 instructions of 64 clocks each, so the independent ones of a
-// kind go to different warps (the solver waits for this kernel three times an
-// iteration).
+// One block per system.
 __global__ void __launch_bounds__(256)
 bicg_finalize_kernel(int kind, const double *__restrict__ partial, int nb, BicgScalars *sc,
                      int *status, double *hist, int hist_len) {
@@ -167,62 +165,7 @@ bicg_finalize_kernel(int kind, const double *__restrict__ partial, int nb, BicgS
   }
   if (kind == FIN_ALPHA || kind == FIN_OMEGA || kind == FIN_RHO) {
     if (st != ST_ACTIVE) return;
-    __shared__ double sum[3];
-    __shared__ double2 quot[2];
-    __shared__ double root[2];
-    BicgScalars &S = sc[r];
-    double v[3];
-    reduce_partials<3>(partial, nb, r, v);
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) sum[q] = v[q];
-    }
-    __syncthreads();
-    const double2 d = make_double2(sum[0], sum[1]);
-    const double n2 = sum[2];
-    if (threadIdx.x == 0) {
-      if (kind == FIN_ALPHA) quot[0] = cdiv(S.rho, d);
-      else if (kind == FIN_OMEGA) quot[0].x = n2 == 0.0 ? 0.0 : d.x / n2;
-      else quot[0] = cdiv(d, S.rho);   // rho / rho_old
-    } else if (threadIdx.x == 32) {
-      if (kind == FIN_OMEGA) quot[0].y = n2 == 0.0 ? 0.0 : d.y / n2;
-      else root[0] = sqrt(n2);
-    } else if (threadIdx.x == 64 && kind != FIN_OMEGA) {
-      root[1] = hypot(d.x, d.y);
-    } else if (threadIdx.x == 96 && kind == FIN_RHO) {
-      quot[1] = cdiv(S.alpha, S.omega);
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    if (kind == FIN_ALPHA) {  // <r_hat, v>, ||v||^2
-      S.mvp += 1;
-      if (root[1] <= 1e-30 * S.rhat_norm * root[0]) {
-        status[r] = ST_BREAKDOWN;
-        return;
-      }
-      S.alpha = quot[0];
-    } else if (kind == FIN_OMEGA) {  // <t, s>, ||t||^2
-      // t = A s = 0 means s = 0: omega = 0, x += alpha p finishes
-      if (n2 != 0.0) S.mvp += 1;
-      S.omega = quot[0];
-    } else {  // FIN_RHO: <r_hat, r>, ||r||^2
-      const double rnorm = root[0], rel = rnorm / S.bnorm;
-      const double2 beta = cmul(quot[0], quot[1]);
-      S.beta = beta;
-      S.mbo = cneg(cmul(beta, S.omega));
-      S.rho_old = S.rho;
-      S.rho = d;
-      S.rnorm = rnorm;
-      S.iters += 1;
-      if (hist != nullptr && S.iters <= hist_len)
-        hist[(long long)r * hist_len + S.iters - 1] = rel;
-      if (rel <= S.tol)
-        status[r] = ST_RECURSIVE;
-      else if (S.iters >= S.max_iter)
-        status[r] = ST_MAXITER;
-      else if (root[1] <= 1e-30 * S.rhat_norm * rnorm)
-        status[r] = ST_BREAKDOWN;
-    }
+    fin_system(kind, partial, nb, sc, status, hist, hist_len, r);
     return;
   }
   if (kind == FIN_TRUE) {  // ||b - A x||^2 (NQ = 1)

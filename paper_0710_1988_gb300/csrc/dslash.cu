@@ -14,6 +14,7 @@
 // Optional fused epilogues write one block-partial (3 doubles) per block for
 // the BiCGStab scalars: EPI_DOT   <aux, out>, <out, out>   (aux = r_hat)
 //                       EPI_TSTT  <out, in>,  <out, out>
+#include "bicg_fin.cuh"
 #include "cplx.cuh"
 #include "wd_internal.h"
 #include "kernels.cuh"
@@ -291,7 +292,7 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
                  const double2 *__restrict__ in64, double2 *__restrict__ out, LatticeGeom g,
                  size_t tiled, double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
                  double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
-                 unsigned long long *__restrict__ sites) {
+                 unsigned long long *__restrict__ sites, FinArgs fin) {
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
@@ -373,6 +374,7 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
     if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, in>: the conjugate
     const long long nsb = gridDim.x / (unsigned)nrhs;
     fx_block_dots<2 * FX_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
+    fin_last_block(fin, partial, r);
   }
 }
 
@@ -403,7 +405,7 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
                      const double2 *__restrict__ in, double2 *__restrict__ out, LatticeGeom g,
                      double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
                      double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
-                     unsigned long long *__restrict__ sites) {
+                     unsigned long long *__restrict__ sites, FinArgs fin) {
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
@@ -534,6 +536,7 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
     if (EPI == EPI_TSTT && lane == 16) dd.x = -dd.x;   // <out, in>: the conjugate
     const long long nsb = gridDim.x / (unsigned)nrhs;
     fx_block_dots<FX_FEW_SITES / 2>(dd, sums, partial + ((long long)r * nsb + sb) * 3);
+    fin_last_block(fin, partial, r);
   }
 }
 
@@ -581,13 +584,13 @@ cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nr
 static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 *in, double2 *out,
                                     int nrhs, int dagger, int epi, const double2 *aux,
                                     double *partial, const int *status, cudaStream_t s,
-                                    unsigned mask, unsigned long long *cnt) {
+                                    unsigned mask, unsigned long long *cnt, const FinArgs &fin) {
   const unsigned grid = (unsigned)((h->V + FX_SITES - 1) / FX_SITES) * (unsigned)nrhs;
   const LatticeGeom g = geom_of(h);
 #define WFX(D, E)                                                                                \
   wilson_fx_kernel<D, E><<<grid, 2 * FX_SITES, FX_SMEM, s>>>(h->links_fx, h->links, f, in, out, g,              \
                                               fx_sites(h->V), h->kappa,                       \
-                                              h->mu, nrhs, aux, partial, status, mask, cnt)
+                                              h->mu, nrhs, aux, partial, status, mask, cnt, fin)
   static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
   if (attr_device != h->device) {
     const void *k[6] = {(const void *)wilson_fx_kernel<false, EPI_NONE>, (const void *)wilson_fx_kernel<false, EPI_DOT>,
@@ -615,13 +618,13 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
 static cudaError_t launch_wilson_fx_few(const wd_context *h, const double2 *in, double2 *out, int nrhs,
                                         int dagger, int epi, const double2 *aux, double *partial,
                                         const int *status, cudaStream_t s, unsigned mask,
-                                        unsigned long long *cnt) {
+                                        unsigned long long *cnt, const FinArgs &fin) {
   const unsigned grid = (unsigned)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES) * (unsigned)nrhs;
   const LatticeGeom g = geom_of(h);
 #define WFEW(D, E)                                                                              \
   wilson_fx_few_kernel<D, E><<<grid, 16 * FX_FEW_SITES, 0, s>>>(h->links_fx, h->links, in, out, g, \
                                                                 h->kappa, h->mu, nrhs, aux,       \
-                                                                partial, status, mask, cnt)
+                                                                partial, status, mask, cnt, fin)
   if (dagger) {
     if (epi == EPI_DOT) WFEW(true, EPI_DOT);
     else if (epi == EPI_TSTT) WFEW(true, EPI_TSTT);
@@ -655,7 +658,7 @@ int eo_blocks(const wd_context *h);
 cudaError_t launch_schur_f64_epi(const wd_context *h, const double2 *in, double2 *out, int nrhs,
                                  int dagger, int epi, const double2 *aux, double *partial,
                                  const int *status, cudaStream_t s, unsigned mask,
-                                 const FxVec *pre);
+                                 const FxVec *pre, const FinArgs *fin);
 
 int wilson_blocks(const wd_context *h, int nrhs) {
   if (fx_few(h, nrhs, EPI_DOT)) return (int)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES);
@@ -669,24 +672,25 @@ bool wilson_takes_encoded(const wd_context *h, int nrhs) {
 cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double2 *out,
                                   int nrhs, int dagger, int epi, const double2 *aux,
                                   double *partial, const int *status, cudaStream_t s,
-                                  unsigned mask, const FxVec *pre) {
+                                  unsigned mask, const FxVec *pre, const FinArgs *fin) {
+  const FinArgs f = fin ? *fin : FinArgs{};
   if (h->eo)  // even-odd Schur operator on even half vectors
-    return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, pre);
+    return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, pre, fin);
   ProfLaunch prof(PC_DSLASH, s);
   unsigned long long *cnt = prof_site_counter();
   if (fx_few(h, nrhs, epi))
-    return launch_wilson_fx_few(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
+    return launch_wilson_fx_few(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt, f);
   if (h->links_fx != nullptr && (long long)wilson_blocks(h, nrhs) * nrhs <= 0x7fffffffLL) {
     if (pre != nullptr)
-      return launch_wilson_fx(h, *pre, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
+      return launch_wilson_fx(h, *pre, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt, f);
     // scratch for the encoded input, stream-ordered; without it the FP64 kernel
     const size_t nv = (size_t)nrhs * fx_sites(h->V);
     int4 *buf = nullptr;
     if (cudaMallocFromPoolAsync((void **)&buf, nv * (12 * sizeof(int4) + sizeof(int)), h->pool, s) == cudaSuccess) {
-      const FxVec f{buf, reinterpret_cast<int *>(buf + 12 * nv)};
-      cudaError_t e = launch_fx_encode(in, f, h->V, nrhs, status, mask, s);
+      const FxVec enc{buf, reinterpret_cast<int *>(buf + 12 * nv)};
+      cudaError_t e = launch_fx_encode(in, enc, h->V, nrhs, status, mask, s);
       if (e == cudaSuccess)
-        e = launch_wilson_fx(h, f, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt);
+        e = launch_wilson_fx(h, enc, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, cnt, f);
       cudaError_t e2 = cudaFreeAsync(buf, s);
       return e != cudaSuccess ? e : e2;
     }
@@ -709,7 +713,9 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
     else
       wilson_f64_kernel<false, EPI_NONE><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
   }
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || fin == nullptr) return e;
+  return launch_bicg_finalize(f.kind, partial, f.nb, f.sc, f.status, f.hist, f.hist_len, nrhs, s);
 }
 
 cudaError_t launch_wilson_f64(const wd_context *h, const double2 *in, double2 *out, int nrhs,

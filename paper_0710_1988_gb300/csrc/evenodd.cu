@@ -11,6 +11,7 @@
 // kernels swap projectors and the diagonal terms flip mu, as in dslash.cu.
 #include <cmath>
 
+#include "bicg_fin.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -198,7 +199,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
                     double kappa, double mu, double inv_1mu2, int nrhs,
                     const double2 *__restrict__ aux, double *__restrict__ partial,
                     const int *__restrict__ status, unsigned mask,
-                    unsigned long long *__restrict__ sites) {
+                    unsigned long long *__restrict__ sites, FinArgs fin) {
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;
@@ -332,6 +333,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, same>: the conjugate
     const long long nsb = gridDim.x / (unsigned)nrhs;
     fx_block_dots<2 * EO_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
+    fin_last_block(fin, partial, r);
   }
 }
 
@@ -339,7 +341,7 @@ template <bool DAG, int MODE, int EPI>
 static cudaError_t launch_eo_fx1(const wd_context *h, FxVec src, const double2 *src64,
                                  const double2 *same, double2 *out, FxVec outfx, int pout, int nrhs,
                                  const double2 *aux, double *partial, const int *status,
-                                 unsigned mask, unsigned long long *cnt, cudaStream_t s) {
+                                 unsigned mask, unsigned long long *cnt, const FinArgs &fin, cudaStream_t s) {
   static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
   if (attr_device != h->device) {
     const cudaError_t e = cudaFuncSetAttribute(wilson_eo_fx_kernel<DAG, MODE, EPI>,
@@ -351,7 +353,7 @@ static cudaError_t launch_eo_fx1(const wd_context *h, FxVec src, const double2 *
   const double inv = 1.0 / std::fma(h->mu, h->mu, 1.0);
   wilson_eo_fx_kernel<DAG, MODE, EPI><<<grid, 2 * EO_SITES, EO_SMEM, s>>>(
       h->links_fx, h->links, src, src64, same, out, outfx, geom_of(h), fx_sites(h->V / 2), pout,
-      h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt);
+      h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt, fin);
   return cudaGetLastError();
 }
 
@@ -413,7 +415,8 @@ static int ensure_eo_tmp(wd_context *h, int nrhs) {
 cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double2 *out, int nrhs,
                                  int dagger, int epi, const double2 *aux, double *partial,
                                  const int *status, cudaStream_t s, unsigned mask,
-                                 const FxVec *pre) {
+                                 const FxVec *pre, const FinArgs *fin) {
+  const FinArgs none{};
   wd_context *h = const_cast<wd_context *>(hc);
   if (ensure_eo_tmp(h, nrhs)) return cudaErrorMemoryAllocation;
   ProfLaunch prof(PC_DSLASH, s);
@@ -424,12 +427,14 @@ cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double
     cudaError_t e = cudaSuccess;
     if (!pre) e = launch_fx_encode(in, src, h->V / 2, nrhs, status, mask, s);
     if (e != cudaSuccess) return e;
-#define EO_FX(D, M, E, SRC, SRC64, SAME, OUT, OUTFX, POUT, CNT)                                     \
-  launch_eo_fx1<D, M, E>(h, SRC, SRC64, SAME, OUT, OUTFX, POUT, nrhs, aux, partial, status, mask, CNT, s)
+#define EO_FX(D, M, E, SRC, SRC64, SAME, OUT, OUTFX, POUT, CNT, FIN)                                \
+  launch_eo_fx1<D, M, E>(h, SRC, SRC64, SAME, OUT, OUTFX, POUT, nrhs, aux, partial, status, mask, CNT, \
+                         FIN, s)
 #define EO_FX_PAIR(D, E)                                                                            \
   {                                                                                                 \
-    e = EO_FX(D, EO_SCHUR1, EPI_NONE, src, in, nullptr, h->eo_tmp, tmp, 1, nullptr);                \
-    return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, tmp, h->eo_tmp, in, out, tmp, 0, cnt);       \
+    e = EO_FX(D, EO_SCHUR1, EPI_NONE, src, in, nullptr, h->eo_tmp, tmp, 1, nullptr, none);          \
+    return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, tmp, h->eo_tmp, in, out, tmp, 0, cnt,        \
+                                              fin ? *fin : none);                                  \
   }
     if (dagger) {
       if (epi == EPI_DOT) EO_FX_PAIR(true, EPI_DOT)
@@ -449,7 +454,9 @@ cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double
     launch_eo<false>(EO_SCHUR1, EPI_NONE, grid, s, h, in, nullptr, h->eo_tmp, 1, nullptr, nullptr, status, mask, nullptr);
     launch_eo<false>(EO_SCHUR2, epi, grid, s, h, h->eo_tmp, in, out, 0, aux, partial, status, mask, cnt);
   }
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || fin == nullptr) return e;
+  return launch_bicg_finalize(fin->kind, partial, fin->nb, fin->sc, fin->status, fin->hist, fin->hist_len, nrhs, s);
 }
 
 // ----------------------------------------------------------------- split / merge / diagonal
@@ -506,7 +513,7 @@ static cudaError_t launch_eo_axpy(const wd_context *h, const double2 *src, const
     const cudaError_t e = launch_fx_encode(src, fx.f[0], h->V / 2, nrhs, nullptr, M_ALL, s);
     return e != cudaSuccess ? e
                             : launch_eo_fx1<false, EO_AXPY, EPI_NONE>(h, fx.f[0], src, same, out, FxVec{nullptr, nullptr}, pout, nrhs,
-                                                                      nullptr, nullptr, nullptr, M_ALL, nullptr, s);
+                                                                      nullptr, nullptr, nullptr, M_ALL, nullptr, FinArgs{}, s);
   }
   launch_eo<false>(EO_AXPY, EPI_NONE, dim3(eo_blocks(h), nrhs), s, h, src, same, out, pout, nullptr,
                    nullptr, nullptr, M_ALL, nullptr);

@@ -6,8 +6,8 @@
 // 112 bytes in 3, 2.2 and 5.3.  So p, x and the dots are formed in integers
 // (fx.cuh: shared exponent, two slices, three multiply-adds a real product, one
 // FP64 addition a real), and s and r, four FMAs an entry each, stay on the FP64
-// pipe beside them.  A warp works on 16 sites (192 entries, six a lane) that
-// share one exponent per operand; a scalar has its own.  Products are kept at
+// pipe beside them.  A warp works on a tile of N entries a lane that share one
+// exponent per operand; a scalar has its own.  Products are kept at
 // 2^-58 of (scalar x largest entry) and leave out 2^-56 of it at most, 2^-58 in
 // the mean: below the two roundings of the FP64 form.  Tiles with infinities,
 // NaN or magnitudes near the ends of FP64's range take FP64.  p and s also leave
@@ -17,6 +17,7 @@
 // 16^4, 10 systems, us a launch (FP64 with its separate encoding -> here):
 // p 173 -> 124 (all FP64 but one term: 148), s 97 -> 84 (in integers 111),
 // x and r 285 -> 189 (r in integers too: 219; its memory takes 130).
+#include "bicg_fin.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -27,7 +28,6 @@ namespace wd {
 namespace {
 
 constexpr int FXS_WARPS = 8, FXS_THREADS = 32 * FXS_WARPS;
-constexpr int FXS_TILE = 192;   // entries of a warp's tile
 
 // a scalar in slices against its own exponent field e (0: not held)
 struct FxScalar {
@@ -86,32 +86,34 @@ struct FxsTile {
   int nz[16];
 };
 
-// The warp's 16 sites of x (entry q 32 + lane) into the operator's form;
-// first: its first site, count: its entries.
-__device__ __forceinline__ void fxs_emit(FxsTile &t, const double2 (&x)[6], FxVec fx, int r,
+// The warp's 32 N / 12 sites of x (entry q 32 + lane; N = 3 or 6) into the
+// operator's form; first: its first site, count: its entries.
+template <int N>
+__device__ __forceinline__ void fxs_emit(FxsTile &t, const double2 (&x)[N], FxVec fx, int r,
                                          long long sites, size_t tiled, long long first, int count) {
+  constexpr int NS = 32 * N / 12, STEP = 32 / NS;   // sites; components a pass of the warp writes
   const int lane = threadIdx.x & 31;
   if (lane < 16) t.e[lane] = t.nz[lane] = 0;
   __syncwarp();
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
+  for (int q = 0; q < N; ++q) {
     const int s = (q * 32 + lane) / 12;
     atomicMax(&t.e[s], max(exp_bits(x[q].x), exp_bits(x[q].y)));
     if ((__double_as_longlong(x[q].x) | __double_as_longlong(x[q].y)) << 1) t.nz[s] = 1;
   }
   __syncwarp();
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
+  for (int q = 0; q < N; ++q) {
     const int c = q * 32 + lane, s = c / 12;
     t.v[c + s] = fx_slices(x[q], max(t.e[s], FX_EMIN));
   }
   __syncwarp();
-  const int site = lane & 15;
+  const int site = lane % NS, c0 = lane / NS;
   if (12 * site < count) {
     int4 *o = fx.v + (size_t)r * 12 * tiled + fx_at((unsigned)(first + site), 12);
 #pragma unroll
-    for (int c = 0; c < 12; c += 2) o[(c + (lane >> 4)) * FX_TILE] = t.v[site * 13 + c + (lane >> 4)];
-    if (lane < 16) fx.e[(size_t)r * sites + first + site] = fx_site_exponent(t.e[site], t.nz[site] == 0);
+    for (int c = 0; c < 12; c += STEP) o[(c + c0) * FX_TILE] = t.v[site * 13 + c + c0];
+    if (c0 == 0) fx.e[(size_t)r * sites + first + site] = fx_site_exponent(t.e[site], t.nz[site] == 0);
   }
   __syncwarp();
 }
@@ -119,7 +121,7 @@ __device__ __forceinline__ void fxs_emit(FxsTile &t, const double2 (&x)[6], FxVe
 }  // namespace
 
 // TWO: out = a + beta out + mbo z (the p update); else out = a - alpha z (s)
-template <bool TWO>
+template <int N, bool TWO>
 __global__ void __launch_bounds__(FXS_THREADS, 2)
 bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, const double2 *__restrict__ z,
                       FxVec fx, size_t tiled, const BicgScalars *__restrict__ sc,
@@ -127,7 +129,7 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
   const int r = blockIdx.y;
   if (!((M_ACTIVE >> status[r]) & 1u)) return;   // uniform per block
   extern __shared__ __align__(16) unsigned char fxs_smem[];
-  FxsTile &tile = reinterpret_cast<FxsTile *>(fxs_smem)[threadIdx.x >> 5];
+  constexpr int FXS_TILE = 32 * N;
   const int lane = threadIdx.x & 31;
   const double2 c1 = TWO ? sc[r].beta : cneg(sc[r].alpha), c2 = TWO ? sc[r].mbo : c1;
   bool held = true;
@@ -138,9 +140,9 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
        t += (long long)gridDim.x * FXS_WARPS) {
     const long long base = t * FXS_TILE;
     const int count = (int)min((long long)FXS_TILE, n - base);
-    double2 y[6], w[6], x[6];
+    double2 y[N], w[N], x[N];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < N; ++q) {
       const int c = q * 32 + lane;
       const size_t i = off + base + c;
       const bool in = c < count;
@@ -157,7 +159,7 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
       ok = ok && o1 && held && fxs_in_range(s1, Ey) && fxs_in_range(s2, Ez);
     }
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < N; ++q) {
       if (TWO)
         x[q] = ok ? fxs_axpy2(x[q], s1, y[q], Ey, s2, w[q], Ez) : cfma(c2, w[q], cfma(c1, y[q], x[q]));
       else
@@ -165,17 +167,23 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
       const int c = q * 32 + lane;
       if (c < count) out[off + base + c] = x[q];
     }
-    if (fx.v != nullptr) fxs_emit(tile, x, fx, r, n / 12, tiled, base / 12, count);
+    if constexpr (N % 3 == 0) {
+      if (fx.v != nullptr)
+        fxs_emit<N>(reinterpret_cast<FxsTile *>(fxs_smem)[threadIdx.x >> 5], x, fx, r, n / 12, tiled,
+                    base / 12, count);
+    }
   }
 }
 
+template <int N>
 __global__ void __launch_bounds__(FXS_THREADS, 2)
 bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, const double2 *__restrict__ p,
                          const double2 *__restrict__ sv, const double2 *__restrict__ t,
                          const double2 *__restrict__ rhat, const BicgScalars *__restrict__ sc,
-                         const int *__restrict__ status, double *__restrict__ partial, long long n) {
+                         const int *__restrict__ status, double *__restrict__ partial, long long n, FinArgs fin) {
   const int r = blockIdx.y;
   if (!((M_ACTIVE >> status[r]) & 1u)) return;
+  constexpr int FXS_TILE = 32 * N;
   __shared__ double sums[FXS_WARPS][3];
   const int lane = threadIdx.x & 31;
   const double2 al = sc[r].alpha, om = sc[r].omega;
@@ -189,9 +197,9 @@ bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, cons
        w += (long long)gridDim.x * FXS_WARPS) {
     const long long base = w * FXS_TILE;
     const int count = (int)min((long long)FXS_TILE, n - base);
-    double2 s[6], u[6], h[6];
+    double2 s[N], u[N], h[N];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < N; ++q) {
       const size_t i = off + base + q * 32 + lane;
       const bool in = q * 32 + lane < count;
       s[q] = in ? sv[i] : zero;
@@ -202,58 +210,85 @@ bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, cons
     const int Es = fx_warp_exponent(s, os), Ep = fx_warp_exponent(u, ok);
     ok = ok && os && held && fxs_in_range(sa, Ep) && fxs_in_range(so, Es);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {   // x += alpha p + omega s
+    for (int q = 0; q < N; ++q) {   // x += alpha p + omega s
       const double2 xi = ok ? fxs_axpy2(h[q], sa, u[q], Ep, so, s[q], Es)
                             : cfma(om, s[q], cfma(al, u[q], h[q]));
       if (q * 32 + lane < count) x[off + base + q * 32 + lane] = xi;
     }
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < N; ++q) {
       const size_t i = off + base + q * 32 + lane;
       const bool in = q * 32 + lane < count;
       u[q] = in ? t[i] : zero;
       h[q] = in ? rhat[i] : zero;
     }
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {   // r = s - omega t
+    for (int q = 0; q < N; ++q) {   // r = s - omega t
       s[q] = cfma(cneg(om), u[q], s[q]);
       if (q * 32 + lane < count) rv[off + base + q * 32 + lane] = s[q];
     }
-    const double2 d = fx_warp_dots<6>(h, s);
+    const double2 d = fx_warp_dots<N>(h, s);
     dots = cadd(dots, d);
   }
   fx_block_dots<FXS_WARPS>(dots, sums, partial + ((long long)r * gridDim.x + blockIdx.x) * 3);
+  fin_last_block(fin, partial, r);
 }
 
-// blocks (per system) of the update kernels: a tile a warp up to four blocks per SM
-int fxs_blocks(long long n) {
-  const long long b = ((n + FXS_TILE - 1) / FXS_TILE + FXS_WARPS - 1) / FXS_WARPS;
+// Entries a lane: six where that gives every SM sixteen warps; below, the time
+// is a warp's chain over its entries, so one (three with the encoded form,
+// whose tiles are whole sites).
+static int fxs_entries(long long n, int nrhs, bool emit) {
+  return n * nrhs >= 192LL * 16 * 152 ? 6 : emit ? 3 : 1;
+}
+
+// blocks (per system): a tile a warp up to four blocks per SM
+static int fxs_grid(long long n, int entries) {
+  const long long b = (n + 32 * entries * FXS_WARPS - 1) / (32 * entries * FXS_WARPS);
   return (int)(b > 608 ? 608 : b < 1 ? 1 : b);
+}
+
+bool fin_fused(long long n, int nrhs) { return fxs_entries(n, nrhs, false) != 6; }
+
+int fxs_blocks(long long n, int nrhs) { return fxs_grid(n, fxs_entries(n, nrhs, false)); }
+
+template <bool TWO>
+static cudaError_t launch_update(double2 *out, const double2 *a, const double2 *z, FxVec fx,
+                                 const BicgScalars *sc, const int *status, long long n, int nrhs,
+                                 cudaStream_t s) {
+  const int N = fxs_entries(n, nrhs, fx.v != nullptr);
+  const dim3 grid(fxs_grid(n, N), nrhs);
+  const size_t smem = fx.v != nullptr ? FXS_WARPS * sizeof(FxsTile) : 0;
+#define FXS_UPDATE(N) \
+  bicg_update_fx_kernel<N, TWO><<<grid, FXS_THREADS, smem, s>>>(out, a, z, fx, fx_sites(n / 12), sc, status, n)
+  if (N == 6) FXS_UPDATE(6);
+  else if (N == 3) FXS_UPDATE(3);
+  else FXS_UPDATE(1);
+#undef FXS_UPDATE
+  return cudaGetLastError();
 }
 
 cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v, FxVec fx,
                                  const BicgScalars *sc, const int *status, long long n,
                                  int nrhs, cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_fx_kernel<true><<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, FXS_WARPS * sizeof(FxsTile), s>>>(
-      p, r, v, fx, fx_sites(n / 12), sc, status, n);
-  return cudaGetLastError();
+  return launch_update<true>(p, r, v, fx, sc, status, n, nrhs, s);
 }
 cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v, FxVec fx,
                                  const BicgScalars *sc, const int *status, long long n,
                                  int nrhs, cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_fx_kernel<false><<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, FXS_WARPS * sizeof(FxsTile), s>>>(
-      sv, r, v, fx, fx_sites(n / 12), sc, status, n);
-  return cudaGetLastError();
+  return launch_update<false>(sv, r, v, fx, sc, status, n, nrhs, s);
 }
 cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, const double2 *sv,
                                   const double2 *t, const double2 *rhat, const BicgScalars *sc,
                                   const int *status, double *partial, long long n, int nrhs,
-                                  cudaStream_t s) {
+                                  const FinArgs &fin, cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  bicg_update_xr_fx_kernel<<<dim3(fxs_blocks(n), nrhs), FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc,
-                                                                             status, partial, n);
+  const dim3 grid(fxs_blocks(n, nrhs), nrhs);
+  if (fxs_entries(n, nrhs, false) == 6)
+    bicg_update_xr_fx_kernel<6><<<grid, FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc, status, partial, n, fin);
+  else
+    bicg_update_xr_fx_kernel<1><<<grid, FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc, status, partial, n, fin);
   return cudaGetLastError();
 }
 

@@ -51,6 +51,18 @@ struct BicgScalars {
   double tol_outer, delta;
 };
 
+// A scalar step of BiCGStab to be done by the last block of the launch that
+// writes its nb partials a system (bicg_fin.cuh): kind FIN_ALPHA, FIN_OMEGA or
+// FIN_RHO; count: a zero a system; count == nullptr: no step.
+struct FinArgs {
+  int kind, nb;
+  BicgScalars *sc;
+  int *status;
+  double *hist;
+  int hist_len;
+  unsigned *count;
+};
+
 LatticeGeom geom_of(const wd_context *h);
 
 // Fixed-point spinors (fx.cuh): v [rhs][tile][12][32], e [rhs][sites].
@@ -69,10 +81,12 @@ cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nr
 // Wilson apply with an optional fused reduction epilogue; blocks of systems
 // whose status is not in `mask` do nothing (status == nullptr: all act).
 // pre: `in` already in fixed point (used when the handle has such links).
+// fin: the scalar step on the epilogue's partials, nrhs systems.
 cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double2 *out,
                                   int nrhs, int dagger, int epi, const double2 *aux,
                                   double *partial, const int *status, cudaStream_t s,
-                                  unsigned mask = M_ACTIVE, const FxVec *pre = nullptr);
+                                  unsigned mask = M_ACTIVE, const FxVec *pre = nullptr,
+                                  const FinArgs *fin = nullptr);
 
 // ----------------------------------------------------------------- BLAS1
 // Number of blocks (per system) every streaming kernel uses; fixed so that
@@ -81,8 +95,11 @@ int stream_blocks(long long n);
 
 // BiCGStab updates of the active systems in fixed point (fx_stream.cu); n a
 // multiple of 12.  fx (v may be nullptr): the result site by site for the
-// operator.  update_xr writes fxs_blocks(n) partials (<rhat, r>, ||r||^2) a system.
-int fxs_blocks(long long n);
+// operator.  update_xr writes fxs_blocks(n, nrhs) partials (<rhat, r>, ||r||^2) a system.
+int fxs_blocks(long long n, int nrhs);
+// Whether the scalar steps of nrhs systems go to the last block of the kernels
+// that form their dots.
+bool fin_fused(long long n, int nrhs);
 cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v, FxVec fx,
                                  const BicgScalars *sc, const int *status, long long n,
                                  int nrhs, cudaStream_t s);
@@ -92,7 +109,7 @@ cudaError_t launch_bicg_update_s(double2 *sv, const double2 *r, const double2 *v
 cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, const double2 *sv,
                                   const double2 *t, const double2 *rhat, const BicgScalars *sc,
                                   const int *status, double *partial, long long n, int nrhs,
-                                  cudaStream_t s);
+                                  const FinArgs &fin, cudaStream_t s);
 // out = a - b, partial <- ||out||^2 ; systems in mask only
 cudaError_t launch_sub_norm(double2 *out, const double2 *a, const double2 *b, const int *status,
                             unsigned mask, double *partial, long long n, int nrhs,

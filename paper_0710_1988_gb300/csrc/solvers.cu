@@ -50,11 +50,12 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   double2 *p = ar.take<double2>(vec), *v = ar.take<double2>(vec);
   double2 *sv = ar.take<double2>(vec), *t = ar.take<double2>(vec);
   const size_t ns = (size_t)(n / 12 + 31) / 32 * 32 * nrhs;
-  const int nbx = fxs_blocks(n);
+  const int nbx = fxs_blocks(n, nrhs);
   double *part_s = ar.take<double>((size_t)nrhs * std::max(nbs, nbx) * 3);
   double *part_w = ar.take<double>((size_t)nrhs * nbw * 3);
   BicgScalars *sc = ar.take<BicgScalars>(nrhs);
   int *status = ar.take<int>(nrhs);
+  unsigned *arrived = ar.take<unsigned>(nrhs);
   double *hist = hist_len > 0 ? ar.take<double>((size_t)nrhs * hist_len) : nullptr;
   if (ar.failed) return WD_OUT_OF_MEMORY;
   // p or s in the operator's fixed-point form, written by their updates
@@ -92,6 +93,14 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   RET_IF(launch_ok(launch_bicg_restart_vectors(rhat, r, p, v, status, M_RESTART, n, nrhs, s), "restart"));
   RET_IF(launch_ok(launch_bicg_finalize(FIN_ACTIVATE, nullptr, 0, sc, status, nullptr, 0, nrhs, s), "activate"));
 
+  // the scalar steps: short vectors by the last block of the kernel that forms
+  // the dots, long ones by a kernel of their own
+  const bool fused = fin_fused(n, nrhs);
+  WD_CK(cudaMemsetAsync(arrived, 0, sizeof(unsigned) * nrhs, s));
+  const FinArgs f_alpha{FIN_ALPHA, nbw, sc, status, hist, hist_len, arrived};
+  const FinArgs f_omega{FIN_OMEGA, nbw, sc, status, hist, hist_len, arrived};
+  const FinArgs f_rho{FIN_RHO, nbx, sc, status, hist, hist_len, arrived};
+
   std::vector<int> hst(nrhs);
   const unsigned M_FINAL_CHECK = (1u << ST_BREAKDOWN) | (1u << ST_MAXITER);
   long long guard = 0;
@@ -99,13 +108,13 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
     if (++guard > (long long)max_iter + 64) break;  // every pass does >= 1 iteration
     for (int it = 0; it < CHUNK; ++it) {
       RET_IF(launch_ok(launch_bicg_update_p(p, r, v, fv, sc, status, n, nrhs, s), "update_p"));
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, p, v, nrhs, 0, EPI_DOT, rhat, part_w, status, s, M_ACTIVE, pre), "wilson_dot"));
-      RET_IF(launch_ok(launch_bicg_finalize(FIN_ALPHA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_alpha"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, p, v, nrhs, 0, EPI_DOT, rhat, part_w, status, s, M_ACTIVE, pre, fused ? &f_alpha : nullptr), "wilson_dot"));
+      if (!fused) RET_IF(launch_ok(launch_bicg_finalize(FIN_ALPHA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_alpha"));
       RET_IF(launch_ok(launch_bicg_update_s(sv, r, v, fv, sc, status, n, nrhs, s), "update_s"));
-      RET_IF(launch_ok(launch_wilson_f64_epi(h, sv, t, nrhs, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, pre), "wilson_tstt"));
-      RET_IF(launch_ok(launch_bicg_finalize(FIN_OMEGA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_omega"));
-      RET_IF(launch_ok(launch_bicg_update_xr(X, r, p, sv, t, rhat, sc, status, part_s, n, nrhs, s), "update_xr"));
-      RET_IF(launch_ok(launch_bicg_finalize(FIN_RHO, part_s, nbx, sc, status, hist, hist_len, nrhs, s), "fin_rho"));
+      RET_IF(launch_ok(launch_wilson_f64_epi(h, sv, t, nrhs, 0, EPI_TSTT, nullptr, part_w, status, s, M_ACTIVE, pre, fused ? &f_omega : nullptr), "wilson_tstt"));
+      if (!fused) RET_IF(launch_ok(launch_bicg_finalize(FIN_OMEGA, part_w, nbw, sc, status, hist, hist_len, nrhs, s), "fin_omega"));
+      RET_IF(launch_ok(launch_bicg_update_xr(X, r, p, sv, t, rhat, sc, status, part_s, n, nrhs, fused ? f_rho : FinArgs{}, s), "update_xr"));
+      if (!fused) RET_IF(launch_ok(launch_bicg_finalize(FIN_RHO, part_s, nbx, sc, status, hist, hist_len, nrhs, s), "fin_rho"));
     }
     WD_CK(cudaMemcpyAsync(hst.data(), status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
     WD_CK(cudaStreamSynchronize(s));
