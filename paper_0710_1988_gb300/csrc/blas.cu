@@ -9,6 +9,7 @@
 #include <cstdio>
 
 #include "bicg_fin.cuh"
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "kernels.cuh"
 #include "wd_internal.h"
@@ -140,8 +141,9 @@ __device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
 
 // One block per system.
 __global__ void __launch_bounds__(256)
-bicg_finalize_kernel(int kind, const double *__restrict__ partial, int nb, BicgScalars *sc,
+bicg_finalize_kernel(int kind, const double *partial, int nb, BicgScalars *sc,
                      int *status, double *hist, int hist_len) {
+  chain_enter();
   const int r = blockIdx.x;
   const int st = status[r];
   if (kind == FIN_INIT) {  // partial: ||b||^2, ||r0||^2 (NQ = 2)
@@ -196,8 +198,7 @@ cudaError_t launch_bicg_finalize(int kind, const double *partial, int nb, BicgSc
                                  int *status, double *hist, int hist_len, int nrhs,
                                  cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  bicg_finalize_kernel<<<nrhs, 256, 0, s>>>(kind, partial, nb, sc, status, hist, hist_len);
-  return cudaGetLastError();
+  return launch_chained(bicg_finalize_kernel, dim3(nrhs), dim3(256), 0, s, kind, partial, nb, sc, status, hist, hist_len);
 }
 
 // ----------------------------------------------------------------- tall-skinny

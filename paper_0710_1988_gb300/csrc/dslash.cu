@@ -15,6 +15,7 @@
 // the BiCGStab scalars: EPI_DOT   <aux, out>, <out, out>   (aux = r_hat)
 //                       EPI_TSTT  <out, in>,  <out, out>
 #include "bicg_fin.cuh"
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "wd_internal.h"
 #include "kernels.cuh"
@@ -291,8 +292,9 @@ __global__ void __launch_bounds__(2 * FX_SITES, 2)
 wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec in,
                  const double2 *__restrict__ in64, double2 *__restrict__ out, LatticeGeom g,
                  size_t tiled, double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
-                 double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
+                 double *__restrict__ partial, const int *status, unsigned mask,
                  unsigned long long *__restrict__ sites, FinArgs fin) {
+  chain_enter();
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
@@ -404,8 +406,9 @@ __global__ void __launch_bounds__(16 * FX_FEW_SITES)
 wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links,
                      const double2 *__restrict__ in, double2 *__restrict__ out, LatticeGeom g,
                      double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
-                     double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
+                     double *__restrict__ partial, const int *status, unsigned mask,
                      unsigned long long *__restrict__ sites, FinArgs fin) {
+  chain_enter();
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;  // uniform per block
@@ -588,9 +591,9 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
   const unsigned grid = (unsigned)((h->V + FX_SITES - 1) / FX_SITES) * (unsigned)nrhs;
   const LatticeGeom g = geom_of(h);
 #define WFX(D, E)                                                                                \
-  wilson_fx_kernel<D, E><<<grid, 2 * FX_SITES, FX_SMEM, s>>>(h->links_fx, h->links, f, in, out, g,              \
-                                              fx_sites(h->V), h->kappa,                       \
-                                              h->mu, nrhs, aux, partial, status, mask, cnt, fin)
+  return launch_chained(wilson_fx_kernel<D, E>, dim3(grid), dim3(2 * FX_SITES), FX_SMEM, s,      \
+                        h->links_fx, h->links, f, in, out, g, fx_sites(h->V), h->kappa, h->mu,   \
+                        nrhs, aux, partial, status, mask, cnt, fin)
   static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
   if (attr_device != h->device) {
     const void *k[6] = {(const void *)wilson_fx_kernel<false, EPI_NONE>, (const void *)wilson_fx_kernel<false, EPI_DOT>,
@@ -604,15 +607,14 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
   }
   if (dagger) {
     if (epi == EPI_DOT) WFX(true, EPI_DOT);
-    else if (epi == EPI_TSTT) WFX(true, EPI_TSTT);
-    else WFX(true, EPI_NONE);
+    if (epi == EPI_TSTT) WFX(true, EPI_TSTT);
+    WFX(true, EPI_NONE);
   } else {
     if (epi == EPI_DOT) WFX(false, EPI_DOT);
-    else if (epi == EPI_TSTT) WFX(false, EPI_TSTT);
-    else WFX(false, EPI_NONE);
+    if (epi == EPI_TSTT) WFX(false, EPI_TSTT);
+    WFX(false, EPI_NONE);
   }
 #undef WFX
-  return cudaGetLastError();
 }
 
 static cudaError_t launch_wilson_fx_few(const wd_context *h, const double2 *in, double2 *out, int nrhs,
@@ -622,20 +624,19 @@ static cudaError_t launch_wilson_fx_few(const wd_context *h, const double2 *in, 
   const unsigned grid = (unsigned)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES) * (unsigned)nrhs;
   const LatticeGeom g = geom_of(h);
 #define WFEW(D, E)                                                                              \
-  wilson_fx_few_kernel<D, E><<<grid, 16 * FX_FEW_SITES, 0, s>>>(h->links_fx, h->links, in, out, g, \
-                                                                h->kappa, h->mu, nrhs, aux,       \
-                                                                partial, status, mask, cnt, fin)
+  return launch_chained(wilson_fx_few_kernel<D, E>, dim3(grid), dim3(16 * FX_FEW_SITES), 0, s,  \
+                        h->links_fx, h->links, in, out, g, h->kappa, h->mu, nrhs, aux, partial, \
+                        status, mask, cnt, fin)
   if (dagger) {
     if (epi == EPI_DOT) WFEW(true, EPI_DOT);
-    else if (epi == EPI_TSTT) WFEW(true, EPI_TSTT);
-    else WFEW(true, EPI_NONE);
+    if (epi == EPI_TSTT) WFEW(true, EPI_TSTT);
+    WFEW(true, EPI_NONE);
   } else {
     if (epi == EPI_DOT) WFEW(false, EPI_DOT);
-    else if (epi == EPI_TSTT) WFEW(false, EPI_TSTT);
-    else WFEW(false, EPI_NONE);
+    if (epi == EPI_TSTT) WFEW(false, EPI_TSTT);
+    WFEW(false, EPI_NONE);
   }
 #undef WFEW
-  return cudaGetLastError();
 }
 
 LatticeGeom geom_of(const wd_context *h) {

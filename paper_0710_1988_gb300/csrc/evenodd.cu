@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "bicg_fin.cuh"
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -198,8 +199,9 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
                     double2 *__restrict__ out, FxVec outfx, LatticeGeom g, size_t tiled, int pout,
                     double kappa, double mu, double inv_1mu2, int nrhs,
                     const double2 *__restrict__ aux, double *__restrict__ partial,
-                    const int *__restrict__ status, unsigned mask,
-                    unsigned long long *__restrict__ sites, FinArgs fin) {
+                    const int *status, unsigned mask, unsigned long long *__restrict__ sites,
+                    FinArgs fin) {
+  chain_enter();
   const int r = (int)(blockIdx.x % (unsigned)nrhs);
   const long long sb = blockIdx.x / (unsigned)nrhs;
   if (status != nullptr && !((mask >> status[r]) & 1u)) return;
@@ -351,10 +353,9 @@ static cudaError_t launch_eo_fx1(const wd_context *h, FxVec src, const double2 *
   }
   const unsigned grid = (unsigned)((h->V / 2 + EO_SITES - 1) / EO_SITES) * (unsigned)nrhs;
   const double inv = 1.0 / std::fma(h->mu, h->mu, 1.0);
-  wilson_eo_fx_kernel<DAG, MODE, EPI><<<grid, 2 * EO_SITES, EO_SMEM, s>>>(
-      h->links_fx, h->links, src, src64, same, out, outfx, geom_of(h), fx_sites(h->V / 2), pout,
-      h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt, fin);
-  return cudaGetLastError();
+  return launch_chained(wilson_eo_fx_kernel<DAG, MODE, EPI>, dim3(grid), dim3(2 * EO_SITES), EO_SMEM, s,
+                        h->links_fx, h->links, src, src64, same, out, outfx, geom_of(h), fx_sites(h->V / 2),
+                        pout, h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt, fin);
 }
 
 // Stream-ordered scratch for `count` encoded batches of half vectors; v is

@@ -18,6 +18,7 @@
 // p 173 -> 124 (all FP64 but one term: 148), s 97 -> 84 (in integers 111),
 // x and r 285 -> 189 (r in integers too: 219; its memory takes 130).
 #include "bicg_fin.cuh"
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -125,7 +126,8 @@ template <int N, bool TWO>
 __global__ void __launch_bounds__(FXS_THREADS, 2)
 bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, const double2 *__restrict__ z,
                       FxVec fx, size_t tiled, const BicgScalars *__restrict__ sc,
-                      const int *__restrict__ status, long long n) {
+                      const int *status, long long n) {
+  chain_enter();
   const int r = blockIdx.y;
   if (!((M_ACTIVE >> status[r]) & 1u)) return;   // uniform per block
   extern __shared__ __align__(16) unsigned char fxs_smem[];
@@ -180,7 +182,8 @@ __global__ void __launch_bounds__(FXS_THREADS, 2)
 bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, const double2 *__restrict__ p,
                          const double2 *__restrict__ sv, const double2 *__restrict__ t,
                          const double2 *__restrict__ rhat, const BicgScalars *__restrict__ sc,
-                         const int *__restrict__ status, double *__restrict__ partial, long long n, FinArgs fin) {
+                         const int *status, double *__restrict__ partial, long long n, FinArgs fin) {
+  chain_enter();
   const int r = blockIdx.y;
   if (!((M_ACTIVE >> status[r]) & 1u)) return;
   constexpr int FXS_TILE = 32 * N;
@@ -259,12 +262,12 @@ static cudaError_t launch_update(double2 *out, const double2 *a, const double2 *
   const dim3 grid(fxs_grid(n, N), nrhs);
   const size_t smem = fx.v != nullptr ? FXS_WARPS * sizeof(FxsTile) : 0;
 #define FXS_UPDATE(N) \
-  bicg_update_fx_kernel<N, TWO><<<grid, FXS_THREADS, smem, s>>>(out, a, z, fx, fx_sites(n / 12), sc, status, n)
+  return launch_chained(bicg_update_fx_kernel<N, TWO>, grid, dim3(FXS_THREADS), smem, s, out, a, z, fx, \
+                        fx_sites(n / 12), sc, status, n)
   if (N == 6) FXS_UPDATE(6);
-  else if (N == 3) FXS_UPDATE(3);
-  else FXS_UPDATE(1);
+  if (N == 3) FXS_UPDATE(3);
+  FXS_UPDATE(1);
 #undef FXS_UPDATE
-  return cudaGetLastError();
 }
 
 cudaError_t launch_bicg_update_p(double2 *p, const double2 *r, const double2 *v, FxVec fx,
@@ -285,11 +288,8 @@ cudaError_t launch_bicg_update_xr(double2 *x, double2 *r, const double2 *p, cons
                                   const FinArgs &fin, cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
   const dim3 grid(fxs_blocks(n, nrhs), nrhs);
-  if (fxs_entries(n, nrhs, false) == 6)
-    bicg_update_xr_fx_kernel<6><<<grid, FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc, status, partial, n, fin);
-  else
-    bicg_update_xr_fx_kernel<1><<<grid, FXS_THREADS, 0, s>>>(x, r, p, sv, t, rhat, sc, status, partial, n, fin);
-  return cudaGetLastError();
+  return launch_chained(fxs_entries(n, nrhs, false) == 6 ? bicg_update_xr_fx_kernel<6> : bicg_update_xr_fx_kernel<1>,
+                        grid, dim3(FXS_THREADS), 0, s, x, r, p, sv, t, rhat, sc, status, partial, n, fin);
 }
 
 }  // namespace wd

@@ -9,6 +9,7 @@
 // The dslash handles R right-hand sides per thread so every link it loads
 // serves R spinors.  Reductions: FP32 within a thread and a warp, FP64
 // across warps and blocks, fixed order.
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "kernels.cuh"
 #include "mixed.h"
@@ -135,8 +136,8 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
                   const float4 *__restrict__ in2, float4 *__restrict__ out, LatticeGeom g,
                   float kappa, float mu, int nrhs, const BicgScalars *__restrict__ sc,
                   const float4 *__restrict__ aux, double *__restrict__ partial,
-                  const int *__restrict__ status, unsigned mask,
-                  unsigned long long *__restrict__ sites) {
+                  const int *status, unsigned mask, unsigned long long *__restrict__ sites) {
+  chain_enter();
   // Blocks are numbered system-row fastest: the nrow blocks that cover the
   // same sites run next to each other and share the links and the
   // neighbour spinors' cache lines through L2.
@@ -265,14 +266,12 @@ static cudaError_t launch_w32(const Mixed32 &m, const float4 *in, const float4 *
   const dim3 grid((unsigned)nblk);
   const float kap = (float)h->kappa, mu = (float)h->mu;
   if (epi == EPI_DOT)
-    wilson_f32_kernel<R, TPB, false, EPI_DOT, false><<<grid, TPB, 0, s>>>(m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
-  else if (epi == EPI_TSTT)
-    wilson_f32_kernel<R, TPB, false, EPI_TSTT, true><<<grid, TPB, 0, s>>>(m.links, in, in2, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
-  else if (dagger)
-    wilson_f32_kernel<R, TPB, true, EPI_NONE, false><<<grid, TPB, 0, s>>>(m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
-  else
-    wilson_f32_kernel<R, TPB, false, EPI_NONE, false><<<grid, TPB, 0, s>>>(m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
-  return cudaGetLastError();
+    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_DOT, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+  if (epi == EPI_TSTT)
+    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_TSTT, true>, grid, dim3(TPB), 0, s, m.links, in, in2, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+  if (dagger)
+    return launch_chained(wilson_f32_kernel<R, TPB, true, EPI_NONE, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+  return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_NONE, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
 }
 
 // Launch shape of the FP32 kernel for nrhs right-hand sides: the autotuned
@@ -517,7 +516,8 @@ __device__ __forceinline__ float4 c2fma(float2 a, float4 b, float4 c) {  // c + 
 __global__ void __launch_bounds__(256)
 bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *__restrict__ r,
                        const float4 *__restrict__ v, const BicgScalars *__restrict__ sc,
-                       const int *__restrict__ status, long long n4) {
+                       const int *status, long long n4) {
+  chain_enter();
   const int q = blockIdx.y;
   if (!on32(status, M_ACTIVE, q)) return;  // uniform per block
   const float2 beta = f2(sc[q].beta), mom = make_float2(-(float)sc[q].omega.x, -(float)sc[q].omega.y);
@@ -534,8 +534,9 @@ __global__ void __launch_bounds__(256)
 bicg32_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r,
                         const float4 *__restrict__ p, const float4 *__restrict__ v,
                         const float4 *__restrict__ t, const float4 *__restrict__ rhat,
-                        const BicgScalars *__restrict__ sc, const int *__restrict__ status,
+                        const BicgScalars *__restrict__ sc, const int *status,
                         double *__restrict__ partial, long long n4) {
+  chain_enter();
   const int q = blockIdx.y;
   if (!on32(status, M_ACTIVE, q)) return;
   const float2 al = f2(sc[q].alpha), om = f2(sc[q].omega);
@@ -600,8 +601,7 @@ cudaError_t launch_bicg32_update_p(float4 *p, const float4 *r, const float4 *v,
                                    const BicgScalars *sc, const int *status, long long n4,
                                    int nrhs, cudaStream_t s) {
   ProfLaunch prof(PC_STREAM_LOW, s);
-  bicg32_update_p_kernel<<<dim3(stream32_blocks(n4), nrhs), 256, 0, s>>>(p, r, v, sc, status, n4);
-  return cudaGetLastError();
+  return launch_chained(bicg32_update_p_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, p, r, v, sc, status, n4);
 }
 
 cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, const float4 *v,
@@ -609,9 +609,8 @@ cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, cons
                                     const int *status, double *partial, long long n4, int nrhs,
                                     cudaStream_t s) {
   ProfLaunch prof(PC_STREAM_LOW, s);
-  bicg32_update_xr_kernel<<<dim3(stream32_blocks(n4), nrhs), 256, 0, s>>>(xs, r, p, v, t, rhat, sc,
-                                                                         status, partial, n4);
-  return cudaGetLastError();
+  return launch_chained(bicg32_update_xr_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, xs, r, p, v, t, rhat,
+                        sc, status, partial, n4);
 }
 
 cudaError_t launch_bicg32_restart(float4 *rhat, const float4 *r, float4 *p, float4 *v,

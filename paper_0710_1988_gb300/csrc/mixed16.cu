@@ -16,6 +16,7 @@
 //    instructions of the rebuild.)
 #include <cuda_fp16.h>
 
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "kernels.cuh"
 #include "mixed.h"
@@ -214,8 +215,9 @@ __global__ void __launch_bounds__(TPB)
 wilson_f16_kernel(const uint2 *__restrict__ links, Half16 in, const float4 *__restrict__ r32,
                   Half16 out, LatticeGeom g, float kappa, float mu, int nrhs,
                   const BicgScalars *__restrict__ sc, const float4 *__restrict__ aux,
-                  double *__restrict__ partial, const int *__restrict__ status, unsigned mask,
+                  double *__restrict__ partial, const int *status, unsigned mask,
                   unsigned long long *__restrict__ sites) {
+  chain_enter();
   // Blocks are numbered system-row fastest: the nrow blocks that cover the
   // same sites run next to each other and share the links and the
   // neighbour spinors' cache lines through L2.
@@ -341,14 +343,12 @@ static cudaError_t launch_w16(const wd_context *h, const uint2 *links, Half16 in
   const dim3 grid((unsigned)nblk);
   const float kap = (float)h->kappa, mu = (float)h->mu;
   if (epi == EPI_DOT)
-    wilson_f16_kernel<R, TPB, false, EPI_DOT, false><<<grid, TPB, 0, s>>>(links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
-  else if (epi == EPI_TSTT)
-    wilson_f16_kernel<R, TPB, false, EPI_TSTT, true><<<grid, TPB, 0, s>>>(links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
-  else if (dagger)
-    wilson_f16_kernel<R, TPB, true, EPI_NONE, false><<<grid, TPB, 0, s>>>(links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
-  else
-    wilson_f16_kernel<R, TPB, false, EPI_NONE, false><<<grid, TPB, 0, s>>>(links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
-  return cudaGetLastError();
+    return launch_chained(wilson_f16_kernel<R, TPB, false, EPI_DOT, false>, grid, dim3(TPB), 0, s, links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
+  if (epi == EPI_TSTT)
+    return launch_chained(wilson_f16_kernel<R, TPB, false, EPI_TSTT, true>, grid, dim3(TPB), 0, s, links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
+  if (dagger)
+    return launch_chained(wilson_f16_kernel<R, TPB, true, EPI_NONE, false>, grid, dim3(TPB), 0, s, links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
+  return launch_chained(wilson_f16_kernel<R, TPB, false, EPI_NONE, false>, grid, dim3(TPB), 0, s, links, in, r32, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, sites);
 }
 
 static int tune_key16(int nrhs) { return nrhs < WD_TUNE_SLOTS ? nrhs : WD_TUNE_SLOTS - 1; }
@@ -519,8 +519,9 @@ __device__ __forceinline__ bool on16(const int *status, unsigned mask, int r) {
 // p (half) = r + beta (p - omega v)
 __global__ void __launch_bounds__(256)
 bicg16_update_p_kernel(Half16 p, const float4 *__restrict__ r, Half16 v,
-                       const BicgScalars *__restrict__ sc, const int *__restrict__ status,
+                       const BicgScalars *__restrict__ sc, const int *status,
                        long long V) {
+  chain_enter();
   const int q = blockIdx.y;
   if (!on16(status, M_ACTIVE, q)) return;  // uniform per block
   const float2 beta = f2of(sc[q].beta), mom = make_float2(-(float)sc[q].omega.x, -(float)sc[q].omega.y);
@@ -540,8 +541,9 @@ bicg16_update_p_kernel(Half16 p, const float4 *__restrict__ r, Half16 v,
 __global__ void __launch_bounds__(256)
 bicg16_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r, Half16 p, Half16 v,
                         Half16 t, const float4 *__restrict__ rhat,
-                        const BicgScalars *__restrict__ sc, const int *__restrict__ status,
+                        const BicgScalars *__restrict__ sc, const int *status,
                         double *__restrict__ partial, long long V) {
+  chain_enter();
   const int q = blockIdx.y;
   if (!on16(status, M_ACTIVE, q)) return;
   const float2 al = f2of(sc[q].alpha), om = f2of(sc[q].omega);
@@ -613,17 +615,15 @@ int stream16_blocks(long long V) { return (int)site_blocks(V); }
 cudaError_t launch_bicg16_update_p(Half16 p, const float4 *r, Half16 v, const BicgScalars *sc,
                                    const int *status, long long V, int nrhs, cudaStream_t s) {
   ProfLaunch prof(PC_STREAM_LOW, s);
-  bicg16_update_p_kernel<<<dim3(site_blocks(V), nrhs), 256, 0, s>>>(p, r, v, sc, status, V);
-  return cudaGetLastError();
+  return launch_chained(bicg16_update_p_kernel, dim3(site_blocks(V), nrhs), dim3(256), 0, s, p, r, v, sc, status, V);
 }
 
 cudaError_t launch_bicg16_update_xr(float4 *xs, float4 *r, Half16 p, Half16 v, Half16 t,
                                     const float4 *rhat, const BicgScalars *sc, const int *status,
                                     double *partial, long long V, int nrhs, cudaStream_t s) {
   ProfLaunch prof(PC_STREAM_LOW, s);
-  bicg16_update_xr_kernel<<<dim3(site_blocks(V), nrhs), 256, 0, s>>>(xs, r, p, v, t, rhat, sc,
-                                                                     status, partial, V);
-  return cudaGetLastError();
+  return launch_chained(bicg16_update_xr_kernel, dim3(site_blocks(V), nrhs), dim3(256), 0, s, xs, r, p, v, t, rhat, sc,
+                        status, partial, V);
 }
 
 cudaError_t launch_bicg16_restart(float4 *rhat, const float4 *r, Half16 p, Half16 v,

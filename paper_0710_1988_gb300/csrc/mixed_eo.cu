@@ -9,6 +9,7 @@
 // mixed.cu on the sites of one parity: float4 [rhs][6][V/2], compact index
 // s / 2 (Lx even: the two sites of an x-pair have opposite parities).  The
 // links are the full-lattice FP32 links of mixed.cu.
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "kernels.cuh"
 #include "mixed.h"
@@ -123,8 +124,8 @@ wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ 
                    const float4 *__restrict__ same2, float4 *__restrict__ out, LatticeGeom g,
                    int pout, float kappa, float mu, const BicgScalars *__restrict__ sc,
                    const float4 *__restrict__ aux, double *__restrict__ partial,
-                   const int *__restrict__ status, unsigned mask,
-                   unsigned long long *__restrict__ sites, int nrhs) {
+                   const int *status, unsigned mask, unsigned long long *__restrict__ sites, int nrhs) {
+  chain_enter();
   // Blocks are numbered system fastest: the nrhs blocks that cover one range
   // of sites run side by side and share the links through L2, which a
   // half-lattice hop reads in full (every link touches one site of each
@@ -245,10 +246,11 @@ cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, const float4 *i
   const dim3 grid((unsigned)schur32_blocks(h) * (unsigned)nrhs);
   const float kap = (float)h->kappa, mu = (float)h->mu;
   unsigned long long *cnt = prof_site_counter_low();
+  cudaError_t e = cudaSuccess;
 #define EO32(D, M, E, FU, SRC, SRC2, SAME, SAME2, OUT, POUT, CNT)                               \
-  wilson_eo32_kernel<D, M, E, FU><<<grid, 128, 0, s>>>(m.links, SRC, SRC2, SAME, SAME2, OUT, g, \
-                                                       POUT, kap, mu, sc, aux, partial, status, \
-                                                       mask, CNT, nrhs)
+  if (e == cudaSuccess)                                                                         \
+  e = launch_chained(wilson_eo32_kernel<D, M, E, FU>, grid, dim3(128), 0, s, m.links, SRC, SRC2, SAME, \
+                     SAME2, OUT, g, POUT, kap, mu, sc, aux, partial, status, mask, CNT, nrhs)
   if (epi == EPI_TSTT) {
     EO32(false, EO32_SCHUR1, EPI_NONE, true, in, in2, nullptr, nullptr, tmp, 1, nullptr);
     EO32(false, EO32_SCHUR2, EPI_TSTT, true, tmp, nullptr, in, in2, out, 0, cnt);
@@ -263,7 +265,7 @@ cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, const float4 *i
     EO32(false, EO32_SCHUR2, EPI_NONE, false, tmp, nullptr, in, nullptr, out, 0, cnt);
   }
 #undef EO32
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace wd
