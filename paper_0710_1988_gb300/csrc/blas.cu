@@ -315,7 +315,8 @@ ts_dot_kernel(const double2 *__restrict__ V, int k, const double2 *__restrict__ 
 // so the loads overlap instead of forming one dependent chain.
 __global__ void ts_dot_finalize_kernel(const double2 *__restrict__ partial, int gx, int gy,
                                        int JT, int RT, int k, int nrhs, double2 *C, int ldc,
-                                       double2 *C2, int ldc2, const int *__restrict__ status) {
+                                       double2 *C2, int ldc2, const int *status) {
+  chain_enter();
   if (status != nullptr && *status != 0) return;
   const int P = k * nrhs;
   const int lane = threadIdx.x & 31;
@@ -360,9 +361,8 @@ cudaError_t launch_ts_dot_finalize_grid(const double2 *partial, int gx, int gy, 
                                         int nrhs, double2 *C, int ldc, double2 *C2, int ldc2,
                                         const int *status, cudaStream_t s) {
   const int P = k * nrhs;  // one warp per pair, four warps per block
-  ts_dot_finalize_kernel<<<(P + 3) / 4, 128, 0, s>>>(partial, gx, gy, JT, RT, k, nrhs, C, ldc, C2,
-                                                     ldc2, status);
-  return cudaGetLastError();
+  return launch_chained(ts_dot_finalize_kernel, dim3((P + 3) / 4), dim3(128), 0, s, partial, gx, gy, JT, RT, k, nrhs,
+                        C, ldc, C2, ldc2, status);
 }
 
 cudaError_t launch_ts_dot_finalize(const double2 *partial, long long n, int k, int nrhs,
@@ -441,6 +441,7 @@ __global__ void arnoldi_normalize_finalize_kernel(const double *__restrict__ pw,
                                                   const double *__restrict__ pw0, int nb0,
                                                   double2 *H, int ldh, int j, double lucky,
                                                   int *status, int *m_eff) {
+  chain_enter();
   if (*status != 0) return;
   double a[1] = {0.0}, b[1] = {0.0};
   for (int i = threadIdx.x; i < nb; i += blockDim.x) a[0] += pw[(long long)i * 2];
@@ -462,9 +463,8 @@ cudaError_t launch_arnoldi_normalize_finalize(const double *partial_w, int nb,
                                               int ldh, int j, double lucky, int *status,
                                               int *m_eff, cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  arnoldi_normalize_finalize_kernel<<<1, 256, 0, s>>>(partial_w, nb, partial_w0, nb0, H, ldh, j,
-                                                      lucky, status, m_eff);
-  return cudaGetLastError();
+  return launch_chained(arnoldi_normalize_finalize_kernel, dim3(1), dim3(256), 0, s, partial_w, nb, partial_w0, nb0, H,
+                        ldh, j, lucky, status, m_eff);
 }
 
 __global__ void norm_finalize_kernel(const double *__restrict__ partial, int nb, int stride,

@@ -21,6 +21,7 @@
 //
 // Chunks with infinities, NaN or magnitudes near the ends of FP64's range
 // have exponent FX_SPECIAL and take their products in FP64.
+#include "chain.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -76,7 +77,8 @@ __device__ __forceinline__ int fxb_exponent(const double2 (&x)[4], int *raw, int
 __global__ void __launch_bounds__(FXB_THREADS)
 fxb_encode_kernel(const double2 *w, const double2 *__restrict__ H, int idx, double2 *v, int2 *__restrict__ hi,
                   int2 *__restrict__ lo, int *__restrict__ ex, FxVec fx, long long n,
-                  const int *__restrict__ status) {
+                  const int *status) {
+  chain_enter();
   if (status != nullptr && *status != 0) return;
   __shared__ int red[2 * FXB_THREADS / 32];
   __shared__ int site_e[FXB_CHUNK / 12], site_nz[FXB_CHUNK / 12];
@@ -127,9 +129,8 @@ cudaError_t launch_fxb_encode(const double2 *w, const double2 *H, int idx, doubl
                               cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
   const long long nc = fxb_chunks(n);
-  fxb_encode_kernel<<<dim3((unsigned)nc, count), FXB_THREADS, 0, s>>>(
-      w, H, idx, v, b.hi + j * n, b.lo + j * n, b.ex + j * nc, fx, n, status);
-  return cudaGetLastError();
+  return launch_chained(fxb_encode_kernel, dim3((unsigned)nc, count), dim3(FXB_THREADS), 0, s, w, H, idx, v,
+                        b.hi + j * n, b.lo + j * n, b.ex + j * nc, fx, n, status);
 }
 
 // ----------------------------------------------------------------- operands in flight
@@ -186,7 +187,8 @@ __device__ __forceinline__ long long fxb_warp_sum(long long a, long long b) {
 // for its jb <= 16 vectors and handles chunks bx, bx + gx, ...
 __global__ void __launch_bounds__(FXB_THREADS, 3)
 fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const double2 *__restrict__ W,
-               int g5, long long n, double2 *__restrict__ partial, const int *__restrict__ status) {
+               int g5, long long n, double2 *__restrict__ partial, const int *status) {
+  chain_enter();
   if (status != nullptr && *status != 0) return;
   extern __shared__ __align__(16) unsigned char fxb_smem[];
   FxbRing &ring = *reinterpret_cast<FxbRing *>(fxb_smem);
@@ -197,23 +199,26 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long nc = (n + FXB_CHUNK - 1) / FXB_CHUNK;
   const int mine = 2 * (int)threadIdx.x;   // first entry of the thread in a chunk
-  // operand u = vector j0 + u % nj of chunk bx + (u / nj) gx
-  auto fetch = [&](int slot, long long c, int jj) {
-    if (c < nc) {
-      const long long at = c * FXB_CHUNK + mine;
-      const bool in0 = at < n, in1 = at + FXB_CHUNK / 2 < n;
-      const long long o = (long long)(j0 + jj) * n + (in0 ? at : 0);
-      fxb_fetch(ring, slot, b.hi + o, b.lo + o, in0, in1);
+  // the next operand to fetch: vector j0 + fj of chunk fc
+  long long fc = blockIdx.x, fo = 0;   // fo: its first entry of this thread in the planes
+  int fj = 0;
+  bool in0 = false, in1 = false;
+  auto fetch = [&](int slot) {
+    if (fc < nc) {
+      if (fj == 0) {
+        const long long at = fc * FXB_CHUNK + mine;
+        in0 = at < n;
+        in1 = at + FXB_CHUNK / 2 < n;
+        fo = (long long)j0 * n + (in0 ? at : 0);
+      }
+      fxb_fetch(ring, slot, b.hi + fo, b.lo + fo, in0, in1);
+      fo += n;
+      if (++fj == nj) fj = 0, fc += gridDim.x;
     }
     fxb_commit();
   };
-  long long fc = blockIdx.x;   // next operand to fetch
-  int fj = 0;
 #pragma unroll
-  for (int u = 0; u < FXB_DEPTH - 1; ++u) {
-    fetch(u, fc, fj);
-    if (++fj == nj) fj = 0, fc += gridDim.x;
-  }
+  for (int u = 0; u < FXB_DEPTH - 1; ++u) fetch(u);
   int slot = 0;
   double sum = 0.0;   // lane l: value l (2 jj, 2 jj + 1: re, im of vector jj)
   for (long long c = blockIdx.x; c < nc; c += gridDim.x) {
@@ -232,8 +237,7 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
 #pragma unroll
     for (int q = 0; q < 4; ++q) w[q] = fx_slices(x[q], raw);
     for (int jj = 0; jj < nj; ++jj) {
-      fetch((slot + FXB_DEPTH - 1) % FXB_DEPTH, fc, fj);
-      if (++fj == nj) fj = 0, fc += gridDim.x;
+      fetch((slot + FXB_DEPTH - 1) % FXB_DEPTH);
       fxb_wait<FXB_DEPTH - 1>();
       long long rh = 0, rm = 1LL << 28, ih = 0, im = 1LL << 28;
 #pragma unroll
@@ -256,15 +260,14 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
     }
     __syncwarp();
     const int jl = lane >> 1;   // this lane's vector
-    if (jl < nj) {
-      const int Ev = b.ex[(long long)(j0 + jl) * nc + c];
-      if (Ew != FX_SPECIAL && Ev != FX_SPECIAL) sum += fx_scaled(tsum[warp][lane], Ev + Ew - 1019);
-    }
-    __syncwarp();
+    const int Ev = jl < nj ? b.ex[(long long)(j0 + jl) * nc + c] : 0;
+    const bool held = Ew != FX_SPECIAL && Ev != FX_SPECIAL;
+    if (jl < nj && held) sum += fx_scaled(tsum[warp][lane], Ev + Ew - 1019);
+    const unsigned other = __ballot_sync(0xffffffffu, jl < nj && !held);
     // chunks that fixed point does not hold, in FP64
-    for (int jj = 0; jj < nj; ++jj) {
+    for (int jj = 0; other != 0 && jj < nj; ++jj) {
+      if (!((other >> (2 * jj)) & 1u)) continue;
       const long long j = j0 + jj;
-      if (Ew != FX_SPECIAL && b.ex[j * nc + c] != FX_SPECIAL) continue;
       double2 a = make_double2(0.0, 0.0);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -337,8 +340,7 @@ cudaError_t launch_fxb_dot(FxBasis b, const double2 *V, int k, const double2 *w,
   static thread_local int device = -1;
   cudaError_t e = fxb_allow_smem((const void *)fxb_dot_kernel, &device);
   if (e != cudaSuccess) return e;
-  fxb_dot_kernel<<<grid, FXB_THREADS, sizeof(FxbRing), s>>>(b, V, k, jb, w, g5, n, partial, status);
-  e = cudaGetLastError();
+  e = launch_chained(fxb_dot_kernel, grid, dim3(FXB_THREADS), sizeof(FxbRing), s, b, V, k, jb, w, g5, n, partial, status);
   if (e != cudaSuccess) return e;
   return launch_ts_dot_finalize_grid(partial, (int)grid.x, (int)grid.y, jb, 1, k, 1, C, ldc, C2, ldc2, status, s);
 }
@@ -349,7 +351,8 @@ cudaError_t launch_fxb_dot(FxBasis b, const double2 *V, int k, const double2 *w,
 // sum V h in fixed point against the largest |h_j| 2^(E_j) of the chunk.
 __global__ void __launch_bounds__(FXB_THREADS, 3)
 fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2 *__restrict__ h, int ldh,
-                  int add, double2 *w, long long n, const int *__restrict__ status) {
+                  int add, double2 *w, long long n, const int *status) {
+  chain_enter();
   if (status != nullptr && *status != 0) return;
   __shared__ int4 g[128];       // h_j in slices
   __shared__ int top[FXB_THREADS / 32], bad[FXB_THREADS / 32];
@@ -455,8 +458,8 @@ cudaError_t launch_fxb_update(FxBasis b, const double2 *V, int k, const double2 
   static thread_local int device = -1;
   cudaError_t e = fxb_allow_smem((const void *)fxb_update_kernel, &device);
   if (e != cudaSuccess) return e;
-  fxb_update_kernel<<<(unsigned)fxb_chunks(n), FXB_THREADS, sizeof(FxbRing), s>>>(b, V, k, h, ldh, add, w, n, status);
-  return cudaGetLastError();
+  return launch_chained(fxb_update_kernel, dim3((unsigned)fxb_chunks(n)), dim3(FXB_THREADS), sizeof(FxbRing), s, b,
+                        V, k, h, ldh, add, w, n, status);
 }
 
 // ----------------------------------------------------------------- correction
@@ -475,7 +478,8 @@ __global__ void __launch_bounds__(FXB_THREADS)
 fxb_correction_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2 *__restrict__ h,
                       const double2 *__restrict__ hsum, int ldh, const double *__restrict__ part_w,
                       int nbw, double2 *w, long long n, double *__restrict__ part_n,
-                      const int *__restrict__ status) {
+                      const int *status) {
+  chain_enter();
   if (status != nullptr && *status != 0) return;
   __shared__ float2 hf[128];
   __shared__ int use32, bad;
@@ -552,9 +556,8 @@ cudaError_t launch_fxb_correction(FxBasis b, const double2 *V, int k, const doub
                                   cudaStream_t s) {
   ProfLaunch prof_(PC_TS, s);
   if (k < 1 || k > 128) return cudaErrorInvalidValue;
-  fxb_correction_kernel<<<(unsigned)fxb_chunks(n), FXB_THREADS, 0, s>>>(b, V, k, h, hsum, ldh, part_w,
-                                                                        nbw, w, n, part_n, status);
-  return cudaGetLastError();
+  return launch_chained(fxb_correction_kernel, dim3((unsigned)fxb_chunks(n)), dim3(FXB_THREADS), 0, s, b, V, k, h,
+                        hsum, ldh, part_w, nbw, w, n, part_n, status);
 }
 
 }  // namespace wd
