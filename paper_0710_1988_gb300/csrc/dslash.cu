@@ -280,15 +280,15 @@ __device__ __noinline__ void hops_f64(const double2 *__restrict__ psi,
 }
 
 // wilson_f64_kernel's result with the hops in fixed point; `in` is the
-// encoded form of in64.  A block covers 128 sites, two lanes (l, l + 16) a
-// site.  Blocks are numbered system fastest: the nrhs blocks of one range of
+// encoded form of in64.  A block covers 64 sites, two lanes (l, l + 16) a
+// site; four fit an SM (16 warps, the registers' limit).  With two of 128 sites
+// more of the SM waits for a block's last warp (0.274 against 0.267 ms, 10
+// systems at 16^4).  Blocks are numbered system fastest: the nrhs blocks of one range of
 // sites share its links through L2.
-constexpr int FX_SITES = 128;
-
-constexpr size_t FX_SMEM = 2 * FX_SITES / 32 * 2 * sizeof(FxStage);   // two stages a warp
+constexpr size_t FX_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);   // two stages a warp
 
 template <bool DAG, int EPI>
-__global__ void __launch_bounds__(2 * FX_SITES, 2)
+__global__ void __launch_bounds__(2 * WILSON_SITES, 4)
 wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec in,
                  const double2 *__restrict__ in64, double2 *__restrict__ out, LatticeGeom g,
                  size_t tiled, double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
@@ -301,7 +301,7 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   if (sites != nullptr && sb == 0 && threadIdx.x == 0)
     atomicAdd(sites, (unsigned long long)g.V);  // work accounting for the profiler
   const int sp = (threadIdx.x >> 4) & 1;
-  const long long at = sb * FX_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+  const long long at = sb * WILSON_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
   const bool valid = at < g.V;
   const unsigned s = valid ? (unsigned)at : (unsigned)g.V - 1;   // idle lanes repeat the last site
   const size_t V = (size_t)g.V;
@@ -316,6 +316,9 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   }
   extern __shared__ __align__(128) unsigned char fx_smem[];
   FxStage *stage = reinterpret_cast<FxStage *>(fx_smem) + 2 * (threadIdx.x >> 5);
+  const long long first = sb * WILSON_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
+  const size_t base = ((size_t)r * V + first) * 12;
+  const int count = 12 * (int)max(0LL, min(16LL, g.V - first));
   longlong2 up[3], low[3];
   {
     const int4 *psi = in.v + (size_t)r * 12 * tiled;
@@ -326,12 +329,13 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
         stage, [&](int m, bool fwd) {
           return L + fx_at(fwd ? here : other + (nb.dn[m] >> half), 36) + m * 9 * FX_TILE;
         },
-        [&](int m, bool fwd) { return psi + fx_at(fwd ? nb.up[m] : nb.dn[m], 12); }, sp, E, eu, ed,
+        [&](int m, bool fwd) { return psi + fx_at(fwd ? nb.up[m] : nb.dn[m], 12); },
+        [&](double2 *own) { fx_fetch_own(own, in64 + base, count); }, sp, E, eu, ed,
         up, low);
   }
   // the warp's 16 sites of hop sums through shared memory, so that its reads
   // and writes of the FP64 vectors are contiguous
-  double2 *hop = reinterpret_cast<double2 *>(stage);   // 13 a site: no bank conflicts
+  double2 *hop = reinterpret_cast<double2 *>(stage + 1);   // 13 a site: no bank conflicts
   double2 *mine = hop + (threadIdx.x & 15) * 13;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -342,17 +346,16 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   if (E == FX_SPECIAL && sp == 0 && valid) {
     hops_f64<DAG>(in64 + (size_t)r * 12 * V, links, nb, s, mine);
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
+  const double2 *own = reinterpret_cast<const double2 *>(stage);
   double2 dv[6], da[6];   // the epilogue's operands
-  const long long first = sb * FX_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
-  const size_t base = ((size_t)r * V + first) * 12;
-  const int count = 12 * (int)max(0LL, min(16LL, g.V - first));
   const double tmu = DAG ? -mu : mu;
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const int c = q * 32 + (threadIdx.x & 31);
     if (c < count) {
-      const double2 p = __ldg(in64 + base + c), d = hop[c + c / 12];
+      const double2 p = own[c], d = hop[c + c / 12];
       double2 v;
       v.x = fma(-kappa, d.x, p.x);
       v.y = fma(-kappa, d.y, p.y);
@@ -371,11 +374,11 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
     }
   }
   if (EPI != EPI_NONE) {  // <aux, out> or <out, in>, and <out, out>
-    __shared__ double sums[2 * FX_SITES / 32][3];
+    __shared__ double sums[2 * WILSON_SITES / 32][3];
     double2 d = fx_warp_dots<6>(da, dv);
     if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, in>: the conjugate
     const long long nsb = gridDim.x / (unsigned)nrhs;
-    fx_block_dots<2 * FX_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
+    fx_block_dots<2 * WILSON_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
     fin_last_block(fin, partial, r);
   }
 }
@@ -588,23 +591,12 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
                                     int nrhs, int dagger, int epi, const double2 *aux,
                                     double *partial, const int *status, cudaStream_t s,
                                     unsigned mask, unsigned long long *cnt, const FinArgs &fin) {
-  const unsigned grid = (unsigned)((h->V + FX_SITES - 1) / FX_SITES) * (unsigned)nrhs;
+  const unsigned grid = (unsigned)((h->V + WILSON_SITES - 1) / WILSON_SITES) * (unsigned)nrhs;
   const LatticeGeom g = geom_of(h);
 #define WFX(D, E)                                                                                \
-  return launch_chained(wilson_fx_kernel<D, E>, dim3(grid), dim3(2 * FX_SITES), FX_SMEM, s,      \
+  return launch_chained(wilson_fx_kernel<D, E>, dim3(grid), dim3(2 * WILSON_SITES), FX_SMEM, s,      \
                         h->links_fx, h->links, f, in, out, g, fx_sites(h->V), h->kappa, h->mu,   \
                         nrhs, aux, partial, status, mask, cnt, fin)
-  static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
-  if (attr_device != h->device) {
-    const void *k[6] = {(const void *)wilson_fx_kernel<false, EPI_NONE>, (const void *)wilson_fx_kernel<false, EPI_DOT>,
-                        (const void *)wilson_fx_kernel<false, EPI_TSTT>, (const void *)wilson_fx_kernel<true, EPI_NONE>,
-                        (const void *)wilson_fx_kernel<true, EPI_DOT>, (const void *)wilson_fx_kernel<true, EPI_TSTT>};
-    for (const void *f : k) {
-      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
-      if (e != cudaSuccess) return e;
-    }
-    attr_device = h->device;
-  }
   if (dagger) {
     if (epi == EPI_DOT) WFX(true, EPI_DOT);
     if (epi == EPI_TSTT) WFX(true, EPI_TSTT);
@@ -663,7 +655,7 @@ cudaError_t launch_schur_f64_epi(const wd_context *h, const double2 *in, double2
 
 int wilson_blocks(const wd_context *h, int nrhs) {
   if (fx_few(h, nrhs, EPI_DOT)) return (int)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES);
-  return h->eo ? eo_blocks(h) : (int)((h->V + 127) / 128);
+  return h->eo ? eo_blocks(h) : (int)((h->V + WILSON_SITES - 1) / WILSON_SITES);
 }
 
 bool wilson_takes_encoded(const wd_context *h, int nrhs) {
@@ -701,18 +693,18 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
   LatticeGeom g = geom_of(h);
   if (dagger) {
     if (epi == EPI_DOT)
-      wilson_f64_kernel<true, EPI_DOT><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<true, EPI_DOT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
     else if (epi == EPI_TSTT)
-      wilson_f64_kernel<true, EPI_TSTT><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<true, EPI_TSTT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
     else
-      wilson_f64_kernel<true, EPI_NONE><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<true, EPI_NONE><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
   } else {
     if (epi == EPI_DOT)
-      wilson_f64_kernel<false, EPI_DOT><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<false, EPI_DOT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
     else if (epi == EPI_TSTT)
-      wilson_f64_kernel<false, EPI_TSTT><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<false, EPI_TSTT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
     else
-      wilson_f64_kernel<false, EPI_NONE><<<grid, 128, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
+      wilson_f64_kernel<false, EPI_NONE><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin == nullptr) return e;

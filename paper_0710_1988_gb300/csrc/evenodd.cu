@@ -185,15 +185,14 @@ __device__ __noinline__ void hops_mixed(const double2 *__restrict__ src, const i
   for (int c = 0; c < 12; ++c) out[c] = acc[c];
 }
 
-constexpr int EO_SITES = 128;                                          // per block, two lanes each
-constexpr size_t EO_SMEM = 2 * EO_SITES / 32 * 2 * sizeof(FxStage);    // two stages a warp
+constexpr size_t EO_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);    // two stages a warp
 
 // wilson_eo_kernel's modes with the hops in fixed point (fx.cuh): src is the
 // encoded operand, src64 its FP64 values at least where it has FX_SPECIAL.
 // EO_SCHUR1 writes the odd vector in fixed point (outfx) for the second half
 // hop, and in FP64 (out) only the sites that need it.
 template <bool DAG, int MODE, int EPI>
-__global__ void __launch_bounds__(2 * EO_SITES, 2)
+__global__ void __launch_bounds__(2 * WILSON_SITES, 4)
 wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec src,
                     const double2 *__restrict__ src64, const double2 *__restrict__ same,
                     double2 *__restrict__ out, FxVec outfx, LatticeGeom g, size_t tiled, int pout,
@@ -209,7 +208,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     atomicAdd(sites, (unsigned long long)g.V);  // two half hops = one full MVP of work
   const unsigned Vh = (unsigned)(g.V / 2);
   const int sp = (threadIdx.x >> 4) & 1;
-  const long long at = sb * EO_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+  const long long at = sb * WILSON_SITES + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
   const bool valid = at < Vh;
   const unsigned i = valid ? (unsigned)at : Vh - 1;   // idle lanes repeat the last site
   // the site of parity pout in the x-pair (2i, 2i + 1)
@@ -231,14 +230,18 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
   extern __shared__ __align__(128) unsigned char eo_smem[];
   FxStage *stage = reinterpret_cast<FxStage *>(eo_smem) + 2 * (threadIdx.x >> 5);
   longlong2 up[3], low[3];
+  const size_t off = (size_t)r * 12 * Vh;
+  const long long first = sb * WILSON_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
+  const size_t base = off + (size_t)first * 12;
+  const int count = 12 * (int)max(0LL, min(16LL, (long long)Vh - first));
   const unsigned here = (pout ? Vh : 0u) + i, other = pout ? 0u : Vh;
   fx_hops<(DAG ? +1 : -1)>(
       stage, [&](int m, bool fwd) {
         return L + fx_at(fwd ? here : other + (nb.dn[m] >> 1), 36) + m * 9 * FX_TILE;
       },
-      [&](int m, bool fwd) { return psi + fx_at((fwd ? nb.up[m] : nb.dn[m]) >> 1, 12); }, sp, E,
-      eu, ed, up, low);
-  const size_t off = (size_t)r * 12 * Vh;
+      [&](int m, bool fwd) { return psi + fx_at((fwd ? nb.up[m] : nb.dn[m]) >> 1, 12); },
+      [&](double2 *own) { fx_fetch_own(own, same + base, MODE == EO_SCHUR1 ? 0 : count); }, sp, E, eu,
+      ed, up, low);
   const double tmu = DAG ? -mu : mu;
   if (MODE == EO_SCHUR1 && tmu == 0.0 && __all_sync(0xffffffffu, E != FX_SPECIAL)) {
     // h itself: the sums' slices, without a way through FP64
@@ -258,7 +261,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     return;
   }
   // the warp's 16 sites of hop sums through shared memory
-  double2 *hop = reinterpret_cast<double2 *>(stage);   // 13 a site: no bank conflicts
+  double2 *hop = reinterpret_cast<double2 *>(stage + 1);   // 13 a site: no bank conflicts
   double2 *mine = hop + (threadIdx.x & 15) * 13;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -296,16 +299,16 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     }
     return;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  const double2 *own = reinterpret_cast<const double2 *>(stage);
   double2 dv[6], da[6];   // the epilogue's operands
-  const long long first = sb * EO_SITES + (threadIdx.x >> 5) * 16;   // the warp's first site
-  const size_t base = off + (size_t)first * 12;
-  const int count = 12 * (int)max(0LL, min(16LL, (long long)Vh - first));
   const double k2 = kappa * kappa;
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const int c = q * 32 + (threadIdx.x & 31);
     if (c < count) {
-      const double2 sm = __ldg(same + base + c), h = hop[c + c / 12];
+      const double2 sm = own[c], h = hop[c + c / 12];
       double2 v;
       if (MODE == EO_SCHUR2) {    // (1 + i mu g5) same - kappa^2 h
         double2 d = sm;
@@ -330,11 +333,11 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     }
   }
   if (EPI != EPI_NONE) {  // <aux, out> or <out, same>, and <out, out>
-    __shared__ double sums[2 * EO_SITES / 32][3];
+    __shared__ double sums[2 * WILSON_SITES / 32][3];
     double2 d = fx_warp_dots<6>(da, dv);
     if (EPI == EPI_TSTT && (threadIdx.x & 31) == 16) d.x = -d.x;   // <out, same>: the conjugate
     const long long nsb = gridDim.x / (unsigned)nrhs;
-    fx_block_dots<2 * EO_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
+    fx_block_dots<2 * WILSON_SITES / 32>(d, sums, partial + ((long long)r * nsb + sb) * 3);
     fin_last_block(fin, partial, r);
   }
 }
@@ -344,16 +347,9 @@ static cudaError_t launch_eo_fx1(const wd_context *h, FxVec src, const double2 *
                                  const double2 *same, double2 *out, FxVec outfx, int pout, int nrhs,
                                  const double2 *aux, double *partial, const int *status,
                                  unsigned mask, unsigned long long *cnt, const FinArgs &fin, cudaStream_t s) {
-  static thread_local int attr_device = -1;   // shared memory above 48 KB, once per device
-  if (attr_device != h->device) {
-    const cudaError_t e = cudaFuncSetAttribute(wilson_eo_fx_kernel<DAG, MODE, EPI>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EO_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_device = h->device;
-  }
-  const unsigned grid = (unsigned)((h->V / 2 + EO_SITES - 1) / EO_SITES) * (unsigned)nrhs;
+  const unsigned grid = (unsigned)((h->V / 2 + WILSON_SITES - 1) / WILSON_SITES) * (unsigned)nrhs;
   const double inv = 1.0 / std::fma(h->mu, h->mu, 1.0);
-  return launch_chained(wilson_eo_fx_kernel<DAG, MODE, EPI>, dim3(grid), dim3(2 * EO_SITES), EO_SMEM, s,
+  return launch_chained(wilson_eo_fx_kernel<DAG, MODE, EPI>, dim3(grid), dim3(2 * WILSON_SITES), EO_SMEM, s,
                         h->links_fx, h->links, src, src64, same, out, outfx, geom_of(h), fx_sites(h->V / 2),
                         pout, h->kappa, h->mu, inv, nrhs, aux, partial, status, mask, cnt, fin);
 }
@@ -365,7 +361,7 @@ struct FxScratch {
   int4 *buf = nullptr;
   cudaStream_t s;
   FxScratch(const wd_context *h, int nrhs, int count, cudaStream_t stream) : s(stream) {
-    if (h->links_fx == nullptr || (h->V / 2 + EO_SITES - 1) / EO_SITES * nrhs > 0x7fffffffLL) return;
+    if (h->links_fx == nullptr || (h->V / 2 + WILSON_SITES - 1) / WILSON_SITES * nrhs > 0x7fffffffLL) return;
     const size_t nv = (size_t)nrhs * fx_sites(h->V / 2), one = nv * 12 * sizeof(int4) + nv * sizeof(int);
     if (cudaMallocFromPoolAsync((void **)&buf, count * one, h->pool, s) != cudaSuccess) {
       cudaGetLastError();
@@ -380,7 +376,7 @@ struct FxScratch {
   }
 };
 
-int eo_blocks(const wd_context *h) { return (int)((h->V / 2 + 127) / 128); }
+int eo_blocks(const wd_context *h) { return (int)((h->V / 2 + WILSON_SITES - 1) / WILSON_SITES); }
 
 template <bool DAG>
 static void launch_eo(int mode, int epi, dim3 grid, cudaStream_t s, const wd_context *h,
@@ -390,7 +386,7 @@ static void launch_eo(int mode, int epi, dim3 grid, cudaStream_t s, const wd_con
   const LatticeGeom g = geom_of(h);
   const double inv = 1.0 / std::fma(h->mu, h->mu, 1.0);  // as the device contracts it
 #define EO_LAUNCH(M, E)                                                                   \
-  wilson_eo_kernel<DAG, M, E><<<grid, 128, 0, s>>>(h->links, src, same, out, g, pout, h->kappa, \
+  wilson_eo_kernel<DAG, M, E><<<grid, WILSON_SITES, 0, s>>>(h->links, src, same, out, g, pout, h->kappa, \
                                                    h->mu, inv, aux, partial, status, mask, cnt)
   if (mode == EO_SCHUR1) EO_LAUNCH(EO_SCHUR1, EPI_NONE);
   else if (mode == EO_AXPY) EO_LAUNCH(EO_AXPY, EPI_NONE);

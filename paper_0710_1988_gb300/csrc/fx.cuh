@@ -235,6 +235,16 @@ __device__ __forceinline__ void fx_fetch(FxStage &st, const int4 *l, const int4 
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+// The warp copies its epilogue's operand, count entries from x.
+__device__ __forceinline__ void fx_fetch_own(double2 *own, const double2 *x, int count) {
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int c = q * 32 + (threadIdx.x & 31);
+    if (c < count) cp_async16(own + c, x + c);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
 // The lane's part of one hop, in units 2^(Eq + d - 1079): up += chi, low +=
 // (factor without sgn) chi, low lying in the neighbour's spin cl.
 template <int MU, int S, bool ADJ>
@@ -242,6 +252,7 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
                                        longlong2 (&up)[3], longlong2 (&low)[3]) {
   using W = FxSpin<MU, S>;
   const int site = threadIdx.x & 15, sgn = 1 - 2 * sp;
+  const long long half = (long long)((1ULL << d) >> 1);
   FxArg h[3];
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
@@ -251,11 +262,11 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    FxAcc s = {0, 1LL << 28, 0, 0, 0, 0};
+    FxAcc s = {half, 1LL << 28, 0, 0, 0, 0};
 #pragma unroll
     for (int b = 0; b < 3; ++b) fx_cmac<ADJ>(s, st.u[ADJ ? 3 * b + a : 3 * a + b][site], h[b]);
     longlong2 chi = fx_value<ADJ>(s);
-    if (d != 0) chi = make_longlong2(fx_align(chi.x, d), fx_align(chi.y, d));
+    chi = make_longlong2(chi.x >> d, chi.y >> d);   // rounded: half is in h1, so in both parts
     up[a] = fx_add<0>(up[a], chi);
     low[a] = fx_add<W::R>(low[a], chi);
   }
@@ -269,8 +280,8 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
 // plain loads, 0.332 with copies past L1; the arithmetic alone 0.237).  The y and z hops come first in
 // their lower sums, whose factor sgn is then applied once; between them the
 // lanes exchange the x and y hops' lower sums, which belong to the other.
-template <int F, class LinkAt, class SiteAt>
-__device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, int sp, int E,
+template <int F, class LinkAt, class SiteAt, class Tail>
+__device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, Tail tail, int sp, int E,
                                         const int (&eu)[4], const int (&ed)[4],
                                         longlong2 (&up)[3], longlong2 (&low)[3]) {
 #pragma unroll
@@ -303,7 +314,7 @@ __device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, i
   FX_SIGN
   FX_PAIR(2, 2 + sp, FX_FETCH(0, 3, true), 1)
   FX_SIGN
-  FX_PAIR(3, 2 + sp, , 0)
+  FX_PAIR(3, 2 + sp, tail(reinterpret_cast<double2 *>(&st[0]));, 1)
 #undef FX_PAIR
 #undef FX_SIGN
 #undef FX_READY

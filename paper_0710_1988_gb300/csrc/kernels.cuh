@@ -70,6 +70,7 @@ struct FxVec {
   int4 *v;
   int *e;
 };
+constexpr int WILSON_SITES = 64;   // per block of the FP64 products, in fixed point and in FP64
 // blocks (partials a system) of a product of nrhs systems, and whether it reads `pre`
 int wilson_blocks(const wd_context *h, int nrhs);
 bool wilson_takes_encoded(const wd_context *h, int nrhs);
