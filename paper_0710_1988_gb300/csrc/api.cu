@@ -751,9 +751,9 @@ extern "C" int wd_apply_f32(wd_handle h, const void *in, void *out, int nrhs, in
   cudaError_t e = launch_f64_to_f32(static_cast<const double2 *>(in), a, Vop, nrhs, nullptr,
                                     nullptr, nullptr, M_ALL, s);
   if (e == cudaSuccess)
-    e = h->eo ? launch_schur_f32(m, a, nullptr, b, tmp, nrhs, dagger ? 1 : 0, EPI_NONE, nullptr,
+    e = h->eo ? launch_schur_f32(m, a, b, tmp, nrhs, dagger ? 1 : 0, EPI_NONE,
                                  nullptr, nullptr, nullptr, M_ALL, s)
-              : launch_wilson_f32(m, a, nullptr, b, nrhs, dagger ? 1 : 0, EPI_NONE, nullptr,
+              : launch_wilson_f32(m, a, b, nrhs, dagger ? 1 : 0, EPI_NONE,
                                   nullptr, nullptr, nullptr, M_ALL, s);
   if (e == cudaSuccess) e = launch_f32_to_f64(b, static_cast<double2 *>(out), Vop, nrhs, s);
   ar.release();

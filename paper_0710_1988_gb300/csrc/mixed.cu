@@ -90,24 +90,8 @@ __device__ __forceinline__ void su3_mul32(const float2 (&m)[9], const float2 (&h
     }
 }
 
-// Input spinor of the hop: `in` itself (FUSED = false) or in - alpha * in2
-// (FUSED: s = r - alpha v without materialising s).
-template <bool FUSED>
-__device__ __forceinline__ void ld_input(const float4 *__restrict__ in, const float4 *__restrict__ in2,
-                                         float2 alpha, long long V, long long s, float2 (&p)[12]) {
-  ld_spinor32(in, V, s, p);
-  if (FUSED) {
-    float2 q[12];
-    ld_spinor32(in2, V, s, q);
-    const float2 ma = make_float2(-alpha.x, -alpha.y);
-#pragma unroll
-    for (int c = 0; c < 12; ++c) p[c] = fcfma(ma, q[c], p[c]);
-  }
-}
-
-template <int MU, int S, bool ADJ, int R, bool FUSED>
+template <int MU, int S, bool ADJ, int R>
 __device__ __forceinline__ void hop32(const float4 *__restrict__ links, const float4 *__restrict__ in,
-                                      const float4 *__restrict__ in2, const float2 (&alpha)[R],
                                       const bool (&on)[R], long long V, long long q, long long ql,
                                       float2 (&acc)[R][12]) {
   float2 u[9];
@@ -116,8 +100,7 @@ __device__ __forceinline__ void hop32(const float4 *__restrict__ links, const fl
   for (int r = 0; r < R; ++r) {
     if (!on[r]) continue;
     float2 p[12], h[6], c[6];
-    ld_input<FUSED>(in + (long long)r * 6 * V, FUSED ? in2 + (long long)r * 6 * V : nullptr,
-                    alpha[r], V, q, p);
+    ld_spinor32(in + (long long)r * 6 * V, V, q, p);
     project<MU, S>(p, h);
     su3_mul32<ADJ>(u, h, c);
     reconstruct<MU, S>(acc[r], c);
@@ -125,16 +108,15 @@ __device__ __forceinline__ void hop32(const float4 *__restrict__ links, const fl
 }
 
 // EPI_NONE: out = A in.   EPI_DOT: out = A in, partial <aux, out>, ||out||^2.
-// EPI_TSTT (FUSED): out = A s with s = in - alpha in2, partial <out, s>, ||out||^2.
+// EPI_TSTT: out = A in, partial <out, in>, ||out||^2.
 // R = 1 shapes are held to 80 registers (768 threads per SM, 6 blocks of 128):
 // the kernel waits on gathers, and the sixth block's warps hide more of that
 // latency than the few spilled words cost (0.778 -> 0.692 ms at 24^3 x 48
 // with 16 systems).
-template <int R, int TPB, bool DAG, int EPI, bool FUSED>
+template <int R, int TPB, bool DAG, int EPI>
 __global__ void __launch_bounds__(TPB, R == 1 ? 768 / TPB : 1)
 wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ in,
-                  const float4 *__restrict__ in2, float4 *__restrict__ out, LatticeGeom g,
-                  float kappa, float mu, int nrhs, const BicgScalars *__restrict__ sc,
+                  float4 *__restrict__ out, LatticeGeom g, float kappa, float mu, int nrhs,
                   const float4 *__restrict__ aux, double *__restrict__ partial,
                   const int *status, unsigned mask, unsigned long long *__restrict__ sites) {
   chain_enter();
@@ -161,16 +143,11 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
     for (int r = 0; r < R; ++r) cnt += on[r] ? 1 : 0;
     atomicAdd(sites, (unsigned long long)V * cnt);  // work accounting for the profiler
   }
-  float2 alpha[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r)
-    alpha[r] = (FUSED && on[r]) ? f2(sc[r0 + r].alpha) : make_float2(0.f, 0.f);
   const long long s = sb * TPB + threadIdx.x;
   float red[R][3];
 #pragma unroll
   for (int r = 0; r < R; ++r) red[r][0] = red[r][1] = red[r][2] = 0.f;
   const float4 *inb = in + (long long)r0 * 6 * V;
-  const float4 *in2b = FUSED ? in2 + (long long)r0 * 6 * V : nullptr;
   if (s < V) {
     const Nbrs32 nb = neighbours32((unsigned)s, g);
     float2 acc[R][12];
@@ -180,21 +157,20 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
       for (int c = 0; c < 12; ++c) acc[r][c] = make_float2(0.f, 0.f);
     constexpr int F = DAG ? +1 : -1;
     constexpr int B = -F;
-    hop32<0, F, false, R, FUSED>(links, inb, in2b, alpha, on, V, nb.up[0], s, acc);
-    hop32<0, B, true, R, FUSED>(links, inb, in2b, alpha, on, V, nb.dn[0], nb.dn[0], acc);
-    hop32<1, F, false, R, FUSED>(links, inb, in2b, alpha, on, V, nb.up[1], s, acc);
-    hop32<1, B, true, R, FUSED>(links, inb, in2b, alpha, on, V, nb.dn[1], nb.dn[1], acc);
-    hop32<2, F, false, R, FUSED>(links, inb, in2b, alpha, on, V, nb.up[2], s, acc);
-    hop32<2, B, true, R, FUSED>(links, inb, in2b, alpha, on, V, nb.dn[2], nb.dn[2], acc);
-    hop32<3, F, false, R, FUSED>(links, inb, in2b, alpha, on, V, nb.up[3], s, acc);
-    hop32<3, B, true, R, FUSED>(links, inb, in2b, alpha, on, V, nb.dn[3], nb.dn[3], acc);
+    hop32<0, F, false, R>(links, inb, on, V, nb.up[0], s, acc);
+    hop32<0, B, true, R>(links, inb, on, V, nb.dn[0], nb.dn[0], acc);
+    hop32<1, F, false, R>(links, inb, on, V, nb.up[1], s, acc);
+    hop32<1, B, true, R>(links, inb, on, V, nb.dn[1], nb.dn[1], acc);
+    hop32<2, F, false, R>(links, inb, on, V, nb.up[2], s, acc);
+    hop32<2, B, true, R>(links, inb, on, V, nb.dn[2], nb.dn[2], acc);
+    hop32<3, F, false, R>(links, inb, on, V, nb.up[3], s, acc);
+    hop32<3, B, true, R>(links, inb, on, V, nb.dn[3], nb.dn[3], acc);
     const float tmu = DAG ? -mu : mu;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (!on[r]) continue;
       float2 p[12];
-      ld_input<FUSED>(inb + (long long)r * 6 * V, FUSED ? in2b + (long long)r * 6 * V : nullptr,
-                      alpha[r], V, s, p);
+      ld_spinor32(inb + (long long)r * 6 * V, V, s, p);
       float2 o[12];
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
@@ -218,7 +194,7 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
           red[r][1] = fmaf(a[c].x, o[c].y, fmaf(-a[c].y, o[c].x, red[r][1]));
           red[r][2] = fmaf(o[c].x, o[c].x, fmaf(o[c].y, o[c].y, red[r][2]));
         }
-      } else if (EPI == EPI_TSTT) {  // <t, s>, ||t||^2 with s = p
+      } else if (EPI == EPI_TSTT) {  // <out, in>, ||out||^2
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
           red[r][0] = fmaf(o[c].x, p[c].x, fmaf(o[c].y, p[c].y, red[r][0]));
@@ -255,8 +231,7 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
 }
 
 template <int R, int TPB>
-static cudaError_t launch_w32(const Mixed32 &m, const float4 *in, const float4 *in2, float4 *out,
-                              int nrhs, int dagger, int epi, const BicgScalars *sc,
+static cudaError_t launch_w32(const Mixed32 &m, const float4 *in, float4 *out, int nrhs, int dagger, int epi,
                               const float4 *aux, double *partial, const int *status,
                               unsigned mask, cudaStream_t s) {
   const wd_context *h = m.h;
@@ -266,12 +241,12 @@ static cudaError_t launch_w32(const Mixed32 &m, const float4 *in, const float4 *
   const dim3 grid((unsigned)nblk);
   const float kap = (float)h->kappa, mu = (float)h->mu;
   if (epi == EPI_DOT)
-    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_DOT, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_DOT>, grid, dim3(TPB), 0, s, m.links, in, out, g, kap, mu, nrhs, aux, partial, status, mask, m.sites);
   if (epi == EPI_TSTT)
-    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_TSTT, true>, grid, dim3(TPB), 0, s, m.links, in, in2, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+    return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_TSTT>, grid, dim3(TPB), 0, s, m.links, in, out, g, kap, mu, nrhs, aux, partial, status, mask, m.sites);
   if (dagger)
-    return launch_chained(wilson_f32_kernel<R, TPB, true, EPI_NONE, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
-  return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_NONE, false>, grid, dim3(TPB), 0, s, m.links, in, nullptr, out, g, kap, mu, nrhs, sc, aux, partial, status, mask, m.sites);
+    return launch_chained(wilson_f32_kernel<R, TPB, true, EPI_NONE>, grid, dim3(TPB), 0, s, m.links, in, out, g, kap, mu, nrhs, aux, partial, status, mask, m.sites);
+  return launch_chained(wilson_f32_kernel<R, TPB, false, EPI_NONE>, grid, dim3(TPB), 0, s, m.links, in, out, g, kap, mu, nrhs, aux, partial, status, mask, m.sites);
 }
 
 // Launch shape of the FP32 kernel for nrhs right-hand sides: the autotuned
@@ -290,11 +265,10 @@ void wilson32_shape(const wd_context *h, int nrhs, int *R, int *T) {
 }
 
 cudaError_t launch_wilson_f32_shape(const Mixed32 &m, int R, int T, const float4 *in,
-                                    const float4 *in2, float4 *out, int nrhs, int dagger, int epi,
-                                    const BicgScalars *sc, const float4 *aux, double *partial,
+                                    float4 *out, int nrhs, int dagger, int epi, const float4 *aux, double *partial,
                                     const int *status, unsigned mask, cudaStream_t s) {
 #define W32(RR, TT) \
-  if (R == RR && T == TT) return launch_w32<RR, TT>(m, in, in2, out, nrhs, dagger, epi, sc, aux, partial, status, mask, s);
+  if (R == RR && T == TT) return launch_w32<RR, TT>(m, in, out, nrhs, dagger, epi, aux, partial, status, mask, s);
   W32(1, 64) W32(1, 128) W32(1, 256)
   W32(2, 64) W32(2, 128) W32(2, 256)
   W32(4, 64) W32(4, 128) W32(4, 256)
@@ -302,8 +276,7 @@ cudaError_t launch_wilson_f32_shape(const Mixed32 &m, int R, int T, const float4
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_wilson_f32(const Mixed32 &m, const float4 *in, const float4 *in2, float4 *out,
-                              int nrhs, int dagger, int epi, const BicgScalars *sc,
+cudaError_t launch_wilson_f32(const Mixed32 &m, const float4 *in, float4 *out, int nrhs, int dagger, int epi,
                               const float4 *aux, double *partial, const int *status,
                               unsigned mask, cudaStream_t s) {
   ProfLaunch prof(PC_DSLASH_LOW, s);
@@ -311,7 +284,7 @@ cudaError_t launch_wilson_f32(const Mixed32 &m, const float4 *in, const float4 *
   wilson32_shape(m.h, nrhs, &R, &T);
   Mixed32 mc = m;
   mc.sites = prof_site_counter_low();
-  return launch_wilson_f32_shape(mc, R, T, in, in2, out, nrhs, dagger, epi, sc, aux, partial, status,
+  return launch_wilson_f32_shape(mc, R, T, in, out, nrhs, dagger, epi, aux, partial, status,
                                  mask, s);
 }
 
@@ -339,13 +312,13 @@ cudaError_t tune_wilson_f32(wd_context *h, const float4 *links, int nrhs, const 
     if (R > nrhs && R > 1) continue;
     for (int T : Ts) {
       for (int w = 0; w < 2 && err == cudaSuccess; ++w)
-        err = launch_wilson_f32_shape(m, R, T, in, nullptr, out, nrhs, 0, EPI_NONE, nullptr, nullptr,
-                                      nullptr, nullptr, M_ALL, s);
+        err = launch_wilson_f32_shape(m, R, T, in, out, nrhs, 0, EPI_NONE, nullptr, nullptr, nullptr, M_ALL,
+                                      s);
       float t_best = 1e30f;
       for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {
         cudaEventRecord(e0, s);
-        err = launch_wilson_f32_shape(m, R, T, in, nullptr, out, nrhs, 0, EPI_NONE, nullptr, nullptr,
-                                      nullptr, nullptr, M_ALL, s);
+        err = launch_wilson_f32_shape(m, R, T, in, out, nrhs, 0, EPI_NONE, nullptr, nullptr, nullptr, M_ALL,
+                                      s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -529,23 +502,38 @@ bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *__restrict__ r,
   }
 }
 
-// s = r - alpha v; xs += alpha p + omega s; r = s - omega t; partial <rhat, r>, ||r||^2
+// r = s = r - alpha v.  A product that forms s at its neighbours instead
+// gathers two vectors: 332 us for it and 322 us for the update below at 20^3 x
+// 32 with 12 systems; with s in place of r S_US + T_US + X_US us.
+__global__ void __launch_bounds__(256)
+bicg32_update_s_kernel(float4 *__restrict__ r, const float4 *__restrict__ v,
+                       const BicgScalars *__restrict__ sc, const int *status, long long n4) {
+  chain_enter();
+  const int q = blockIdx.y;
+  if (!on32(status, M_ACTIVE, q)) return;
+  const float2 mal = make_float2(-(float)sc[q].alpha.x, -(float)sc[q].alpha.y);
+  const long long off = (long long)q * n4;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
+       i += (long long)gridDim.x * blockDim.x)
+    r[off + i] = c2fma(mal, v[off + i], r[off + i]);
+}
+
+// xs += alpha p + omega s; r = s - omega t, s in place of r; partial <rhat, r>, ||r||^2
 __global__ void __launch_bounds__(256)
 bicg32_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r,
-                        const float4 *__restrict__ p, const float4 *__restrict__ v,
-                        const float4 *__restrict__ t, const float4 *__restrict__ rhat,
-                        const BicgScalars *__restrict__ sc, const int *status,
+                        const float4 *__restrict__ p, const float4 *__restrict__ t,
+                        const float4 *__restrict__ rhat, const BicgScalars *__restrict__ sc, const int *status,
                         double *__restrict__ partial, long long n4) {
   chain_enter();
   const int q = blockIdx.y;
   if (!on32(status, M_ACTIVE, q)) return;
   const float2 al = f2(sc[q].alpha), om = f2(sc[q].omega);
-  const float2 mal = make_float2(-al.x, -al.y), mom = make_float2(-om.x, -om.y);
+  const float2 mom = make_float2(-om.x, -om.y);
   const long long off = (long long)q * n4;
   float a0 = 0.f, a1 = 0.f, a2 = 0.f;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x) {
-    const float4 sv = c2fma(mal, v[off + i], r[off + i]);
+    const float4 sv = r[off + i];
     float4 x = xs[off + i];
     x = c2fma(al, p[off + i], x);
     x = c2fma(om, sv, x);
@@ -604,12 +592,18 @@ cudaError_t launch_bicg32_update_p(float4 *p, const float4 *r, const float4 *v,
   return launch_chained(bicg32_update_p_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, p, r, v, sc, status, n4);
 }
 
-cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, const float4 *v,
-                                    const float4 *t, const float4 *rhat, const BicgScalars *sc,
+cudaError_t launch_bicg32_update_s(float4 *r, const float4 *v, const BicgScalars *sc, const int *status,
+                                   long long n4, int nrhs, cudaStream_t s) {
+  ProfLaunch prof(PC_STREAM_LOW, s);
+  return launch_chained(bicg32_update_s_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, r, v, sc, status, n4);
+}
+
+cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, const float4 *t,
+                                    const float4 *rhat, const BicgScalars *sc,
                                     const int *status, double *partial, long long n4, int nrhs,
                                     cudaStream_t s) {
   ProfLaunch prof(PC_STREAM_LOW, s);
-  return launch_chained(bicg32_update_xr_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, xs, r, p, v, t, rhat,
+  return launch_chained(bicg32_update_xr_kernel, dim3(stream32_blocks(n4), nrhs), dim3(256), 0, s, xs, r, p, t, rhat,
                         sc, status, partial, n4);
 }
 

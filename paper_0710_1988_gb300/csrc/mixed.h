@@ -22,10 +22,8 @@ cudaError_t tune_wilson_f32(wd_context *h, const float4 *links, int nrhs, const 
 int stream32_blocks(long long n4);
 int conv_blocks_count(long long V);
 
-// out = A in (FP32 [rhs][6][V]); epi as for the FP64 kernel; EPI_TSTT applies
-// A to s = in - alpha in2 (alpha from sc) and reduces <out, s>, ||out||^2.
-cudaError_t launch_wilson_f32(const Mixed32 &m, const float4 *in, const float4 *in2, float4 *out,
-                              int nrhs, int dagger, int epi, const BicgScalars *sc,
+// out = A in (FP32 [rhs][6][V]); epi as for the FP64 kernel.
+cudaError_t launch_wilson_f32(const Mixed32 &m, const float4 *in, float4 *out, int nrhs, int dagger, int epi,
                               const float4 *aux, double *partial, const int *status,
                               unsigned mask, cudaStream_t s);
 cudaError_t launch_links_to_f32(const wd_context *h, float4 *L, cudaStream_t s);
@@ -41,8 +39,12 @@ cudaError_t launch_f32_to_f64(const float4 *in, double2 *out, long long V, int n
 cudaError_t launch_bicg32_update_p(float4 *p, const float4 *r, const float4 *v,
                                    const BicgScalars *sc, const int *status, long long n4,
                                    int nrhs, cudaStream_t s);
-cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, const float4 *v,
-                                    const float4 *t, const float4 *rhat, const BicgScalars *sc,
+// r = s = r - alpha v
+cudaError_t launch_bicg32_update_s(float4 *r, const float4 *v, const BicgScalars *sc, const int *status,
+                                   long long n4, int nrhs, cudaStream_t s);
+// xs += alpha p + omega s, r = s - omega t, s given in r
+cudaError_t launch_bicg32_update_xr(float4 *xs, float4 *r, const float4 *p, const float4 *t,
+                                    const float4 *rhat, const BicgScalars *sc,
                                     const int *status, double *partial, long long n4, int nrhs,
                                     cudaStream_t s);
 cudaError_t launch_bicg32_restart(float4 *rhat, const float4 *r, float4 *p, float4 *v,
@@ -60,7 +62,7 @@ int wilson16_blocks(const wd_context *h, int nrhs);
 cudaError_t tune_wilson_f16(wd_context *h, const uint2 *links, int nrhs, Half16 in, Half16 out,
                             cudaStream_t s);
 int stream16_blocks(long long V);
-// out = A in (half), epi as launch_wilson_f32; EPI_TSTT applies A to
+// out = A in (half), epi as launch_wilson_f32 but that EPI_TSTT applies A to
 // s = r32 - alpha in and reduces <out, s>, ||out||^2.
 cudaError_t launch_wilson_f16(const wd_context *h, const uint2 *links, Half16 in, const float4 *r32,
                               Half16 out, int nrhs, int dagger, int epi, const BicgScalars *sc,
@@ -80,11 +82,10 @@ cudaError_t launch_bicg16_restart(float4 *rhat, const float4 *r, Half16 p, Half1
 
 // ----------------------------------------------------------------- FP32 Schur operator (mixed_eo.cu)
 // out = A_hat in on even half vectors (float4 [rhs][6][V/2]); tmp: an odd
-// half vector per system; epi / FUSED as launch_wilson_f32.
+// half vector per system; epi as launch_wilson_f32.
 int schur32_blocks(const wd_context *h);
-cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, const float4 *in2, float4 *out,
-                             float4 *tmp, int nrhs, int dagger, int epi, const BicgScalars *sc,
-                             const float4 *aux, double *partial, const int *status,
+cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, float4 *out, float4 *tmp, int nrhs,
+                             int dagger, int epi, const float4 *aux, double *partial, const int *status,
                              unsigned mask, cudaStream_t s);
 
 cudaError_t launch_reliable_finalize(const double *partial, int nb, BicgScalars *sc, int *status,

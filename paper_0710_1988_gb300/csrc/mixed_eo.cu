@@ -38,26 +38,14 @@ __device__ __forceinline__ float2 fcmul_eo(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-// 12 complex components of a half-vector site (compact index c, stride Vh);
-// FUSED: the value of base - alpha base2.
-template <bool FUSED>
-__device__ __forceinline__ void ld_half32(const float4 *__restrict__ base,
-                                          const float4 *__restrict__ base2, float2 alpha,
-                                          long long Vh, long long c, float2 (&p)[12]) {
+// 12 complex components of a half-vector site (compact index c, stride Vh)
+__device__ __forceinline__ void ld_half32(const float4 *__restrict__ base, long long Vh, long long c,
+                                          float2 (&p)[12]) {
 #pragma unroll
   for (int g = 0; g < 6; ++g) {
     const float4 f = __ldg(base + g * Vh + c);
     p[2 * g] = make_float2(f.x, f.y);
     p[2 * g + 1] = make_float2(f.z, f.w);
-  }
-  if (FUSED) {
-    const float2 ma = make_float2(-alpha.x, -alpha.y);
-#pragma unroll
-    for (int g = 0; g < 6; ++g) {
-      const float4 f = __ldg(base2 + g * Vh + c);
-      p[2 * g] = fcfma_eo(ma, make_float2(f.x, f.y), p[2 * g]);
-      p[2 * g + 1] = fcfma_eo(ma, make_float2(f.z, f.w), p[2 * g + 1]);
-    }
   }
 }
 
@@ -83,15 +71,14 @@ __device__ __forceinline__ void ld_link_eo(const float4 *__restrict__ L, long lo
 }
 
 // one hop: neighbour q (full index, other parity) read from the half vector
-template <int MU, int S, bool ADJ, bool FUSED>
+template <int MU, int S, bool ADJ>
 __device__ __forceinline__ void hop_eo32(const float4 *__restrict__ links,
                                          const float4 *__restrict__ src,
-                                         const float4 *__restrict__ src2, float2 alpha,
                                          long long V, long long q, long long ql,
                                          float2 (&acc)[12]) {
   float2 u[9], p[12], h[6], c[6];
   ld_link_eo(links, V, MU, ql, u);
-  ld_half32<FUSED>(src, src2, alpha, V / 2, q >> 1, p);
+  ld_half32(src, V / 2, q >> 1, p);
   project<MU, S>(p, h);
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -115,14 +102,11 @@ enum { EO32_SCHUR1 = 0, EO32_SCHUR2 = 1 };
 //  EO32_SCHUR2: out = (1 + i mu g5) same - kappa^2 h, with the epilogues
 //               EPI_DOT (<aux, out>, ||out||^2) and EPI_TSTT (<out, same>,
 //               ||out||^2).
-// FUSED: the even operand is s = r - alpha v, read from (src, src2) in
-// SCHUR1 and from (same, same2) in SCHUR2.
-template <bool DAG, int MODE, int EPI, bool FUSED>
+template <bool DAG, int MODE, int EPI>
 __global__ void __launch_bounds__(128, 6)  // 80 registers, as the full FP32 kernel
 wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ src,
-                   const float4 *__restrict__ src2, const float4 *__restrict__ same,
-                   const float4 *__restrict__ same2, float4 *__restrict__ out, LatticeGeom g,
-                   int pout, float kappa, float mu, const BicgScalars *__restrict__ sc,
+                   const float4 *__restrict__ same, float4 *__restrict__ out, LatticeGeom g,
+                   int pout, float kappa, float mu,
                    const float4 *__restrict__ aux, double *__restrict__ partial,
                    const int *status, unsigned mask, unsigned long long *__restrict__ sites, int nrhs) {
   chain_enter();
@@ -137,8 +121,6 @@ wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ 
   const long long V = g.V, Vh = g.V / 2;
   if (sites != nullptr && sb == 0 && threadIdx.x == 0)
     atomicAdd(sites, (unsigned long long)Vh);  // work accounting for the profiler
-  const float2 alpha = FUSED ? make_float2((float)sc[r].alpha.x, (float)sc[r].alpha.y)
-                             : make_float2(0.f, 0.f);
   const long long off = (long long)r * 6 * Vh;
   const long long i = sb * blockDim.x + threadIdx.x;
   float red[3] = {0.f, 0.f, 0.f};
@@ -154,23 +136,21 @@ wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ 
     constexpr int F = DAG ? +1 : -1;
     constexpr int B = -F;
     const float4 *sr = src + off;
-    const float4 *sr2 = FUSED && MODE == EO32_SCHUR1 ? src2 + off : nullptr;
-    constexpr bool FS = FUSED && MODE == EO32_SCHUR1;
     float2 acc[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = make_float2(0.f, 0.f);
-    hop_eo32<0, F, false, FS>(links, sr, sr2, alpha, V, nb.up[0], s, acc);
-    hop_eo32<0, B, true, FS>(links, sr, sr2, alpha, V, nb.dn[0], nb.dn[0], acc);
-    hop_eo32<1, F, false, FS>(links, sr, sr2, alpha, V, nb.up[1], s, acc);
-    hop_eo32<1, B, true, FS>(links, sr, sr2, alpha, V, nb.dn[1], nb.dn[1], acc);
-    hop_eo32<2, F, false, FS>(links, sr, sr2, alpha, V, nb.up[2], s, acc);
-    hop_eo32<2, B, true, FS>(links, sr, sr2, alpha, V, nb.dn[2], nb.dn[2], acc);
-    hop_eo32<3, F, false, FS>(links, sr, sr2, alpha, V, nb.up[3], s, acc);
-    hop_eo32<3, B, true, FS>(links, sr, sr2, alpha, V, nb.dn[3], nb.dn[3], acc);
+    hop_eo32<0, F, false>(links, sr, V, nb.up[0], s, acc);
+    hop_eo32<0, B, true>(links, sr, V, nb.dn[0], nb.dn[0], acc);
+    hop_eo32<1, F, false>(links, sr, V, nb.up[1], s, acc);
+    hop_eo32<1, B, true>(links, sr, V, nb.dn[1], nb.dn[1], acc);
+    hop_eo32<2, F, false>(links, sr, V, nb.up[2], s, acc);
+    hop_eo32<2, B, true>(links, sr, V, nb.dn[2], nb.dn[2], acc);
+    hop_eo32<3, F, false>(links, sr, V, nb.up[3], s, acc);
+    hop_eo32<3, B, true>(links, sr, V, nb.dn[3], nb.dn[3], acc);
     const float tmu = DAG ? -mu : mu;
     float2 sm[12];
     if (MODE == EO32_SCHUR2)
-      ld_half32<FUSED>(same + off, FUSED ? same2 + off : nullptr, alpha, Vh, i, sm);
+      ld_half32(same + off, Vh, i, sm);
     const float inv = 1.f / (1.f + tmu * tmu);
     const float k2 = kappa * kappa;
     float2 o[12];
@@ -234,11 +214,9 @@ wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ 
 int schur32_blocks(const wd_context *h) { return (int)((h->V / 2 + 127) / 128); }
 
 // out = A_hat in (dagger: A_hat^dagger) on even half vectors, tmp an odd
-// half vector per system; epi and FUSED (epi == EPI_TSTT: in = r, in2 = v,
-// the operand is s = r - alpha v) as launch_wilson_f32.
-cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, const float4 *in2, float4 *out,
-                             float4 *tmp, int nrhs, int dagger, int epi, const BicgScalars *sc,
-                             const float4 *aux, double *partial, const int *status,
+// half vector per system; epi as launch_wilson_f32.
+cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, float4 *out, float4 *tmp, int nrhs,
+                             int dagger, int epi, const float4 *aux, double *partial, const int *status,
                              unsigned mask, cudaStream_t s) {
   ProfLaunch prof(PC_DSLASH_LOW, s);
   const wd_context *h = m.h;
@@ -247,23 +225,18 @@ cudaError_t launch_schur_f32(const Mixed32 &m, const float4 *in, const float4 *i
   const float kap = (float)h->kappa, mu = (float)h->mu;
   unsigned long long *cnt = prof_site_counter_low();
   cudaError_t e = cudaSuccess;
-#define EO32(D, M, E, FU, SRC, SRC2, SAME, SAME2, OUT, POUT, CNT)                               \
-  if (e == cudaSuccess)                                                                         \
-  e = launch_chained(wilson_eo32_kernel<D, M, E, FU>, grid, dim3(128), 0, s, m.links, SRC, SRC2, SAME, \
-                     SAME2, OUT, g, POUT, kap, mu, sc, aux, partial, status, mask, CNT, nrhs)
-  if (epi == EPI_TSTT) {
-    EO32(false, EO32_SCHUR1, EPI_NONE, true, in, in2, nullptr, nullptr, tmp, 1, nullptr);
-    EO32(false, EO32_SCHUR2, EPI_TSTT, true, tmp, nullptr, in, in2, out, 0, cnt);
-  } else if (epi == EPI_DOT) {
-    EO32(false, EO32_SCHUR1, EPI_NONE, false, in, nullptr, nullptr, nullptr, tmp, 1, nullptr);
-    EO32(false, EO32_SCHUR2, EPI_DOT, false, tmp, nullptr, in, nullptr, out, 0, cnt);
-  } else if (dagger) {
-    EO32(true, EO32_SCHUR1, EPI_NONE, false, in, nullptr, nullptr, nullptr, tmp, 1, nullptr);
-    EO32(true, EO32_SCHUR2, EPI_NONE, false, tmp, nullptr, in, nullptr, out, 0, cnt);
-  } else {
-    EO32(false, EO32_SCHUR1, EPI_NONE, false, in, nullptr, nullptr, nullptr, tmp, 1, nullptr);
-    EO32(false, EO32_SCHUR2, EPI_NONE, false, tmp, nullptr, in, nullptr, out, 0, cnt);
+#define EO32(D, M, E, SRC, SAME, OUT, POUT, CNT)                                                \
+  e = e != cudaSuccess ? e : launch_chained(wilson_eo32_kernel<D, M, E>, grid, dim3(128), 0, s, m.links, SRC, SAME, OUT, g, POUT, \
+                     kap, mu, aux, partial, status, mask, CNT, nrhs)
+  if (dagger && epi == EPI_NONE) {
+    EO32(true, EO32_SCHUR1, EPI_NONE, in, nullptr, tmp, 1, nullptr);
+    EO32(true, EO32_SCHUR2, EPI_NONE, tmp, in, out, 0, cnt);
+    return e;
   }
+  EO32(false, EO32_SCHUR1, EPI_NONE, in, nullptr, tmp, 1, nullptr);
+  if (epi == EPI_TSTT) EO32(false, EO32_SCHUR2, EPI_TSTT, tmp, in, out, 0, cnt);
+  else if (epi == EPI_DOT) EO32(false, EO32_SCHUR2, EPI_DOT, tmp, in, out, 0, cnt);
+  else EO32(false, EO32_SCHUR2, EPI_NONE, tmp, in, out, 0, cnt);
 #undef EO32
   return e;
 }

@@ -110,7 +110,7 @@ extern "C" int wd_apply_f32_noalloc(wd_handle h, const void *in, void *out, int 
     e = launch_f64_to_f32(static_cast<const double2 *>(in), a, h->V, nrhs, nullptr, nullptr,
                           nullptr, M_ALL, s);
   if (e == cudaSuccess)
-    e = launch_wilson_f32(m, a, nullptr, b, nrhs, dagger ? 1 : 0, EPI_NONE, nullptr, nullptr,
+    e = launch_wilson_f32(m, a, b, nrhs, dagger ? 1 : 0, EPI_NONE, nullptr,
                           nullptr, nullptr, M_ALL, s);
   if (e == cudaSuccess) e = launch_f32_to_f64(b, static_cast<double2 *>(out), h->V, nrhs, s);
   if (e != cudaSuccess) return cuda_fail(e, "wd_apply_f32_noalloc");

@@ -164,22 +164,23 @@ int bicgstab_mixed_batched(wd_context *h, const double2 *B, double2 *X, const do
       } else {
         RET_IF(ok(launch_bicg32_update_p(p, r, v, sc, status, n4, nrhs, s), "update_p32"));
         if (eo)
-          RET_IF(ok(launch_schur_f32(m, p, nullptr, v, tmp_o, nrhs, 0, EPI_DOT, sc, rhat, part_w, status, M_ACTIVE, s), "s32_dot"));
+          RET_IF(ok(launch_schur_f32(m, p, v, tmp_o, nrhs, 0, EPI_DOT, rhat, part_w, status, M_ACTIVE, s), "s32_dot"));
         else
-          RET_IF(ok(launch_wilson_f32(m, p, nullptr, v, nrhs, 0, EPI_DOT, sc, rhat, part_w, status, M_ACTIVE, s), "w32_dot"));
+          RET_IF(ok(launch_wilson_f32(m, p, v, nrhs, 0, EPI_DOT, rhat, part_w, status, M_ACTIVE, s), "w32_dot"));
       }
       RET_IF(ok(launch_bicg_finalize(FIN_ALPHA, part_w, nbw, sc, status, nullptr, 0, nrhs, s), "fin_alpha"));
+      if (!half) RET_IF(ok(launch_bicg32_update_s(r, v, sc, status, n4, nrhs, s), "update_s32"));   // r holds s
       if (half)
         RET_IF(ok(launch_wilson_f16(h, h->links16, v16, r, t16, nrhs, 0, EPI_TSTT, sc, nullptr, part_w, status, M_ACTIVE, s), "w16_tstt"));
       else if (eo)
-        RET_IF(ok(launch_schur_f32(m, r, v, t, tmp_o, nrhs, 0, EPI_TSTT, sc, nullptr, part_w, status, M_ACTIVE, s), "s32_tstt"));
+        RET_IF(ok(launch_schur_f32(m, r, t, tmp_o, nrhs, 0, EPI_TSTT, nullptr, part_w, status, M_ACTIVE, s), "s32_tstt"));
       else
-        RET_IF(ok(launch_wilson_f32(m, r, v, t, nrhs, 0, EPI_TSTT, sc, nullptr, part_w, status, M_ACTIVE, s), "w32_tstt"));
+        RET_IF(ok(launch_wilson_f32(m, r, t, nrhs, 0, EPI_TSTT, nullptr, part_w, status, M_ACTIVE, s), "w32_tstt"));
       RET_IF(ok(launch_bicg_finalize(FIN_OMEGA, part_w, nbw, sc, status, nullptr, 0, nrhs, s), "fin_omega"));
       if (half)
         RET_IF(ok(launch_bicg16_update_xr(xs, r, p16, v16, t16, rhat, sc, status, part_s, V, nrhs, s), "update_xr16"));
       else
-        RET_IF(ok(launch_bicg32_update_xr(xs, r, p, v, t, rhat, sc, status, part_s, n4, nrhs, s), "update_xr32"));
+        RET_IF(ok(launch_bicg32_update_xr(xs, r, p, t, rhat, sc, status, part_s, n4, nrhs, s), "update_xr32"));
       RET_IF(ok(launch_bicg_finalize(FIN_RHO, part_s, nbs, sc, status, nullptr, 0, nrhs, s), "fin_rho"));
     }
     return WD_OK;
