@@ -140,7 +140,7 @@ __device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
 }
 
 // One block per system.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 bicg_finalize_kernel(int kind, const double *partial, int nb, BicgScalars *sc,
                      int *status, double *hist, int hist_len) {
   chain_enter();
@@ -198,7 +198,7 @@ cudaError_t launch_bicg_finalize(int kind, const double *partial, int nb, BicgSc
                                  int *status, double *hist, int hist_len, int nrhs,
                                  cudaStream_t s) {
   ProfLaunch prof_(PC_STREAM, s);
-  return launch_chained(bicg_finalize_kernel, dim3(nrhs), dim3(256), 0, s, kind, partial, nb, sc, status, hist, hist_len);
+  return launch_chained(bicg_finalize_kernel, dim3(nrhs), dim3(nb > 1024 ? 1024 : 256), 0, s, kind, partial, nb, sc, status, hist, hist_len);
 }
 
 // ----------------------------------------------------------------- tall-skinny

@@ -116,3 +116,20 @@ def test_bicgstab_steps_match_oracle(wdl, dims, kind, iters):
             continue
         assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
     op.close()
+
+
+@pytest.mark.parametrize("dims", [(8, 8, 16, 1), (43, 8, 3, 1), (10, 10, 10, 6), (26, 16, 16, 10)])
+@pytest.mark.parametrize("scale", [1.0, 1e-130])
+def test_scalar_steps_over_partials(wdl, dims, scale):
+    """The dots' block partials (bicg_fin.cuh): 128, 129, 750 and 1040 of them,
+    in fixed point and, for squares below its range, in FP64.  Two steps at
+    kappa = 0.1: 1e-12, as above."""
+    U = L.gauge_field(dims, 0.5, 97)
+    A, _ = oracle_ops(U, dims, 0.1)
+    b = L.gaussian_spinor(dims, 98).ravel()
+    ref, _ = krylov.bicgstab(A, b, tol=1e-15, max_iter=2)
+    op = wdl.WilsonOperator(dims, cuda(U), 0.1)
+    X = cuda(np.zeros_like(b)[None])
+    op.dbicgstab(cuda(scale * b[None]), X, None, tol=1e-15, max_iter=2)
+    assert np.linalg.norm(host(X)[0] / scale - ref) <= 1e-12 * np.linalg.norm(ref)
+    op.close()
