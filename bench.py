@@ -46,10 +46,15 @@ SM_MAX_MHZ = 2070.0
 
 DSLASH_FLOPS_PER_SITE = 1368      # 1320 hopping + 48 for 1 - kappa*D
 DSLASH_BYTES_PER_SITE = 960       # 192 in + 192 out + 4 links x 144 (FP64)
-# DRAM bytes (read + write) per site update of wilson_f64_kernel from one ncu
-# capture of a 10-system launch at 16^4 (383.6 + 111.4 MB / 655,360 site
+# DRAM bytes (read + write) per site update of wilson_fx_kernel from one ncu
+# capture of a 10-system launch at 16^4 (316.6 + 110.7 MB / 655,360 site
 # updates); the bench scales it to a launch by the site updates it processed.
-DSLASH_DRAM_BYTES_PER_SITE_UPDATE = 495.0e6 / 655360
+DSLASH_DRAM_BYTES_PER_SITE_UPDATE = 427.3e6 / 655360
+# The FP64 operator's products are formed in fixed point: 8 hops x 6 components
+# x 3 terms x 9 integer multiply-adds (32 x 32 + 64 bits) a site update, which a
+# throughput probe of independent chains issues at 53 per clock and SM.
+DSLASH_WIDE_MADS_PER_SITE = 1296
+WIDE_MADS_PER_CLK_PER_SM = 53
 METRIC = "D-BiCGStab solves/s at rel. residual 1e-10; dslash GB/s vs HBM roofline"
 
 
@@ -515,20 +520,26 @@ def roofline(res, peaks, fp64_peak):
     flops = DSLASH_FLOPS_PER_SITE * sites_per_launch
     tflops = flops / (avg_ms * 1e-3) / 1e12
     gbs = DSLASH_BYTES_PER_SITE * sites_per_launch / (avg_ms * 1e-3) / 1e9
+    peak = (WIDE_MADS_PER_CLK_PER_SM * SMS * SM_MAX_MHZ * 1e6 / DSLASH_WIDE_MADS_PER_SITE
+            * DSLASH_FLOPS_PER_SITE / 1e12)
     out = {
-        "kernel": "wilson_f64_kernel (FP64 dslash)",
+        "kernel": "wilson_fx_kernel (FP64 dslash, products in fixed point)",
         "bound": "alu",
         "achieved": round(tflops, 4),
-        "peak": fp64_peak["tflops"],
+        "peak": round(peak, 4),
         "unit": "TFLOP/s",
-        "frac": round(tflops / fp64_peak["tflops"], 4),
-        "peak_source": fp64_peak["source"],
-        "peak_derived": fp64_peak["derived_tflops"],
-        "frac_of_derived": round(tflops / fp64_peak["derived_tflops"], 4),
-        "peak_derived_source": fp64_peak["derived_source"],
+        "frac": round(tflops / peak, 4),
+        "peak_source": (f"{DSLASH_WIDE_MADS_PER_SITE} 32 x 32 + 64-bit multiply-adds a site update at "
+                        f"{WIDE_MADS_PER_CLK_PER_SM} per clock and SM (throughput probe), {SMS} SMs, "
+                        f"{SM_MAX_MHZ:.0f} MHz, counted as the {DSLASH_FLOPS_PER_SITE} FP64 flops they stand for"),
+        "fp64_pipe_peak": fp64_peak["tflops"],
+        "times_fp64_pipe_peak": round(tflops / fp64_peak["tflops"], 4),
+        "fp64_pipe_peak_source": fp64_peak["source"],
+        "fp64_pipe_peak_derived": fp64_peak["derived_tflops"],
+        "fp64_pipe_peak_derived_source": fp64_peak["derived_source"],
         "traffic": round(DSLASH_DRAM_BYTES_PER_SITE_UPDATE * sites_per_launch),
         "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 16^4 "
-                          "10-system launch (755 B per site update), scaled to the average "
+                          "10-system launch (652 B per site update), scaled to the average "
                           "launch by site updates",
         "algorithmic_flops_per_launch": flops,
         "avg_launch_ms": avg_ms,
@@ -638,13 +649,16 @@ def main():
 # JSON line.
 
 # FP32 / FP16 bytes per site and system of the mixed solver's kernels
-LOW_DSLASH_BYTES = {32: 3 * 96, 16: 52 + 52 + 96}   # in + out + (r_hat or r) per site update
+# per site update: in + out, and r_hat for the first product of a step (FP32) or
+# r_hat or r (FP16)
+LOW_DSLASH_BYTES = {32: (3 * 96 + 2 * 96) / 2, 16: 52 + 52 + 96}
 LOW_LINK_BYTES = {32: 4 * 48, 16: 4 * 24}            # links (rows 0, 1), read once per launch
 # even-odd Schur apply (FP32), per even site and system: v = A_hat p moves
 # SCHUR1 in + tmp and SCHUR2 tmp + p + out + r_hat; t = A_hat (r - alpha v) moves
-# SCHUR1 r + v + tmp and SCHUR2 tmp + r + v + out; the mean of the two applies
+# SCHUR1 r + v + tmp and SCHUR2 tmp + r + v + out; the mean of the two applies.
+# (The kernels read s = r - alpha v, which an update pass writes: 11 of these 13.)
 LOW_SCHUR_BYTES = {32: (2 * 96 + 4 * 96 + 3 * 96 + 4 * 96) / 2}
-LOW_UPDATE_BYTES = {32: 4 * 96 + 8 * 96,             # p = r + beta (p - omega v); x, r update
+LOW_UPDATE_BYTES = {32: 4 * 96 + 3 * 96 + 7 * 96,    # p = r + beta (p - omega v); s; x, r update
                     16: (96 + 3 * 52) + (4 * 96 + 3 * 52 + 2 * 96)}
 
 
@@ -693,7 +707,8 @@ def timed_steps(args, step, op, flush, stream, world, dev, prof_mask=0):
 def low_rooflines(prof, bits, V, peaks, iters_total, eo=False):
     """HBM rooflines of the mixed solver's FP32/FP16 kernels from a profiled
     step: the Wilson apply (site updates counted on the device) and the two
-    per-iteration vector updates (one pass of each per system iteration).
+    per-iteration vector updates (one pass of each per system iteration; FP16
+    forms s inside its product and update).
     On the even-odd Schur system (eo) one profiled launch is a Schur apply: two
     half-lattice hop kernels, each reading every link, with V/2 counted site
     updates per system (LOW_SCHUR_BYTES each); the vector updates run over V/2
@@ -719,7 +734,7 @@ def low_rooflines(prof, bits, V, peaks, iters_total, eo=False):
     if u["launches"]:
         byt = LOW_UPDATE_BYTES[bits] * (V // 2 if eo else V) * iters_total
         gbs = byt / (u["ms"] * 1e-3) / 1e9
-        out["updates"] = {"kernel": f"bicg{bits}_update_p + bicg{bits}_update_xr", "bound": "hbm",
+        out["updates"] = {"kernel": f"bicg{bits}_update_p{' + bicg32_update_s' if bits == 32 else ''} + bicg{bits}_update_xr", "bound": "hbm",
                           "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",
                           "frac": round(gbs / hbm, 4) if hbm else None, "traffic": None,
                           "avg_launch_ms": u["ms"] / u["launches"], "launches": u["launches"],

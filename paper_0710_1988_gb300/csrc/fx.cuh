@@ -276,10 +276,15 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
 // spin 2 + sp, in units 2^(E - 1079).  The next hop's operands are copied to
 // shared memory (st: two stages of this warp) while one hop is computed: the
 // copies wait for L2 and hold no registers (through L1, which serves a third
-// of them: a 10-system apply at 16^4 0.288 ms with the staging, 0.301 with
-// plain loads, 0.332 with copies past L1; the arithmetic alone 0.237).  The y and z hops come first in
-// their lower sums, whose factor sgn is then applied once; between them the
-// lanes exchange the x and y hops' lower sums, which belong to the other.
+// of them).  A 10-system apply at 16^4 took 0.301 ms with plain loads, 0.332 with
+// copies past L1, 0.288 so, of which 0.237 without any copy; with a hop's shift
+// rounded in its first sum (no additions, no branch for d = 0) and blocks of
+// half the size 0.267, with the epilogue's operand copied during the last hop
+// (tail) 0.257.  Now the LSU's data pipe (78 % of its wavefronts) and the
+// multiply-adds (54 %) bound it, at the 16 warps an SM that 128 registers leave.
+// The y and z hops come first in their lower sums, whose factor sgn is then
+// applied once; between them the lanes exchange the x and y hops' lower sums,
+// which belong to the other.
 template <int F, class LinkAt, class SiteAt, class Tail>
 __device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, Tail tail, int sp, int E,
                                         const int (&eu)[4], const int (&ed)[4],

@@ -138,7 +138,7 @@ cudaError_t launch_fxb_encode(const double2 *w, const double2 *H, int idx, doubl
 // A thread's entries of the next FXB_DEPTH vectors travel to shared memory
 // while it works on one: 16-byte copies into its own slots, so no barrier and
 // no registers (with the loads in registers the kernels wait for them: the
-// dot 397 us where this form takes 121, 61 vectors on average at 16^4).
+// dot 397 us where this form takes 116, 61 vectors on average at 16^4).
 constexpr int FXB_DEPTH = 4;
 struct FxbRing {
   int4 w[FXB_DEPTH][4][FXB_THREADS];   // hi and lo of both halves of the chunk

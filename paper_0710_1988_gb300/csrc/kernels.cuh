@@ -65,7 +65,7 @@ struct FinArgs {
 
 LatticeGeom geom_of(const wd_context *h);
 
-// Fixed-point spinors (fx.cuh): v [rhs][tile][12][32], e [rhs][sites].
+// Fixed-point spinors (fx.cuh): v [rhs][tile of 32 sites][12][32], e [rhs][sites].
 struct FxVec {
   int4 *v;
   int *e;
