@@ -280,8 +280,8 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
 // copies past L1, 0.288 so, of which 0.237 without any copy; with a hop's shift
 // rounded in its first sum (no additions, no branch for d = 0) and blocks of
 // half the size 0.267, with the epilogue's operand copied during the last hop
-// (tail) 0.257.  Now the LSU's data pipe (78 % of its wavefronts) and the
-// multiply-adds (54 %) bound it, at the 16 warps an SM that 128 registers leave.
+// (tail) 0.257.  Now the LSU's data pipe (83 % of its wavefronts) and the
+// multiply-adds (56 %) bound it, at the 16 warps an SM that 128 registers leave.
 // The y and z hops come first in their lower sums, whose factor sgn is then
 // applied once; between them the lanes exchange the x and y hops' lower sums,
 // which belong to the other.
