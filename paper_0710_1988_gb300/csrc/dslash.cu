@@ -548,11 +548,13 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
 
 // Whether the few-site kernel serves nrhs systems of the full operator: up to
 // where the two forms take the same time, sites x systems (us an apply, this
-// kernel against encoding + wilson_fx_kernel): 256: 7.6 / 18.3, 4096: 10.3 /
-// 18.5, 8192: 14.4 / 18.5, 10395: 16.5 / 26.3, 16384: 24.6 / 18.5.  The solvers'
-// products (epi) come with their input encoded, 4.8 us less.
+// kernel / encoding + wilson_fx_kernel).  Even extents: 256: 9.2 / 12.4, 4096: 9.5 /
+// 12.4, 8192: 12.5 / 12.5, 16384: 21.8 / 15.0.  With an odd extent, where the links
+// are not stored by parity, 3465: 9.6 / 14.4, 10395: 14.6 / 18.5.  The
+// solvers' products (epi) come with their input encoded, some 3 us less.
 static bool fx_few(const wd_context *h, int nrhs, int epi) {
-  return !h->eo && h->links_fx != nullptr && h->V * nrhs <= (epi == EPI_NONE ? 12288 : 6144);
+  const long long most = epi != EPI_NONE ? 6144 : geom_of(h).split ? 8192 : 12288;
+  return !h->eo && h->links_fx != nullptr && h->V * nrhs <= most;
 }
 
 // The handle's fixed-point links, or none where they do not fit fx.cuh's
