@@ -35,6 +35,7 @@ __device__ __forceinline__ void fin_warp_sum(const double (&x)[N][3], double (&s
     }
     e = __reduce_max_sync(0xffffffffu, e);
     if (e <= FX_EMAX && (e >= FX_EMIN || !__any_sync(0xffffffffu, any))) {
+      e = max(e, FX_EMIN);   // zeros are shifted out, also where all entries are zero
       long long t = 0;
 #pragma unroll
       for (int i = 0; i < N; ++i) {
