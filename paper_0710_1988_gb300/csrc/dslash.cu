@@ -263,20 +263,13 @@ fx_encode_kernel(const double2 *__restrict__ in, FxVec out, long long sites, siz
   for (int c = 0; c < 12; ++c) o[c * FX_TILE] = fx_slices(p[c], max(e, FX_EMIN));
 }
 
-// sum over the eight hops of one site in FP64: the sites next to a value that
-// fixed point does not hold
+// fx_exact on FP64 spinors; a call, so that the kernel's registers are not its own
 template <bool DAG>
-__device__ __noinline__ void hops_f64(const double2 *__restrict__ psi,
-                                      const double2 *__restrict__ links, const Nbrs32 &nb,
-                                      long long s, double2 *acc) {
-  constexpr int F = DAG ? +1 : -1;
-  double2 t[12];
-  hop_pair<0, F, true>(psi, links, nb.up[0], s, nb.dn[0], t);
-  hop_pair<1, F, false>(psi, links, nb.up[1], s, nb.dn[1], t);
-  hop_pair<2, F, false>(psi, links, nb.up[2], s, nb.dn[2], t);
-  hop_pair<3, F, false>(psi, links, nb.up[3], s, nb.dn[3], t);
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = t[c];
+__device__ __noinline__ void hops_f64(const double2 *psi, const double2 *__restrict__ links,
+                                      const LatticeGeom &g, unsigned s, int sp, bool special, int lost, double2 *out) {
+  const Nbrs32 nb = neighbours32(s, g);
+  fx_exact<DAG, true>([&](unsigned q, int c) { return psi[(size_t)q * 12 + c]; }, links, nb.up, nb.dn, s, sp,
+                      special, lost, out);
 }
 
 // wilson_f64_kernel's result with the hops in fixed point; `in` is the
@@ -320,12 +313,13 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   const size_t base = ((size_t)r * V + first) * 12;
   const int count = 12 * (int)max(0LL, min(16LL, g.V - first));
   longlong2 up[3], low[3];
+  uint2 reach;
   {
     const int4 *psi = in.v + (size_t)r * 12 * tiled;
     const unsigned half = g.split, odd = (unsigned)(g.V / 2);
     const unsigned here = g.split ? (nb.par ? odd : 0u) + (s >> 1) : s;
     const unsigned other = g.split && !nb.par ? odd : 0u;
-    fx_hops<(DAG ? +1 : -1)>(
+    reach = fx_hops<(DAG ? +1 : -1)>(
         stage, [&](int m, bool fwd) {
           return L + fx_at(fwd ? here : other + (nb.dn[m] >> half), 36) + m * 9 * FX_TILE;
         },
@@ -342,10 +336,10 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
     mine[3 * sp + a] = make_double2(fx_to_double(up[a].x, E), fx_to_double(up[a].y, E));
     mine[6 + 3 * sp + a] = make_double2(fx_to_double(low[a].x, E), fx_to_double(low[a].y, E));
   }
+  const int lost = E != 0 ? fx_lost(reach, FX_REACH) : 0;   // E = 0: all neighbours are zero
   __syncwarp();
-  if (E == FX_SPECIAL && sp == 0 && valid) {
-    hops_f64<DAG>(in64 + (size_t)r * 12 * V, links, nb, s, mine);
-  }
+  if (__any_sync(0xffffffffu, E == FX_SPECIAL || lost != 0))
+    hops_f64<DAG>(in64 + (size_t)r * 12 * V, links, g, s, sp, E == FX_SPECIAL, lost, mine);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
   const double2 *own = reinterpret_cast<const double2 *>(stage);
@@ -403,6 +397,43 @@ __device__ __forceinline__ longlong2 shfl_xor(longlong2 v, int lane) {
 // site are summed over lanes; no encoded copy, one launch.  It issues about
 // twice the instructions a site of wilson_fx_kernel.
 constexpr int FX_FEW_SITES = 8;   // sites a block, two a warp
+
+// fx_exact in the layout of this kernel: the four lanes of a direction form both
+// its hops.  q: the lane's neighbour; reached_by: the lanes whose terms reach the
+// lane's component, of colour j.  Returns whether the site's sums are in out.
+template <bool DAG>
+__device__ __noinline__ bool few_f64(const double2 *psi, const double2 *__restrict__ links, unsigned s, int m, bool fwd,
+                                     unsigned q, int sp, unsigned reached_by, int j, bool special, bool lost,
+                                     double2 *out) {
+  const int lane = threadIdx.x & 31;
+  auto ld = [&](unsigned at, int c) { return psi[(size_t)at * 12 + c]; };
+  bool need = special;
+  if (__any_sync(0xffffffffu, lost && !special)) {
+    const int t = fx_terms(ld, links + ((size_t)(fwd ? s : q) * 4 + m) * 9, !fwd, q, sp, m < 2 ? 3 - sp : 2 + sp);
+    const unsigned t0 = __ballot_sync(0xffffffffu, t & 1), t1 = __ballot_sync(0xffffffffu, t & 2),
+                   t2 = __ballot_sync(0xffffffffu, t & 4);
+    need = need || (lost && ((j == 0 ? t0 : j == 1 ? t1 : t2) & reached_by) != 0);
+  }
+  const unsigned any = __ballot_sync(0xffffffffu, need);
+  if (any == 0) return false;
+  need = ((any >> (lane & 16)) & 0xffffu) != 0;
+  const unsigned other = __shfl_xor_sync(0xffffffffu, q, 1);
+  double2 acc[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
+  fx_pair_f64<true>(ld, links, m, DAG ? +1 : -1, fwd ? q : other, s, fwd ? other : q, acc);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+#pragma unroll
+    for (int o = 2; o <= 4; o <<= 1) {
+      acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, o);
+      acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, o);
+    }
+    if ((lane & 15) == c) out[c] = acc[c];
+  }
+  __syncwarp();
+  return need;
+}
 
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(16 * FX_FEW_SITES)
@@ -505,17 +536,26 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
       sum[a] = make_longlong2(sum[a].x + v.x, sum[a].y + v.y);
     }
   }
+  // by colour: the lanes whose terms are long enough (fx.cuh); those of this
+  // lane's component are the hops of its spin, or for a lower spin the z and t hops
+  // of the upper one that it goes with and the x and y hops of the other
+  unsigned term[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int hr = (int)(up[a].x >> 32), hi = (int)(up[a].y >> 32);
+    term[a] = __ballot_sync(0xffffffffu, ((hr ^ (hr >> 31)) | (hi ^ (hi >> 31))) >= 1 << (FX_REACH - 1));
+  }
   const int j = lane & 3;   // colour of this lane's entry (3: none)
+  const unsigned reached_by = (lower ? (sp ? 0xf00fu : 0x0ff0u) : (sp ? 0xff00u : 0x00ffu)) << (lane & 16);
+  const bool lost = j < 3 && E != 0 && ((j == 0 ? term[0] : j == 1 ? term[1] : term[2]) & reached_by) == 0;
   const longlong2 T = j == 0 ? sum[0] : j == 1 ? sum[1] : sum[2];
   double2 hop = make_double2(fx_to_double(T.x, E), fx_to_double(T.y, E));
   const int c = 3 * ((lower ? 2 : 0) + sp) + j;
-  // values that fixed point does not hold
-  __shared__ double2 exact[FX_FEW_SITES][12];
-  if (__any_sync(0xffffffffu, E == FX_SPECIAL)) {
-    if (E == FX_SPECIAL && (lane & 15) == 0)
-      hops_f64<DAG>(in + (size_t)r * 12 * V, links, neighbours32(s, g), s, exact[local]);
-    __syncwarp();
-    if (E == FX_SPECIAL && j < 3) hop = exact[local][c];
+  if (__any_sync(0xffffffffu, E == FX_SPECIAL || lost)) {
+    __shared__ double2 exact[FX_FEW_SITES][12];
+    if (few_f64<DAG>(in + (size_t)r * 12 * V, links, s, m, fwd, q, sp, reached_by, j, E == FX_SPECIAL, lost,
+                     exact[local]) && j < 3)
+      hop = exact[local][c];
   }
   double2 dv[1] = {make_double2(0.0, 0.0)}, da[1] = {make_double2(0.0, 0.0)};
   if (valid && j < 3) {

@@ -146,51 +146,28 @@ wilson_eo_kernel(const double2 *__restrict__ links, const double2 *__restrict__ 
 
 // ----------------------------------------------------------------- fixed-point form
 
-// D_{pout, 1-pout} src at site s in FP64, from the FP64 values of the sites
-// that fixed point does not hold and the fixed-point ones of the others: the
-// sites next to such a value.
-template <int MU, int S, bool ADJ>
-__device__ __forceinline__ void hop_mixed(const double2 *__restrict__ src, const int4 *__restrict__ psi,
-                                          const int *__restrict__ e, const double2 *__restrict__ links,
-                                          unsigned q, long long ql, double2 (&acc)[12]) {
-  double2 p[12], h[6], c[6];
-  const int E = e[q >> 1];
-  const int4 *x = psi + fx_at(q >> 1, 12);
-#pragma unroll
-  for (int i = 0; i < 12; ++i)
-    p[i] = E == FX_SPECIAL ? src[(size_t)(q >> 1) * 12 + i] : fx_decode(x[i * FX_TILE], E);
-  project<MU, S>(p, h);
-  su3_mul_eo<ADJ>(links + (ql * 4 + MU) * 9, h, c);
-  reconstruct<MU, S>(acc, c);
-}
-
+// fx_exact for D_{pout, 1-pout} src at site s.  whole: src has every site's FP64
+// values; else those that fixed point does not hold, and psi, e the others.
 template <bool DAG>
-__device__ __noinline__ void hops_mixed(const double2 *__restrict__ src, const int4 *__restrict__ psi,
-                                        const int *__restrict__ e, const double2 *__restrict__ links,
-                                        const Nbrs32 nb, unsigned s, double2 *out) {
-  constexpr int F = DAG ? +1 : -1;
-  constexpr int B = -F;
-  double2 acc[12];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
-  hop_mixed<0, F, false>(src, psi, e, links, nb.up[0], s, acc);
-  hop_mixed<0, B, true>(src, psi, e, links, nb.dn[0], nb.dn[0], acc);
-  hop_mixed<1, F, false>(src, psi, e, links, nb.up[1], s, acc);
-  hop_mixed<1, B, true>(src, psi, e, links, nb.dn[1], nb.dn[1], acc);
-  hop_mixed<2, F, false>(src, psi, e, links, nb.up[2], s, acc);
-  hop_mixed<2, B, true>(src, psi, e, links, nb.dn[2], nb.dn[2], acc);
-  hop_mixed<3, F, false>(src, psi, e, links, nb.up[3], s, acc);
-  hop_mixed<3, B, true>(src, psi, e, links, nb.dn[3], nb.dn[3], acc);
-#pragma unroll
-  for (int c = 0; c < 12; ++c) out[c] = acc[c];
+__device__ __noinline__ bool hops_mixed(const double2 *src, const int4 *psi, const int *e, bool whole,
+                                        const double2 *__restrict__ links, const Nbrs32 nb, unsigned s, int sp,
+                                        bool special, int lost, double2 *out) {
+  auto ld = [&](unsigned q, int c) {
+    const unsigned i = q >> 1;
+    if (whole || e[i] == FX_SPECIAL) return src[(size_t)i * 12 + c];
+    return fx_decode(psi[fx_at(i, 12) + c * FX_TILE], e[i]);
+  };
+  return fx_exact<DAG, false>(ld, links, nb.up, nb.dn, s, sp, special, lost, out);
 }
 
 constexpr size_t EO_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);    // two stages a warp
 
 // wilson_eo_kernel's modes with the hops in fixed point (fx.cuh): src is the
-// encoded operand, src64 its FP64 values at least where it has FX_SPECIAL.
-// EO_SCHUR1 writes the odd vector in fixed point (outfx) for the second half
-// hop, and in FP64 (out) only the sites that need it.
+// encoded operand, src64 its FP64 values, for EO_SCHUR2 only where it has
+// FX_SPECIAL.  EO_SCHUR1 writes the odd vector in fixed point (outfx) for the
+// second half hop, and in FP64 (out) the sites that need it: values that fixed
+// point does not hold, or components so far below their site's largest that its
+// unit would be coarser than FP64's rounding of their terms.
 template <bool DAG, int MODE, int EPI>
 __global__ void __launch_bounds__(2 * WILSON_SITES, 4)
 wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec src,
@@ -235,7 +212,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
   const size_t base = off + (size_t)first * 12;
   const int count = 12 * (int)max(0LL, min(16LL, (long long)Vh - first));
   const unsigned here = (pout ? Vh : 0u) + i, other = pout ? 0u : Vh;
-  fx_hops<(DAG ? +1 : -1)>(
+  const uint2 reach = fx_hops<(DAG ? +1 : -1)>(
       stage, [&](int m, bool fwd) {
         return L + fx_at(fwd ? here : other + (nb.dn[m] >> 1), 36) + m * 9 * FX_TILE;
       },
@@ -243,10 +220,16 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
       [&](double2 *own) { fx_fetch_own(own, same + base, MODE == EO_SCHUR1 ? 0 : count); }, sp, E, eu,
       ed, up, low);
   const double tmu = DAG ? -mu : mu;
-  if (MODE == EO_SCHUR1 && tmu == 0.0 && __all_sync(0xffffffffu, E != FX_SPECIAL)) {
-    // h itself: the sums' slices, without a way through FP64
-    int bits = fx_sum_bits(up, low);
+  int bits = 0, least = FX_REACH;
+  if (MODE == EO_SCHUR1) {   // a stored site's unit is 2^(bits - 56): terms of 2^-7 of the largest sum
+    bits = fx_sum_bits(up, low);
     bits = max(bits, __shfl_xor_sync(0xffffffffu, bits, 16));
+    least = max(least, bits - 38);
+  }
+  const int lost = E != 0 ? fx_lost(reach, least) : 0;   // E = 0: all neighbours are zero
+  const bool exact = __any_sync(0xffffffffu, E == FX_SPECIAL || lost != 0);
+  if (MODE == EO_SCHUR1 && tmu == 0.0 && !exact) {
+    // h itself: the sums' slices, without a way through FP64
     if (valid) {
       int4 *o = outfx.v + (size_t)r * 12 * tiled + fx_at(i, 12);
 #pragma unroll
@@ -269,7 +252,9 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     mine[6 + 3 * sp + a] = make_double2(fx_to_double(low[a].x, E), fx_to_double(low[a].y, E));
   }
   __syncwarp();
-  if (E == FX_SPECIAL && sp == 0 && valid) hops_mixed<DAG>(src64 + off, psi, ev, links, nb, s, mine);
+  bool in64 = false;   // the site's sums are FP64's
+  if (exact)
+    in64 = hops_mixed<DAG>(src64 + off, psi, ev, MODE != EO_SCHUR2, links, nb, s, sp, E == FX_SPECIAL, lost, mine);
   __syncwarp();
   if (MODE == EO_SCHUR1) {   // (1 - i mu g5) h / (1 + mu^2)
     double2 v[6];
@@ -286,7 +271,7 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
     }
     e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
     any |= __shfl_xor_sync(0xffffffffu, any, 16);
-    const int Eo = fx_site_exponent(e, any == 0);
+    const int Eo = in64 ? FX_SPECIAL : fx_site_exponent(e, any == 0);
     if (valid) {
       int4 *o = outfx.v + (size_t)r * 12 * tiled + fx_at(i, 12);
 #pragma unroll

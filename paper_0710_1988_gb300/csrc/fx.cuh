@@ -23,11 +23,17 @@
 // to FP64 at the end.  Its error is a few units of 2^-57 of the largest
 // neighbour entry; the eight hops' FP64 roundings leave more (2-norm against
 // 64-bit torch arithmetic, whose own rounding is in both: 1.0e-16 against
-// 1.1e-16).
+// 1.1e-16).  That holds for a component whose own terms are of the size of the
+// largest entry.  A component that only smaller entries reach (colours that a
+// diagonal link does not mix, spins that a large neighbour's projector leaves out)
+// would keep fewer bits than in FP64: fx_hops tells the terms' size, and
+// components whose terms all lie below 2^52 units, where FP64 would leave less
+// than a few units, are formed in FP64 (fx_exact).
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include "cplx.cuh"
 #include "spin.cuh"
 
 namespace wd {
@@ -246,10 +252,12 @@ __device__ __forceinline__ void fx_fetch_own(double2 *own, const double2 *x, int
 }
 
 // The lane's part of one hop, in units 2^(Eq + d - 1079): up += chi, low +=
-// (factor without sgn) chi, low lying in the neighbour's spin cl.
+// (factor without sgn) chi, low lying in the neighbour's spin cl.  reach: the
+// high words of the forward hops' |chi|, or-ed, by colour: four hops tell the terms'
+// size, at half the cost of eight (10-system apply at 16^4: 266 us, eight 271, none 257).
 template <int MU, int S, bool ADJ>
 __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
-                                       longlong2 (&up)[3], longlong2 (&low)[3]) {
+                                       longlong2 (&up)[3], longlong2 (&low)[3], int (&reach)[3]) {
   using W = FxSpin<MU, S>;
   const int site = threadIdx.x & 15, sgn = 1 - 2 * sp;
   const long long half = (long long)((1ULL << d) >> 1);
@@ -267,9 +275,30 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
     for (int b = 0; b < 3; ++b) fx_cmac<ADJ>(s, st.u[ADJ ? 3 * b + a : 3 * a + b][site], h[b]);
     longlong2 chi = fx_value<ADJ>(s);
     chi = make_longlong2(chi.x >> d, chi.y >> d);   // rounded: half is in h1, so in both parts
+    const int hr = (int)(chi.x >> 32), hi = (int)(chi.y >> 32);
+    if (!ADJ) reach[a] |= (hr ^ (hr >> 31)) | (hi ^ (hi >> 31));
     up[a] = fx_add<0>(up[a], chi);
     low[a] = fx_add<W::R>(low[a], chi);
   }
+}
+
+// bit lengths of three words, a byte each
+__device__ __forceinline__ unsigned fx_lengths(const int (&m)[3]) {
+  return (32u - __clz(m[0])) | (32u - __clz(m[1])) << 8 | (32u - __clz(m[2])) << 16;
+}
+
+constexpr int FX_REACH = 21;   // least bit length of a high word: terms of 2^52 units
+
+// The lane's components whose terms are all shorter than `least`, as bits: up's
+// colours 0 .. 2, low's 3 .. 5.
+__device__ __forceinline__ int fx_lost(uint2 reach, int least) {
+  int lost = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lost |= (int)((reach.x >> (8 * a)) & 0xffu) < least ? 1 << a : 0;
+    lost |= (int)((reach.y >> (8 * a)) & 0xffu) < least ? 8 << a : 0;
+  }
+  return lost;
 }
 
 // The eight hops of a site for one lane: up is the sum's spin sp, low its
@@ -284,13 +313,18 @@ __device__ __forceinline__ void fx_hop(const FxStage &st, int sp, int cl, int d,
 // multiply-adds (56 %) bound it, at the 16 warps an SM that 128 registers leave.
 // The y and z hops come first in their lower sums, whose factor sgn is then
 // applied once; between them the lanes exchange the x and y hops' lower sums,
-// which belong to the other.
+// which belong to the other.  Returned: the bit lengths of the high words of the
+// largest forward |chi| in each component's sum, by colour a byte: .x of up, .y of
+// low.  On fields whose sites are of one size a component's four stay below 2^52 units
+// once in 1e8 sites; where one neighbour exceeds the others by 2^4 or more some per
+// cent of the sites go to FP64.
 template <int F, class LinkAt, class SiteAt, class Tail>
-__device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, Tail tail, int sp, int E,
-                                        const int (&eu)[4], const int (&ed)[4],
-                                        longlong2 (&up)[3], longlong2 (&low)[3]) {
+__device__ __forceinline__ uint2 fx_hops(FxStage *st, LinkAt link, SiteAt site, Tail tail, int sp, int E,
+                                         const int (&eu)[4], const int (&ed)[4],
+                                         longlong2 (&up)[3], longlong2 (&low)[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) up[a] = low[a] = make_longlong2(0, 0);
+  int reach[3] = {0, 0, 0};
 #define FX_FETCH(B, M, FWD) fx_fetch(st[B], link(M, FWD), site(M, FWD));
 #define FX_READY(N)                                            \
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); \
@@ -302,11 +336,11 @@ __device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, T
 #define FX_PAIR(M, CL, NEXT, WAIT)                                      \
   FX_FETCH(1, M, false)                                                 \
   FX_READY(1)                                                           \
-  fx_hop<M, F, false>(st[0], sp, CL, min(E - eu[M], 63), up, low);      \
+  fx_hop<M, F, false>(st[0], sp, CL, min(E - eu[M], 63), up, low, reach); \
   __syncwarp();                                                         \
   NEXT                                                                  \
   FX_READY(WAIT)                                                        \
-  fx_hop<M, -F, true>(st[1], sp, CL, min(E - ed[M], 63), up, low);      \
+  fx_hop<M, -F, true>(st[1], sp, CL, min(E - ed[M], 63), up, low, reach); \
   __syncwarp();
   FX_FETCH(0, 1, true)
   FX_PAIR(1, 3 - sp, FX_FETCH(0, 0, true), 1)
@@ -316,14 +350,137 @@ __device__ __forceinline__ void fx_hops(FxStage *st, LinkAt link, SiteAt site, T
   for (int a = 0; a < 3; ++a)
     low[a] = make_longlong2(__shfl_xor_sync(0xffffffffu, low[a].x, 16),
                             __shfl_xor_sync(0xffffffffu, low[a].y, 16));
+  const unsigned xy = fx_lengths(reach);
+  reach[0] = reach[1] = reach[2] = 0;
   FX_SIGN
   FX_PAIR(2, 2 + sp, FX_FETCH(0, 3, true), 1)
   FX_SIGN
   FX_PAIR(3, 2 + sp, tail(reinterpret_cast<double2 *>(&st[0]));, 1)
+  const unsigned zt = fx_lengths(reach);
+  return make_uint2(__vmaxu4(xy, zt), __vmaxu4(zt, __shfl_xor_sync(0xffffffffu, xy, 16)));
 #undef FX_PAIR
 #undef FX_SIGN
 #undef FX_READY
 #undef FX_FETCH
+}
+
+// ----------------------------------------------------------------- in FP64
+
+__device__ __forceinline__ double2 fx_turned(double2 b, int f) {   // i^f b
+  const double x = f & 1 ? b.y : b.x, y = f & 1 ? b.x : b.y;
+  return make_double2(f == 1 || f == 2 ? -x : x, f >= 2 ? -y : y);
+}
+
+// Which colours of the half spinor U h_sp have a nonzero term, h_sp from the
+// spins sp and cl of site q: bits 0 .. 2.  ld(q, c): component c of site q.
+template <class Load>
+__device__ __forceinline__ int fx_terms(Load ld, const double2 *u, bool adj, unsigned q, int sp, int cl) {
+  auto nonzero = [](double2 z) {
+    return ((__double_as_longlong(z.x) | __double_as_longlong(z.y)) << 1) != 0;
+  };
+  int bits = 0;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    if (!nonzero(ld(q, 3 * sp + b)) && !nonzero(ld(q, 3 * cl + b))) continue;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) bits |= nonzero(__ldg(u + (adj ? 3 * b + a : 3 * a + b))) ? 1 << a : 0;
+  }
+  return bits;
+}
+
+// Both hops of direction m added to acc in FP64, with the terms of the FP64
+// kernels (SUM: the full operator's, which starts the backward product at the
+// forward one and takes the difference from the two).  S: sign of the forward
+// projector; m and S at run time, so that lanes with different m run together.
+template <bool SUM, class Load>
+__device__ __forceinline__ void fx_pair_f64(Load ld, const double2 *__restrict__ links, int m, int S, unsigned qf,
+                                            unsigned s, unsigned qb, double2 (&acc)[12]) {
+  // projection of 1 - gamma_m for the upper spins 0, 1 and reconstruction of 1 + gamma_m
+  const int p0 = m == 3 ? 2 : m != 1, p1 = m == 0 ? 1 : m == 2 ? 3 : 2;
+  const int r0 = m == 1 ? 2 : m != 3, r1 = m == 0 ? 1 : m == 2 ? 3 : 0;
+  const int c0 = m < 2 ? 9 : 6, c1 = m < 2 ? 6 : 9;   // the lower spins that go with them
+  double2 h[6], f[6], sum[6];
+#pragma unroll
+  for (int back = 0; back < 2; ++back) {
+    const unsigned q = back ? qb : qf;
+    const int flip = (back ? -S : S) > 0 ? 2 : 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      h[b] = cadd(ld(q, b), fx_turned(ld(q, c0 + b), (p0 + flip) & 3));
+      h[3 + b] = cadd(ld(q, 3 + b), fx_turned(ld(q, c1 + b), (p1 + flip) & 3));
+    }
+    const double2 *u = links + ((size_t)(back ? qb : s) * 4 + m) * 9;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int sp = 0; sp < 2; ++sp) {
+        double2 x = SUM && back ? f[3 * sp + a] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const double2 e = __ldg(u + (back ? 3 * b + a : 3 * a + b));
+          x = back ? cfmac(e, h[3 * sp + b], x) : cfma(e, h[3 * sp + b], x);
+        }
+        (back ? sum : f)[3 * sp + a] = x;
+      }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    double2 d[2];
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp) {
+      const double2 cf = f[3 * sp + a], cb = sum[3 * sp + a];   // cb: with SUM the sum of both
+      acc[3 * sp + a] = cadd(acc[3 * sp + a], SUM ? cb : cadd(cf, cb));
+      d[sp] = SUM ? make_double2(fma(2.0, cf.x, -cb.x), fma(2.0, cf.y, -cb.y)) : csub(cf, cb);
+    }
+    const int flip = S > 0 ? 0 : 2;
+    const double2 l0 = fx_turned(d[0], (r0 + flip) & 3), l1 = fx_turned(d[1], (r1 + flip) & 3);
+    acc[6 + a] = cadd(acc[6 + a], m < 2 ? l1 : l0);
+    acc[9 + a] = cadd(acc[9 + a], m < 2 ? l0 : l1);
+  }
+}
+
+// FP64 hop sums of a warp's 16 sites for those that need them: special (values
+// that fixed point does not hold), or lost components (fx_lost) with any nonzero
+// term.  The whole warp calls it, a site's two lanes taking two directions each.
+// Returns whether the site's sums were written to out.
+template <bool DAG, bool SUM, class Load>
+__device__ __forceinline__ bool fx_exact(Load ld, const double2 *__restrict__ links, const unsigned (&nup)[4],
+                                         const unsigned (&ndn)[4], unsigned s, int sp, bool special, int lost,
+                                         double2 *out) {
+  constexpr int F = DAG ? +1 : -1;
+  bool need = special;
+  if (__any_sync(0xffffffffu, lost != 0 && !special)) {
+    int up = 0, low = 0, xy = 0;
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) {
+      const int m = i >> 1;
+      const bool fwd = !(i & 1);
+      const unsigned q = fwd ? nup[m] : ndn[m];
+      const int t = fx_terms(ld, links + ((size_t)(fwd ? s : q) * 4 + m) * 9, !fwd, q, sp, m < 2 ? 3 - sp : 2 + sp);
+      up |= t;
+      if (m < 2) xy |= t;
+      else low |= t;
+    }
+    low |= __shfl_xor_sync(0xffffffffu, xy, 16);
+    need = need || (lost & (up | low << 3)) != 0;
+  }
+  need = __shfl_xor_sync(0xffffffffu, (int)need, 16) || need;
+  if (!__any_sync(0xffffffffu, need)) return false;
+  double2 acc[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) acc[c] = make_double2(0.0, 0.0);
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    const int m = 2 * i + sp;
+    fx_pair_f64<SUM>(ld, links, m, F, nup[m], s, ndn[m], acc);
+  }
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, 16);
+    acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, 16);
+    if (need && sp == c / 6) out[c] = acc[c];
+  }
+  return need;
 }
 
 // ----------------------------------------------------------------- a warp's entries

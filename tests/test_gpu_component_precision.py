@@ -1,0 +1,119 @@
+"""Entries far below their neighbours keep FP64's precision: the fixed-point
+kernels share exponents over sites, chunks and tiles, and have to fall back to
+FP64 where a result rests on entries that the shared exponent does not hold.
+
+Fields: (colours) links that are diagonal in colour and colours of 1, 2^-40 and
+2^-80, which the operator never mixes; (point) one site 1e20 above the others
+with a single spin, which does not reach every spin of its neighbours.
+
+Bar of an operator product, component by component: FP64 leaves at most 64
+units of 2^-53 times the sum of the magnitudes of the terms that reach the
+component (48 products, their sums and projections: at most some 60 roundings
+of partial sums no larger than it; in practice a few units), per half hop for
+the Schur operator, so 128.  Exact zeros stay zero.
+"""
+import numpy as np
+import pytest
+
+from inputs import lattice as L
+from oracle import dirac, evenodd
+
+from .gpu_util import cuda, host
+
+pytestmark = pytest.mark.gpu
+
+SCALE = 2.0 ** np.array([0.0, -40.0, -80.0])
+
+
+@pytest.fixture(scope="module")
+def wdl():
+    import paper_0710_1988_gb300 as wdl
+    wdl.lib()
+    return wdl
+
+
+def _links(dims, kind):
+    if kind == "point":
+        return L.gauge_field(dims, 0.9, 21)
+    rng = np.random.Generator(np.random.PCG64(22))
+    ph = np.exp(2j * np.pi * rng.uniform(size=(L.volume(dims), 4, 3)))
+    U = np.zeros((L.volume(dims), 4, 3, 3), dtype=np.complex128)
+    for c in range(3):
+        U[:, :, c, c] = ph[:, :, c]
+    return U
+
+
+def _field(dims, kind, nrhs):
+    psi = L.gaussian_spinor(dims, 23, nrhs=nrhs).reshape(nrhs, -1, 4, 3)
+    if kind == "colours":
+        return psi * SCALE
+    p = psi.copy()
+    for r in range(nrhs):
+        at = (5 * r) % p.shape[1]
+        p[r, at] = 0.0
+        p[r, at, r % 4] = 1e20
+    return p
+
+
+def _hop_abs(U, a, dims):
+    """sum over the hops of |U| (|psi_s| + |psi_partner|): the terms' magnitudes."""
+    n = dims[::-1]
+    v = L.volume(dims)
+    aU = np.abs(U)
+    out = np.zeros((v, 4, 3))
+    site = np.arange(v).reshape(n)
+    for mu in range(4):
+        part = [3, 2, 1, 0] if mu < 2 else [2, 3, 0, 1]
+        h = a + a[:, part]
+        up = np.roll(site, -1, 3 - mu).reshape(-1)
+        dn = np.roll(site, 1, 3 - mu).reshape(-1)
+        out += np.einsum("sab,sib->sia", aU[:, mu], h[up])
+        out += np.einsum("sba,sib->sia", aU[dn, mu], h[dn])
+    return out
+
+
+@pytest.mark.parametrize("dims,nrhs", [((4, 4, 4, 4), 1), ((3, 5, 7, 2), 3), ((8, 4, 4, 8), 12), ((9, 7, 5, 11), 4)])
+@pytest.mark.parametrize("kind", ["colours", "point"])
+@pytest.mark.parametrize("dagger,mu", [(False, 0.0), (True, 0.07)])
+def test_product(wdl, dims, nrhs, kind, dagger, mu):
+    import torch
+    U, psi = _links(dims, kind), _field(dims, kind, nrhs)
+    op = wdl.WilsonOperator(dims, cuda(U), 0.14, mu)
+    out = torch.empty(psi.size, dtype=torch.complex128, device="cuda:0")
+    op.apply(cuda(psi), out, dagger=dagger)
+    got = host(out).reshape(psi.shape)
+    op.close()
+    f = dirac.apply_A_dagger if dagger else dirac.apply_A
+    for r in range(nrhs):
+        ref = f(U, psi[r], dims, 0.14, mu)
+        a = np.abs(psi[r])
+        bound = 64 * 2.0 ** -53 * ((1 + mu) * a + 0.14 * _hop_abs(U, a, dims))
+        assert np.all(np.abs(got[r] - ref) <= bound)
+
+
+@pytest.mark.parametrize("dims,nrhs", [((4, 4, 4, 4), 1), ((2, 6, 4, 8), 5), ((8, 8, 4, 6), 3)])
+@pytest.mark.parametrize("kind", ["colours", "point"])
+@pytest.mark.parametrize("dagger,mu", [(False, 0.0), (True, 0.07), (False, 0.07)])
+def test_schur_product(wdl, dims, nrhs, kind, dagger, mu):
+    import torch
+    U = _links(dims, kind)
+    v = L.volume(dims)
+    half = np.ascontiguousarray(_field(dims, kind, nrhs)[:, : v // 2])
+    op = wdl.WilsonOperator(dims, cuda(U), 0.14, mu)
+    op.set_operator(True)
+    out = torch.empty(half.size, dtype=torch.complex128, device="cuda:0")
+    op.apply(cuda(half), out, dagger=dagger)
+    got = host(out).reshape(half.shape)
+    op.close()
+    s = np.indices(dims[::-1]).sum(0).reshape(-1) % 2 == 0
+    g5 = lambda z: dirac.gamma5(z.reshape(-1, 4, 3))
+    for r in range(nrhs):
+        if dagger:
+            ref = g5(evenodd.schur_apply(U, dims, 0.14, -mu, g5(half[r]).ravel()))
+        else:
+            ref = evenodd.schur_apply(U, dims, 0.14, mu, half[r].ravel())
+        full = np.zeros((v, 4, 3))
+        full[s] = np.abs(half[r])
+        two = _hop_abs(U, _hop_abs(U, full, dims), dims)[s] * (1 + mu)
+        bound = 128 * 2.0 ** -53 * ((1 + mu) * np.abs(half[r]) + 0.14 ** 2 * two)
+        assert np.all(np.abs(got[r] - ref.reshape(-1, 4, 3)) <= bound)
