@@ -55,7 +55,7 @@ enum wd_status {
   WD_BAD_ARG = 1,              /* invalid size, pointer or parameter */
   WD_NOT_CONVERGED = 2,        /* tolerance not reached; x and stats still
                                   written (the paper's "F", Sec. 3) */
-  WD_BREAKDOWN = 3,            /* a Krylov scalar vanished (rho, <r_hat,v>) */
+  WD_BREAKDOWN = 3,            /* a Krylov scalar vanished (<r_hat,v>; rho for the fourth time) */
   WD_SINGULAR_PROJECTION = 4,  /* U^dagger A V numerically singular */
   WD_TIMEOUT = 5,              /* a bounded device-side wait expired */
   WD_CUDA_ERROR = 6,           /* a CUDA call failed (see detail) */
@@ -70,7 +70,8 @@ typedef struct {
   long long mvp_extra;
   int iters;         /* BiCGStab iterations (2 MVPs each) */
   int cycles;        /* GMRES-DR cycles */
-  int restarts;      /* BiCGStab restarts from the true residual */
+  int restarts;      /* BiCGStab restarts: from the true residual, and with a
+                        new shadow vector r_hat = r where <r_hat, r> vanished */
   int converged;     /* 1 if true residual <= tol */
   int breakdown;
   double rel_res;    /* recursive (BiCGStab) or least-squares (GMRES-DR)

@@ -71,6 +71,24 @@ __device__ __forceinline__ void fin_partials(const double *src, int b, int step,
   fin_warp_sum(x, sum);
 }
 
+// The recurrence starts anew from r_hat = r, p = v = 0; rr = ||r||^2.
+__device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
+  S.rho = make_double2(rr, 0.0);  // r_hat = r, so <r_hat, r> = ||r||^2
+  S.rho_old = make_double2(1.0, 0.0);
+  S.alpha = make_double2(1.0, 0.0);
+  S.omega = make_double2(1.0, 0.0);
+  S.beta = S.rho;
+  S.mbo = cneg(S.rho);
+  S.rhat_norm = sqrt(rr);
+  S.rnorm = sqrt(rr);
+}
+
+// FIN_RHO with <r_hat, r> = 0 starts the recurrence anew from r this often.  It
+// happens at the first step to sources on one site, whose r is orthogonal to them:
+// A A b has no part at the site, as (1 - gamma)(1 + gamma) = 0.  In FP64 sums the
+// rounding of alpha mostly hides it, with the more exact ones it shows.
+constexpr int SHADOWS_MAX = 3;
+
 // FIN_ALPHA, FIN_OMEGA or FIN_RHO of system r, status ST_ACTIVE, by a block of
 // 128 threads or more.  What takes time is one chain: up to 128 partials are
 // summed by each warp that needs them, without a barrier; the scalars are
@@ -157,7 +175,11 @@ static __device__ __noinline__ void fin_system(int kind, const double *partial, 
       status[r] = ST_RECURSIVE;
     else if (iters >= max_iter)
       status[r] = ST_MAXITER;
-    else if (vanishes)
+    else if (vanishes && S.shadows < SHADOWS_MAX) {   // the host loop resets the vectors
+      S.shadows += 1;
+      reset_recurrence(S, n2);
+      status[r] = ST_RESTART;
+    } else if (vanishes)
       status[r] = ST_BREAKDOWN;
   }
 }

@@ -128,17 +128,6 @@ __device__ void reduce_partials(const double *partial, int nb, int r, double (&v
   block_sum<NQ>(v);
 }
 
-__device__ __forceinline__ void reset_recurrence(BicgScalars &S, double rr) {
-  S.rho = make_double2(rr, 0.0);  // r_hat = r, so <r_hat, r> = ||r||^2
-  S.rho_old = make_double2(1.0, 0.0);
-  S.alpha = make_double2(1.0, 0.0);
-  S.omega = make_double2(1.0, 0.0);
-  S.beta = S.rho;
-  S.mbo = cneg(S.rho);
-  S.rhat_norm = sqrt(rr);
-  S.rnorm = sqrt(rr);
-}
-
 // One block per system.
 __global__ void __launch_bounds__(1024)
 bicg_finalize_kernel(int kind, const double *partial, int nb, BicgScalars *sc,

@@ -44,6 +44,7 @@ struct BicgScalars {
   double2 beta, mbo;   // of the next p = r + beta p + mbo v: (rho / rho_old)(alpha / omega), -beta omega
   double bnorm, rhat_norm, rnorm, true_rel, tol;
   int iters, max_iter, restarts, max_restarts;
+  int shadows;   // restarts with a new shadow vector (bicg_fin.cuh)
   long long mvp, mvp_extra;
   // mixed solver only: tol is the target of the low-precision recursion;
   // tol_outer the FP64 true-residual target; delta > 0 selects restarted

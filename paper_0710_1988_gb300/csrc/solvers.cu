@@ -118,12 +118,17 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
     }
     WD_CK(cudaMemcpyAsync(hst.data(), status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
     WD_CK(cudaStreamSynchronize(s));
-    bool active = false, recursive = false;
+    bool active = false, recursive = false, again = false;
     for (int q : hst) {
       active |= q == ST_ACTIVE;
       recursive |= q == ST_RECURSIVE;
+      again |= q == ST_RESTART;   // <r_hat, r> vanished: r_hat = r
     }
-    if (active) continue;
+    if (again) {
+      RET_IF(launch_ok(launch_bicg_restart_vectors(rhat, r, p, v, status, M_RESTART, n, nrhs, s), "new shadow"));
+      RET_IF(launch_ok(launch_bicg_finalize(FIN_ACTIVATE, nullptr, 0, sc, status, nullptr, 0, nrhs, s), "activate"));
+    }
+    if (active || again) continue;
     if (!recursive) break;
     // true residual r = b - A x for the systems whose recursive residual converged
     RET_IF(launch_ok(launch_wilson_f64_epi(h, X, t, nrhs, 0, EPI_NONE, nullptr, nullptr, status, s, M_RECURSIVE), "wilson_true"));
@@ -150,7 +155,7 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
       o.mvp = S.mvp;
       o.mvp_extra += S.mvp_extra;
       o.iters = S.iters;
-      o.restarts = S.restarts;
+      o.restarts = S.restarts + S.shadows;
       o.converged = st == ST_DONE ? 1 : 0;
       o.breakdown = st == ST_BREAKDOWN ? 1 : 0;
       o.rel_res = S.bnorm > 0 ? S.rnorm / S.bnorm : 0.0;

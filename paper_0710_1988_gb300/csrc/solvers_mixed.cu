@@ -199,6 +199,16 @@ int bicgstab_mixed_batched(wd_context *h, const double2 *B, double2 *X, const do
     WD_CK(cudaGraphInstantiate(&graph.x, graph.g, 0));
   }
 
+  // systems to restart: r_hat = r, p = v = 0, then active again
+  auto restart_vectors = [&]() -> int {
+    if (half)
+      RET_IF(ok(launch_bicg16_restart(rhat, r, p16, v16, status, M_RESTART, V, nrhs, s), "restart16"));
+    else
+      RET_IF(ok(launch_bicg32_restart(rhat, r, p, v, status, M_RESTART, n4, nrhs, s), "restart32"));
+    RET_IF(ok(launch_bicg_finalize(FIN_ACTIVATE, nullptr, 0, sc, status, nullptr, 0, nrhs, s), "activate"));
+    return WD_OK;
+  };
+
   std::vector<int> hst(nrhs);
   const unsigned M_RU = M_ACTIVE | M_RECURSIVE;
   int since = 0;
@@ -213,11 +223,13 @@ int bicgstab_mixed_batched(wd_context *h, const double2 *B, double2 *X, const do
     since += chunk;
     WD_CK(cudaMemcpyAsync(hst.data(), status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
     WD_CK(cudaStreamSynchronize(s));
-    bool active = false, recursive = false;
+    bool active = false, recursive = false, again = false;
     for (int q : hst) {
-      active |= q == ST_ACTIVE;
+      active |= q == ST_ACTIVE || q == ST_RESTART;
       recursive |= q == ST_RECURSIVE;
+      again |= q == ST_RESTART;   // <r_hat, r> vanished
     }
+    if (again) RET_IF(restart_vectors());
     if (!active && !recursive) break;
     const bool due = since >= every;
     if (recursive || !active || due) {
@@ -235,13 +247,7 @@ int bicgstab_mixed_batched(wd_context *h, const double2 *B, double2 *X, const do
         left |= q == ST_ACTIVE || q == ST_RESTART;
         restarted |= q == ST_RESTART;
       }
-      if (restarted) {  // restarted refinement: r_hat = r, p = v = 0, then active again
-        if (half)
-          RET_IF(ok(launch_bicg16_restart(rhat, r, p16, v16, status, M_RESTART, V, nrhs, s), "restart16"));
-        else
-          RET_IF(ok(launch_bicg32_restart(rhat, r, p, v, status, M_RESTART, n4, nrhs, s), "restart32"));
-        RET_IF(ok(launch_bicg_finalize(FIN_ACTIVATE, nullptr, 0, sc, status, nullptr, 0, nrhs, s), "activate"));
-      }
+      if (restarted) RET_IF(restart_vectors());   // restarted refinement
       if (!left) break;
     }
   }
@@ -264,7 +270,7 @@ int bicgstab_mixed_batched(wd_context *h, const double2 *B, double2 *X, const do
       o.mvp = S.mvp;
       o.mvp_extra += S.mvp_extra;
       o.iters = S.iters;
-      o.restarts = S.restarts;
+      o.restarts = S.restarts + S.shadows;
       o.converged = hst[q] == ST_DONE ? 1 : 0;
       o.breakdown = hst[q] == ST_BREAKDOWN ? 1 : 0;
       o.rel_res = S.bnorm > 0 ? S.rnorm / S.bnorm : 0.0;
