@@ -485,8 +485,17 @@ __device__ __forceinline__ bool fx_exact(Load ld, const double2 *__restrict__ li
 
 // ----------------------------------------------------------------- a warp's entries
 
-// Shared exponent of N entries a lane over the warp: the largest exponent
-// field (at least FX_EMIN) and, in ok, whether fixed point holds every value.
+// Exponent field of an entry's larger part (at least FX_EMIN); ok becomes false
+// where fixed point does not hold the entry.
+__device__ __forceinline__ int fx_entry_exponent(double2 x, bool &ok) {
+  const int e = max(exp_bits(x.x), exp_bits(x.y));
+  const bool zero = ((__double_as_longlong(x.x) | __double_as_longlong(x.y)) << 1) == 0;
+  ok = ok && (zero || (e >= FX_EMIN && e <= FX_EMAX));
+  return max(e, FX_EMIN);
+}
+
+// Shared exponent of N entries a lane over the warp: the largest exponent field
+// (FX_EMIN: all are zero) and, in ok, whether fixed point holds every value.
 template <int N>
 __device__ __forceinline__ int fx_warp_exponent(const double2 (&x)[N], bool &ok) {
   int e = 0;
@@ -497,16 +506,18 @@ __device__ __forceinline__ int fx_warp_exponent(const double2 (&x)[N], bool &ok)
     any |= (unsigned long long)(__double_as_longlong(x[i].x) | __double_as_longlong(x[i].y)) << 1;
   }
   e = __reduce_max_sync(0xffffffffu, e);
-  ok = e <= FX_EMAX && (e >= FX_EMIN || !__any_sync(0xffffffffu, any != 0));
+  ok = e <= FX_EMAX && (e > FX_EMIN || !__any_sync(0xffffffffu, any != 0));
   return max(e, FX_EMIN);
 }
 
 // <a, v> and ||v||^2 over N <= 8 entries a lane of a warp, in fixed point
 // against the warp's exponents: lane 0 returns (re, ||v||^2), lane 16 (im, ).
 // A lane's sums are below 2^58 (middle 2^60), the warp's below 2^63; a product
-// leaves out 2^-56 of the maxima's, a lane's sum is rounded at 2^-54.  In FP64 this is
-// six FMAs an entry, 76 clocks of a subpartition each for a warp, and as many
-// for every addition of the warp's reduction.
+// leaves out 2^-56 of the maxima's, a lane's sum is rounded at 2^-54.  That is below
+// FP64's roundings unless the vectors have their large entries apart: a sum below
+// 2^-5 of the maxima's product (2^48 units; one warp in 1e4 on even fields) is formed
+// in FP64.  In FP64 this is six FMAs an entry, 76 clocks of a subpartition each
+// for a warp, and as many for every addition of the warp's reduction.
 template <int N>
 __device__ __forceinline__ double2 fx_warp_dots(const double2 (&a)[N], const double2 (&v)[N]) {
   bool oka, okv;
@@ -543,9 +554,11 @@ __device__ __forceinline__ double2 fx_warp_dots(const double2 (&a)[N], const dou
       t += __shfl_xor_sync(0xffffffffu, t, o);
       u += __shfl_xor_sync(0xffffffffu, u, o);
     }
-    return make_double2(fx_scaled(t, ea + ev - 1019), fx_scaled(u, ev + ev - 1019));
+    const bool zero = ea == FX_EMIN || ev == FX_EMIN;
+    if (zero || __any_sync(0xffffffffu, t >= 1LL << 48 || t <= -(1LL << 48)))
+      return make_double2(fx_scaled(t, ea + ev - 1019), fx_scaled(u, ev + ev - 1019));
   }
-  double s[3] = {0.0, 0.0, 0.0};   // values that fixed point does not hold
+  double s[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     s[0] = fma(a[i].x, v[i].x, fma(a[i].y, v[i].y, s[0]));

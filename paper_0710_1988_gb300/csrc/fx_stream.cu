@@ -6,11 +6,12 @@
 // 112 bytes in 3, 2.2 and 5.3.  So p, x and the dots are formed in integers
 // (fx.cuh: shared exponent, two slices, three multiply-adds a real product, one
 // FP64 addition a real), and s and r, four FMAs an entry each, stay on the FP64
-// pipe beside them.  A warp works on a tile of N entries a lane that share one
-// exponent per operand; a scalar has its own.  Products are kept at
-// 2^-58 of (scalar x largest entry) and leave out 2^-56 of it at most, 2^-58 in
-// the mean: below the two roundings of the FP64 form.  Tiles with infinities,
-// NaN or magnitudes near the ends of FP64's range take FP64.  p and s also leave
+// pipe beside them.  Every entry of p, v and s has its own exponent (its larger
+// part's), so has a scalar: a product of the two is kept at 2^-58 of it and leaves
+// out 2^-56 of it at most, 2^-58 in the mean, below the two roundings of the FP64
+// form, entry by entry.  The dots share exponents over a warp's tile of N entries a
+// lane (fx_warp_dots).  Entries that are infinite, NaN or near the ends of FP64's
+// range take FP64.  p and s also leave
 // in the operator's form, site by site, through shared memory so that the
 // writes are contiguous.
 //
@@ -70,9 +71,11 @@ __device__ __forceinline__ bool fxs_in_range(const FxScalar &c, int E) {
   return u >= 70 && u <= 1970;
 }
 
-// a + c1 z1 + c2 z2: E1, E2 the shared exponents of z1, z2
-__device__ __forceinline__ double2 fxs_axpy2(double2 a, const FxScalar &c1, double2 z1, int E1,
-                                             const FxScalar &c2, double2 z2, int E2) {
+// a + k1 z1 + k2 z2; c1, c2: k1, k2 in slices, held: whether both are
+__device__ __forceinline__ double2 fxs_axpy2(double2 a, double2 k1, const FxScalar &c1, double2 z1,
+                                             double2 k2, const FxScalar &c2, double2 z2, bool held) {
+  const int E1 = fx_entry_exponent(z1, held), E2 = fx_entry_exponent(z2, held);
+  if (!held || !fxs_in_range(c1, E1) || !fxs_in_range(c2, E2)) return cfma(k2, z2, cfma(k1, z1, a));
   const longlong2 t = fxs_mul(c1, fx_cut30(z1, E1)), u = fxs_mul(c2, fx_cut30(z2, E2));
   const int E = c1.e + E1 - 1023, F = c2.e + E2 - 1023;
   const int dt = min(max(F - E, 0), 63), du = min(max(E - F, 0), 63);
@@ -152,18 +155,10 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
       w[q] = in ? z[i] : make_double2(0.0, 0.0);
       if (TWO) y[q] = in ? out[i] : make_double2(0.0, 0.0);
     }
-    bool ok = false;
-    int Ey = FX_EMIN, Ez = FX_EMIN;
-    if (TWO) {
-      bool o1;
-      Ez = fx_warp_exponent(w, ok);
-      Ey = fx_warp_exponent(y, o1);
-      ok = ok && o1 && held && fxs_in_range(s1, Ey) && fxs_in_range(s2, Ez);
-    }
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       if (TWO)
-        x[q] = ok ? fxs_axpy2(x[q], s1, y[q], Ey, s2, w[q], Ez) : cfma(c2, w[q], cfma(c1, y[q], x[q]));
+        x[q] = fxs_axpy2(x[q], c1, s1, y[q], c2, s2, w[q], held);
       else
         x[q] = cfma(c1, w[q], x[q]);
       const int c = q * 32 + lane;
@@ -209,13 +204,9 @@ bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, cons
       u[q] = in ? p[i] : zero;
       h[q] = in ? x[i] : zero;
     }
-    bool os, ok;
-    const int Es = fx_warp_exponent(s, os), Ep = fx_warp_exponent(u, ok);
-    ok = ok && os && held && fxs_in_range(sa, Ep) && fxs_in_range(so, Es);
 #pragma unroll
     for (int q = 0; q < N; ++q) {   // x += alpha p + omega s
-      const double2 xi = ok ? fxs_axpy2(h[q], sa, u[q], Ep, so, s[q], Es)
-                            : cfma(om, s[q], cfma(al, u[q], h[q]));
+      const double2 xi = fxs_axpy2(h[q], al, sa, u[q], om, so, s[q], held);
       if (q * 32 + lane < count) x[off + base + q * 32 + lane] = xi;
     }
 #pragma unroll
