@@ -20,7 +20,11 @@
 // partial sum (2^-53 of it, 2 k times an entry in the update).
 //
 // Chunks with infinities, NaN or magnitudes near the ends of FP64's range
-// have exponent FX_SPECIAL and take their products in FP64.
+// have exponent FX_SPECIAL and take their products in FP64.  So do results that
+// rest on entries far below their chunk's largest, for which its unit is coarser
+// than FP64's rounding: a warp's dot below 2^-5 of the maxima's product, and an
+// entry of the update whose own value and partial sums all stay below 2^-6 of
+// the largest |h_j| 2^(E_j).
 #include "chain.cuh"
 #include "cplx.cuh"
 #include "fx.cuh"
@@ -38,6 +42,10 @@ long long fxb_chunks(long long n) { return (n + FXB_CHUNK - 1) / FXB_CHUNK; }
 // A thread's four entries of a chunk: pairs 2 tid, 2 tid + 1 of both halves.
 __device__ __forceinline__ int fxb_entry(int q) {
   return (q >> 1) * (FXB_CHUNK / 2) + 2 * (int)threadIdx.x + (q & 1);
+}
+
+__device__ __forceinline__ bool fxb_nonzero(double2 x) {
+  return ((__double_as_longlong(x.x) | __double_as_longlong(x.y)) << 1) != 0;
 }
 
 // Largest exponent field over the block's entries and whether all are zero,
@@ -261,19 +269,29 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
     __syncwarp();
     const int jl = lane >> 1;   // this lane's vector
     const int Ev = jl < nj ? b.ex[(long long)(j0 + jl) * nc + c] : 0;
-    const bool held = Ew != FX_SPECIAL && Ev != FX_SPECIAL;
-    if (jl < nj && held) sum += fx_scaled(tsum[warp][lane], Ev + Ew - 1019);
+    const long long T = jl < nj ? tsum[warp][lane] : 0;
+    // long enough (2^47 units; one in 1e4 is not on even fields), or a chunk of zeros
+    const bool mine_long = T >= 1LL << 47 || T <= -(1LL << 47) || Ev == 0 || Ew == 0;
+    const bool longer = __shfl_xor_sync(0xffffffffu, (int)mine_long, 1) || mine_long;
+    const bool held = Ew != FX_SPECIAL && Ev != FX_SPECIAL && longer;
+    if (jl < nj && held) sum += fx_scaled(T, Ev + Ew - 1019);
     const unsigned other = __ballot_sync(0xffffffffu, jl < nj && !held);
-    // chunks that fixed point does not hold, in FP64
+    const unsigned spec = __ballot_sync(0xffffffffu, Ew == FX_SPECIAL || Ev == FX_SPECIAL);
+    // the others in FP64
     for (int jj = 0; other != 0 && jj < nj; ++jj) {
       if (!((other >> (2 * jj)) & 1u)) continue;
       const long long j = j0 + jj;
-      double2 a = make_double2(0.0, 0.0);
+      double2 a = make_double2(0.0, 0.0), v[4];
+      bool terms = (spec >> (2 * jj)) & 1u;   // infinities times zero count
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const long long i = base + fxb_entry(q);
-        if (i < n) a = cfmac(V[j * n + i], x[q], a);
+        v[q] = i < n ? V[j * n + i] : make_double2(0.0, 0.0);
+        terms = terms || (fxb_nonzero(v[q]) && fxb_nonzero(x[q]));
       }
+      if (!__any_sync(0xffffffffu, terms)) continue;   // as in regions that a source has not reached
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a = cfmac(v[q], x[q], a);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
@@ -410,8 +428,19 @@ fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2
 #pragma unroll
   for (int q = 0; q < 4; ++q) x[q] = (q < 2 ? in0 : in1) ? w[base + fxb_entry(q)] : make_double2(0.0, 0.0);
   long long rh[4], rm[4], ih[4], im[4];
+  int reach[4];   // high words of the partial sums, or-ed; 2^47 units where x is large enough itself
 #pragma unroll
-  for (int q = 0; q < 4; ++q) rh[q] = ih[q] = 0;
+  for (int q = 0; q < 4; ++q) {
+    rh[q] = ih[q] = 0;
+    reach[q] = max(exp_bits(x[q].x), exp_bits(x[q].y)) >= G - 1028 ? 1 << 15 : 0;
+  }
+  auto track = [&]() {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int a = (int)(rh[q] >> 32), c2 = (int)(ih[q] >> 32);
+      reach[q] |= (a ^ (a >> 31)) | (c2 ^ (c2 >> 31));
+    }
+  };
   for (int j0 = 0; j0 < k; j0 += 32) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) rm[q] = im[q] = 1LL << 28;
@@ -431,6 +460,7 @@ fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2
         fxb_mac(ih[q], im[q], ah, al, y.z, y.w);
         fxb_mac(ih[q], im[q], bh, bl, y.x, y.y);
       }
+      if ((j & 3) == 3) track();
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -438,11 +468,21 @@ fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2
       ih[q] += im[q] >> 29;
     }
   }
+  track();
   // units 2^(58 - 2 * 1078 + G)
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (!(q < 2 ? in0 : in1)) continue;
     double re = fx_scaled(rh[q], G - 1019), im2 = fx_scaled(ih[q], G - 1019);
+    if (reach[q] < 1 << 15 && G != 0) {   // G = 0: all products are zero
+      double2 acc = make_double2(0.0, 0.0);
+      for (int j = 0; j < k; ++j) {
+        const double2 v = V[(long long)j * n + base + fxb_entry(q)];
+        if (fxb_nonzero(v)) acc = cfma(v, h[(long long)j * ldh], acc);
+      }
+      re = acc.x;
+      im2 = acc.y;
+    }
     if (add) {
       re = -re;
       im2 = -im2;
@@ -468,7 +508,8 @@ cudaError_t launch_fxb_update(FxBasis b, const double2 *V, int k, const double2 
 // partial of ||w||^2 afterwards.  The coefficients h are of the order of the
 // first pass's rounding (|h| ~ eps ||w||): the correction V h then needs only
 // FP32 accuracy relative to itself, far below FP64 rounding of w, and reads
-// only the high plane (half the bytes of V).  FP32 path, taken when ||h||^2 <=
+// only the high plane (half the bytes of V; entries that are below 2^-4 of their
+// chunk's largest in every vector are read from V).  FP32 path, taken when ||h||^2 <=
 // 1e-20 (||w0||^2 - ||hsum||^2) (the correction below 1e-10 of the vector it
 // corrects; ||w0||^2 from the Wilson kernel's partials, hsum the coefficients
 // of both passes); products and sums in FP32, w updated in FP64.  Otherwise,
@@ -517,16 +558,33 @@ fxb_correction_kernel(FxBasis b, const double2 *__restrict__ V, int k, const dou
     if (i >= n) continue;
     double2 o0 = w[i], o1 = w[i + 1];
     if (fp32) {
-      float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f;
+      float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, am = 0.f, bm = 0.f;
 #pragma unroll 8
       for (int r = 0; r < k; ++r) {
         const int4 v = __ldg(reinterpret_cast<const int4 *>(b.hi + (long long)r * n + i));
         const float2 y = hf[r];
         const float p = (float)v.x, q = (float)v.y, s = (float)v.z, t = (float)v.w;
+        am = fmaxf(am, fmaxf(fabsf(p), fabsf(q)));
+        bm = fmaxf(bm, fmaxf(fabsf(s), fabsf(t)));
         ax = fmaf(p, y.x, fmaf(-q, y.y, ax));
         ay = fmaf(p, y.y, fmaf(q, y.x, ay));
         bx = fmaf(s, y.x, fmaf(-t, y.y, bx));
         by = fmaf(s, y.y, fmaf(t, y.x, by));
+      }
+      // entries whose high parts have fewer than FP32's 24 bits in every vector: from V
+      for (int one = 0; one < 2; ++one) {
+        if ((one ? bm : am) >= 0x1p23f) continue;
+        float2 c2 = make_float2(0.f, 0.f);
+        for (int r = 0; r < k; ++r) {
+          const double2 v = V[(long long)r * n + i + one];
+          if (!fxb_nonzero(v)) continue;
+          const int E = b.ex[(long long)r * nc + c];
+          const float p = (float)ldexp(v.x, 1049 - E), q = (float)ldexp(v.y, 1049 - E);
+          c2.x = fmaf(p, hf[r].x, fmaf(-q, hf[r].y, c2.x));
+          c2.y = fmaf(p, hf[r].y, fmaf(q, hf[r].x, c2.y));
+        }
+        if (one) bx = c2.x, by = c2.y;
+        else ax = c2.x, ay = c2.y;
       }
       o0 = make_double2(o0.x - (double)ax, o0.y - (double)ay);
       o1 = make_double2(o1.x - (double)bx, o1.y - (double)by);

@@ -139,3 +139,28 @@ def test_bicgstab_carries_every_colour(wdl, dims, nrhs, even_odd):
     op.close()
     for c in (1, 2):
         assert np.linalg.norm(x[..., c] - x[..., 0]) <= 1e-12 * np.linalg.norm(x[..., 0])
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (5, 13, 3, 2), (8, 8, 8, 4)])
+@pytest.mark.parametrize("m,k", [(12, 0), (40, 12)])
+def test_gmresdr_carries_every_colour(wdl, dims, m, k):
+    """The same through the Gram-Schmidt products: a basis vector's colours stay
+    equal up to the power of two, and so does the solution; 1e-11 as for two
+    runs that differ by rounding (condition of the least squares below 1e3)."""
+    import torch
+    ph = _links(dims, "colours")
+    for c in (1, 2):
+        ph[:, :, c, c] = ph[:, :, 0, 0]
+    op = wdl.WilsonOperator(dims, cuda(ph), 0.12)
+    b = (L.gaussian_spinor(dims, 25)[..., :1] * SCALE).reshape(-1)
+    X = cuda(np.zeros_like(b))
+    V = torch.zeros(max(k, 1) * b.size, dtype=torch.complex128, device="cuda:0")
+    op.gmresdr(cuda(b), X, m, k, 1e-14, m + (m - k if k else 0), V_out=V if k else None)
+    x = host(X).reshape(-1, 3) / SCALE
+    op.close()
+    for c in (1, 2):
+        assert np.linalg.norm(x[:, c] - x[:, 0]) <= 1e-11 * np.linalg.norm(x[:, 0])
+    if k:
+        w = host(V).reshape(-1, 3) / SCALE
+        for c in (1, 2):
+            assert np.linalg.norm(w[:, c] - w[:, 0]) <= 1e-11 * np.linalg.norm(w[:, 0])
