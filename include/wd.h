@@ -115,7 +115,12 @@ int wd_set_params(wd_handle h, double kappa, double mu);
 
 /* out = A in (dagger = 0) or A^dagger in (dagger = 1) for nrhs spinors.
  * in, out: device pointers, boundary spinor layout, nrhs*n complex128
- * each, in != out (no aliasing).  Sec. 1. */
+ * each, in != out (no aliasing).  Sec. 1.
+ * On near-unitary links the hops run in fixed point; above a few thousand
+ * sites x nrhs that takes scratch from the handle's pool (196 bytes a site and
+ * vector, kept for the next call), and without it they run in FP64.  On a stream
+ * that is being captured no scratch is taken: the graph holds kernels only, and
+ * can be instantiated again and cloned. */
 int wd_apply(wd_handle h, const void *in, void *out, int nrhs, int dagger,
              wd_stream stream);
 

@@ -695,6 +695,12 @@ cudaError_t launch_schur_f64_epi(const wd_context *h, const double2 *in, double2
                                  const int *status, cudaStream_t s, unsigned mask,
                                  const FxVec *pre, const FinArgs *fin);
 
+bool being_captured(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();   // the legacy stream beside a capture
+  return st != cudaStreamCaptureStatusNone;
+}
+
 int wilson_blocks(const wd_context *h, int nrhs) {
   if (fx_few(h, nrhs, EPI_DOT)) return (int)((h->V + FX_FEW_SITES - 1) / FX_FEW_SITES);
   return h->eo ? eo_blocks(h) : (int)((h->V + WILSON_SITES - 1) / WILSON_SITES);
@@ -721,7 +727,8 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
     // scratch for the encoded input, stream-ordered; without it the FP64 kernel
     const size_t nv = (size_t)nrhs * fx_sites(h->V);
     int4 *buf = nullptr;
-    if (cudaMallocFromPoolAsync((void **)&buf, nv * (12 * sizeof(int4) + sizeof(int)), h->pool, s) == cudaSuccess) {
+    if (!being_captured(s) &&
+        cudaMallocFromPoolAsync((void **)&buf, nv * (12 * sizeof(int4) + sizeof(int)), h->pool, s) == cudaSuccess) {
       const FxVec enc{buf, reinterpret_cast<int *>(buf + 12 * nv)};
       cudaError_t e = launch_fx_encode(in, enc, h->V, nrhs, status, mask, s);
       if (e == cudaSuccess)

@@ -346,7 +346,7 @@ struct FxScratch {
   int4 *buf = nullptr;
   cudaStream_t s;
   FxScratch(const wd_context *h, int nrhs, int count, cudaStream_t stream) : s(stream) {
-    if (h->links_fx == nullptr || (h->V / 2 + WILSON_SITES - 1) / WILSON_SITES * nrhs > 0x7fffffffLL) return;
+    if (h->links_fx == nullptr || being_captured(s) || (h->V / 2 + WILSON_SITES - 1) / WILSON_SITES * nrhs > 0x7fffffffLL) return;
     const size_t nv = (size_t)nrhs * fx_sites(h->V / 2), one = nv * 12 * sizeof(int4) + nv * sizeof(int);
     if (cudaMallocFromPoolAsync((void **)&buf, count * one, h->pool, s) != cudaSuccess) {
       cudaGetLastError();

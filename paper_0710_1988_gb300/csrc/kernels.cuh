@@ -76,6 +76,10 @@ constexpr int WILSON_SITES = 64;   // per block of the FP64 products, in fixed p
 int wilson_blocks(const wd_context *h, int nrhs);
 bool wilson_takes_encoded(const wd_context *h, int nrhs);
 cudaError_t fx_links_create(wd_context *h);
+// Whether s records a graph.  Products then take no scratch, hence the FP64
+// kernels above the few-site size: a graph with allocation nodes could be
+// neither instantiated twice nor cloned.
+bool being_captured(cudaStream_t s);
 // Encode nrhs vectors of `sites` sites (systems in mask).
 cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,
                              const int *status, unsigned mask, cudaStream_t s);
