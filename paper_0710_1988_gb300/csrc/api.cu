@@ -116,6 +116,17 @@ int bad_alloc() {
 
 using namespace wd;
 
+// call(), and once more without the handle's fixed-point links when there was no
+// memory: they are given back and the FP64 kernels serve from then on.  The
+// solvers take their memory before they touch X, except that a deflated start or
+// an earlier shift may have improved it.
+template <class F> static int with_memory(wd_handle h, F call) {
+  const int rc = call();
+  if (rc != WD_OUT_OF_MEMORY || h == nullptr || h->links_fx == nullptr) return rc;
+  fx_links_release(h);
+  return call();
+}
+
 // ------------------------------------------------------------------ handles
 
 extern "C" int wd_create(const int lat[4], const void *links, double kappa, double mu,
@@ -188,7 +199,7 @@ extern "C" int wd_create(const int lat[4], const void *links, double kappa, doub
   if (e != cudaSuccess) {
     int rc = cuda_fail(e, "wd_create");
     if (h->links) cudaFree(h->links);
-    if (h->links_fx) cudaFree(h->links_fx);
+    fx_links_release(h);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     h->prof.destroy();
     delete h;
@@ -207,7 +218,7 @@ extern "C" int wd_set_operator(wd_handle h, int even_odd) {
   return WD_OK;
 }
 
-extern "C" int wd_eo_prepare(wd_handle h, const void *B, void *Bhat, int nrhs, wd_stream stream) {
+static int wd_eo_prepare_once(wd_handle h, const void *B, void *Bhat, int nrhs, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr || B == nullptr || Bhat == nullptr) return bad("wd_eo_prepare: NULL argument");
   if (!h->eo) return bad("wd_eo_prepare: the handle is not in even-odd mode");
@@ -226,7 +237,11 @@ extern "C" int wd_eo_prepare(wd_handle h, const void *B, void *Bhat, int nrhs, w
   return e == cudaSuccess ? WD_OK : cuda_fail(e, "wd_eo_prepare");
 }
 
-extern "C" int wd_eo_reconstruct(wd_handle h, const void *B, const void *Xe, void *X, int nrhs,
+extern "C" int wd_eo_prepare(wd_handle h, const void *B, void *Bhat, int nrhs, wd_stream stream) {
+  return with_memory(h, [&] { return wd_eo_prepare_once(h, B, Bhat, nrhs, stream); });
+}
+
+static int wd_eo_reconstruct_once(wd_handle h, const void *B, const void *Xe, void *X, int nrhs,
                                  wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr || B == nullptr || Xe == nullptr || X == nullptr) return bad("wd_eo_reconstruct: NULL argument");
@@ -247,6 +262,10 @@ extern "C" int wd_eo_reconstruct(wd_handle h, const void *B, const void *Xe, voi
   return e == cudaSuccess ? WD_OK : cuda_fail(e, "wd_eo_reconstruct");
 }
 
+extern "C" int wd_eo_reconstruct(wd_handle h, const void *B, const void *Xe, void *X, int nrhs, wd_stream stream) {
+  return with_memory(h, [&] { return wd_eo_reconstruct_once(h, B, Xe, X, nrhs, stream); });
+}
+
 extern "C" int wd_set_params(wd_handle h, double kappa, double mu) {
   if (h == nullptr) return bad("wd_set_params: NULL handle");
   h->kappa = kappa;
@@ -265,7 +284,7 @@ extern "C" void wd_destroy(wd_handle h) {
   if (h->ev_in) cudaEventDestroy(h->ev_in);
   if (h->ev_out) cudaEventDestroy(h->ev_out);
   if (h->links) cudaFree(h->links);
-  if (h->links_fx) cudaFree(h->links_fx);
+  fx_links_release(h);
   if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
 }
@@ -292,7 +311,7 @@ extern "C" int wd_profile_read(wd_handle h, wd_profile *out) {
   return WD_OK;
 }
 
-extern "C" int wd_apply(wd_handle h, const void *in, void *out, int nrhs, int dagger,
+static int wd_apply_once(wd_handle h, const void *in, void *out, int nrhs, int dagger,
                         wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr) return bad("wd_apply: NULL handle");
@@ -312,6 +331,10 @@ extern "C" int wd_apply(wd_handle h, const void *in, void *out, int nrhs, int da
   return WD_OK;
 }
 
+extern "C" int wd_apply(wd_handle h, const void *in, void *out, int nrhs, int dagger, wd_stream stream) {
+  return with_memory(h, [&] { return wd_apply_once(h, in, out, nrhs, dagger, stream); });
+}
+
 // ------------------------------------------------------------------ GMRES-DR
 
 extern "C" int gmresdr_history(wd_handle h, double *out, int len) {
@@ -324,7 +347,7 @@ extern "C" int gmresdr_history(wd_handle h, double *out, int len) {
   return c;
 }
 
-extern "C" int gmresdr_solve(wd_handle h, const void *b, void *x, int m, int k, double tol,
+static int gmresdr_solve_once(wd_handle h, const void *b, void *x, int m, int k, double tol,
                              int max_mv, void *V_out, void *Hbar_out, void *theta_out,
                              wd_stats *stats, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
@@ -371,9 +394,13 @@ extern "C" int gmresdr_solve(wd_handle h, const void *b, void *x, int m, int k, 
   return rc;
 }
 
+extern "C" int gmresdr_solve(wd_handle h, const void *b, void *x, int m, int k, double tol, int max_mv, void *V_out, void *Hbar_out, void *theta_out, wd_stats *stats, wd_stream stream) {
+  return with_memory(h, [&] { return gmresdr_solve_once(h, b, x, m, k, tol, max_mv, V_out, Hbar_out, theta_out, stats, stream); });
+}
+
 // ------------------------------------------------------------------ deflation
 
-extern "C" int wd_deflation_create(wd_handle h, const void *V, const void *U, int k,
+static int wd_deflation_create_once(wd_handle h, const void *V, const void *U, int k,
                                    wd_deflation *out, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (out == nullptr) return bad("wd_deflation_create: out is NULL");
@@ -415,6 +442,10 @@ extern "C" int wd_deflation_create(wd_handle h, const void *V, const void *U, in
   return WD_OK;
 }
 
+extern "C" int wd_deflation_create(wd_handle h, const void *V, const void *U, int k, wd_deflation *out, wd_stream stream) {
+  return with_memory(h, [&] { return wd_deflation_create_once(h, V, U, k, out, stream); });
+}
+
 extern "C" void wd_deflation_destroy(wd_deflation d) {
   if (d == nullptr) return;
   cudaDeviceSynchronize();
@@ -428,7 +459,7 @@ extern "C" void wd_deflation_destroy(wd_deflation d) {
 
 // ------------------------------------------------------------------ D-BiCGStab
 
-extern "C" int dbicgstab_solve_deflated(wd_handle h, wd_deflation d, const void *B, void *X,
+static int dbicgstab_solve_deflated_once(wd_handle h, wd_deflation d, const void *B, void *X,
                                         int nrhs, double tol, int max_iter, wd_stats *stats,
                                         wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
@@ -503,6 +534,10 @@ extern "C" int dbicgstab_solve_deflated(wd_handle h, wd_deflation d, const void 
   return rc;
 }
 
+extern "C" int dbicgstab_solve_deflated(wd_handle h, wd_deflation d, const void *B, void *X, int nrhs, double tol, int max_iter, wd_stats *stats, wd_stream stream) {
+  return with_memory(h, [&] { return dbicgstab_solve_deflated_once(h, d, B, X, nrhs, tol, max_iter, stats, stream); });
+}
+
 extern "C" int dbicgstab_solve(wd_handle h, const void *B, void *X, int nrhs, const void *V,
                                const void *U, int k, double tol, int max_iter, wd_stats *stats,
                                wd_stream stream) {
@@ -521,7 +556,7 @@ extern "C" int dbicgstab_solve(wd_handle h, const void *B, void *X, int nrhs, co
 
 // ------------------------------------------------------------------ Sec. 4 shifts
 
-extern "C" int tm_multishift_solve(wd_handle h, const void *B, void *X, int nrhs,
+static int tm_multishift_solve_once(wd_handle h, const void *B, void *X, int nrhs,
                                    const double *mus, int nshift, double tol, int max_iter,
                                    int project, int mixed, wd_stats *stats, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
@@ -541,6 +576,10 @@ extern "C" int tm_multishift_solve(wd_handle h, const void *B, void *X, int nrhs
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess && rc != WD_CUDA_ERROR) rc = cuda_fail(e, "tm_multishift_solve");
   return rc;
+}
+
+extern "C" int tm_multishift_solve(wd_handle h, const void *B, void *X, int nrhs, const double *mus, int nshift, double tol, int max_iter, int project, int mixed, wd_stats *stats, wd_stream stream) {
+  return with_memory(h, [&] { return tm_multishift_solve_once(h, B, X, nrhs, mus, nshift, tol, max_iter, project, mixed, stats, stream); });
 }
 
 // ------------------------------------------------------------------ differentiation
@@ -595,7 +634,7 @@ extern "C" int dbicgstab_solve_adjoint_mixed(wd_handle h, wd_deflation d, const 
   return adjoint_solve(h, d, G, LAM, nrhs, tol, max_iter, 1, reliable_every, stats, stream);
 }
 
-extern "C" int wd_gradients(wd_handle h, const void *lam, const void *x, void *force,
+static int wd_gradients_once(wd_handle h, const void *lam, const void *x, void *force,
                             double *dkappa, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr || lam == nullptr || x == nullptr) return bad("wd_gradients: NULL argument");
@@ -632,9 +671,13 @@ extern "C" int wd_gradients(wd_handle h, const void *lam, const void *x, void *f
   return WD_OK;
 }
 
+extern "C" int wd_gradients(wd_handle h, const void *lam, const void *x, void *force, double *dkappa, wd_stream stream) {
+  return with_memory(h, [&] { return wd_gradients_once(h, lam, x, force, dkappa, stream); });
+}
+
 // ------------------------------------------------------------------ mixed precision
 
-extern "C" int dbicgstab_solve_mixed(wd_handle h, wd_deflation d, const void *B, void *X,
+static int dbicgstab_solve_mixed_once(wd_handle h, wd_deflation d, const void *B, void *X,
                                      int nrhs, double tol, int max_iter, int reliable_every,
                                      wd_stats *stats, wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
@@ -728,7 +771,11 @@ extern "C" int dbicgstab_solve_mixed(wd_handle h, wd_deflation d, const void *B,
   return rc;
 }
 
-extern "C" int wd_apply_f32(wd_handle h, const void *in, void *out, int nrhs, int dagger,
+extern "C" int dbicgstab_solve_mixed(wd_handle h, wd_deflation d, const void *B, void *X, int nrhs, double tol, int max_iter, int reliable_every, wd_stats *stats, wd_stream stream) {
+  return with_memory(h, [&] { return dbicgstab_solve_mixed_once(h, d, B, X, nrhs, tol, max_iter, reliable_every, stats, stream); });
+}
+
+static int wd_apply_f32_once(wd_handle h, const void *in, void *out, int nrhs, int dagger,
                             wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr) return bad("wd_apply_f32: NULL handle");
@@ -761,7 +808,11 @@ extern "C" int wd_apply_f32(wd_handle h, const void *in, void *out, int nrhs, in
   return WD_OK;
 }
 
-extern "C" int wd_apply_f16(wd_handle h, const void *in, void *out, int nrhs, int dagger,
+extern "C" int wd_apply_f32(wd_handle h, const void *in, void *out, int nrhs, int dagger, wd_stream stream) {
+  return with_memory(h, [&] { return wd_apply_f32_once(h, in, out, nrhs, dagger, stream); });
+}
+
+static int wd_apply_f16_once(wd_handle h, const void *in, void *out, int nrhs, int dagger,
                             wd_stream stream) {
   ProfScope prof_scope_(h ? &h->prof : nullptr);
   if (h == nullptr) return bad("wd_apply_f16: NULL handle");
@@ -790,7 +841,11 @@ extern "C" int wd_apply_f16(wd_handle h, const void *in, void *out, int nrhs, in
   return WD_OK;
 }
 
-extern "C" int wd_autotune_f16(wd_handle h, int nrhs, int *R, int *threads, float *ms,
+extern "C" int wd_apply_f16(wd_handle h, const void *in, void *out, int nrhs, int dagger, wd_stream stream) {
+  return with_memory(h, [&] { return wd_apply_f16_once(h, in, out, nrhs, dagger, stream); });
+}
+
+static int wd_autotune_f16_once(wd_handle h, int nrhs, int *R, int *threads, float *ms,
                                wd_stream stream) {
   if (h == nullptr) return bad("wd_autotune_f16: NULL handle");
   if (h->eo) return bad("wd_autotune_f16: the FP16 kernel acts on the full operator");
@@ -815,6 +870,10 @@ extern "C" int wd_autotune_f16(wd_handle h, int nrhs, int *R, int *threads, floa
   if (threads) *threads = h->tune16_T[key];
   if (ms) *ms = h->tune16_ms[key];
   return WD_OK;
+}
+
+extern "C" int wd_autotune_f16(wd_handle h, int nrhs, int *R, int *threads, float *ms, wd_stream stream) {
+  return with_memory(h, [&] { return wd_autotune_f16_once(h, nrhs, R, threads, ms, stream); });
 }
 
 extern "C" int wd_set_f16_shape(wd_handle h, int nrhs, int R, int threads) {
@@ -904,7 +963,7 @@ extern "C" int wd_set_mixed_storage(wd_handle h, int bits) {
 
 // ------------------------------------------------------------------ autotuner
 
-extern "C" int wd_autotune_f32(wd_handle h, int nrhs, int *R, int *threads, float *ms,
+static int wd_autotune_f32_once(wd_handle h, int nrhs, int *R, int *threads, float *ms,
                                wd_stream stream) {
   if (h == nullptr) return bad("wd_autotune_f32: NULL handle");
   if (h->eo) return bad("wd_autotune_f32: the FP32 kernel acts on the full operator");
@@ -927,6 +986,10 @@ extern "C" int wd_autotune_f32(wd_handle h, int nrhs, int *R, int *threads, floa
   if (threads) *threads = h->tune_T[key];
   if (ms) *ms = h->tune_ms[key];
   return WD_OK;
+}
+
+extern "C" int wd_autotune_f32(wd_handle h, int nrhs, int *R, int *threads, float *ms, wd_stream stream) {
+  return with_memory(h, [&] { return wd_autotune_f32_once(h, nrhs, R, threads, ms, stream); });
 }
 
 extern "C" int wd_set_f32_shape(wd_handle h, int nrhs, int R, int threads) {

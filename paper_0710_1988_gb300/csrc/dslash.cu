@@ -598,12 +598,17 @@ static bool fx_few(const wd_context *h, int nrhs, int epi) {
 }
 
 // The handle's fixed-point links, or none where they do not fit fx.cuh's
-// bounds or the memory: the FP64 kernel then serves.
+// bounds or the memory, of which they may take a quarter of what is free: the
+// FP64 kernel then serves.
 cudaError_t fx_links_create(wd_context *h) {
   h->links_fx = nullptr;
   if (h->V >= (1LL << 31)) return cudaSuccess;
   int *bad = nullptr, hbad = 1;
-  if (cudaMalloc(&h->links_fx, sizeof(int4) * 36 * fx_sites(h->V)) != cudaSuccess) {
+  const size_t bytes = sizeof(int4) * 36 * fx_sites(h->V);
+  size_t free_bytes = 0, all = 0;
+  if (bytes > ((size_t)64 << 20) && cudaMemGetInfo(&free_bytes, &all) == cudaSuccess && bytes > free_bytes / 4)
+    return cudaSuccess;
+  if (cudaMalloc(&h->links_fx, bytes) != cudaSuccess) {
     cudaGetLastError();
     h->links_fx = nullptr;
     return cudaSuccess;
@@ -621,6 +626,15 @@ cudaError_t fx_links_create(wd_context *h) {
     h->links_fx = nullptr;
   }
   return e;
+}
+
+void fx_links_release(wd_context *h) {
+  if (h->links_fx == nullptr) return;
+  cudaDeviceSynchronize();
+  cudaFree(h->links_fx);
+  h->links_fx = nullptr;
+  if (h->pool) cudaMemPoolTrimTo(h->pool, 0);
+  cudaGetLastError();   // of the allocation that failed
 }
 
 cudaError_t launch_fx_encode(const double2 *in, FxVec f, long long sites, int nrhs,

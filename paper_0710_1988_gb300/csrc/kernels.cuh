@@ -76,6 +76,7 @@ constexpr int WILSON_SITES = 64;   // per block of the FP64 products, in fixed p
 int wilson_blocks(const wd_context *h, int nrhs);
 bool wilson_takes_encoded(const wd_context *h, int nrhs);
 cudaError_t fx_links_create(wd_context *h);
+void fx_links_release(wd_context *h);   // waits for the device
 // Whether s records a graph.  Products then take no scratch, hence the FP64
 // kernels above the few-site size: a graph with allocation nodes could be
 // neither instantiated twice nor cloned.

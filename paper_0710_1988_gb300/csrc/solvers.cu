@@ -40,6 +40,16 @@ int launch_ok(cudaError_t e, const char *what) {
 
 // --------------------------------------------------------------------- BiCGStab
 
+// Vectors of ns (padded) sites in the operator's fixed-point form, or none where it
+// does not read such, or without the memory: the operator then encodes for
+// itself, or runs in FP64.
+static FxVec take_encoded(const wd_context *h, int nrhs, size_t ns, Arena &ar) {
+  FxVec f{nullptr, nullptr};
+  if (!wilson_takes_encoded(h, nrhs)) return f;
+  f = FxVec{ar.take_or_null<int4>(12 * ns), ar.take_or_null<int>(ns)};
+  return f.v != nullptr && f.e != nullptr ? f : FxVec{nullptr, nullptr};
+}
+
 int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 *R0,
                      int nrhs, double tol, int max_iter, wd_stats *stats, cudaStream_t s,
                      double *hist_host, int hist_len, Arena &ar) {
@@ -59,15 +69,7 @@ int bicgstab_batched(wd_context *h, const double2 *B, double2 *X, const double2 
   double *hist = hist_len > 0 ? ar.take<double>((size_t)nrhs * hist_len) : nullptr;
   if (ar.failed) return WD_OUT_OF_MEMORY;
   // p or s in the operator's fixed-point form, written by their updates
-  FxVec fv{nullptr, nullptr};   // without the memory the operator encodes for itself, or runs in FP64
-  if (wilson_takes_encoded(h, nrhs)) {
-    fv = FxVec{ar.take<int4>(12 * ns), ar.take<int>(ns)};
-    if (ar.failed) {
-      cudaGetLastError();
-      ar.failed = false;
-      fv = FxVec{nullptr, nullptr};
-    }
-  }
+  const FxVec fv = take_encoded(h, nrhs, ns, ar);
   const FxVec *pre = fv.v != nullptr ? &fv : nullptr;
 
   std::vector<BicgScalars> hsc(nrhs);
@@ -299,8 +301,6 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
   FxBasis fb{ar.take<int2>((size_t)(m + 1) * n), ar.take<int2>((size_t)(m + 1) * n),
              ar.take<int>((size_t)(m + 1) * nc)};
   const size_t ns = (size_t)(n / 12 + 31) / 32 * 32;
-  FxVec fv{nullptr, nullptr};
-  if (wilson_takes_encoded(h, 1)) fv = FxVec{ar.take<int4>(12 * ns), ar.take<int>(ns)};
   double *part_w = ar.take<double>((size_t)nbw * 3);
   double *part_n = ar.take<double>((size_t)std::max<long long>(nbs, nc) * 2);
   double2 *H = ar.take<double2>((size_t)(m + 1) * m);
@@ -326,6 +326,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
       tc_restart ? ar.take<unsigned char>(ts_update_tc_scratch_bytes(m + 1, k + 1, n)) : nullptr;
   int *tc_err = ar.take<int>(1);
   if (ar.failed) return WD_OUT_OF_MEMORY;
+  const FxVec fv = take_encoded(h, 1, ns, ar);
   WD_CK(cudaMemsetAsync(tc_err, 0, sizeof(int), s));
 
   long long mvp = 0, mvp_extra = 0;

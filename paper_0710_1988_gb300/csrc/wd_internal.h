@@ -55,6 +55,19 @@ struct Arena {
     for (void *p : ptrs) cudaFreeAsync(p, stream);
     ptrs.clear();
   }
+  Arena() = default;
+  Arena(const Arena &) = delete;
+  ~Arena() { release(); }   // also where a function leaves because one was refused
+  // as take(), for a buffer that can be done without
+  template <class T> T *take_or_null(size_t count) {
+    if (failed) return nullptr;
+    T *p = take<T>(count);
+    if (p == nullptr) {
+      cudaGetLastError();
+      failed = false;
+    }
+    return p;
+  }
 };
 
 inline size_t aligned_bytes(size_t b) { return (b + 255) & ~size_t(255); }
