@@ -302,7 +302,7 @@ ts_dot_kernel(const double2 *__restrict__ V, int k, const double2 *__restrict__ 
 // One warp per (j, r) pair: the lanes load the gx block partials of the pair
 // together (lane b, b + 32, ...) and reduce them with a fixed shuffle tree,
 // so the loads overlap instead of forming one dependent chain.
-__global__ void ts_dot_finalize_kernel(const double2 *__restrict__ partial, int gx, int gy,
+__global__ void ts_dot_finalize_kernel(const double2 *partial, int gx, int gy,
                                        int JT, int RT, int k, int nrhs, double2 *C, int ldc,
                                        double2 *C2, int ldc2, const int *status) {
   chain_enter();
@@ -426,8 +426,8 @@ cudaError_t launch_ts_update(const double2 *V, int kv, const double2 *Y, int ldy
 
 // ----------------------------------------------------------------- Arnoldi helpers
 
-__global__ void arnoldi_normalize_finalize_kernel(const double *__restrict__ pw, int nb,
-                                                  const double *__restrict__ pw0, int nb0,
+__global__ void arnoldi_normalize_finalize_kernel(const double *pw, int nb,
+                                                  const double *pw0, int nb0,
                                                   double2 *H, int ldh, int j, double lucky,
                                                   int *status, int *m_eff) {
   chain_enter();

@@ -4,9 +4,12 @@
 // lets the next one be launched; launch_chained() permits the early launch.
 // Every block has to pass chain_enter(), also one that has nothing to do: a
 // kernel that could end before its predecessor would let its successor start
-// too early.  The first read after it is the system's status through an ordinary
-// load, which the wait's memory clobber orders; everything else follows the
-// branch on that status.
+// too early.  The kernel is resident while its predecessor still writes, so what
+// another kernel of the chain writes is read by ordinary loads after the wait,
+// which its memory clobber orders.  Loads through __ldg or from const __restrict__
+// parameters are defined for memory that nobody writes while the kernel lives:
+// they are for links, and for the shadow vector r_hat, which only the restart
+// kernels write, outside the chain (launched in the ordinary way they run alone).
 #pragma once
 
 #include <cuda_runtime.h>

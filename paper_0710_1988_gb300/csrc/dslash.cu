@@ -283,7 +283,7 @@ constexpr size_t FX_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);   // two
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(2 * WILSON_SITES, 4)
 wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec in,
-                 const double2 *__restrict__ in64, double2 *__restrict__ out, LatticeGeom g,
+                 const double2 *in64, double2 *__restrict__ out, LatticeGeom g,
                  size_t tiled, double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
                  double *__restrict__ partial, const int *status, unsigned mask,
                  unsigned long long *__restrict__ sites, FinArgs fin) {
@@ -303,8 +303,8 @@ wilson_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, 
   int eu[4], ed[4], E = 0;
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    eu[m] = __ldg(ev + nb.up[m]);
-    ed[m] = __ldg(ev + nb.dn[m]);
+    eu[m] = ev[nb.up[m]];
+    ed[m] = ev[nb.dn[m]];
     E = max(E, max(eu[m], ed[m]));
   }
   extern __shared__ __align__(128) unsigned char fx_smem[];
@@ -438,7 +438,7 @@ __device__ __noinline__ bool few_f64(const double2 *psi, const double2 *__restri
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(16 * FX_FEW_SITES)
 wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links,
-                     const double2 *__restrict__ in, double2 *__restrict__ out, LatticeGeom g,
+                     const double2 *in, double2 *__restrict__ out, LatticeGeom g,
                      double kappa, double mu, int nrhs, const double2 *__restrict__ aux,
                      double *__restrict__ partial, const int *status, unsigned mask,
                      unsigned long long *__restrict__ sites, FinArgs fin) {
@@ -481,8 +481,8 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
   double2 pu[3], pl[3];
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
-    pu[b] = __ldg(psi + 3 * sp + b);
-    pl[b] = __ldg(psi + 3 * low_spin + b);
+    pu[b] = psi[3 * sp + b];
+    pl[b] = psi[3 * low_spin + b];
   }
   int e = 0;
   unsigned long long any = 0;
@@ -560,7 +560,7 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
   double2 dv[1] = {make_double2(0.0, 0.0)}, da[1] = {make_double2(0.0, 0.0)};
   if (valid && j < 3) {
     const size_t i = ((size_t)r * V + s) * 12 + c;
-    const double2 p = __ldg(in + i);
+    const double2 p = in[i];
     const double tmu = DAG ? -mu : mu;
     double2 v;
     v.x = fma(-kappa, hop.x, p.x);

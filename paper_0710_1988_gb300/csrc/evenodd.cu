@@ -171,7 +171,7 @@ constexpr size_t EO_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);    // tw
 template <bool DAG, int MODE, int EPI>
 __global__ void __launch_bounds__(2 * WILSON_SITES, 4)
 wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ links, FxVec src,
-                    const double2 *__restrict__ src64, const double2 *__restrict__ same,
+                    const double2 *src64, const double2 *same,
                     double2 *__restrict__ out, FxVec outfx, LatticeGeom g, size_t tiled, int pout,
                     double kappa, double mu, double inv_1mu2, int nrhs,
                     const double2 *__restrict__ aux, double *__restrict__ partial,
@@ -200,8 +200,8 @@ wilson_eo_fx_kernel(const int4 *__restrict__ L, const double2 *__restrict__ link
   int eu[4], ed[4], E = 0;
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    eu[m] = __ldg(ev + (nb.up[m] >> 1));
-    ed[m] = __ldg(ev + (nb.dn[m] >> 1));
+    eu[m] = ev[nb.up[m] >> 1];
+    ed[m] = ev[nb.dn[m] >> 1];
     E = max(E, max(eu[m], ed[m]));
   }
   extern __shared__ __align__(128) unsigned char eo_smem[];

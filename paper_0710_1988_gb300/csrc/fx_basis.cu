@@ -83,7 +83,7 @@ __device__ __forceinline__ int fxb_exponent(const double2 (&x)[4], int *raw, int
 // (unless nullptr or w itself) and, for the next operator product, the
 // site-wise fixed point of fx.cuh (fx.v != nullptr; one vector).
 __global__ void __launch_bounds__(FXB_THREADS)
-fxb_encode_kernel(const double2 *w, const double2 *__restrict__ H, int idx, double2 *v, int2 *__restrict__ hi,
+fxb_encode_kernel(const double2 *w, const double2 *H, int idx, double2 *v, int2 *__restrict__ hi,
                   int2 *__restrict__ lo, int *__restrict__ ex, FxVec fx, long long n,
                   const int *status) {
   chain_enter();
@@ -194,7 +194,7 @@ __device__ __forceinline__ long long fxb_warp_sum(long long a, long long b) {
 // j = by jb + jj < k; g5: w is gamma5 w.  A block encodes its chunk of w once
 // for its jb <= 16 vectors and handles chunks bx, bx + gx, ...
 __global__ void __launch_bounds__(FXB_THREADS, 3)
-fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const double2 *__restrict__ W,
+fxb_dot_kernel(FxBasis b, const double2 *V, int k, int jb, const double2 *W,
                int g5, long long n, double2 *__restrict__ partial, const int *status) {
   chain_enter();
   if (status != nullptr && *status != 0) return;
@@ -235,7 +235,7 @@ fxb_dot_kernel(FxBasis b, const double2 *__restrict__ V, int k, int jb, const do
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const long long i = base + fxb_entry(q);
-      x[q] = i < n ? __ldg(W + i) : make_double2(0.0, 0.0);
+      x[q] = i < n ? W[i] : make_double2(0.0, 0.0);
       if (g5 && fxb_entry(q) % 12 >= 6) x[q] = cneg(x[q]);
     }
     int raw;
@@ -368,7 +368,7 @@ cudaError_t launch_fxb_dot(FxBasis b, const double2 *V, int k, const double2 *w,
 // w -= V h (add: w += V h) for k vectors: a block's chunk of w in FP64, the
 // sum V h in fixed point against the largest |h_j| 2^(E_j) of the chunk.
 __global__ void __launch_bounds__(FXB_THREADS, 3)
-fxb_update_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2 *__restrict__ h, int ldh,
+fxb_update_kernel(FxBasis b, const double2 *V, int k, const double2 *h, int ldh,
                   int add, double2 *w, long long n, const int *status) {
   chain_enter();
   if (status != nullptr && *status != 0) return;
@@ -516,8 +516,8 @@ cudaError_t launch_fxb_update(FxBasis b, const double2 *V, int k, const double2 
 // and for chunks with FX_SPECIAL, FP64.  Every block forms the decision from
 // the same device data in the same order, so all take the same path.
 __global__ void __launch_bounds__(FXB_THREADS)
-fxb_correction_kernel(FxBasis b, const double2 *__restrict__ V, int k, const double2 *__restrict__ h,
-                      const double2 *__restrict__ hsum, int ldh, const double *__restrict__ part_w,
+fxb_correction_kernel(FxBasis b, const double2 *V, int k, const double2 *h,
+                      const double2 *hsum, int ldh, const double *part_w,
                       int nbw, double2 *w, long long n, double *__restrict__ part_n,
                       const int *status) {
   chain_enter();
@@ -561,7 +561,7 @@ fxb_correction_kernel(FxBasis b, const double2 *__restrict__ V, int k, const dou
       float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, am = 0.f, bm = 0.f;
 #pragma unroll 8
       for (int r = 0; r < k; ++r) {
-        const int4 v = __ldg(reinterpret_cast<const int4 *>(b.hi + (long long)r * n + i));
+        const int4 v = *reinterpret_cast<const int4 *>(b.hi + (long long)r * n + i);
         const float2 y = hf[r];
         const float p = (float)v.x, q = (float)v.y, s = (float)v.z, t = (float)v.w;
         am = fmaxf(am, fmaxf(fabsf(p), fabsf(q)));
@@ -591,8 +591,8 @@ fxb_correction_kernel(FxBasis b, const double2 *__restrict__ V, int k, const dou
     } else {
       double2 a0 = make_double2(0.0, 0.0), a1 = a0;
       for (int r = 0; r < k; ++r) {
-        a0 = cfma(__ldg(V + (long long)r * n + i), h[r], a0);
-        a1 = cfma(__ldg(V + (long long)r * n + i + 1), h[r], a1);
+        a0 = cfma(V[(long long)r * n + i], h[r], a0);
+        a1 = cfma(V[(long long)r * n + i + 1], h[r], a1);
       }
       o0 = csub(o0, a0);
       o1 = csub(o1, a1);

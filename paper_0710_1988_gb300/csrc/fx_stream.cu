@@ -127,8 +127,8 @@ __device__ __forceinline__ void fxs_emit(FxsTile &t, const double2 (&x)[N], FxVe
 // TWO: out = a + beta out + mbo z (the p update); else out = a - alpha z (s)
 template <int N, bool TWO>
 __global__ void __launch_bounds__(FXS_THREADS, 2)
-bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, const double2 *__restrict__ z,
-                      FxVec fx, size_t tiled, const BicgScalars *__restrict__ sc,
+bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *a, const double2 *z,
+                      FxVec fx, size_t tiled, const BicgScalars *sc,
                       const int *status, long long n) {
   chain_enter();
   const int r = blockIdx.y;
@@ -174,9 +174,9 @@ bicg_update_fx_kernel(double2 *__restrict__ out, const double2 *__restrict__ a, 
 
 template <int N>
 __global__ void __launch_bounds__(FXS_THREADS, 2)
-bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, const double2 *__restrict__ p,
-                         const double2 *__restrict__ sv, const double2 *__restrict__ t,
-                         const double2 *__restrict__ rhat, const BicgScalars *__restrict__ sc,
+bicg_update_xr_fx_kernel(double2 *__restrict__ x, double2 *__restrict__ rv, const double2 *p,
+                         const double2 *sv, const double2 *t,
+                         const double2 *__restrict__ rhat, const BicgScalars *sc,
                          const int *status, double *__restrict__ partial, long long n, FinArgs fin) {
   chain_enter();
   const int r = blockIdx.y;

@@ -37,8 +37,19 @@ __device__ __forceinline__ float2 fcmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-__device__ __forceinline__ void ld_spinor32(const float4 *__restrict__ base, long long V,
+__device__ __forceinline__ void ld_spinor32(const float4 *base, long long V,
                                             long long s, float2 (&p)[12]) {
+#pragma unroll
+  for (int g = 0; g < 6; ++g) {
+    const float4 f = base[g * V + s];
+    p[2 * g] = make_float2(f.x, f.y);
+    p[2 * g + 1] = make_float2(f.z, f.w);
+  }
+}
+
+// the same of a vector that the chain does not write (chain.cuh)
+__device__ __forceinline__ void ld_fixed32(const float4 *__restrict__ base, long long V,
+                                           long long s, float2 (&p)[12]) {
 #pragma unroll
   for (int g = 0; g < 6; ++g) {
     const float4 f = __ldg(base + g * V + s);
@@ -91,7 +102,7 @@ __device__ __forceinline__ void su3_mul32(const float2 (&m)[9], const float2 (&h
 }
 
 template <int MU, int S, bool ADJ, int R>
-__device__ __forceinline__ void hop32(const float4 *__restrict__ links, const float4 *__restrict__ in,
+__device__ __forceinline__ void hop32(const float4 *__restrict__ links, const float4 *in,
                                       const bool (&on)[R], long long V, long long q, long long ql,
                                       float2 (&acc)[R][12]) {
   float2 u[9];
@@ -115,7 +126,7 @@ __device__ __forceinline__ void hop32(const float4 *__restrict__ links, const fl
 // with 16 systems).
 template <int R, int TPB, bool DAG, int EPI>
 __global__ void __launch_bounds__(TPB, R == 1 ? 768 / TPB : 1)
-wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ in,
+wilson_f32_kernel(const float4 *__restrict__ links, const float4 *in,
                   float4 *__restrict__ out, LatticeGeom g, float kappa, float mu, int nrhs,
                   const float4 *__restrict__ aux, double *__restrict__ partial,
                   const int *status, unsigned mask, unsigned long long *__restrict__ sites) {
@@ -187,7 +198,7 @@ wilson_f32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ i
       st_spinor32(out + (long long)(r0 + r) * 6 * V, V, s, o);
       if (EPI == EPI_DOT) {
         float2 a[12];
-        ld_spinor32(aux + (long long)(r0 + r) * 6 * V, V, s, a);
+        ld_fixed32(aux + (long long)(r0 + r) * 6 * V, V, s, a);
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
           red[r][0] = fmaf(a[c].x, o[c].x, fmaf(a[c].y, o[c].y, red[r][0]));
@@ -487,8 +498,8 @@ __device__ __forceinline__ float4 c2fma(float2 a, float4 b, float4 c) {  // c + 
 
 // p = r + beta (p - omega v)
 __global__ void __launch_bounds__(256)
-bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *__restrict__ r,
-                       const float4 *__restrict__ v, const BicgScalars *__restrict__ sc,
+bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *r,
+                       const float4 *v, const BicgScalars *sc,
                        const int *status, long long n4) {
   chain_enter();
   const int q = blockIdx.y;
@@ -506,8 +517,8 @@ bicg32_update_p_kernel(float4 *__restrict__ p, const float4 *__restrict__ r,
 // gathers two vectors: 332 us for it and 322 us for the update below at 20^3 x
 // 32 with 12 systems; with s in place of r 117 + 196 + 279 us.
 __global__ void __launch_bounds__(256)
-bicg32_update_s_kernel(float4 *__restrict__ r, const float4 *__restrict__ v,
-                       const BicgScalars *__restrict__ sc, const int *status, long long n4) {
+bicg32_update_s_kernel(float4 *__restrict__ r, const float4 *v,
+                       const BicgScalars *sc, const int *status, long long n4) {
   chain_enter();
   const int q = blockIdx.y;
   if (!on32(status, M_ACTIVE, q)) return;
@@ -521,8 +532,8 @@ bicg32_update_s_kernel(float4 *__restrict__ r, const float4 *__restrict__ v,
 // xs += alpha p + omega s; r = s - omega t, s in place of r; partial <rhat, r>, ||r||^2
 __global__ void __launch_bounds__(256)
 bicg32_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r,
-                        const float4 *__restrict__ p, const float4 *__restrict__ t,
-                        const float4 *__restrict__ rhat, const BicgScalars *__restrict__ sc, const int *status,
+                        const float4 *p, const float4 *t,
+                        const float4 *__restrict__ rhat, const BicgScalars *sc, const int *status,
                         double *__restrict__ partial, long long n4) {
   chain_enter();
   const int q = blockIdx.y;

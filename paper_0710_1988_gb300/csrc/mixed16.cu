@@ -57,13 +57,13 @@ __device__ __forceinline__ float2 f2of(double2 a) { return make_float2((float)a.
 }  // namespace
 
 // The stored half values of a site without its norm (the caller applies k).
-__device__ __forceinline__ float ld_h_raw(const uint4 *__restrict__ base,
-                                          const float *__restrict__ nrm, long long V, long long s,
+__device__ __forceinline__ float ld_h_raw(const uint4 *base,
+                                          const float *nrm, long long V, long long s,
                                           float2 (&p)[12]) {
-  const float k = __ldg(nrm + s);
+  const float k = nrm[s];
 #pragma unroll
   for (int g = 0; g < 3; ++g) {
-    const uint4 q = __ldg(base + g * V + s);
+    const uint4 q = base[g * V + s];
     p[4 * g] = h2f(q.x);
     p[4 * g + 1] = h2f(q.y);
     p[4 * g + 2] = h2f(q.z);
@@ -72,12 +72,12 @@ __device__ __forceinline__ float ld_h_raw(const uint4 *__restrict__ base,
   return k;
 }
 
-__device__ __forceinline__ void ld_h(const uint4 *__restrict__ base, const float *__restrict__ nrm,
+__device__ __forceinline__ void ld_h(const uint4 *base, const float *nrm,
                                      long long V, long long s, float2 (&p)[12]) {
-  const float k = __ldg(nrm + s);
+  const float k = nrm[s];
 #pragma unroll
   for (int g = 0; g < 3; ++g) {
-    const uint4 q = __ldg(base + g * V + s);
+    const uint4 q = base[g * V + s];
     const float2 a = h2f(q.x), b = h2f(q.y), c = h2f(q.z), d = h2f(q.w);
     p[4 * g] = make_float2(a.x * k, a.y * k);
     p[4 * g + 1] = make_float2(b.x * k, b.y * k);
@@ -104,8 +104,19 @@ __device__ __forceinline__ void st_h(uint4 *__restrict__ base, float *__restrict
   }
 }
 
-__device__ __forceinline__ void ld_f(const float4 *__restrict__ base, long long V, long long s,
+__device__ __forceinline__ void ld_f(const float4 *base, long long V, long long s,
                                      float2 (&p)[12]) {
+#pragma unroll
+  for (int g = 0; g < 6; ++g) {
+    const float4 f = base[g * V + s];
+    p[2 * g] = make_float2(f.x, f.y);
+    p[2 * g + 1] = make_float2(f.z, f.w);
+  }
+}
+
+// the same of a vector that the chain does not write (chain.cuh)
+__device__ __forceinline__ void ld_fixed16(const float4 *__restrict__ base, long long V, long long s,
+                                           float2 (&p)[12]) {
 #pragma unroll
   for (int g = 0; g < 6; ++g) {
     const float4 f = __ldg(base + g * V + s);
@@ -138,8 +149,8 @@ __device__ __forceinline__ void ld_link16(const uint2 *__restrict__ L, long long
 // vector (p holds its stored values; the hop scales its product once), 1
 // for the fused input (the norm is folded into alpha).
 template <bool FUSED>
-__device__ __forceinline__ float ld_hop16(const uint4 *__restrict__ in, const float *__restrict__ in_n,
-                                          const float4 *__restrict__ r32, float2 alpha, long long V,
+__device__ __forceinline__ float ld_hop16(const uint4 *in, const float *in_n,
+                                          const float4 *r32, float2 alpha, long long V,
                                           long long s, float2 (&p)[12]) {
   if (FUSED) {
     float2 q[12];
@@ -154,8 +165,8 @@ __device__ __forceinline__ float ld_hop16(const uint4 *__restrict__ in, const fl
 }
 
 template <bool FUSED>
-__device__ __forceinline__ void ld_in16(const uint4 *__restrict__ in, const float *__restrict__ in_n,
-                                        const float4 *__restrict__ r32, float2 alpha, long long V,
+__device__ __forceinline__ void ld_in16(const uint4 *in, const float *in_n,
+                                        const float4 *r32, float2 alpha, long long V,
                                         long long s, float2 (&p)[12]) {
   if (FUSED) {
     float2 q[12];
@@ -186,7 +197,7 @@ __device__ __forceinline__ void su3_mul16(const float2 (&m)[9], const float2 (&h
 
 template <int MU, int S, bool ADJ, int R, bool FUSED>
 __device__ __forceinline__ void hop16(const uint2 *__restrict__ links, const Half16 &in,
-                                      const float4 *__restrict__ r32, const float2 (&alpha)[R],
+                                      const float4 *r32, const float2 (&alpha)[R],
                                       const bool (&on)[R], int r0, long long V, long long q,
                                       long long ql, float2 (&acc)[R][12]) {
   float2 u[9];
@@ -212,9 +223,9 @@ __device__ __forceinline__ void hop16(const uint2 *__restrict__ links, const Hal
 // in = v, r32 = r): out = A s with s = r - alpha v, + <out, s>, ||out||^2.
 template <int R, int TPB, bool DAG, int EPI, bool FUSED>
 __global__ void __launch_bounds__(TPB)
-wilson_f16_kernel(const uint2 *__restrict__ links, Half16 in, const float4 *__restrict__ r32,
+wilson_f16_kernel(const uint2 *__restrict__ links, Half16 in, const float4 *r32,
                   Half16 out, LatticeGeom g, float kappa, float mu, int nrhs,
-                  const BicgScalars *__restrict__ sc, const float4 *__restrict__ aux,
+                  const BicgScalars *sc, const float4 *__restrict__ aux,
                   double *__restrict__ partial, const int *status, unsigned mask,
                   unsigned long long *__restrict__ sites) {
   chain_enter();
@@ -289,7 +300,7 @@ wilson_f16_kernel(const uint2 *__restrict__ links, Half16 in, const float4 *__re
       st_h(out.v + (long long)q * 3 * V, out.n + (long long)q * V, V, s, o);
       if (EPI == EPI_DOT) {
         float2 a[12];
-        ld_f(aux + (long long)q * 6 * V, V, s, a);
+        ld_fixed16(aux + (long long)q * 6 * V, V, s, a);
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
           red[r][0] = fmaf(a[c].x, o[c].x, fmaf(a[c].y, o[c].y, red[r][0]));
@@ -517,9 +528,9 @@ __device__ __forceinline__ bool on16(const int *status, unsigned mask, int r) {
 }
 
 // p (half) = r + beta (p - omega v)
-__global__ void __launch_bounds__(256)
-bicg16_update_p_kernel(Half16 p, const float4 *__restrict__ r, Half16 v,
-                       const BicgScalars *__restrict__ sc, const int *status,
+__global__ void __launch_bounds__(256, 4)
+bicg16_update_p_kernel(Half16 p, const float4 *r, Half16 v,
+                       const BicgScalars *sc, const int *status,
                        long long V) {
   chain_enter();
   const int q = blockIdx.y;
@@ -538,10 +549,10 @@ bicg16_update_p_kernel(Half16 p, const float4 *__restrict__ r, Half16 v,
 }
 
 // s = r - alpha v; xs += alpha p + omega s; r = s - omega t; partial <rhat, r>, ||r||^2
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 bicg16_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r, Half16 p, Half16 v,
                         Half16 t, const float4 *__restrict__ rhat,
-                        const BicgScalars *__restrict__ sc, const int *status,
+                        const BicgScalars *sc, const int *status,
                         double *__restrict__ partial, long long V) {
   chain_enter();
   const int q = blockIdx.y;
@@ -557,7 +568,7 @@ bicg16_update_xr_kernel(float4 *__restrict__ xs, float4 *__restrict__ r, Half16 
     ld_h(p.v + (long long)q * 3 * V, p.n + (long long)q * V, V, s, pv);
     ld_h(t.v + (long long)q * 3 * V, t.n + (long long)q * V, V, s, tv);
     ld_f(xs + (long long)q * 6 * V, V, s, xv);
-    ld_f(rhat + (long long)q * 6 * V, V, s, hv);
+    ld_fixed16(rhat + (long long)q * 6 * V, V, s, hv);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
       const float2 sv = fcfma16(mal, vv[c], rv[c]);

@@ -39,11 +39,11 @@ __device__ __forceinline__ float2 fcmul_eo(float2 a, float2 b) {
 }
 
 // 12 complex components of a half-vector site (compact index c, stride Vh)
-__device__ __forceinline__ void ld_half32(const float4 *__restrict__ base, long long Vh, long long c,
+__device__ __forceinline__ void ld_half32(const float4 *base, long long Vh, long long c,
                                           float2 (&p)[12]) {
 #pragma unroll
   for (int g = 0; g < 6; ++g) {
-    const float4 f = __ldg(base + g * Vh + c);
+    const float4 f = base[g * Vh + c];
     p[2 * g] = make_float2(f.x, f.y);
     p[2 * g + 1] = make_float2(f.z, f.w);
   }
@@ -73,7 +73,7 @@ __device__ __forceinline__ void ld_link_eo(const float4 *__restrict__ L, long lo
 // one hop: neighbour q (full index, other parity) read from the half vector
 template <int MU, int S, bool ADJ>
 __device__ __forceinline__ void hop_eo32(const float4 *__restrict__ links,
-                                         const float4 *__restrict__ src,
+                                         const float4 *src,
                                          long long V, long long q, long long ql,
                                          float2 (&acc)[12]) {
   float2 u[9], p[12], h[6], c[6];
@@ -104,8 +104,8 @@ enum { EO32_SCHUR1 = 0, EO32_SCHUR2 = 1 };
 //               ||out||^2).
 template <bool DAG, int MODE, int EPI>
 __global__ void __launch_bounds__(128, 6)  // 80 registers, as the full FP32 kernel
-wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *__restrict__ src,
-                   const float4 *__restrict__ same, float4 *__restrict__ out, LatticeGeom g,
+wilson_eo32_kernel(const float4 *__restrict__ links, const float4 *src,
+                   const float4 *same, float4 *__restrict__ out, LatticeGeom g,
                    int pout, float kappa, float mu,
                    const float4 *__restrict__ aux, double *__restrict__ partial,
                    const int *status, unsigned mask, unsigned long long *__restrict__ sites, int nrhs) {
