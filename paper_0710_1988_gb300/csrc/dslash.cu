@@ -587,13 +587,17 @@ wilson_fx_few_kernel(const int4 *__restrict__ L, const double2 *__restrict__ lin
 }
 
 // Whether the few-site kernel serves nrhs systems of the full operator: up to
-// where the two forms take the same time, sites x systems (us an apply, this
-// kernel / encoding + wilson_fx_kernel).  Even extents: 256: 9.2 / 12.4, 4096: 9.5 /
-// 12.4, 8192: 12.5 / 12.5, 16384: 21.8 / 15.0.  With an odd extent, where the links
-// are not stored by parity, 3465: 9.6 / 14.4, 10395: 14.6 / 18.5.  The
-// solvers' products (epi) come with their input encoded, some 3 us less.
+// where the two forms take the same time, in sites x systems.
+// us an apply, this kernel / encoding + wilson_fx_kernel: even extents 4096 8.2 /
+// 12.4, 12288 13.9 / 16.1, 14336 15.4 / 16.2, 16384 17.4 / 16.4; with an odd extent,
+// where the links are not stored by parity, 3969 8.7 / 14.5, 11979 12.5 / 18.5,
+// 20449 18.5 / 20.6, 24167 21.1 / 20.0 (one system; seven to 56 alike).
+// us a BiCGStab iteration (epi), whose products come with their input encoded:
+// even 4096 49.7 / 54.1, 4608 53.6 / 54.4, 5120 57.7 / 56.6, 8192 68.0 / 65.6; odd 8019
+// 67.4 / 68.8, 11025 71.9 / 79.4, 11979 83.6 / 83.6, 14641 92.7 / 83.2.
 static bool fx_few(const wd_context *h, int nrhs, int epi) {
-  const long long most = epi != EPI_NONE ? 6144 : geom_of(h).split ? 8192 : 12288;
+  const bool even = geom_of(h).split;
+  const long long most = epi != EPI_NONE ? (even ? 4608 : 11264) : even ? 14336 : 21504;
   return !h->eo && h->links_fx != nullptr && h->V * nrhs <= most;
 }
 
