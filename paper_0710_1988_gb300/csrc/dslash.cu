@@ -657,15 +657,10 @@ static cudaError_t launch_wilson_fx(const wd_context *h, FxVec f, const double2 
   return launch_chained(wilson_fx_kernel<D, E>, dim3(grid), dim3(2 * WILSON_SITES), FX_SMEM, s,      \
                         h->links_fx, h->links, f, in, out, g, fx_sites(h->V), h->kappa, h->mu,   \
                         nrhs, aux, partial, status, mask, cnt, fin)
-  if (dagger) {
-    if (epi == EPI_DOT) WFX(true, EPI_DOT);
-    if (epi == EPI_TSTT) WFX(true, EPI_TSTT);
-    WFX(true, EPI_NONE);
-  } else {
-    if (epi == EPI_DOT) WFX(false, EPI_DOT);
-    if (epi == EPI_TSTT) WFX(false, EPI_TSTT);
-    WFX(false, EPI_NONE);
-  }
+  if (epi == EPI_DOT) WFX(false, EPI_DOT);
+  if (epi == EPI_TSTT) WFX(false, EPI_TSTT);
+  if (dagger) WFX(true, EPI_NONE);
+  WFX(false, EPI_NONE);
 #undef WFX
 }
 
@@ -679,15 +674,10 @@ static cudaError_t launch_wilson_fx_few(const wd_context *h, const double2 *in, 
   return launch_chained(wilson_fx_few_kernel<D, E>, dim3(grid), dim3(16 * FX_FEW_SITES), 0, s,  \
                         h->links_fx, h->links, in, out, g, h->kappa, h->mu, nrhs, aux, partial, \
                         status, mask, cnt, fin)
-  if (dagger) {
-    if (epi == EPI_DOT) WFEW(true, EPI_DOT);
-    if (epi == EPI_TSTT) WFEW(true, EPI_TSTT);
-    WFEW(true, EPI_NONE);
-  } else {
-    if (epi == EPI_DOT) WFEW(false, EPI_DOT);
-    if (epi == EPI_TSTT) WFEW(false, EPI_TSTT);
-    WFEW(false, EPI_NONE);
-  }
+  if (epi == EPI_DOT) WFEW(false, EPI_DOT);
+  if (epi == EPI_TSTT) WFEW(false, EPI_TSTT);
+  if (dagger) WFEW(true, EPI_NONE);
+  WFEW(false, EPI_NONE);
 #undef WFEW
 }
 
@@ -733,6 +723,7 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
                                   double *partial, const int *status, cudaStream_t s,
                                   unsigned mask, const FxVec *pre, const FinArgs *fin) {
   const FinArgs f = fin ? *fin : FinArgs{};
+  if (dagger && epi != EPI_NONE) return cudaErrorInvalidValue;   // no solver iterates A^dagger
   if (h->eo)  // even-odd Schur operator on even half vectors
     return launch_schur_f64_epi(h, in, out, nrhs, dagger, epi, aux, partial, status, s, mask, pre, fin);
   ProfLaunch prof(PC_DSLASH, s);
@@ -758,21 +749,14 @@ cudaError_t launch_wilson_f64_epi(const wd_context *h, const double2 *in, double
   }
   dim3 grid(wilson_blocks(h, nrhs), nrhs);
   LatticeGeom g = geom_of(h);
-  if (dagger) {
-    if (epi == EPI_DOT)
-      wilson_f64_kernel<true, EPI_DOT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-    else if (epi == EPI_TSTT)
-      wilson_f64_kernel<true, EPI_TSTT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-    else
-      wilson_f64_kernel<true, EPI_NONE><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-  } else {
-    if (epi == EPI_DOT)
-      wilson_f64_kernel<false, EPI_DOT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-    else if (epi == EPI_TSTT)
-      wilson_f64_kernel<false, EPI_TSTT><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-    else
-      wilson_f64_kernel<false, EPI_NONE><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, status, mask, cnt);
-  }
+#define W64(D, E)                                                                                        \
+  wilson_f64_kernel<D, E><<<grid, WILSON_SITES, 0, s>>>(h->links, in, out, g, h->kappa, h->mu, aux, partial, \
+                                                        status, mask, cnt)
+  if (epi == EPI_DOT) W64(false, EPI_DOT);
+  else if (epi == EPI_TSTT) W64(false, EPI_TSTT);
+  else if (dagger) W64(true, EPI_NONE);
+  else W64(false, EPI_NONE);
+#undef W64
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || fin == nullptr) return e;
   return launch_bicg_finalize(f.kind, partial, f.nb, f.sc, f.status, f.hist, f.hist_len, nrhs, s);

@@ -375,8 +375,8 @@ static void launch_eo(int mode, int epi, dim3 grid, cudaStream_t s, const wd_con
                                                    h->mu, inv, aux, partial, status, mask, cnt)
   if (mode == EO_SCHUR1) EO_LAUNCH(EO_SCHUR1, EPI_NONE);
   else if (mode == EO_AXPY) EO_LAUNCH(EO_AXPY, EPI_NONE);
-  else if (epi == EPI_DOT) EO_LAUNCH(EO_SCHUR2, EPI_DOT);
-  else if (epi == EPI_TSTT) EO_LAUNCH(EO_SCHUR2, EPI_TSTT);
+  else if (epi == EPI_DOT) EO_LAUNCH(EO_SCHUR2, DAG ? EPI_NONE : EPI_DOT);   // never with DAG
+  else if (epi == EPI_TSTT) EO_LAUNCH(EO_SCHUR2, DAG ? EPI_NONE : EPI_TSTT);
   else EO_LAUNCH(EO_SCHUR2, EPI_NONE);
 #undef EO_LAUNCH
 }
@@ -418,11 +418,7 @@ cudaError_t launch_schur_f64_epi(const wd_context *hc, const double2 *in, double
     return e != cudaSuccess ? e : EO_FX(D, EO_SCHUR2, E, tmp, h->eo_tmp, in, out, tmp, 0, cnt,        \
                                               fin ? *fin : none);                                  \
   }
-    if (dagger) {
-      if (epi == EPI_DOT) EO_FX_PAIR(true, EPI_DOT)
-      if (epi == EPI_TSTT) EO_FX_PAIR(true, EPI_TSTT)
-      EO_FX_PAIR(true, EPI_NONE)
-    }
+    if (dagger) EO_FX_PAIR(true, EPI_NONE)
     if (epi == EPI_DOT) EO_FX_PAIR(false, EPI_DOT)
     if (epi == EPI_TSTT) EO_FX_PAIR(false, EPI_TSTT)
     EO_FX_PAIR(false, EPI_NONE)
