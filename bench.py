@@ -51,10 +51,9 @@ DSLASH_BYTES_PER_SITE = 960       # 192 in + 192 out + 4 links x 144 (FP64)
 # updates); the bench scales it to a launch by the site updates it processed.
 DSLASH_DRAM_BYTES_PER_SITE_UPDATE = 430.4e6 / 655360
 # The FP64 operator's products are formed in fixed point: 8 hops x 6 components
-# x 3 terms x 9 integer multiply-adds (32 x 32 + 64 bits) a site update, which a
-# throughput probe of independent chains issues at 53 per clock and SM.
+# x 3 terms x 9 integer multiply-adds (32 x 32 + 64 bits) a site update; the rate
+# is measured live (wd_probe_wide_mad_peak, 53 per clock and SM).
 DSLASH_WIDE_MADS_PER_SITE = 1296
-WIDE_MADS_PER_CLK_PER_SM = 53
 METRIC = "D-BiCGStab solves/s at rel. residual 1e-10; dslash GB/s vs HBM roofline"
 
 
@@ -501,7 +500,9 @@ def measured_fp64_peak(local_rank, iters=1 << 15, reps=20):
     clocks.start()
     tf, ms = wdl.probe_fp64_peak(iters=iters, reps=reps)
     clk = clocks.stop()
-    return {"tflops": round(tf, 4), "ms_per_launch": round(ms, 3), "clocks": clk,
+    wdl.probe_wide_mad_peak(iters=iters // 4, reps=2)
+    tmads, _ = wdl.probe_wide_mad_peak(iters=iters // 4, reps=reps)
+    return {"tflops": round(tf, 4), "wide_tmads": round(tmads, 3), "ms_per_launch": round(ms, 3), "clocks": clk,
             "derived_tflops": round(derived, 4),
             "source": (f"measured live: wd_probe_fp64_peak (8 independent DFMA chains per "
                        f"thread, 4 x 256 threads per SM, {reps} launches of {ms:.1f} ms, CUDA "
@@ -520,8 +521,7 @@ def roofline(res, peaks, fp64_peak):
     flops = DSLASH_FLOPS_PER_SITE * sites_per_launch
     tflops = flops / (avg_ms * 1e-3) / 1e12
     gbs = DSLASH_BYTES_PER_SITE * sites_per_launch / (avg_ms * 1e-3) / 1e9
-    peak = (WIDE_MADS_PER_CLK_PER_SM * SMS * SM_MAX_MHZ * 1e6 / DSLASH_WIDE_MADS_PER_SITE
-            * DSLASH_FLOPS_PER_SITE / 1e12)
+    peak = fp64_peak["wide_tmads"] / DSLASH_WIDE_MADS_PER_SITE * DSLASH_FLOPS_PER_SITE
     out = {
         "kernel": "wilson_fx_kernel (FP64 dslash, products in fixed point)",
         "bound": "alu",
@@ -530,8 +530,8 @@ def roofline(res, peaks, fp64_peak):
         "unit": "TFLOP/s",
         "frac": round(tflops / peak, 4),
         "peak_source": (f"{DSLASH_WIDE_MADS_PER_SITE} 32 x 32 + 64-bit multiply-adds a site update at "
-                        f"{WIDE_MADS_PER_CLK_PER_SM} per clock and SM (throughput probe), {SMS} SMs, "
-                        f"{SM_MAX_MHZ:.0f} MHz, counted as the {DSLASH_FLOPS_PER_SITE} FP64 flops they stand for"),
+                        f"{fp64_peak['wide_tmads']}e12 a second (measured live: wd_probe_wide_mad_peak), "
+                        f"counted as the {DSLASH_FLOPS_PER_SITE} FP64 flops they stand for"),
         "fp64_pipe_peak": fp64_peak["tflops"],
         "times_fp64_pipe_peak": round(tflops / fp64_peak["tflops"], 4),
         "fp64_pipe_peak_source": fp64_peak["source"],
@@ -656,8 +656,10 @@ LOW_LINK_BYTES = {32: 4 * 48, 16: 4 * 24}            # links (rows 0, 1), read o
 # even-odd Schur apply (FP32), per even site and system: v = A_hat p moves
 # SCHUR1 in + tmp and SCHUR2 tmp + p + out + r_hat; t = A_hat (r - alpha v) moves
 # SCHUR1 r + v + tmp and SCHUR2 tmp + r + v + out; the mean of the two applies.
-# (The kernels read s = r - alpha v, which an update pass writes: 11 of these 13.)
 LOW_SCHUR_BYTES = {32: (2 * 96 + 4 * 96 + 3 * 96 + 4 * 96) / 2}
+# as the kernels move them: t = A_hat s reads s, which an update pass writes (and
+# LOW_UPDATE_BYTES counts), SCHUR1 s + tmp and SCHUR2 tmp + s + out.
+LOW_SCHUR_MOVED_BYTES = {32: (2 * 96 + 4 * 96 + 2 * 96 + 3 * 96) / 2}
 LOW_UPDATE_BYTES = {32: 4 * 96 + 3 * 96 + 7 * 96,    # p = r + beta (p - omega v); s; x, r update
                     16: (96 + 3 * 52) + (4 * 96 + 3 * 52 + 2 * 96)}
 
@@ -704,21 +706,21 @@ def timed_steps(args, step, op, flush, stream, world, dev, prof_mask=0):
     return ms_steps, last, prof, clocks.stop()
 
 
-def low_rooflines(prof, bits, V, peaks, iters_total, eo=False):
+def low_rooflines(prof, bits, V, peaks, iters_total, eo=False, schur_bytes=None):
     """HBM rooflines of the mixed solver's FP32/FP16 kernels from a profiled
     step: the Wilson apply (site updates counted on the device) and the two
     per-iteration vector updates (one pass of each per system iteration; FP16
     forms s inside its product and update).
     On the even-odd Schur system (eo) one profiled launch is a Schur apply: two
     half-lattice hop kernels, each reading every link, with V/2 counted site
-    updates per system (LOW_SCHUR_BYTES each); the vector updates run over V/2
-    sites."""
+    updates per system (schur_bytes each, LOW_SCHUR_BYTES by default); the vector
+    updates run over V/2 sites."""
     hbm = peaks.get("hbm_gbs")
     out = {}
     d = prof["dslash_low"]
     if d["launches"]:
         if eo:
-            byt = (LOW_SCHUR_BYTES[bits] * prof["dslash_low_site_updates"]
+            byt = ((schur_bytes or LOW_SCHUR_BYTES)[bits] * prof["dslash_low_site_updates"]
                    + 2 * LOW_LINK_BYTES[bits] * V * d["launches"])
         else:
             byt = (LOW_DSLASH_BYTES[bits] * prof["dslash_low_site_updates"]
@@ -897,7 +899,7 @@ def twisted_arm(args, cfg, rank, world, local_rank):
     op.profile(mask=0)
     peaks = load_json(MEASURED_PEAKS, {}) or {}
     roof = low_rooflines(prof, args.storage, v, peaks, sum(q["iters"] for row in sts_p for q in row),
-                         eo=args.even_odd)
+                         eo=args.even_odd, schur_bytes=LOW_SCHUR_MOVED_BYTES)
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
     e0.record(stream)
@@ -1217,7 +1219,8 @@ def growth_twisted(local_rank, peaks, mus=(0.064, 0.032)):
     sts_p = run()
     prof = op.profile_read()
     op.profile(mask=0)
-    roof = low_rooflines(prof, 32, v, peaks, sum(q["iters"] for row in sts_p for q in row), eo=True)
+    roof = low_rooflines(prof, 32, v, peaks, sum(q["iters"] for row in sts_p for q in row), eo=True,
+                         schur_bytes=LOW_SCHUR_MOVED_BYTES)
     op.close()
     units = cfg.n_rhs * len(mus)
     return {"workload": f"{cfg.name}: A_W + i mu gamma5 at kappa_c, shifts {list(mus)} heaviest "

@@ -406,6 +406,11 @@ int wd_profile_read(wd_handle h, wd_profile *out);
  * 1 <= reps <= 1000, else WD_BAD_ARG. */
 int wd_probe_fp64_peak(int iters, int reps, double *tflops, double *ms, wd_stream stream);
 
+/* 32 x 32 + 64-bit integer multiply-add throughput of the current device,
+ * measured in the same way (the denominator of the fixed-point kernels'
+ * roofline): *tmads = 1e12 multiply-adds a second. */
+int wd_probe_wide_mad_peak(int iters, int reps, double *tmads, double *ms, wd_stream stream);
+
 /* BF16 tensor-core throughput of the current device, measured (not part of
  * the paper's method: the rate the exact-split contraction of
  * wd_set_contraction draws on).  One CTA per SM issues `iters` tcgen05 MMAs

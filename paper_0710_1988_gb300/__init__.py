@@ -62,6 +62,15 @@ def probe_fp64_peak(iters: int = 1 << 15, reps: int = 3, stream=None):
     return tf.value, ms.value
 
 
+def probe_wide_mad_peak(iters: int = 1 << 15, reps: int = 3, stream=None):
+    """Measured 32 x 32 + 64-bit integer multiply-add throughput of the current
+    device: (1e12 a second, ms per launch), timed by CUDA events."""
+    t, ms = ctypes.c_double(), ctypes.c_double()
+    check(lib().wd_probe_wide_mad_peak(int(iters), int(reps), ctypes.byref(t), ctypes.byref(ms),
+                                       _stream(stream)))
+    return t.value, ms.value
+
+
 def tsgemm(V, kv: int, Y, ncol: int, OUT, IN=None, sign: float = 1.0,
            tensor_cores: bool = True, ldy: Optional[int] = None, stream=None):
     """OUT[c] = (IN[c] if IN is given else 0) + sign * sum_r V[r] Y[r, c] for

@@ -71,6 +71,7 @@ SIGNATURES = {
     "gmresdr_solve": (I, [P, P, P, I, I, D, I, P, P, P, ctypes.POINTER(WdStats), P]),
     "gmresdr_history": (I, [P, P, I]),
     "wd_probe_fp64_peak": (I, [I, I, P, P, P]),
+    "wd_probe_wide_mad_peak": (I, [I, I, P, P, P]),
     "wd_probe_bf16_mma_peak": (I, [I, I, P, P, P]),
     "wd_set_contraction": (I, [P, I]),
     "wd_set_eigen_estimates": (I, [P, I]),

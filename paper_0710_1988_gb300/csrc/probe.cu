@@ -68,6 +68,61 @@ extern "C" int wd_probe_fp64_peak(int iters, int reps, double *tflops, double *m
   return WD_OK;
 }
 
+// ----------------------------------------------------------------- integer multiply-adds
+//
+// The same for the 32 x 32 + 64-bit multiply-adds of the fixed-point products:
+// kChains independent 64-bit sums a thread.
+namespace wd {
+namespace {
+__global__ void __launch_bounds__(kThreads) wide_mad_probe_kernel(int iters, int a, int b) {
+  long long acc[kChains];
+  const int x = a + (int)threadIdx.x;
+#pragma unroll
+  for (int c = 0; c < kChains; ++c) acc[c] = threadIdx.x + c;
+  for (int i = 0; i < iters; ++i) {
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) asm volatile("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[c]) : "r"(x), "r"(b + c));
+  }
+  long long s = 0;
+#pragma unroll
+  for (int c = 0; c < kChains; ++c) s += acc[c];
+  if (s == -1) g_probe_sink = (double)s;   // never: positive products below 2^20 each
+}
+}  // namespace
+}  // namespace wd
+
+extern "C" int wd_probe_wide_mad_peak(int iters, int reps, double *tmads, double *ms, wd_stream stream) {
+  if (iters < 1 || iters > (1 << 24) || reps < 1 || reps > 1000 || tmads == nullptr) {
+    set_error("wd_probe_wide_mad_peak: iters in [1, 2^24], reps in [1, 1000], tmads not NULL");
+    return WD_BAD_ARG;
+  }
+  int dev = 0, sms = 0;
+  WD_CK(cudaGetDevice(&dev));
+  WD_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int blocks = 4 * sms;
+  cudaStream_t s = (cudaStream_t)stream;
+  wide_mad_probe_kernel<<<blocks, kThreads, 0, s>>>(iters, 3, 5);  // warm-up
+  WD_CK_LAUNCH("wide_mad_probe_kernel");
+  cudaEvent_t e0, e1;
+  WD_CK(cudaEventCreate(&e0));
+  WD_CK(cudaEventCreate(&e1));
+  cudaError_t e = cudaEventRecord(e0, s);
+  for (int r = 0; r < reps && e == cudaSuccess; ++r) {
+    wide_mad_probe_kernel<<<blocks, kThreads, 0, s>>>(iters, 3, 5);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+  if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+  float t = 0.f;
+  if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (e != cudaSuccess) return cuda_fail(e, "wd_probe_wide_mad_peak");
+  *tmads = (double)kChains * iters * blocks * kThreads * reps / (t * 1e-3) / 1e12;
+  if (ms) *ms = t / reps;
+  return WD_OK;
+}
+
 // ----------------------------------------------------------------- BF16 MMA throughput
 //
 // tcgen05 BF16 MMAs with FP32 accumulation, M = 128, N = 256, K = 16, one
