@@ -47,12 +47,12 @@ SM_MAX_MHZ = 2070.0
 DSLASH_FLOPS_PER_SITE = 1368      # 1320 hopping + 48 for 1 - kappa*D
 DSLASH_BYTES_PER_SITE = 960       # 192 in + 192 out + 4 links x 144 (FP64)
 # DRAM bytes (read + write) per site update of wilson_fx_kernel from one ncu
-# capture of a 10-system launch at 16^4 (318.0 + 112.4 MB / 655,360 site
+# capture of a 10-system launch at 16^4 (317.8 + 120.6 MB / 655,360 site
 # updates); the bench scales it to a launch by the site updates it processed.
-DSLASH_DRAM_BYTES_PER_SITE_UPDATE = 430.4e6 / 655360
+DSLASH_DRAM_BYTES_PER_SITE_UPDATE = 438.4e6 / 655360
 # The FP64 operator's products are formed in fixed point: 8 hops x 6 components
 # x 3 terms x 9 integer multiply-adds (32 x 32 + 64 bits) a site update; the rate
-# is measured live (wd_probe_wide_mad_peak, 53 per clock and SM).
+# is measured live (wd_probe_wide_mad_peak, 60 per clock and SM).
 DSLASH_WIDE_MADS_PER_SITE = 1296
 METRIC = "D-BiCGStab solves/s at rel. residual 1e-10; dslash GB/s vs HBM roofline"
 
@@ -539,7 +539,7 @@ def roofline(res, peaks, fp64_peak):
         "fp64_pipe_peak_derived_source": fp64_peak["derived_source"],
         "traffic": round(DSLASH_DRAM_BYTES_PER_SITE_UPDATE * sites_per_launch),
         "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 16^4 "
-                          "10-system launch (657 B per site update), scaled to the average "
+                          "10-system launch (669 B per site update), scaled to the average "
                           "launch by site updates",
         "algorithmic_flops_per_launch": flops,
         "avg_launch_ms": avg_ms,

@@ -275,7 +275,7 @@ __device__ __noinline__ void hops_f64(const double2 *psi, const double2 *__restr
 // wilson_f64_kernel's result with the hops in fixed point; `in` is the
 // encoded form of in64.  A block covers 64 sites, two lanes (l, l + 16) a
 // site; four fit an SM (16 warps, the registers' limit).  With two of 128 sites
-// more of the SM waits for a block's last warp (0.274 against 0.267 ms, 10
+// more of the SM waits for a block's last warp (0.274 against 0.267 ms then, 10
 // systems at 16^4).  Blocks are numbered system fastest: the nrhs blocks of one range of
 // sites share its links through L2.
 constexpr size_t FX_SMEM = 2 * WILSON_SITES / 32 * 2 * sizeof(FxStage);   // two stages a warp

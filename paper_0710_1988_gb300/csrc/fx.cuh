@@ -2,8 +2,8 @@
 //
 // This GPU issues 1.7 FP64 FMAs per clock and SM (DFMA probe), so a site
 // update's ~930 FP64 instructions take 550 clocks of its SM; integer
-// multiply-adds of 32 x 32 + 64 bits go at about 30, 32-bit integer adds at
-// 120.  The hops' products are therefore formed in integers.  A spinor site
+// multiply-adds of 32 x 32 + 64 bits go at 60 (27 to 35 reached inside these
+// kernels), 32-bit integer adds at 120.  The hops' products are therefore formed in integers.  A spinor site
 // (24 reals) shares the largest exponent field E of its entries and holds
 // each as X = round(x 2^(1078 - E)), |X| <= 2^56: entries down to 2^-3 of the
 // site's largest are held exactly, smaller ones to 2^-57 of it.  X is stored
@@ -309,8 +309,9 @@ __device__ __forceinline__ int fx_lost(uint2 reach, int least) {
 // copies past L1, 0.288 so, of which 0.237 without any copy; with a hop's shift
 // rounded in its first sum (no additions, no branch for d = 0) and blocks of
 // half the size 0.267, with the epilogue's operand copied during the last hop
-// (tail) 0.257.  Now the LSU's data pipe (83 % of its wavefronts) and the
-// multiply-adds (56 %) bound it, at the 16 warps an SM that 128 registers leave.
+// (tail) 0.257, with the terms' lengths (reach) 0.266.  Now the LSU's data pipe (82 %
+// of its wavefronts) and the multiply-adds (59 %) bound it, at the 16 warps an SM that
+// 128 registers leave.
 // The y and z hops come first in their lower sums, whose factor sgn is then
 // applied once; between them the lanes exchange the x and y hops' lower sums,
 // which belong to the other.  Returned: the bit lengths of the high words of the
