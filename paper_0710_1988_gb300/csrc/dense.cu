@@ -117,7 +117,7 @@ __device__ __forceinline__ double2 warp_csum_all(double2 v) {
 }
 
 // In-place LU with partial pivoting of the k x k matrix A (leading dim ld).
-// Returns 1 if an exactly zero pivot was met.  Every thread of the block calls it.
+// Returns 1 if a pivot was exactly zero or NaN.  Every thread of the block calls it.
 __device__ int lu_factor_block(double2 *A, int ld, int k, int *piv) {
   int singular = 0;
   for (int j = 0; j < k; ++j) {
@@ -131,7 +131,7 @@ __device__ int lu_factor_block(double2 *A, int ld, int k, int *piv) {
       }
     }
     block_argmax(best, bi);
-    const int p = bi;
+    const int p = bi < k ? bi : j;   // a column of NaN has no largest entry
     if (threadIdx.x == 0) piv[j] = p;
     if (p != j) {
       for (int c = threadIdx.x; c < k; c += blockDim.x) {
@@ -142,7 +142,7 @@ __device__ int lu_factor_block(double2 *A, int ld, int k, int *piv) {
     }
     __syncthreads();
     const double2 pv = A[j * ld + j];
-    if (pv.x == 0.0 && pv.y == 0.0) {
+    if (!(cabs1(pv) > 0.0)) {
       singular = 1;
       continue;
     }
@@ -1310,10 +1310,14 @@ __global__ void __launch_bounds__(HRR_THREADS) harmonic_ritz_refine_kernel(Cycle
 }
 
 // Order (|theta|, Re, Im, index) of the m values th: the ranks of the k
-// smallest into sel.  Block-wide; ends with a barrier.
+// smallest into sel, in range also where NaN leaves ranks out.  Block-wide; ends
+// with a barrier.
 __device__ void select_smallest(const double2 *th, int m, int k, int *sel) {
   __shared__ double s_abs[CE_MAXM];
-  for (int i = threadIdx.x; i < m; i += blockDim.x) s_abs[i] = cabs_(th[i]);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    s_abs[i] = cabs_(th[i]);
+    if (i < k) sel[i] = i;
+  }
   __syncthreads();
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     const double2 ti = th[i];
