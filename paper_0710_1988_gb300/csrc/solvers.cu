@@ -358,10 +358,13 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     return WD_OK;
   }
   WD_CK(cudaMemsetAsync(H, 0, sizeof(double2) * (m + 1) * m, s));
+  WD_CK(cudaMemsetAsync(Hk, 0, sizeof(double2) * (k + 1) * (k > 0 ? k : 1), s));   // outputs of a solve that never restarts
+  WD_CK(cudaMemsetAsync(theta, 0, sizeof(double2) * (k > 0 ? k : 1), s));
   RET_IF(launch_ok(launch_fxb_encode(r, c, 0, Va, fb, 0, 1, fv, n, nullptr, s), "v1"));
 
   double2 *V = Va, *Vn = Vb;
   int j0 = 0, cycles = 0, rc = WD_NOT_CONVERGED;
+  int valid = k;   // basis vectors that exist
   const int zero = 0;
   double last_rel = 1.0;
   std::vector<double> hist;
@@ -418,6 +421,7 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
       break;
     }
     const bool lucky = hflags[1] != 0;
+    if (lucky) valid = hme;
     const bool done = lucky || last_rel <= tol;
     if (!lucky) {
       // V_{k+1} = V_{m+1} P_{k+1} (also after the last cycle, to emit V)
@@ -455,7 +459,8 @@ int gmresdr_run(wd_context *h, const double2 *b, double2 *x, int m, int k, doubl
     RET_IF(launch_ok(launch_fxb_encode(vk, nrm, 0, vk, fb, k, 1, fv, n, nullptr, s), "v_{k+1}"));
     j0 = k;
   }
-  // outputs
+  // outputs; vectors that a lucky breakdown left out are zero
+  if (valid < k) WD_CK(cudaMemsetAsync(V + (size_t)valid * n, 0, sizeof(double2) * (k - valid) * n, s));
   if (V_out && k > 0) WD_CK(cudaMemcpyAsync(V_out, V, sizeof(double2) * k * n, cudaMemcpyDeviceToDevice, s));
   if (Hbar_host && k > 0) WD_CK(cudaMemcpyAsync(Hbar_host, Hk, sizeof(double2) * (k + 1) * k, cudaMemcpyDeviceToHost, s));
   if (theta_host && k > 0) WD_CK(cudaMemcpyAsync(theta_host, theta, sizeof(double2) * k, cudaMemcpyDeviceToHost, s));

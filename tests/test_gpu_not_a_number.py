@@ -1,6 +1,7 @@
 """NaN and infinities that reach the small dense problems: an error or a result,
 never an index out of range.  The LU of the projected matrix (a column of NaN has
-no pivot) and the order of harmonic Ritz values that are NaN."""
+no pivot), the order of harmonic Ritz values that are NaN, and the basis of a
+GMRES-DR solve that ended before it had k vectors."""
 import numpy as np
 import pytest
 
@@ -36,6 +37,26 @@ def test_deflation_space_with_nan_is_singular(wdl, k):
     V[k // 2, 5] = 1.0
     d = op.deflation(cuda(V), k)          # the handle is as good as before
     d.close()
+    op.close()
+
+
+def test_vectors_after_a_lucky_breakdown_are_zero(wdl):
+    """A source in an invariant subspace of two vectors (unit links, momenta 0
+    and (pi, 0, 0, 0)): the basis ends there, the other vectors are zero."""
+    import torch
+    dims = (4, 2, 2, 2)
+    v = L.volume(dims)
+    op = wdl.WilsonOperator(dims, cuda(L.unit_gauge_field(dims)), 0.1)
+    b = np.zeros((v, 4, 3), dtype=np.complex128)
+    b[:, 0, 0] = 1.0
+    b[:, 0, 1] = (-1.0) ** (np.arange(v) % 4)
+    x = cuda(np.zeros(op.n, dtype=np.complex128))
+    V = torch.full((6 * op.n,), float("nan"), dtype=torch.complex128, device="cuda:0")
+    rc, st, hbar, theta = op.gmresdr(cuda(b.ravel()), x, 12, 6, 1e-12, 100, V_out=V)
+    assert rc == 0 and st["mvp"] == 2
+    w = host(V).reshape(6, -1)
+    assert np.all(np.isfinite(w)) and not w[2:].any() and w[:2].any()
+    assert np.all(np.isfinite(hbar)) and np.all(np.isfinite(theta))
     op.close()
 
 
