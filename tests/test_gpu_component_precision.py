@@ -72,7 +72,8 @@ def _hop_abs(U, a, dims):
     return out
 
 
-@pytest.mark.parametrize("dims,nrhs", [((4, 4, 4, 4), 1), ((3, 5, 7, 2), 3), ((8, 4, 4, 8), 12), ((9, 7, 5, 11), 4)])
+@pytest.mark.parametrize("dims,nrhs", [((4, 4, 4, 4), 1), ((3, 5, 7, 2), 3), ((8, 4, 4, 8), 12), ((9, 7, 5, 11), 4),
+                                       ((8, 4, 4, 8), 16), ((9, 7, 5, 11), 7)])   # the batched form
 @pytest.mark.parametrize("kind", ["colours", "point"])
 @pytest.mark.parametrize("dagger,mu", [(False, 0.0), (True, 0.07)])
 def test_product(wdl, dims, nrhs, kind, dagger, mu):
