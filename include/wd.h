@@ -116,7 +116,7 @@ int wd_set_params(wd_handle h, double kappa, double mu);
 /* out = A in (dagger = 0) or A^dagger in (dagger = 1) for nrhs spinors.
  * in, out: device pointers, boundary spinor layout, nrhs*n complex128
  * each, in != out (no aliasing).  Sec. 1.
- * On near-unitary links the hops run in fixed point; above a few thousand
+ * On near-unitary links the hops run in fixed point; above some ten thousand
  * sites x nrhs that takes scratch from the handle's pool (196 bytes a site and
  * vector, kept for the next call), and without it they run in FP64.  On a stream
  * that is being captured no scratch is taken: the graph holds kernels only, and
